@@ -213,8 +213,14 @@ int gep_create(gep_handle_t* out, void* stream) {
   cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev);
   if (cudaMalloc((void**)&h->d_status, 256) != cudaSuccess) { delete h; return GEP_ERR_CUDA; }
   if (cudaMemset(h->d_status, 0, 256) != cudaSuccess) { cudaFree(h->d_status); delete h; return GEP_ERR_CUDA; }
-  h->splitk_bytes = (size_t)32 << 20;
-  if (cudaMalloc((void**)&h->d_splitk, h->splitk_bytes) != cudaSuccess) {
+  if (cudaMalloc((void**)&h->d_splitk, SPLITK_DOUBLES * sizeof(double) + SPLITK_TILES * sizeof(int)) != cudaSuccess) {
+    cudaFree(h->d_status);
+    delete h;
+    return GEP_ERR_CUDA;
+  }
+  h->d_splitk_count = (int*)(h->d_splitk + SPLITK_DOUBLES);
+  if (cudaMemset(h->d_splitk_count, 0, SPLITK_TILES * sizeof(int)) != cudaSuccess) {
+    cudaFree(h->d_splitk);
     cudaFree(h->d_status);
     delete h;
     return GEP_ERR_CUDA;

@@ -15,8 +15,8 @@ struct gep_handle_s {
   size_t ws_bytes = 0;
   char* eng_ws = nullptr;    // scratch of the split-BF16 product engine
   size_t eng_bytes = 0;
-  double* d_splitk = nullptr;  // handle-owned partial sums of split-K FP64 products
-  size_t splitk_bytes = 0;
+  double* d_splitk = nullptr;     // handle-owned partial tiles of FP64 products with a split depth
+  int* d_splitk_count = nullptr;  // arrivals per output tile, zero between products
   long long launches = 0;
   int sm_count = 152;
   // bounded device-side waits: their limit, and a test hook that drops the progress
@@ -114,6 +114,9 @@ inline int check_launch(gep_handle_t h) {
       return GEP_ERR_CUDA;                                                           \
     }                                                                                \
   } while (0)
+
+constexpr int SPLITK_TILES = 2048;          // output tiles of a product with a split depth
+constexpr int SPLITK_DOUBLES = 1 << 18;     // doubles of their partial tiles
 
 // ---- dense contraction engines (gemm_f64.cu, gemm_oz.cu) ----
 // Structure of op(A) a product may exploit: rows [128 r, 128 r + 128) of op(A) are exactly

@@ -272,3 +272,31 @@ def test_solve_edge_sizes(gep, oracle_lib):
         w, Y, info = gep.solve(dev(A), dev(B))
         assert info == 0
         _check_solution(A, B, host(w), host(Y), w_ref)
+
+
+# The FP64 product's tile choice: 16 x 16 tiles with a split depth, 32 x 32 and 64 x 64 tiles, and
+# their ragged edges, each operand form; tolerance: k roundings of the largest product, twice over.
+@pytest.mark.parametrize("m,n,k", [(16, 16, 4096), (17, 15, 33), (64, 64, 63), (65, 130, 1025), (130, 33, 2049),
+                                   (500, 500, 96), (901, 803, 40), (1700, 1601, 20)])
+@pytest.mark.parametrize("ta,tb,uplo", [("N", "N", "F"), ("N", "T", "L"), ("T", "N", "F"), ("T", "T", "F")])
+def test_dgemm_fp64_tile_choices(gep, ta, tb, uplo, m, n, k):
+    rng = np.random.default_rng(m + n + k)
+    n = m if uplo == "L" else n
+    A = rng.standard_normal((k, m) if ta == "T" else (m, k))
+    B = rng.standard_normal((n, k) if tb == "T" else (k, n))
+    C = rng.standard_normal((m, n))
+    ref = 1.5 * (A.T if ta == "T" else A) @ (B.T if tb == "T" else B) + 0.5 * C
+    if uplo == "L":
+        ref = np.tril(ref) + np.triu(C, 1)
+    out = host(gep.dgemm(dev(A), dev(B), ta, tb, alpha=1.5, beta=0.5, C=dev(C), uplo=uplo))
+    tol = 2 * k * EPS * 1.5 * np.max(np.abs(A)) * np.max(np.abs(B)) + 1e-14
+    assert np.max(np.abs(out - ref)) <= tol
+
+
+def test_dgemm_fp64_symmetric_operand_split_depth(gep):
+    rng = np.random.default_rng(5)
+    A = rng.standard_normal((700, 700))
+    S = np.tril(A) + np.tril(A, -1).T
+    B = rng.standard_normal((700, 20))
+    out = host(gep.dgemm(dev(np.tril(A)), dev(B), "S", "N"))
+    assert np.max(np.abs(out - S @ B)) <= 2 * 700 * EPS * np.max(np.abs(A)) * np.max(np.abs(B)) + 1e-14
