@@ -4,11 +4,14 @@
 //                                  "ELPA style" (R = L^-1 formed, then C = R A R^T)
 //   Eq. 6  Y = L^-T Z              blocked back-substitution
 // plus the triangular building blocks they share.  Every nb x nb diagonal block
-// of L is factored and inverted by one CTA in shared memory; everything else is
+// of L is factored and inverted by one cluster of CTAs; everything else is
 // a dense product on the GEMM engine, so the O(M^3) work runs as matrix products.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "gep_internal.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace gep {
 namespace {
@@ -58,66 +61,154 @@ __device__ void store_inv(const double* S, int r, double* out) {
   }
 }
 
-// Factor the diagonal block B(kb:kb+r, kb:kb+r) (already updated by earlier trailing
-// products) and store L_kk in place plus L_kk^-1 into invD.
-__global__ void __launch_bounds__(256) k_potrf_diag(int r, double* B, int ldb, double* invD, int kb,
-                                                    int* st) {
-  extern __shared__ double sm[];
-  double* S = sm;
-  double* tmp = sm + NB * NB;
-  __shared__ int fail;
-  if (status_bad(st)) return;
-  if (threadIdx.x == 0) fail = 0;
-  for (int idx = threadIdx.x; idx < r * r; idx += blockDim.x) {
-    int i = idx % r, j = idx / r;
-    S[i + j * NB] = (i >= j) ? B[GEP_IX(i, j, ldb)] : 0.0;
+// Cholesky factor of the diagonal block B(kb:kb+r, kb:kb+r) (already updated by earlier
+// trailing products) in place, and its inverse L_kk^-1 into invD, by one cluster of 8 CTAs.
+//
+// Symmetric elimination on the augmented matrix [A | I], kept in place: row i holds A's
+// columns c >= j and the growing inverse's columns c < j at step j.  Warp w of rank q owns row
+// q + 8 w (cyclic, so every CTA keeps work to the end), lane l its columns l, l + 32, ... in
+// registers.  Step j: every row i > j takes row_i -= f_i row_j with f_i = M(i, j) / p_j, and
+// column j becomes -f_i; L(i, j) = f_i sqrt(p_j), and row j of the inverse is row_j / sqrt(p_j).
+// The owner of a finished row pushes it, its pivot and 1 / pivot into the shared memory of all
+// 8 CTAs (st.async, one mbarrier per row; every row has its own slot, so nothing is reused and
+// no cluster barrier is needed inside the loop) and is done.
+//
+// Bound: the FP64 pipe (64 clocks a warp instruction) and the chain of 128 pivots.  On one SM
+// the 0.7 M FMAs alone take 200 us; over 8 SMs they hide behind the chain, a step of which is
+// the next row's 4 FMAs, the reciprocal of its pivot and the push.  The other warps of the CTA
+// that owns the next row therefore wait for that row before they spend FP64 issue slots on this
+// one.  A 128 x 128 block takes 123 us
+// (0.95 us a pivot; one CTA working in shared memory took 636 us), a 64 x 64 one 68 us.
+constexpr int PC = 8;            // CTAs of the cluster
+constexpr int PW = NB / PC;      // rows per CTA = warps
+constexpr int PROW = NB + 2;     // a published row: 128 values, 1 / pivot, pivot
+
+struct PotrfShared {
+  double rows[NB][PROW];           // row j at [lane * 4 + u] for column lane + 32 u
+  double f[PW][NB];                // f_i of this CTA's rows
+  double sq[NB], rs[NB];
+  unsigned long long bar[NB];
+};
+
+__device__ __forceinline__ uint32_t cta_shared(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Bounded wait for a published row (about a second); on expiry records the timeout.
+__device__ __forceinline__ bool row_wait(uint32_t bar, int* st) {
+  for (int it = 0; it < (1 << 22); ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok) : "r"(bar) : "memory");
+    if (ok) return true;
+    if ((it & 1023) == 1023 && *(volatile int*)(st + 1) != 0) return false;
   }
-  // right-looking, one column per step; thread t owns row i = t mod 128 of the trailing
-  // triangle, columns of parity t / 128 (no index division, no idle upper half)
-  __shared__ double rinv;
-  const int i = threadIdx.x & (NB - 1), h = threadIdx.x / NB;
-  for (int j = 0; j < r; ++j) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double p = S[j + j * NB];
-      if (!(p > 0.0) || !isfinite(p)) fail = j + 1;
-      else {
-        const double l = sqrt(p);
-        S[j + j * NB] = l;
-        rinv = 1.0 / l;
+  atomicExch(st + 1, GEP_ERR_TIMEOUT);
+  return false;
+}
+
+__global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_diag(int r, double* B, int ldb,
+                                                                                   double* invD, int kb, int* st) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  PotrfShared& sh = *reinterpret_cast<PotrfShared*>(smraw);
+  constexpr int U = NB / 32;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = cl.block_rank(), w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = rank + PC * w;
+  const bool bad = status_bad(st);  // an earlier stage failed: every warp passes through
+  if (threadIdx.x < NB) {
+    const uint32_t bar = cta_shared(&sh.bar[threadIdx.x]);
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(bar),
+                 "r"(PROW * 8) : "memory");
+  }
+  double x[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int c = lane + 32 * u, a = max(i, c), b = min(i, c);
+    x[u] = a < r ? B[GEP_IX(a, b, ldb)] : (i == c ? 1.0 : 0.0);
+  }
+  cl.sync();
+  auto publish = [&](int j, double pivot) {
+    const double ri = 1.0 / pivot;
+    const uint32_t dst = cta_shared(&sh.rows[j][lane * U]), sc = cta_shared(&sh.rows[j][NB]), bar = cta_shared(&sh.bar[j]);
+#pragma unroll
+    for (int q = 0; q < PC; ++q) {
+      uint32_t rd, rb, rsc;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(dst), "r"(q));
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(bar), "r"(q));
+#pragma unroll
+      for (int u = 0; u < U; u += 2)
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(
+                         rd + 8 * u), "l"(__double_as_longlong(x[u])), "l"(__double_as_longlong(x[u + 1])), "r"(rb)
+                     : "memory");
+      if (lane == q) {
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rsc) : "r"(sc), "r"(q));
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(
+                         rsc), "l"(__double_as_longlong(ri)), "l"(__double_as_longlong(pivot)), "r"(rb)
+                     : "memory");
       }
     }
-    __syncthreads();
-    if (fail) break;
-    if (h == 0 && i > j && i < r) S[i + j * NB] *= rinv;
-    __syncthreads();
-    if (i > j && i < r) {
-      const double lij = S[i + j * NB];
-      int c = j + 1;
-      if ((c & 1) != h) ++c;
-      for (; c + 6 <= i; c += 8) {  // four columns at a time: loads issued before the stores
-        const double l0 = S[c + j * NB], l1 = S[c + 2 + j * NB], l2 = S[c + 4 + j * NB], l3 = S[c + 6 + j * NB];
-        double* x = S + i + c * NB;
-        const double x0 = x[0], x1 = x[2 * NB], x2 = x[4 * NB], x3 = x[6 * NB];
-        x[0] = fma(-lij, l0, x0);
-        x[2 * NB] = fma(-lij, l1, x1);
-        x[4 * NB] = fma(-lij, l2, x2);
-        x[6 * NB] = fma(-lij, l3, x3);
+  };
+  int fail = bad ? -1 : 0;
+  if (i == 0 && !fail) publish(0, __shfl_sync(0xffffffffu, x[0], 0));
+  const int last = i < r ? i : 0;  // rows past the block are identity rows: nothing to do
+#pragma unroll
+  for (int ju = 0; ju < U; ++ju) {
+    for (int jl = 0; jl < 32; ++jl) {
+      const int j = 32 * ju + jl;
+      if (j >= last || fail) break;
+      bool ok = true;
+      if (rank == (j + 1) % PC && i != j + 1) ok = row_wait(cta_shared(&sh.bar[j + 1]), st);
+      if (ok) ok = row_wait(cta_shared(&sh.bar[j]), st);
+      if (!ok) { fail = -1; break; }
+      const double ri = sh.rows[j][NB];  // a bad pivot is found at the end: the rows keep coming
+      const double f = __shfl_sync(0xffffffffu, x[ju], jl) * ri;
+#pragma unroll
+      for (int u = 0; u < U; ++u) x[u] = fma(-f, sh.rows[j][lane * U + u], x[u]);
+      if (lane == jl) x[ju] = -f;
+      if (lane == 0) sh.f[w][j] = f;
+      if (i == j + 1) {
+        double piv = 0.0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+          if (u == (i >> 5)) piv = __shfl_sync(0xffffffffu, x[u], i & 31);
+        publish(i, piv);
       }
-      for (; c <= i; c += 2) S[i + c * NB] = fma(-lij, S[c + j * NB], S[i + c * NB]);
+    }
+  }
+  cl.sync();  // every row that is to come has been pushed, and no CTA has left
+  if (bad) return;
+  // the pivots; the first that is not positive is the leading minor reported
+  __shared__ int first_bad;
+  if (threadIdx.x == 0) first_bad = NB;
+  __syncthreads();
+  if (threadIdx.x < NB) {
+    sh.rs[threadIdx.x] = sh.sq[threadIdx.x] = 1.0;
+    if (threadIdx.x < r) {
+      // (also: no CTA leaves before every push into its shared memory has landed)
+      const double p = row_wait(cta_shared(&sh.bar[threadIdx.x]), st) ? sh.rows[threadIdx.x][NB + 1] : 0.0;
+      if (!(p > 0.0) || !isfinite(p)) {
+        atomicMin(&first_bad, (int)threadIdx.x);
+      } else {
+        const double l = sqrt(p);
+        sh.sq[threadIdx.x] = l;
+        sh.rs[threadIdx.x] = 1.0 / l;
+      }
     }
   }
   __syncthreads();
-  if (fail) {
-    if (threadIdx.x == 0) atomicCAS(st, 0, kb + fail);
+  if (first_bad < NB) {
+    if (rank == 0 && threadIdx.x == 0) atomicCAS(st, 0, kb + first_bad + 1);
     return;
   }
-  for (int idx = threadIdx.x; idx < r * r; idx += blockDim.x) {
-    int i = idx % r, j = idx / r;
-    if (i >= j) B[GEP_IX(i, j, ldb)] = S[i + j * NB];
+  const double ri = sh.rs[i];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int c = lane + 32 * u;
+    if (i < r && c <= i) B[GEP_IX(i, c, ldb)] = c == i ? sh.sq[i] : sh.f[w][c] * sh.sq[c];
+    invD[i + c * NB] = c < i ? x[u] * ri : (c == i ? ri : 0.0);
   }
-  tri_inv_smem(S, tmp, r);
-  store_inv(S, r, invD);
 }
 
 // One CTA per diagonal block of an existing lower triangular L: invert it.
@@ -142,7 +233,7 @@ constexpr size_t kSmemDiag = (size_t)NB * NB * sizeof(double) + NB * sizeof(doub
 int set_smem_attr() {
   static unsigned long long devices = 0;
   if (first_use_on_device(devices)) {
-    cudaFuncSetAttribute(k_potrf_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDiag);
+    cudaFuncSetAttribute(k_potrf_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PotrfShared));
     cudaFuncSetAttribute(k_inv_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDiag);
   }
   return GEP_OK;
@@ -218,7 +309,7 @@ int rlt_rec(gep_handle_t h, int o, int n, int m, const double* L, int ldl, const
 // Eq. 4 on the diagonal block (o, o) of order n; B points at the full matrix.
 int potrf_rec(gep_handle_t h, int o, int n, double* B, int ldb, double* invD, double* tmp, int engine) {
   if (n <= NB) {
-    k_potrf_diag<<<1, 256, kSmemDiag, h->stream>>>(n, B + GEP_IX(o, o, ldb), ldb, invD + (size_t)(o / NB) * NB * NB, o,
+    k_potrf_diag<<<PC, 32 * PW, sizeof(PotrfShared), h->stream>>>(n, B + GEP_IX(o, o, ldb), ldb, invD + (size_t)(o / NB) * NB * NB, o,
                                                    h->d_status);
     return check_launch(h);
   }
