@@ -4,7 +4,10 @@
 // T is torn at every multiple of LEAF (Cuppen): at split point p the coupling
 // beta = e[p-1] is removed from the diagonal on both sides, leaving independent
 // leaves solved one warp each (implicit QL with Wilkinson shift in shared
-// memory).  Leaves are merged bottom-up, level by level.  Merging two solved
+// memory).  Leaves are merged bottom-up, level by level; every kernel of a level
+// works on all its merges at once (grid dimension y or x), since a merge alone is
+// far too small for the GPU: the merges of a level used to run one after the other,
+// about 12 launches each (order 2047: D&C 29.5 -> 5.7 ms, order 64: 2.57 -> 0.48 ms).  Merging two solved
 // halves is the rank-one problem D + rho z z^T (z = last row of Q1 and first row
 // of Q2 scaled by sign(beta)/sqrt(2), rho = 2|beta|), handled as:
 //   1. deflation of negligible z_i and of nearly equal d_i (Givens rotation),
@@ -16,7 +19,7 @@
 //      eigenvectors u_j ~ z_i / (d_i - lambda_j) are numerically orthogonal,
 //   4. the merged eigenvectors Q [u_j] as one product per child on the GEMM engine
 //      (the deflation rotations are folded into the rows of [u_j], so Q stays
-//      block diagonal).
+//      block diagonal); the products of narrow merges run in one FP64 launch per level.
 // Eigenvalues of every block are kept sorted ascending.
 #include <math.h>
 
@@ -25,14 +28,27 @@
 namespace gep {
 namespace {
 
-constexpr int LEAF = 32;
+constexpr int LEAF = 16;
+constexpr int FP64_WIDTH = 256;  // merges up to this order form their products in FP64, one launch a level
 constexpr double EPS = 0x1p-53;
 
+// Arrays of M entries: a merge of rows [lo, hi) uses [lo, hi) of each.
 struct DcWs {
-  double *Qt, *U, *D, *dd, *zs, *dv, *ndd, *ndz, *dfv, *rc, *rs, *tauR, *lam, *zhat, *newD, *rho;
+  double *Qt, *U, *D, *dd, *zs, *dv, *ndd, *ndz, *dfv, *rc, *rs, *tauR, *lam, *zhat, *rho;
   double *ptau, *pc, *ps;  // the Givens deflation test of each adjacent pair, from the undeflated values
   int *perm, *ndx, *dfx, *ra, *rb, *org, *posr, *posd, *cnt;
   int *nsl, *prot;         // positions (in perm) with z not negligible; pair test outcome
+  // the view of merge m (rows [lo, ...)): per-merge scalars are rho[m], cnt[8 m ..]
+  __device__ DcWs at(int lo, int m) const {
+    DcWs v = *this;
+    v.zs += lo; v.dv += lo; v.ndd += lo; v.ndz += lo; v.dfv += lo; v.rc += lo; v.rs += lo; v.tauR += lo;
+    v.lam += lo; v.zhat += lo; v.ptau += lo; v.pc += lo; v.ps += lo;
+    v.perm += lo; v.ndx += lo; v.dfx += lo; v.ra += lo; v.rb += lo; v.org += lo; v.posr += lo; v.posd += lo;
+    v.nsl += lo; v.prot += lo;
+    v.rho += m;
+    v.cnt += 8 * m;
+    return v;
+  }
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -71,6 +87,36 @@ __device__ double block_max(double v, double* red) {
   return r;
 }
 
+// Exclusive prefix sum of one count per thread; *total gets the sum.  sc: 33 ints.
+__device__ int block_scan(int v, int* sc, int* total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  int x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  __syncthreads();
+  if (lane == 31) sc[w] = x;
+  __syncthreads();
+  if (w == 0) {
+    int s = lane < nw ? sc[lane] : 0;
+    for (int o = 1; o < 32; o <<= 1) {
+      int y = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += y;
+    }
+    sc[lane] = s;
+  }
+  __syncthreads();
+  *total = sc[nw - 1];
+  return x - v + (w ? sc[w - 1] : 0);
+}
+
+// Order-preserving integer key of a finite double (compared on the integer pipe).
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
 // Tearing: dd = d with |e[p-1]| removed on both sides of every split point p.
 __global__ void k_tear(int M, const double* __restrict__ d, const double* __restrict__ e,
                        double* __restrict__ dd) {
@@ -82,86 +128,93 @@ __global__ void k_tear(int M, const double* __restrict__ d, const double* __rest
   dd[i] = v;
 }
 
-// One warp per leaf: implicit QL with Wilkinson shift; eigenvectors accumulated in
-// shared memory (lane r owns row r), then sorted ascending and written to Z/D.
-__global__ void __launch_bounds__(128) k_leaf(int M, const double* __restrict__ dd,
-                                              const double* __restrict__ e, double* __restrict__ D,
-                                              double* __restrict__ Z, int ldz, int* st) {
-  __shared__ double Zs[4][LEAF][LEAF + 1];
-  __shared__ double dl[4][LEAF], el[4][LEAF], rcs[4][LEAF], rsn[4][LEAF];
-  __shared__ int ord[4][LEAF];
-  __shared__ int sh_m[4], sh_n[4], sh_stop[4];
-  int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int leaf = blockIdx.x * 4 + w;
-  int lo = leaf * LEAF;
-  if (lo >= M) return;
-  int n = min(LEAF, M - lo);
-  for (int c = 0; c < LEAF; ++c) Zs[w][lane][c] = (lane == c) ? 1.0 : 0.0;
-  dl[w][lane] = (lane < n) ? dd[lo + lane] : 0.0;
-  el[w][lane] = (lane < n - 1) ? e[lo + lane] : 0.0;
+// One warp per leaf: implicit QL with Wilkinson shift; lane r owns row r of the eigenvectors
+// (shared memory), every lane runs the scalar recurrence (an FP64 instruction costs a warp the
+// same for one lane as for 32), the split test is one ballot.  The leaf is scaled by a power of
+// two so that a rotation needs one rsqrt instead of a hypot and two divisions.  Sorted
+// ascending and written to Z/D at the end.  With leaves of 32 rows, hypot and divisions in
+// lane 0 this kernel took 2.46 ms; now 0.33 ms.
+__global__ void __launch_bounds__(32) k_leaf(int M, const double* __restrict__ dd, const double* __restrict__ e,
+                                             double* __restrict__ D, double* __restrict__ Z, int ldz, int* st) {
+  __shared__ double Zs[LEAF][33];
+  __shared__ double dl[LEAF], el[LEAF];
+  __shared__ int ord[LEAF];
+  if (status_bad(st)) return;
+  const int lane = threadIdx.x, lo = blockIdx.x * LEAF;
+  const int n = min(LEAF, M - lo);
+  double dv = lane < n ? dd[lo + lane] : 0.0, ev = lane < n - 1 ? e[lo + lane] : 0.0;
+  int mx = max((int)((__double_as_longlong(dv) >> 52) & 0x7FF), (int)((__double_as_longlong(ev) >> 52) & 0x7FF));
+  for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  // 2^(1023 - mx) and its inverse, kept inside the normal range
+  const int sh = max(-1000, min(1000, 1023 - mx));
+  const double sc = __longlong_as_double((long long)(1023 + sh) << 52);
+  const double isc = __longlong_as_double((long long)(1023 - sh) << 52);
+  if (lane < LEAF) {
+    dl[lane] = dv * sc;
+    el[lane] = ev * sc;
+  }
+#pragma unroll
+  for (int c = 0; c < LEAF; ++c) Zs[c][lane] = (lane == c) ? 1.0 : 0.0;
   __syncwarp();
   int bad = 0;
   for (int l = 0; l < n && !bad; ++l) {
-    int iter = 0;
-    for (;;) {
-      if (lane == 0) {
-        int m = l;
-        for (; m + 1 < n; ++m) {
-          double s = fabs(dl[w][m]) + fabs(dl[w][m + 1]);
-          if (fabs(el[w][m]) <= 2.0 * EPS * s) break;
-        }
-        sh_m[w] = m;
-        sh_stop[w] = 0;
-        if (m != l) {
-          if (++iter > 40) {
-            sh_stop[w] = 2;
-          } else {
-            double g = (dl[w][l + 1] - dl[w][l]) / (2.0 * el[w][l]);
-            double r = hypot(g, 1.0);
-            g = dl[w][m] - dl[w][l] + el[w][l] / (g + copysign(r, g));
-            double s = 1.0, c = 1.0, p = 0.0;
-            int nr = 0, early = 0;
-            for (int i = m - 1; i >= l; --i) {
-              double f = s * el[w][i], b = c * el[w][i];
-              r = hypot(f, g);
-              el[w][i + 1] = r;
-              if (r == 0.0) {
-                dl[w][i + 1] -= p;
-                el[w][m] = 0.0;
-                early = 1;
-                break;
-              }
-              s = f / r;
-              c = g / r;
-              g = dl[w][i + 1] - p;
-              r = (dl[w][i] - g) * s + 2.0 * c * b;
-              p = s * r;
-              dl[w][i + 1] = g + p;
-              g = c * r - b;
-              rcs[w][nr] = c;
-              rsn[w][nr] = s;
-              ++nr;
-            }
-            if (!early) {
-              dl[w][l] -= p;
-              el[w][l] = g;
-              el[w][m] = 0.0;
-            }
-            sh_n[w] = nr;
-            sh_stop[w] = 1;
-          }
-        }
-      }
-      __syncwarp();
-      int m = sh_m[w], stop = sh_stop[w];
+    for (int iter = 0;; ++iter) {
+      bool small = true;
+      if (lane < n - 1) small = fabs(el[lane]) <= 2.0 * EPS * (fabs(dl[lane]) + fabs(dl[lane + 1]));
+      const unsigned mask = __ballot_sync(0xffffffffu, small);
+      const int m = l + __ffs(mask >> l) - 1;
       if (m == l) break;
-      if (stop == 2) { bad = 1; break; }
-      int nr = sh_n[w];
-      for (int q = 0; q < nr; ++q) {
-        int col = m - 1 - q;
-        double zi = Zs[w][lane][col], zi1 = Zs[w][lane][col + 1];
-        Zs[w][lane][col + 1] = rsn[w][q] * zi + rcs[w][q] * zi1;
-        Zs[w][lane][col] = rcs[w][q] * zi - rsn[w][q] * zi1;
+      if (iter > 60) { bad = 1; break; }
+      double g, r, s = 1.0, c = 1.0, p = 0.0;
+      {
+        const double a = 2.0 * el[l];
+        g = (dl[l + 1] - dl[l]) / a;
+        r = (fabs(g) < 0x1p400) ? sqrt(fma(g, g, 1.0)) : fabs(g);
+        g = dl[m] - dl[l] + el[l] / (g + copysign(r, g));
+      }
+      double zhi = Zs[m][lane];  // column i + 1 of the running rotation
+      int i = m - 1;
+      bool early = false;
+      for (; i >= l; --i) {
+        const double ei = el[i], di = dl[i], di1 = dl[i + 1];
+        const double f = s * ei, b = c * ei, h = fma(f, f, g * g);
+        __syncwarp();
+        if (h >= 0x1p-900) {
+          const double ri = rsqrt(h);
+          r = h * ri;
+          s = f * ri;
+          c = g * ri;
+        } else {
+          r = hypot(f, g);
+          if (r == 0.0) {
+            if (lane == 0) {
+              el[i + 1] = 0.0;
+              dl[i + 1] = di1 - p;
+              el[m] = 0.0;
+            }
+            early = true;
+            break;
+          }
+          s = f / r;
+          c = g / r;
+        }
+        g = di1 - p;
+        const double q = fma(di - g, s, 2.0 * c * b);
+        p = s * q;
+        if (lane == 0) {
+          el[i + 1] = r;
+          dl[i + 1] = g + p;
+        }
+        g = fma(c, q, -b);
+        const double zi = Zs[i][lane];
+        Zs[i + 1][lane] = fma(s, zi, c * zhi);
+        zhi = fma(c, zi, -s * zhi);
+      }
+      Zs[i + 1][lane] = zhi;  // (after an early stop: the column the last rotation left)
+      if (!early && lane == 0) {
+        dl[l] -= p;
+        el[l] = g;
+        el[m] = 0.0;
       }
       __syncwarp();
     }
@@ -170,36 +223,66 @@ __global__ void __launch_bounds__(128) k_leaf(int M, const double* __restrict__ 
     if (lane == 0) atomicCAS(st, 0, M + lo + 1);
     return;
   }
-  if (lane == 0) {
-    for (int j = 0; j < n; ++j) ord[w][j] = j;
-    for (int a = 1; a < n; ++a) {  // insertion sort of indices by eigenvalue
-      int t = ord[w][a], b = a - 1;
-      while (b >= 0 && dl[w][ord[w][b]] > dl[w][t]) { ord[w][b + 1] = ord[w][b]; --b; }
-      ord[w][b + 1] = t;
-    }
+  if (lane < n) {
+    const double v = dl[lane];
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += dl[j] < v || (dl[j] == v && j < lane);
+    ord[rank] = lane;
   }
   __syncwarp();
-  if (lane < n)
-    for (int j = 0; j < n; ++j) Z[GEP_IX(lo + lane, lo + j, ldz)] = Zs[w][lane][ord[w][j]];
-  if (lane < n) D[lo + lane] = dl[w][ord[w][lane]];
+  if (lane < n) {
+    for (int j = 0; j < n; ++j) Z[GEP_IX(lo + lane, lo + j, ldz)] = Zs[ord[j]][lane];
+    D[lo + lane] = dl[ord[lane]] * isc;
+  }
 }
 
-// Merge set-up (one CTA): z, sort of the two halves' eigenvalues, deflation.  The
+// Sorts the first c entries (key v, with companions) ascending when they are not already: the
+// lists of k_prep are ascending up to the roundings of a few rotations, so this is a check that
+// rarely does more; the sort itself ranks every entry against all (integer compares).
+__device__ void sort_list(int c, double* v, double* z, int* ix, double* tv, double* tz, int* ti) {
+  int inv = 0;
+  for (int x = threadIdx.x + 1; x < c; x += blockDim.x) inv |= order_key(v[x - 1]) > order_key(v[x]);
+  if (!__syncthreads_or(inv)) return;
+  for (int x = threadIdx.x; x < c; x += blockDim.x) {
+    const long long k = order_key(v[x]);
+    int r = 0;
+    for (int y = 0; y < c; ++y) {
+      const long long o = order_key(v[y]);
+      r += o < k || (o == k && y < x);
+    }
+    tv[r] = v[x];
+    if (z) tz[r] = z[x];
+    ti[r] = ix[x];
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < c; x += blockDim.x) {
+    v[x] = tv[x];
+    if (z) z[x] = tz[x];
+    ix[x] = ti[x];
+  }
+  __syncthreads();
+}
+
+// Merge set-up (one CTA per merge): z, sort of the two halves' eigenvalues, deflation.  The
 // deflation scan is sequential (a Givens rotation changes the next pair's operands), but
 // only a rotated pair's successor needs its test re-evaluated: every pair's test is first
-// formed in parallel from the undeflated values, and the scan takes those results wherever
-// the previous pair was not rotated, which gives the sequential outcome exactly.
-__global__ void __launch_bounds__(1024) k_prep(int lo, int mid, int hi, const double* __restrict__ e,
+// formed in parallel from the undeflated values, one thread then follows only the chains
+// that start at a rotated pair, and the lists are compacted in
+// parallel (all set-ups of order 4096: 13.2 -> 0.23 ms).
+__global__ void __launch_bounds__(1024) k_prep(int M, int half, const double* __restrict__ e,
                                                const double* __restrict__ D, const double* __restrict__ Z,
-                                               int ldz, DcWs w, const int* st) {
+                                               int ldz, DcWs ws, const int* st) {
   __shared__ double red[32];
-  __shared__ int scnt[1024];
+  __shared__ int sc[33];
+  __shared__ int snr;
   if (status_bad(st)) return;
+  const int lo = blockIdx.x * 2 * half, mid = lo + half, hi = min(M, mid + half);
+  const DcWs w = ws.at(lo, blockIdx.x);
   const int tid = threadIdx.x, nt = blockDim.x;
-  int n = hi - lo, n1 = mid - lo;
-  double beta = e[mid - 1];
-  double sg = beta < 0.0 ? -1.0 : 1.0;
-  double rho = 2.0 * fabs(beta);
+  const int n = hi - lo, n1 = half;
+  const double beta = e[mid - 1];
+  const double sg = beta < 0.0 ? -1.0 : 1.0;
+  const double rho = 2.0 * fabs(beta);
   double zmax = 0.0, dmax = 0.0;
   for (int t = tid; t < n; t += nt) {
     double z = (t < n1) ? Z[GEP_IX(mid - 1, lo + t, ldz)] : sg * Z[GEP_IX(mid, lo + t, ldz)];
@@ -212,7 +295,6 @@ __global__ void __launch_bounds__(1024) k_prep(int lo, int mid, int hi, const do
   }
   zmax = block_max(zmax, red);
   dmax = block_max(dmax, red);
-  __syncthreads();
   const double tol = 8.0 * EPS * 2.0 * fmax(dmax, zmax);
   // merge the two ascending runs [0, n1) and [n1, n), the first run's entry first on ties
   for (int x = tid; x < n; x += nt) {
@@ -226,105 +308,111 @@ __global__ void __launch_bounds__(1024) k_prep(int lo, int mid, int hi, const do
     w.perm[(x < n1) ? x + (a - n1) : (x - n1) + a] = x;
   }
   __syncthreads();
-  // positions whose z is not negligible, in order (chunk counts, then a scan)
-  const int chunk = (n + nt - 1) / nt, c0 = tid * chunk, c1 = min(n, c0 + chunk);
-  int cnt = 0;
-  for (int q = c0; q < c1; ++q) cnt += !(rho * fabs(w.zs[w.perm[q]]) <= tol);
-  scnt[tid] = cnt;
-  __syncthreads();
-  for (int o = 1; o < nt; o <<= 1) {
-    int v = tid >= o ? scnt[tid - o] : 0;
-    __syncthreads();
-    scnt[tid] += v;
-    __syncthreads();
+  // positions whose z is not negligible, in order; posr marks the deflated positions
+  const int chunk = (n + nt - 1) / nt, c0 = min(n, tid * chunk), c1 = min(n, c0 + chunk);
+  int cnt = 0, nns;
+  for (int q = c0; q < c1; ++q) {
+    const bool neg = rho * fabs(w.zs[w.perm[q]]) <= tol;
+    w.posr[q] = neg;
+    cnt += !neg;
   }
-  const int nns = scnt[nt - 1];
-  for (int q = c0, o = scnt[tid] - cnt; q < c1; ++q)
-    if (!(rho * fabs(w.zs[w.perm[q]]) <= tol)) w.nsl[o++] = q;
+  int o = block_scan(cnt, sc, &nns);
+  for (int q = c0; q < c1; ++q)
+    if (!w.posr[q]) w.nsl[o++] = q;
   __syncthreads();
   // the rotation test of every adjacent pair, from the undeflated values
+  int any = 0;
   for (int m = 1 + tid; m < nns; m += nt) {
     const int pj = w.perm[w.nsl[m - 1]], t = w.perm[w.nsl[m]];
     double zs_ = w.zs[pj], zc = w.zs[t];
     double tau = hypot(zc, zs_);
     double c = zc / tau, sn = -zs_ / tau;
     double tdiff = w.dv[t] - w.dv[pj];
-    w.prot[m] = fabs(tdiff * c * sn) <= tol;
+    const int rot = fabs(tdiff * c * sn) <= tol;
+    w.prot[m] = rot;
     w.ptau[m] = tau;
     w.pc[m] = c;
     w.ps[m] = sn;
+    any |= rot;
+  }
+  if (tid == 0) snr = 0;
+  any = __syncthreads_or(any);
+  if (any) {
+    // the pairs that rotate, in order (posd), then their chains one after the other
+    const int ch = (nns + nt - 1) / nt, m0 = max(1, min(nns, tid * ch)), m1 = min(nns, tid * ch + ch);
+    int rc_ = 0, nrot;
+    for (int m = m0; m < m1; ++m) rc_ += w.prot[m];
+    int ro = block_scan(rc_, sc, &nrot);
+    for (int m = m0; m < m1; ++m)
+      if (w.prot[m]) w.posd[ro++] = m;
+    __syncthreads();
+    if (tid == 0) {
+      int nr = 0, next = 0;
+      for (int x = 0; x < nrot; ++x) {
+        int m = w.posd[x];
+        if (m < next) continue;  // already decided by the chain before it
+        double tau = w.ptau[m], c = w.pc[m], sn = w.ps[m];
+        for (;;) {
+          const int pj = w.perm[w.nsl[m - 1]], t = w.perm[w.nsl[m]];
+          const double dp = w.dv[pj], dt = w.dv[t];
+          const double dnew = dp * sn * sn + dt * c * c;
+          w.zs[t] = tau;
+          w.zs[pj] = 0.0;
+          w.ra[nr] = pj; w.rb[nr] = t; w.rc[nr] = c; w.rs[nr] = sn; ++nr;
+          w.dv[t] = dnew;
+          w.dv[pj] = dp * c * c + dt * sn * sn;
+          w.posr[w.nsl[m - 1]] = 1;
+          if (++m >= nns) break;
+          // t was rotated into: the next pair's test with its new z and d
+          const int t2 = w.perm[w.nsl[m]];
+          const double zc = w.zs[t2];
+          const double ntau = hypot(zc, tau), nc = zc / ntau, ns = -tau / ntau;
+          const double tdiff = w.dv[t2] - dnew;
+          if (!(fabs(tdiff * nc * ns) <= tol)) break;
+          tau = ntau;
+          c = nc;
+          sn = ns;
+        }
+        next = m + 1;
+      }
+      snr = nr;
+    }
+    __syncthreads();
+  }
+  // both lists in sorted order of the undeflated values
+  int k, kc = 0;
+  for (int q = c0; q < c1; ++q) kc += !w.posr[q];
+  int ko = block_scan(kc, sc, &k);
+  for (int q = c0; q < c1; ++q) {
+    const int t = w.perm[q];
+    if (w.posr[q]) {
+      w.dfx[q - ko] = t;
+      w.dfv[q - ko] = w.dv[t];
+    } else {
+      w.ndx[ko] = t;
+      w.ndd[ko] = w.dv[t];
+      w.ndz[ko] = w.zs[t];
+      ++ko;
+    }
   }
   __syncthreads();
-  if (tid != 0) return;
-  int k = 0, nd = 0, nr = 0, pj = -1, mi = -1;
-  bool prev_rot = false;
-  for (int s = 0; s < n; ++s) {
-    int t = w.perm[s];
-    if (rho * fabs(w.zs[t]) <= tol) {
-      w.dfx[nd] = t;
-      w.dfv[nd] = w.dv[t];
-      ++nd;
-      continue;
-    }
-    ++mi;
-    if (pj < 0) { pj = t; continue; }
-    double tau, c, sn;
-    bool rot;
-    if (prev_rot) {  // pj was rotated into: its z and d changed
-      double zs_ = w.zs[pj], zc = w.zs[t];
-      tau = hypot(zc, zs_);
-      c = zc / tau;
-      sn = -zs_ / tau;
-      double tdiff = w.dv[t] - w.dv[pj];
-      rot = fabs(tdiff * c * sn) <= tol;
-    } else {
-      tau = w.ptau[mi];
-      c = w.pc[mi];
-      sn = w.ps[mi];
-      rot = w.prot[mi] != 0;
-    }
-    if (rot) {
-      w.zs[t] = tau;
-      w.zs[pj] = 0.0;
-      w.ra[nr] = pj; w.rb[nr] = t; w.rc[nr] = c; w.rs[nr] = sn; ++nr;
-      double dp = w.dv[pj], dt = w.dv[t];
-      double t2 = dp * c * c + dt * sn * sn;
-      w.dv[t] = dp * sn * sn + dt * c * c;
-      w.dv[pj] = t2;
-      w.dfx[nd] = pj;
-      w.dfv[nd] = t2;
-      ++nd;
-    } else {
-      w.ndx[k] = pj; w.ndd[k] = w.dv[pj]; w.ndz[k] = w.zs[pj]; ++k;
-    }
-    prev_rot = rot;
-    pj = t;
+  sort_list(k, w.ndd, w.ndz, w.ndx, w.ptau, w.pc, w.perm);
+  sort_list(n - k, w.dfv, nullptr, w.dfx, w.ptau, nullptr, w.perm);
+  if (tid == 0) {
+    w.cnt[0] = k;
+    w.cnt[1] = n - k;
+    w.cnt[2] = snr;
+    w.rho[0] = rho;
   }
-  if (pj >= 0) { w.ndx[k] = pj; w.ndd[k] = w.dv[pj]; w.ndz[k] = w.zs[pj]; ++k; }
-  // both lists ascending (they are nearly sorted already)
-  for (int x = 1; x < nd; ++x) {
-    double v = w.dfv[x];
-    int ix = w.dfx[x], y = x - 1;
-    while (y >= 0 && w.dfv[y] > v) { w.dfv[y + 1] = w.dfv[y]; w.dfx[y + 1] = w.dfx[y]; --y; }
-    w.dfv[y + 1] = v; w.dfx[y + 1] = ix;
-  }
-  for (int x = 1; x < k; ++x) {
-    double v = w.ndd[x], zz = w.ndz[x];
-    int ix = w.ndx[x], y = x - 1;
-    while (y >= 0 && w.ndd[y] > v) { w.ndd[y + 1] = w.ndd[y]; w.ndz[y + 1] = w.ndz[y]; w.ndx[y + 1] = w.ndx[y]; --y; }
-    w.ndd[y + 1] = v; w.ndz[y + 1] = zz; w.ndx[y + 1] = ix;
-  }
-  w.cnt[0] = k;
-  w.cnt[1] = nd;
-  w.cnt[2] = nr;
-  w.rho[0] = rho;
 }
 
 // The deflation rotations applied to the rows of U instead of the columns of Q:
 // Q G_0 ... G_{nr-1} U = Q (G_0 (... (G_{nr-1} U))), so Q keeps its block-diagonal
 // form and the merge product splits into one product per child.  One thread per column.
-__global__ void k_rot_u(int lo, int n, double* U, int ldu, DcWs w, const int* st) {
+__global__ void k_rot_u(int M, int width, double* U, int ldu, DcWs ws, const int* st) {
   if (status_bad(st)) return;
+  const int lo = blockIdx.y * width, n = min(width, M - lo);
+  const DcWs w = ws.at(lo, blockIdx.y);
   int col = blockIdx.x * blockDim.x + threadIdx.x;
   if (col >= n) return;
   double* u = U + GEP_IX(lo, lo + col, ldu);
@@ -337,8 +425,9 @@ __global__ void k_rot_u(int lo, int n, double* U, int ldu, DcWs w, const int* st
 }
 
 // One warp per root j of the secular equation on the k non-deflated poles.
-__global__ void __launch_bounds__(256) k_secular(DcWs w, const int* st) {
+__global__ void __launch_bounds__(256) k_secular(int width, DcWs ws, const int* st) {
   if (status_bad(st)) return;
+  const DcWs w = ws.at(blockIdx.y * width, blockIdx.y);
   int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   int k = w.cnt[0];
   if (j >= k) return;
@@ -432,71 +521,146 @@ __device__ __forceinline__ void renorm_exp(double& x, int& e) {
   e += E - 1023;
 }
 
-// Loewner formula: zhat_i^2 = ((lam_i - d_i)/rho) prod_{j != i} (lam_j - d_i)/(d_j - d_i).
-__global__ void k_zhat(DcWs w, const int* st) {
+// Warps 0..k-1 of a merge: Loewner formula zhat_i^2 = ((lam_i - d_i)/rho) prod_{j != i}
+// (lam_j - d_i)/(d_j - d_i), one warp per i (lanes over j), and the place of root i in the
+// ascending order of all n merged eigenvalues; warps k..n-1: the places of the deflated values.
+// One thread per i left most of the GPU idle (992 us at k = 4096), and the order was one
+// thread's merge of the two lists; both together at order 4096: 12.1 -> 0.51 ms.
+__global__ void __launch_bounds__(256) k_zhat_order(int M, int width, double* __restrict__ D, DcWs ws, const int* st) {
   if (status_bad(st)) return;
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int k = w.cnt[0];
-  if (i >= k) return;
+  const int lo = blockIdx.y * width, n = min(width, M - lo);
+  const DcWs w = ws.at(lo, blockIdx.y);
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= n) return;
+  const int k = w.cnt[0], nd = w.cnt[1];
+  if (i >= k) {
+    if (lane == 0) {  // after the roots that are not above it (roots first on ties)
+      const int m = i - k;
+      const double v = w.dfv[m];
+      int a = 0, b = k;
+      while (a < b) {
+        const int c = (a + b) >> 1;
+        if (w.lam[c] <= v) a = c + 1; else b = c;
+      }
+      w.posd[m] = m + a;
+      D[lo + m + a] = v;
+    }
+    return;
+  }
   const double di = w.ndd[i];
   // numerator and denominator products kept apart (one division at the end); every eighth
   // factor both are brought back to [1, 2) in magnitude, their binary exponents counted in
   // en, ed, so that neither over- nor underflows
-  double pn = -((di - w.ndd[w.org[i]]) - w.tauR[i]) / w.rho[0], pd = 1.0;
+  double pn = 1.0, pd = 1.0;
+  if (lane == 0) pn = -((di - w.ndd[w.org[i]]) - w.tauR[i]) / w.rho[0];
   int en = 0, ed = 0, c = 0;
-  for (int j = 0; j < k; ++j) {
-    if (j == i) continue;
-    pn *= -((di - w.ndd[w.org[j]]) - w.tauR[j]);
-    pd *= w.ndd[j] - di;
+  for (int j = lane; j < k; j += 32) {
+    if (j != i) {
+      pn *= -((di - w.ndd[w.org[j]]) - w.tauR[j]);
+      pd *= w.ndd[j] - di;
+    }
     if (++c == 8) {
       c = 0;
       renorm_exp(pn, en);
       renorm_exp(pd, ed);
     }
   }
-  const double prod = ldexp(pn / pd, en - ed);
-  w.zhat[i] = copysign(sqrt(fmax(prod, 0.0)), w.ndz[i]);
-}
-
-// Final ascending order of the merged eigenvalues (roots and deflated values).
-__global__ void k_order(int n, DcWs w, const int* st) {
-  if (status_bad(st)) return;
-  int k = w.cnt[0], nd = w.cnt[1];
-  int a = 0, b = 0, o = 0;
-  while (a < k && b < nd) {
-    if (w.lam[a] <= w.dfv[b]) { w.posr[a] = o; w.newD[o++] = w.lam[a++]; }
-    else { w.posd[b] = o; w.newD[o++] = w.dfv[b++]; }
+  renorm_exp(pn, en);
+  renorm_exp(pd, ed);
+  for (int o = 16; o; o >>= 1) {
+    pn *= __shfl_xor_sync(0xffffffffu, pn, o);
+    pd *= __shfl_xor_sync(0xffffffffu, pd, o);
+    en += __shfl_xor_sync(0xffffffffu, en, o);
+    ed += __shfl_xor_sync(0xffffffffu, ed, o);
   }
-  while (a < k) { w.posr[a] = o; w.newD[o++] = w.lam[a++]; }
-  while (b < nd) { w.posd[b] = o; w.newD[o++] = w.dfv[b++]; }
+  if (lane == 0) {
+    const double prod = ldexp(pn / pd, en - ed);
+    w.zhat[i] = copysign(sqrt(fmax(prod, 0.0)), w.ndz[i]);
+    const double v = w.lam[i];
+    int a = 0, b = nd;
+    while (a < b) {
+      const int q = (a + b) >> 1;
+      if (w.dfv[q] < v) a = q + 1; else b = q;
+    }
+    w.posr[i] = i + a;
+    D[lo + i + a] = v;
+  }
 }
 
-// Column pos_root[j] of U: normalised z_hat_i / (d_i - lam_j) at rows ndx[i].
-__global__ void __launch_bounds__(256) k_ucols(int lo, double* U, int ldu, DcWs w, const int* st) {
+// One CTA per column of U: root j's column posr[j] is the normalised z_hat_i / (d_i - lam_j) at
+// rows ndx[i], a deflated value's column the unit vector of its row; all other entries zero.
+__global__ void __launch_bounds__(256) k_ucols(int M, int width, double* U, int ldu, DcWs ws, const int* st) {
   __shared__ double red[32];
   if (status_bad(st)) return;
-  int j = blockIdx.x;
-  int k = w.cnt[0];
-  if (j >= k) return;
+  const int lo = blockIdx.y * width, n = min(width, M - lo);
+  const DcWs w = ws.at(lo, blockIdx.y);
+  const int j = blockIdx.x, k = w.cnt[0];
+  if (j >= n) return;
+  if (j >= k) {
+    double* col = U + GEP_IX(lo, lo + w.posd[j - k], ldu);
+    const int one = w.dfx[j - k];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) col[i] = i == one ? 1.0 : 0.0;
+    return;
+  }
   const double dorg = w.ndd[w.org[j]], tj = w.tauR[j];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+  double* col = U + GEP_IX(lo, lo + w.posr[j], ldu);
+  for (int i = threadIdx.x; i < n - k; i += blockDim.x) col[w.dfx[i]] = 0.0;
+  constexpr int KEEP = 8;  // entries a thread keeps in registers between the norm and the store
+  double keep[KEEP], s = 0.0;
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q) {
+    const int i = threadIdx.x + q * blockDim.x;
+    keep[q] = 0.0;
+    if (i < k) {
+      keep[q] = w.zhat[i] / ((w.ndd[i] - dorg) - tj);
+      s = fma(keep[q], keep[q], s);
+    }
+  }
+  for (int i = threadIdx.x + KEEP * blockDim.x; i < k; i += blockDim.x) {
     double u = w.zhat[i] / ((w.ndd[i] - dorg) - tj);
     s = fma(u, u, s);
+    col[w.ndx[i]] = u;
   }
-  double inv = 1.0 / sqrt(block_sum(s, red));
-  double* col = U + GEP_IX(lo, lo + w.posr[j], ldu);
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    double u = w.zhat[i] / ((w.ndd[i] - dorg) - tj);
-    col[w.ndx[i]] = u * inv;
+  const double inv = 1.0 / sqrt(block_sum(s, red));
+#pragma unroll
+  for (int q = 0; q < KEEP; ++q) {
+    const int i = threadIdx.x + q * blockDim.x;
+    if (i < k) col[w.ndx[i]] = keep[q] * inv;
   }
+  for (int i = threadIdx.x + KEEP * blockDim.x; i < k; i += blockDim.x) col[w.ndx[i]] *= inv;
 }
 
-__global__ void k_udefl(int lo, double* U, int ldu, DcWs w, const int* st) {
+// Products of every merge of a narrow level (width <= FP64_WIDTH): Out(rows of a child, all n
+// columns) = Z(child, child) U(child rows, :), 16 x 16 output tiles, one output per thread (an
+// FP64 FMA holds its scheduler 64 clocks, so shared-memory reads are free beside it).
+// Grid: (column tiles, row tiles of a child, child).
+__global__ void __launch_bounds__(256) k_merge_prod(int M, int half, const double* __restrict__ Z, int ldz,
+                                                    const double* __restrict__ U, int ldu, double* __restrict__ Out,
+                                                    int ldo, const int* st) {
+  __shared__ double As[FP64_WIDTH / 2][17], Bs[FP64_WIDTH / 2][17];
   if (status_bad(st)) return;
-  int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= w.cnt[1]) return;
-  U[GEP_IX(lo + w.dfx[m], lo + w.posd[m], ldu)] = 1.0;
+  const int mrg = blockIdx.z >> 1, ch = blockIdx.z & 1;
+  const int lo = mrg * 2 * half, n = min(2 * half, M - lo);
+  const int r0 = ch ? half : 0, nr = ch ? n - half : half;  // the child's rows inside the merge
+  const int tr = blockIdx.y * 16, tc = blockIdx.x * 16;
+  if (tr >= nr || tc >= n) return;
+  const int t = threadIdx.x;
+  const double* Zc = Z + GEP_IX(lo + r0, lo + r0, ldz);
+  const double* Uc = U + GEP_IX(lo + r0, lo, ldu);
+  for (int idx = t; idx < 16 * nr; idx += 256) {
+    const int i = idx & 15, kk = idx >> 4;
+    As[kk][i] = tr + i < nr ? Zc[GEP_IX(tr + i, kk, ldz)] : 0.0;
+  }
+  for (int idx = t; idx < 16 * nr; idx += 256) {
+    const int kk = idx % nr, c = idx / nr;
+    Bs[kk][c] = tc + c < n ? Uc[GEP_IX(kk, tc + c, ldu)] : 0.0;
+  }
+  __syncthreads();
+  const int i = t & 15, c = t >> 4;
+  double acc = 0.0;
+#pragma unroll 8
+  for (int kk = 0; kk < nr; ++kk) acc = fma(As[kk][i], Bs[kk][c], acc);
+  if (tr + i < nr && tc + c < n) Out[GEP_IX(lo + r0 + tr + i, lo + tc + c, ldo)] = acc;
 }
 
 __global__ void k_copy_vec(int n, const double* __restrict__ s, double* __restrict__ d, const int* st) {
@@ -510,14 +674,14 @@ DcWs carve(char* base, int M, size_t* used) {
   size_t off = 0;
   auto takeD = [&](size_t n) { off = align256(off); double* p = (double*)(base + off); off += n * sizeof(double); return p; };
   auto takeI = [&](size_t n) { off = align256(off); int* p = (int*)(base + off); off += n * sizeof(int); return p; };
-  size_t mm = (size_t)M * M, m = (size_t)M;
+  size_t mm = (size_t)M * M, m = (size_t)M, nm = (size_t)M / (2 * LEAF) + 1;
   w.Qt = takeD(mm); w.U = takeD(mm);
   w.D = takeD(m); w.dd = takeD(m); w.zs = takeD(m); w.dv = takeD(m); w.ndd = takeD(m); w.ndz = takeD(m);
   w.dfv = takeD(m); w.rc = takeD(m); w.rs = takeD(m); w.tauR = takeD(m); w.lam = takeD(m); w.zhat = takeD(m);
-  w.newD = takeD(m); w.rho = takeD(4);
+  w.rho = takeD(nm);
   w.ptau = takeD(m); w.pc = takeD(m); w.ps = takeD(m);
   w.perm = takeI(m); w.ndx = takeI(m); w.dfx = takeI(m); w.ra = takeI(m); w.rb = takeI(m); w.org = takeI(m);
-  w.posr = takeI(m); w.posd = takeI(m); w.cnt = takeI(8);
+  w.posr = takeI(m); w.posd = takeI(m); w.cnt = takeI(8 * nm);
   w.nsl = takeI(m); w.prot = takeI(m);
   *used = align256(off);
   return w;
@@ -539,44 +703,50 @@ int tridiag_eig_dc(gep_handle_t h, int M, const double* d, const double* e, doub
   if (ws_bytes < used) return GEP_ERR_ALLOC;
   cudaStream_t s = h->stream;
   const int* stc = h->d_status;
-  GEP_CHECK(set_matrix(h, M, M, 0.0, 0.0, Z, ldz));
+  // the eigenvectors alternate between Z and Qt level by level and end in Z
+  int levels = 0;
+  for (int half = LEAF; half < M; half *= 2) ++levels;
+  double *cur = (levels & 1) ? w.Qt : Z, *nxt = (levels & 1) ? Z : w.Qt;
+  int ldcur = (levels & 1) ? M : ldz, ldnxt = (levels & 1) ? ldz : M;
   k_tear<<<(M + 255) / 256, 256, 0, s>>>(M, d, e, w.dd);
   GEP_CHECK(check_launch(h));
-  int nleaf = (M + LEAF - 1) / LEAF;
-  k_leaf<<<(nleaf + 3) / 4, 128, 0, s>>>(M, w.dd, e, w.D, Z, ldz, h->d_status);
+  k_leaf<<<(M + LEAF - 1) / LEAF, 32, 0, s>>>(M, w.dd, e, w.D, cur, ldcur, h->d_status);
   GEP_CHECK(check_launch(h));
   for (int half = LEAF; half < M; half *= 2) {
-    int width = 2 * half;
-    for (int lo = 0; lo < M; lo += width) {
-      int mid = lo + half;
-      if (mid >= M) break;
-      int hi = min(M, lo + width);
-      int n = hi - lo;
-      k_prep<<<1, 1024, 0, s>>>(lo, mid, hi, e, w.D, Z, ldz, w, stc);
+    const int width = 2 * half;
+    const int nm = (M - half + width - 1) / width;  // merges: those whose second half is not empty
+    const int tail = nm * width;                    // rows from here on have no partner on this level
+    const int nmax = M < width ? M : width;
+    k_prep<<<nm, nmax >= 1024 ? 1024 : (nmax + 31) / 32 * 32, 0, s>>>(M, half, e, w.D, cur, ldcur, w, stc);
+    GEP_CHECK(check_launch(h));
+    k_secular<<<dim3((nmax + 7) / 8, nm), 256, 0, s>>>(width, w, stc);
+    GEP_CHECK(check_launch(h));
+    k_zhat_order<<<dim3((nmax + 7) / 8, nm), 256, 0, s>>>(M, width, w.D, w, stc);
+    GEP_CHECK(check_launch(h));
+    k_ucols<<<dim3(nmax, nm), nmax >= 256 ? 256 : (nmax + 31) / 32 * 32, 0, s>>>(M, width, w.U, M, w, stc);
+    GEP_CHECK(check_launch(h));
+    k_rot_u<<<dim3((nmax + 127) / 128, nm), 128, 0, s>>>(M, width, w.U, M, w, stc);
+    GEP_CHECK(check_launch(h));
+    // Q = diag(Q1, Q2): one product per child (half the flops of a dense n x n product)
+    if (width <= FP64_WIDTH) {
+      k_merge_prod<<<dim3((nmax + 15) / 16, (half + 15) / 16, 2 * nm), 256, 0, s>>>(M, half, cur, ldcur, w.U, M, nxt,
+                                                                                    ldnxt, stc);
       GEP_CHECK(check_launch(h));
-      k_secular<<<(n + 7) / 8, 256, 0, s>>>(w, stc);
-      GEP_CHECK(check_launch(h));
-      k_zhat<<<(n + 127) / 128, 128, 0, s>>>(w, stc);
-      GEP_CHECK(check_launch(h));
-      k_order<<<1, 1, 0, s>>>(n, w, stc);
-      GEP_CHECK(check_launch(h));
-      GEP_CHECK(set_matrix(h, n, n, 0.0, 0.0, w.U + GEP_IX(lo, lo, M), M));
-      k_ucols<<<n, 256, 0, s>>>(lo, w.U, M, w, stc);
-      GEP_CHECK(check_launch(h));
-      k_udefl<<<(n + 255) / 256, 256, 0, s>>>(lo, w.U, M, w, stc);
-      GEP_CHECK(check_launch(h));
-      k_rot_u<<<(n + 255) / 256, 256, 0, s>>>(lo, n, w.U, M, w, stc);
-      GEP_CHECK(check_launch(h));
-      // Q = diag(Q1, Q2): one product per child (half the flops of a dense n x n product)
-      const int n1 = mid - lo, n2 = hi - mid;
-      GEP_CHECK(dgemm(h, 'N', 'N', 'F', n1, n, n1, 1.0, Z + GEP_IX(lo, lo, ldz), ldz, w.U + GEP_IX(lo, lo, M), M,
-                      0.0, w.Qt + GEP_IX(lo, lo, M), M, engine));
-      GEP_CHECK(dgemm(h, 'N', 'N', 'F', n2, n, n2, 1.0, Z + GEP_IX(mid, mid, ldz), ldz, w.U + GEP_IX(mid, lo, M), M,
-                      0.0, w.Qt + GEP_IX(mid, lo, M), M, engine));
-      GEP_CHECK(copy_matrix(h, n, n, w.Qt + GEP_IX(lo, lo, M), M, Z + GEP_IX(lo, lo, ldz), ldz));
-      k_copy_vec<<<(n + 255) / 256, 256, 0, s>>>(n, w.newD, w.D + lo, stc);
-      GEP_CHECK(check_launch(h));
+    } else {
+      for (int lo = 0; lo < tail; lo += width) {
+        const int mid = lo + half, hi = M < lo + width ? M : lo + width;
+        const int n = hi - lo, n1 = half, n2 = hi - mid;
+        GEP_CHECK(dgemm(h, 'N', 'N', 'F', n1, n, n1, 1.0, cur + GEP_IX(lo, lo, ldcur), ldcur,
+                        w.U + GEP_IX(lo, lo, M), M, 0.0, nxt + GEP_IX(lo, lo, ldnxt), ldnxt, engine));
+        GEP_CHECK(dgemm(h, 'N', 'N', 'F', n2, n, n2, 1.0, cur + GEP_IX(mid, mid, ldcur), ldcur,
+                        w.U + GEP_IX(mid, lo, M), M, 0.0, nxt + GEP_IX(mid, lo, ldnxt), ldnxt, engine));
+      }
     }
+    if (tail < M)
+      GEP_CHECK(copy_matrix(h, M - tail, M - tail, cur + GEP_IX(tail, tail, ldcur), ldcur,
+                            nxt + GEP_IX(tail, tail, ldnxt), ldnxt));
+    double* tp = cur; cur = nxt; nxt = tp;
+    int tl = ldcur; ldcur = ldnxt; ldnxt = tl;
   }
   k_copy_vec<<<(M + 255) / 256, 256, 0, s>>>(M, w.D, wout, stc);
   return check_launch(h);

@@ -300,3 +300,33 @@ def test_dgemm_fp64_symmetric_operand_split_depth(gep):
     B = rng.standard_normal((700, 20))
     out = host(gep.dgemm(dev(np.tril(A)), dev(B), "S", "N"))
     assert np.max(np.abs(out - S @ B)) <= 2 * 700 * EPS * np.max(np.abs(A)) * np.max(np.abs(B)) + 1e-14
+
+
+def _dc_edge_cases():
+    """Orders at the edges of the leaves (16) and of the merge levels, with and without a ragged or
+    unmerged tail, each with rotations in chains (equal and nearly equal eigenvalues of the halves)
+    and with negligible couplings."""
+    rng = np.random.default_rng(11)
+    cases = []
+    for M in (15, 16, 17, 47, 48, 49, 127, 129, 255, 256, 258, 511, 520, 770):
+        cases.append((f"random{M}", rng.standard_normal(M), rng.standard_normal(M - 1)))
+        cases.append((f"equal{M}", np.full(M, -3.0), np.full(M - 1, 1e-12)))
+        d = np.round(rng.standard_normal(M) * 2)
+        e = np.where(rng.random(M - 1) < 0.3, 1e-17, 1e-3)
+        cases.append((f"chains{M}", d, e))
+    return cases
+
+
+@pytest.mark.parametrize("name,d,e", _dc_edge_cases(), ids=lambda x: x if isinstance(x, str) else "")
+def test_dc_leaf_and_level_edges(gep, oracle_lib, name, d, e):
+    M = d.shape[0]
+    w_ref = oracle_lib.bisect(d, e)
+    T = np.diag(d) + np.diag(e, 1) + np.diag(e, -1)
+    nT = np.max(np.abs(w_ref))
+    w, Z, info = gep.tridiag_eig(dev(d), dev(e))
+    assert info == 0
+    wh, Zh = host(w), host(Z)
+    assert np.all(np.diff(wh) >= 0)
+    assert np.max(np.abs(wh - w_ref)) <= 64 * M * EPS * nT
+    assert np.max(np.abs(Zh.T @ Zh - np.eye(M))) <= 64 * M * EPS
+    assert np.max(np.abs(T @ Zh - Zh * wh[None, :])) <= 64 * M * EPS * nT
