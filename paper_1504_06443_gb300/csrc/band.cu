@@ -308,7 +308,7 @@ __device__ __forceinline__ int bulge_steps(int M, int b, int s) { return (M - 2 
 struct BulgeArgs {
   int M, b, ldab, Q;  // Q = (M - 2) / b: groups 0..Q of b sweeps
   double* AB;
-  int* prog;          // prog[s] = steps of sweep s completed
+  int* prog;          // prog[s] = steps of sweep s completed (k_bulge_ws: see there)
   double* q2;         // diamond storage (or null)
   int* st;
   unsigned long long wait_ns;  // limit of each progress wait
@@ -375,89 +375,6 @@ __device__ void two_sided(double* D, int len, const double* v, double tau, doubl
   __syncthreads();
 }
 
-// One chasing step k >= 1 of a full block (b = len = BMAX = 64, 256 threads), the same
-// arithmetic as the general step below with a fixed thread map: thread t owns row
-// i = t mod 64 and columns q = t / 64 + 4 r (r < 16) of B and of the diagonal block D.
-// B and the lower triangle of D are fetched in one round of coalesced loads.
-__device__ __forceinline__ void bulge_step_full(const BulgeArgs& a, int stp, int st_k, double* Bm, double* Dm,
-                                                const double* vp, double* vc, double* xv, double* pw, double* red,
-                                                double* hs, double taup) {
-  constexpr int N = BMAX, LD = BMAX + 1, R = N / 4;
-  const int t = threadIdx.x, i = t & (N - 1), part = t >> 6;
-  const int ldab = a.ldab;
-  const double* AB = a.AB;
-#pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const int q = part + 4 * r;
-    Bm[i * LD + q] = __ldcg(AB + (N + i - q) + (size_t)(stp + q) * ldab);
-    if (q <= i) Dm[i * LD + q] = __ldcg(AB + (i - q) + (size_t)(st_k + q) * ldab);
-  }
-  __syncthreads();
-  {  // B <- B H(s, k-1): y = B vp, B -= taup y vp^T (the thread's own row: no barrier between)
-    double y = 0.0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) y += Bm[i * LD + part + 4 * r] * vp[part + 4 * r];
-    red[part * N + i] = y;
-    __syncthreads();
-    const double yi = taup * (red[i] + red[N + i] + red[2 * N + i] + red[3 * N + i]);
-#pragma unroll
-    for (int r = 0; r < R; ++r) Bm[i * LD + part + 4 * r] -= yi * vp[part + 4 * r];
-    if (part == 0) xv[i] = Bm[i * LD];
-  }
-  __syncthreads();
-  house(xv, N, vc, hs, N);
-  const double tk = hs[0];
-  {  // B(:, 1:) <- H B(:, 1:): u = tau B^T v over rows i = part + 4 r
-    const int q = i;
-    double u = 0.0;
-    if (q >= 1)
-#pragma unroll
-      for (int r = 0; r < R; ++r) u += vc[part + 4 * r] * Bm[(part + 4 * r) * LD + q];
-    red[part * N + q] = u;
-    __syncthreads();
-    if (t < N) pw[t] = tk * (red[t] + red[N + t] + red[2 * N + t] + red[3 * N + t]);
-    __syncthreads();
-    const double beta = hs[1];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int qq = part + 4 * r;
-      const double x = (qq == 0) ? (i == 0 ? beta : 0.0) : Bm[i * LD + qq] - vc[i] * pw[qq];
-      a.AB[(N + i - qq) + (size_t)(stp + qq) * ldab] = x;
-    }
-  }
-  {  // D <- H D H on the lower triangle (D read symmetric from its lower half)
-    double y = 0.0;
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int q = part + 4 * r;
-      y += (q <= i ? Dm[i * LD + q] : Dm[q * LD + i]) * vc[q];
-    }
-    red[part * N + i] = y;
-    __syncthreads();
-    if (t < N) pw[t] = tk * (red[t] + red[N + t] + red[2 * N + t] + red[3 * N + t]);
-    __syncthreads();
-    if (t < 32) {  // K = tau/2 p^T v
-      double kk = 0.0;
-      for (int q = t; q < N; q += 32) kk += pw[q] * vc[q];
-      for (int o = 16; o; o >>= 1) kk += __shfl_xor_sync(0xffffffffu, kk, o);
-      if (t == 0) red[4 * N] = 0.5 * tk * kk;
-    }
-    __syncthreads();
-    const double K = red[4 * N];
-    if (t < N) pw[t] -= K * vc[t];
-    __syncthreads();
-    const double vi = vc[i], wi = pw[i];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int q = part + 4 * r;
-      if (q <= i) {
-        const double x = Dm[i * LD + q] - (vi * pw[q] + wi * vc[q]);
-        a.AB[(i - q) + (size_t)(st_k + q) * ldab] = x;
-      }
-    }
-  }
-}
-
 __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
   extern __shared__ double sm[];
   double* Bm = sm;                          // BMAX x (BMAX+1), [row][col]
@@ -494,9 +411,7 @@ __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
       if (abort_flag) return;
       const int st_k = s + 1 + k * b;
       const int len = (M - st_k) < b ? (M - st_k) : b;
-      if (k > 0 && b == BMAX && len == BMAX) {
-        bulge_step_full(a, st_k - b, st_k, Bm, Dm, vp, vc, xv, pw, red, hs, taup);
-      } else {
+      {
         if (k == 0) {
           for (int i = t; i < len; i += blockDim.x) xv[i] = __ldcg(a.AB + (1 + i) + (size_t)s * ldab);
           __syncthreads();
@@ -576,6 +491,531 @@ __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
       }
     }
   }
+}
+
+// ---- bulge chasing for b = N = 32 or 64: fixed point, warp-specialised
+//
+// Arithmetic.  The band is held as 64-bit integers q with C = q 2^-sh, sh chosen so that the
+// largest absolute row sum of the band (a bound on its 2-norm, which no similarity changes) is
+// at most 2^61; reflectors have v in Q62 (|v_i| <= 1 by construction), tau in Q61.  The norms
+// in play (v^T v <= 2, tau |v| <= 2, w = tau C v - ... at most 2 |C|) keep every intermediate
+// below 2^63.  A product drops only the low x low limb: its error is about half a unit, 2^-62
+// of the row-sum bound, where an FP64 operation rounds its result at 2^-54.  Only a
+// reflector's scalars (norm, reciprocal, tau, beta) are FP64, from the column scaled up to
+// full width.  An FP64 instruction holds a scheduler for 64 clocks on this part; the three
+// 32 x 32 -> 64 multiply-adds of a fixed-point product and their shifts take about 20.
+//
+// Schedule.  A sweep's reflectors form a chain of their own: x of step k + 1 is column 0 of
+// B_{k+1} H(s, k), which needs H(s, k) but not the updates of step k.  So the finder warps run
+// that chain one step ahead of the appliers, of which one group updates B of the step and the
+// other D; they hand over through shared memory (two buffers, mbarriers).  Likewise step k of
+// sweep s + 1 needs of step k + 1 of sweep s only the element beta = (H B)(0, 0) before its
+// reflector, and the rest of that step (the last row of its D) only before its D update.  Two
+// progress counters per sweep publish the two events: prog[s] counts steps whose beta is
+// stored, prog[M + s] steps stored completely; one warp of a group polls.
+//
+// Bound: latency, one find + apply + flag through L2 per sweep.  Measured (the FP64 kernel at
+// b = 64 with one role -> this one at b = 64 / b = 32): order 516 14.9 -> 5.4 / 2.6 ms, 2047
+// 64 -> 24 / 11 ms, 8192 262 -> 100 / 60 ms (7.3 us a sweep; an FP64 build of the same schedule
+// took 222 / 102 ms).
+constexpr int BC = 8;  // columns per warp in every role: N / BC finder warps, as many for B and for D
+typedef long long ll;
+
+// A fixed-point number as two balanced limbs, value = hi 2^32 + lo with lo in [-2^31, 2^31).
+__device__ __forceinline__ int2 qsplit(ll a) {
+  const int lo = (int)a;
+  return make_int2(lo, (int)(a >> 32) - (lo >> 31));
+}
+__device__ __forceinline__ ll qjoin(int2 a) { return ((ll)a.y << 32) + a.x; }
+__device__ __forceinline__ ll qhh(int2 a, int2 b) { return (ll)a.y * b.y; }
+__device__ __forceinline__ ll qmid(int2 a, int2 b, ll c) { return (ll)a.y * b.x + ((ll)a.x * b.y + c); }
+// a b 2^-S, rounded (the low x low limb product, at most half a unit, is dropped)
+template <int S>
+__device__ __forceinline__ ll qmul(int2 a, int2 b) {
+  return (qhh(a, b) << (64 - S)) + (qmid(a, b, 1ll << (S - 33)) >> (S - 32));
+}
+
+// Sum over the warp (it has to fit 64 bits) by three 32-bit warp reductions.
+__device__ __forceinline__ ll qwarp_sum(ll v) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0xFFFFFu);
+  const unsigned mi = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 20) & 0xFFFFFu);
+  const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 40));
+  return ((ll)hi << 40) + ((ll)mi << 20) + lo;
+}
+// The double nearest below in magnitude of a positive integer (its 53 leading bits).
+__device__ __forceinline__ double qdouble(unsigned long long x) {
+  if (x == 0) return 0.0;
+  const int lz = __clzll((ll)x);
+  return __longlong_as_double((ll)(((unsigned long long)(1085 - lz) << 52) + ((x << lz) >> 11)));
+}
+// x 2^e as an integer, for a positive normal x with x 2^e < 2^63 (rounded half up).
+__device__ __forceinline__ ll qint(double x, int e) {
+  const ll bits = __double_as_longlong(x);
+  const int sh = (int)(bits >> 52) - 1075 + e;
+  const ll m = (bits & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+  return sh >= 0 ? m << sh : (sh > -54 ? (m + (1ll << (-sh - 1))) >> -sh : 0);
+}
+// 1 / sqrt(x) and 1 / x for normal x: the hardware's seeds (about 20 bits) and one third-order
+// step each, y += y e (1/2 + 3/8 e) with e = 1 - x y^2, and r += r (e + e^2) with e = 1 - x r.
+__device__ __forceinline__ double qrsqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double qrcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+template <int N>
+struct BulgeShared {
+  ll Bs[2][N][N + 1];  // [column][row] of the step's block
+  ll Ds[N][N + 1];     // diagonal block, both triangles
+  ll redA[N / BC][N], x0[N];
+  ll redU[N / BC][N], redD[N / BC][N];
+  int2 yv[2][N], vp[2][N], vc[2][N];  // split into limbs
+  ll sc[2][2];                        // tau (Q61), beta
+  double taud[2];
+  unsigned long long full_y[2], full_v[2], empty[2];
+  int abort_a[2], abort_u[2];
+};
+
+__device__ __forceinline__ uint32_t sm32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mb_init(unsigned long long* b, int n) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sm32(b)), "r"(n) : "memory");
+}
+__device__ __forceinline__ void mb_arrive(unsigned long long* b) {
+  asm volatile("{ .reg .b64 t; mbarrier.arrive.shared::cta.b64 t, [%0]; }" ::"r"(sm32(b)) : "memory");
+}
+// Bounded wait inside the CTA: gives up when an error has been recorded, or records a timeout.
+__device__ bool mb_wait(unsigned long long* b, uint32_t parity, const BulgeArgs& a) {
+  unsigned long long t0 = 0;
+  for (int it = 0;; ++it) {
+    uint32_t ok;
+    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                 : "=r"(ok) : "r"(sm32(b)), "r"(parity) : "memory");
+    if (ok) return true;
+    if ((it & 63) == 63) {
+      if (*(volatile int*)(a.st + 1) != 0) return false;
+      const unsigned long long now = gclock();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > a.wait_ns + 2000000000ull) {
+        atomicExch(a.st + 1, GEP_ERR_TIMEOUT);
+        return false;
+      }
+    }
+  }
+}
+// Bounded wait of a warp until *p >= need and *q >= needq (lanes 0 and 1 poll together).
+__device__ __forceinline__ bool prog_wait(const int* p, int need, const int* q, int needq, const BulgeArgs& a) {
+  const int lane = threadIdx.x & 31, want = lane ? needq : need;
+  const int* w = lane ? q : p;
+  unsigned long long t0 = 0;
+  for (int it = 0;; ++it) {
+    const int ok = lane < 2 ? ld_acquire(w) >= want : 1;
+    if (__all_sync(0xffffffffu, ok)) {
+      __syncwarp();
+      return true;
+    }
+    if ((it & 15) == 15) {
+      const unsigned long long now = gclock();
+      if (t0 == 0) t0 = now;
+      int dead = *(volatile int*)(a.st + 1) != 0;
+      if (!dead && now - t0 > a.wait_ns) {
+        atomicExch(a.st + 1, GEP_ERR_TIMEOUT);
+        dead = 1;
+      }
+      if (__any_sync(0xffffffffu, dead)) return false;
+    }
+  }
+}
+template <int ID, int WARPS>
+__device__ __forceinline__ void group_sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(32 * WARPS) : "memory"); }
+
+template <int N>
+constexpr int bulge_threads() { return 32 * 3 * (N / BC); }
+
+template <int N>
+__global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
+  constexpr int R = N / 32, LD = 2 * N;  // rows per lane, band leading dimension
+  constexpr int G = N / BC, C = BC;      // warps of a group, columns per warp
+  extern __shared__ __align__(16) unsigned char smraw[];
+  BulgeShared<N>& sh = *reinterpret_cast<BulgeShared<N>*>(smraw);
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5, M = a.M;
+  ll* AB = reinterpret_cast<ll*>(a.AB);
+  if (t == 0) {
+    for (int q = 0; q < 2; ++q) {
+      mb_init(&sh.full_y[q], 32 * G);
+      mb_init(&sh.full_v[q], 32);
+      mb_init(&sh.empty[q], 64 * G);
+      sh.abort_a[q] = sh.abort_u[q] = 0;
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  if (status_bad(a.st)) return;
+  int* progA = a.prog;
+  int* progF = a.prog + M;
+  int g = 0;  // steps of this CTA so far (every role counts the same)
+  if (wid < G) {
+    // ---------------- finders
+    const int w = wid;
+    for (int s = blockIdx.x; s <= M - 2; s += gridDim.x) {
+      const int ns = bulge_steps(M, N, s), pns = s > 0 ? bulge_steps(M, N, s - 1) : 0;
+      int2 v[R], taup = make_int2(0, 0);
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = make_int2(0, 0);
+      for (int k = 0; k < ns; ++k, ++g) {
+        const int buf = g & 1;
+        if (w == 0) {
+          bool ok = s == 0 || prog_wait(progF + s - 1, min(k + 1, pns), progA + s - 1, min(k + 2, pns), a);
+          if (ok && g >= 2) ok = mb_wait(&sh.empty[buf], ((uint32_t)(g >> 1) & 1u) ^ 1u, a);
+          if (!ok) sh.abort_a[buf] = 1;
+        }
+        group_sync<1, G>();
+        if (sh.abort_a[buf]) return;
+        const int st_k = s + 1 + k * N, stp = st_k - N, len = min(M - st_k, N);
+        ll x[R];
+        if (k == 0) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int i = lane + 32 * r;
+            x[r] = i < len ? __ldcg(AB + (1 + i) + (size_t)s * LD) : 0;
+          }
+        } else {
+          ll b[R][C];
+          const ll* Bp = AB + (size_t)stp * LD + N + lane + w * C * (LD - 1);
+#pragma unroll
+          for (int q = 0; q < C; ++q)
+#pragma unroll
+            for (int r = 0; r < R; ++r) b[r][q] = lane + 32 * r < len ? __ldcg(Bp + 32 * r + q * (LD - 1)) : 0;
+          int2 vsel = v[0];
+          if (R > 1 && w >= G / R) vsel = v[R - 1];  // the half of v that holds this warp's columns
+          ll hh[R], mm[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) { hh[r] = 0; mm[r] = C / 2; }  // (C / 2: the floors of C shifts)
+#pragma unroll
+          for (int q = 0; q < C; ++q) {
+            int2 vq;
+            vq.x = __shfl_sync(0xffffffffu, vsel.x, (w * C + q) & 31);
+            vq.y = __shfl_sync(0xffffffffu, vsel.y, (w * C + q) & 31);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const int2 bb = qsplit(b[r][q]);
+              hh[r] += qhh(bb, vq);
+              mm[r] += qmid(bb, vq, 0) >> 30;
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int i = lane + 32 * r;
+            sh.redA[w][i] = (hh[r] << 2) + mm[r];
+            if (w == 0) {
+              sh.x0[i] = b[r][0];
+              sh.vp[buf][i] = v[r];
+            }
+          }
+          group_sync<1, G>();
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int i = lane + 32 * r;
+            ll ys = 0;
+#pragma unroll
+            for (int q = 0; q < G; ++q) ys += sh.redA[q][i];
+            const ll y = qmul<61>(qsplit(ys), taup);
+            x[r] = sh.x0[i] - y;
+            if (w == 0) sh.yv[buf][i] = qsplit(y);
+          }
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int q = 0; q < C; ++q) sh.Bs[buf][w * C + q][lane + 32 * r] = b[r][q];
+        }
+        mb_arrive(&sh.full_y[buf]);
+        // reflector of x, formed by every finder warp for itself: x scaled up so that its largest
+        // entry fills [2^59, 2^60), squares in units of 2^63 (2^-55 of the largest or finer)
+        int lz = 64;
+#pragma unroll
+        for (int r = 0; r < R; ++r) lz = min(lz, __clzll(x[r] < 0 ? ~x[r] : x[r]));
+        const int up = min((int)__reduce_min_sync(0xffffffffu, (unsigned)lz), 62) - 4;  // may be negative
+        ll s2 = 0;
+        int2 xs[R];
+        ll x00 = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const ll z = up >= 0 ? x[r] << up : x[r] >> -up;
+          if (r == 0) x00 = z;
+          xs[r] = qsplit(z);
+          if (lane + 32 * r > 0) s2 += qmul<63>(xs[r], xs[r]);
+        }
+        s2 = qwarp_sum(s2);
+        const ll alpha_q = __shfl_sync(0xffffffffu, x[0], 0), xa = __shfl_sync(0xffffffffu, x00, 0);
+        ll beq = alpha_q, tauq = 0;
+        double tau = 0.0;
+        if (s2 > 0) {
+          // be = -sign(alpha) |x|, v = x / (alpha - be), tau = 1 + |alpha| / |x|
+          const double al = qdouble(xa < 0 ? -xa : xa), n2 = fma(al, al, qdouble(s2) * 0x1p63);
+          const double ri = qrsqrt(n2), nrm = n2 * ri;
+          const ll m = qint(qrcp(al + nrm), 121);
+          const int2 mq = qsplit(xa < 0 ? -m : m);
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[r] = qsplit(qmul<59>(xs[r], mq));
+          tau = fma(al, ri, 1.0);
+          tauq = qint(tau, 61);
+          beq = qint(nrm, -up);
+          if (xa >= 0) beq = -beq;
+        } else {
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[r] = make_int2(0, 0);
+        }
+        taup = qsplit(tauq);
+        if (lane == 0) v[0] = make_int2(0, 1 << 30);
+        if (w == 0) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) sh.vc[buf][lane + 32 * r] = v[r];
+          if (lane == 0) {
+            sh.sc[buf][0] = tauq;
+            sh.sc[buf][1] = beq;
+            sh.taud[buf] = tau;
+            AB[k == 0 ? 1 + (size_t)s * LD : N + (size_t)stp * LD] = beq;
+          }
+          mb_arrive(&sh.full_v[buf]);
+          if (lane == 0 && s != a.drop_sweep) st_release(progA + s, k + 1);
+        }
+      }
+    }
+  } else if (wid < 2 * G) {
+    // ---------------- appliers of B: B <- H(s,k) (B H(s,k-1)), lane = column, 8 rows a warp
+    const int u = wid - G;
+    for (int s = blockIdx.x; s <= M - 2; s += gridDim.x) {
+      const int ns = bulge_steps(M, N, s);
+      for (int k = 0; k < ns; ++k, ++g) {
+        const int buf = g & 1;
+        const uint32_t ph = (uint32_t)(g >> 1) & 1u;
+        const int st_k = s + 1 + k * N, stp = st_k - N, len = min(M - st_k, N);
+        bool ok = mb_wait(&sh.full_y[buf], ph, a);
+        ll b[R][C];  // column c = lane + 32 r, rows u C + q
+        if (k > 0) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int c = lane + 32 * r;
+            const int2 vpc = sh.vp[buf][c];
+#pragma unroll
+            for (int q = 0; q < C; ++q) b[r][q] = sh.Bs[buf][c][u * C + q] - qmul<62>(sh.yv[buf][u * C + q], vpc);
+          }
+        }
+        if (ok) ok = mb_wait(&sh.full_v[buf], ph, a);
+        if (!ok) sh.abort_u[buf] = 1;
+        if (k > 0) {
+          ll zh[R], zm[R];
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            zh[r] = 0;
+            zm[r] = C / 2;  // the floors of C shifts
+          }
+#pragma unroll
+          for (int q = 0; q < C; ++q) {
+            const int2 vq = sh.vc[buf][u * C + q];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const int2 bb = qsplit(b[r][q]);
+              zh[r] += qhh(bb, vq);
+              zm[r] += qmid(bb, vq, 0) >> 30;
+            }
+          }
+#pragma unroll
+          for (int r = 0; r < R; ++r) sh.redU[u][lane + 32 * r] = (zh[r] << 2) + zm[r];
+          group_sync<2, G>();
+          const int2 tau = qsplit(sh.sc[buf][0]);
+          const ll be = sh.sc[buf][1];
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int c = lane + 32 * r;
+            ll zs = 0;
+#pragma unroll
+            for (int q = 0; q < G; ++q) zs += sh.redU[q][c];
+            const int2 zc = qsplit(qmul<61>(qsplit(zs), tau));
+#pragma unroll
+            for (int q = 0; q < C; ++q) {
+              const int i = u * C + q;
+              const ll x = b[r][q] - qmul<62>(zc, sh.vc[buf][i]);
+              sh.Bs[buf][c][i] = c == 0 ? (i == 0 ? be : 0) : x;
+            }
+          }
+          group_sync<2, G>();  // stored with lane = row, so that a warp's stores are contiguous
+          ll* Bp = AB + (size_t)stp * LD + N + lane + u * C * (LD - 1);
+#pragma unroll
+          for (int q = 0; q < C; ++q)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+              const int i = lane + 32 * r, c = u * C + q;
+              if (i < len && (i | c) != 0) Bp[32 * r + q * (LD - 1)] = sh.Bs[buf][c][i];
+            }
+        } else if (u == 0) {
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int i = lane + 32 * r;
+            if (i > 0 && i < len) AB[(1 + i) + (size_t)s * LD] = 0;
+          }
+        }
+        if (a.q2 && u == G - 1) {  // reflector into diamond (j, k), column c
+          const int j = s / N, c = s - j * N;
+          double* D0 = a.q2 + diamond_index(a.Q, j, k) * diamond_elems(N);
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+            if (lane + 32 * r < len)
+              D0[(c + lane + 32 * r) + (size_t)c * 2 * N] = (double)qjoin(sh.vc[buf][lane + 32 * r]) * 0x1p-62;
+          if (lane == 0) D0[(size_t)2 * N * N + c] = sh.taud[buf];
+        }
+        mb_arrive(&sh.empty[buf]);
+        group_sync<4, 2 * G>();  // the stores of both groups precede the release
+        if (sh.abort_u[buf]) return;
+      }
+    }
+  } else {
+    // ---------------- appliers of D: D <- H D H on the lower triangle, lane = row, 8 columns a warp
+    const int u = wid - 2 * G;
+    for (int s = blockIdx.x; s <= M - 2; s += gridDim.x) {
+      const int ns = bulge_steps(M, N, s), pns = s > 0 ? bulge_steps(M, N, s - 1) : 0;
+      for (int k = 0; k < ns; ++k, ++g) {
+        const int buf = g & 1;
+        const uint32_t ph = (uint32_t)(g >> 1) & 1u;
+        const int st_k = s + 1 + k * N, len = min(M - st_k, N);
+        if (u == 0 && s > 0) {
+          const int need = min(k + 2, pns);
+          if (!prog_wait(progF + s - 1, need, progF + s - 1, need, a)) sh.abort_u[buf] = 1;
+        }
+        group_sync<3, G>();
+        ll dv[R][C];
+        ll* Dp = AB + (size_t)st_k * LD + lane + u * C * (LD - 1);
+#pragma unroll
+        for (int q = 0; q < C; ++q)
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int i = lane + 32 * r, c = u * C + q;
+            dv[r][q] = (i >= c && i < len) ? __ldcg(Dp + 32 * r + q * (LD - 1)) : 0;
+          }
+#pragma unroll
+        for (int q = 0; q < C; ++q)
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int i = lane + 32 * r, c = u * C + q;
+            if (i >= c) {
+              sh.Ds[c][i] = dv[r][q];
+              sh.Ds[i][c] = dv[r][q];
+            }
+          }
+        if (!mb_wait(&sh.full_v[buf], ph, a)) sh.abort_u[buf] = 1;
+        group_sync<3, G>();
+        const int2 tau = qsplit(sh.sc[buf][0]);
+        int2 vr[R];
+        ll hh[R], mm[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          vr[r] = sh.vc[buf][lane + 32 * r];
+          hh[r] = 0;
+          mm[r] = C / 2;
+        }
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+          const int2 vq = sh.vc[buf][u * C + q];
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int2 dd = qsplit(sh.Ds[u * C + q][lane + 32 * r]);
+            hh[r] += qhh(dd, vq);
+            mm[r] += qmid(dd, vq, 0) >> 30;
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) sh.redD[u][lane + 32 * r] = (hh[r] << 2) + mm[r];
+        group_sync<3, G>();
+        ll p[R], K = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          ll ps = 0;
+#pragma unroll
+          for (int q = 0; q < G; ++q) ps += sh.redD[q][lane + 32 * r];
+          p[r] = qmul<61>(qsplit(ps), tau);
+          K += qmul<62>(qsplit(p[r]), vr[r]);
+        }
+        const int2 Kh = qsplit(qmul<62>(qsplit(qwarp_sum(K)), tau));  // tau / 2 p^T v
+        int2 wv[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) wv[r] = qsplit(p[r] - qmul<62>(Kh, vr[r]));
+        int2 wsel = wv[0];
+        if (R > 1 && u >= G / R) wsel = wv[R - 1];
+#pragma unroll
+        for (int q = 0; q < C; ++q) {
+          const int c = u * C + q;
+          int2 wc;
+          wc.x = __shfl_sync(0xffffffffu, wsel.x, c & 31);
+          wc.y = __shfl_sync(0xffffffffu, wsel.y, c & 31);
+          const int2 vq = sh.vc[buf][c];
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int i = lane + 32 * r;
+            if (32 * r + 31 < c) continue;  // the whole warp lies above the diagonal
+            const ll x = dv[r][q] - qmul<62>(vr[r], wc) - qmul<62>(wv[r], vq);
+            if (i >= c && i < len) Dp[32 * r + q * (LD - 1)] = x;
+          }
+        }
+        mb_arrive(&sh.empty[buf]);
+        group_sync<4, 2 * G>();  // the stores of both groups precede the release
+        if (sh.abort_u[buf]) return;
+        if (u == 0 && lane == 0 && s != a.drop_sweep) st_release(progF + s, k + 1);
+      }
+    }
+  }
+}
+
+// Largest absolute row sum of the band matrix (bits of a non-negative double, by atomicMax).
+__global__ void k_band_rowsum(int M, int b, const double* __restrict__ AB, int ldab, unsigned long long* mx,
+                              const int* st) {
+  if (status_bad(st)) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  double s = 0.0;
+  if (i < M) {
+    for (int o = 0; o <= b && i + o < M; ++o) s += fabs(AB[o + (size_t)i * ldab]);
+    for (int o = 1; o <= b && o <= i; ++o) s += fabs(AB[o + (size_t)(i - o) * ldab]);
+  }
+  unsigned long long v = (unsigned long long)__double_as_longlong(s);
+  for (int o = 16; o; o >>= 1) {
+    const unsigned long long q = __shfl_xor_sync(0xffffffffu, v, o);
+    if (q > v) v = q;
+  }
+  if ((threadIdx.x & 31) == 0 && v) atomicMax(mx, v);
+}
+
+// sh with (largest row sum) 2^sh in (2^60, 2^61]
+__device__ __forceinline__ int band_shift(const unsigned long long* mx) {
+  const int E = (int)(*mx >> 52);  // sum < 2^(E - 1022)
+  return E ? 61 - (E - 1022) : 0;
+}
+__device__ __forceinline__ double scale2(double x, int e) {  // x 2^e, e within +-2100
+  const int a = e / 2, c = e - a;
+  return x * __longlong_as_double((ll)(1023 + a) << 52) * __longlong_as_double((ll)(1023 + c) << 52);
+}
+
+__global__ void k_band_fix(int M, double* AB, int ldab, const unsigned long long* mx, const int* st) {
+  if (status_bad(st)) return;
+  const int sh = band_shift(mx);
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)M * ldab; i += (size_t)gridDim.x * blockDim.x) {
+    const double x = AB[i];
+    reinterpret_cast<ll*>(AB)[i] = x == 0.0 ? 0 : __double2ll_rn(scale2(x, sh));
+  }
+}
+
+__global__ void k_band_diag_fix(int M, const double* __restrict__ AB, int ldab, const unsigned long long* mx,
+                                double* __restrict__ d, double* __restrict__ e, const int* st) {
+  if (status_bad(st)) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, sh = band_shift(mx);
+  if (i >= M) return;
+  const ll* q = reinterpret_cast<const ll*>(AB);
+  d[i] = scale2((double)q[(size_t)i * ldab], -sh);
+  if (i + 1 < M) e[i] = scale2((double)q[1 + (size_t)i * ldab], -sh);
 }
 
 __global__ void k_band_diag(int M, const double* __restrict__ AB, int ldab, double* __restrict__ d,
@@ -735,7 +1175,7 @@ size_t band_ws_elems(int M, int b) {
   size_t reduce = 2 * rr(G * BMAX) + 2 * rr(BMAX) + rr(32) + 4 * rr((size_t)M * b) +
                   2 * rr((size_t)M * 2 * BAND_GROUP * b) + 5 * rr((size_t)2 * b * b) +
                   rr((size_t)2 * BAND_GROUP * b * b) + rr(oz_sym_planes_bytes(M, 9) / sizeof(double) + 1);
-  size_t chase = rr((size_t)2 * b * M) + rr((size_t)M);  // band + progress counters
+  size_t chase = rr((size_t)2 * b * M) + rr((size_t)M) + rr(1);  // band, progress counters, norm bound
   return reduce > chase ? reduce : chase;
 }
 
@@ -947,15 +1387,23 @@ int band_to_tridiag(gep_handle_t h, int M, const double* C, int ldc, int b, doub
   k_band_copy<<<M, ldab, 0, h->stream>>>(M, b, C, ldc, AB, ldab, h->d_status);
   GEP_CHECK(check_launch(h));
   if (M >= 2) {
-    GEP_CUDA(cudaMemsetAsync(prog, 0, sizeof(int) * (size_t)M, h->stream));
+    GEP_CUDA(cudaMemsetAsync(prog, 0, sizeof(int) * 2 * (size_t)M, h->stream));
     const int Q = (M - 2) / b;
     if (q2) GEP_CUDA(cudaMemsetAsync(q2, 0, q2_elems(M, b) * sizeof(double), h->stream));
-    size_t smem = bulge_smem_bytes();
+    // b = 32 and 64 take the fixed-point kernel, other widths the general one
+    const bool fixed = b == 32 || b == 64;
+    unsigned long long* mx = reinterpret_cast<unsigned long long*>(prog + rr((size_t)M) * 2);
+    const void* kern = b == 32 ? (const void*)k_bulge_ws<32> : b == 64 ? (const void*)k_bulge_ws<64> : (const void*)k_bulge;
+    const size_t smem = b == 32 ? sizeof(BulgeShared<32>) : b == 64 ? sizeof(BulgeShared<64>) : bulge_smem_bytes();
     static unsigned long long attr_devices = 0;
-    if (first_use_on_device(attr_devices))
-      GEP_CUDA(cudaFuncSetAttribute(k_bulge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (first_use_on_device(attr_devices)) {
+      GEP_CUDA(cudaFuncSetAttribute(k_bulge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bulge_smem_bytes()));
+      GEP_CUDA(cudaFuncSetAttribute(k_bulge_ws<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BulgeShared<32>)));
+      GEP_CUDA(cudaFuncSetAttribute(k_bulge_ws<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BulgeShared<64>)));
+    }
     int per_sm = 0;
-    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bulge, 256, smem));
+    const int threads = b == 32 ? bulge_threads<32>() : b == 64 ? bulge_threads<64>() : 256;
+    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
     if (per_sm < 1) return GEP_ERR_UNSUPPORTED;
     // The sweeps form a dependency chain (step k of sweep s waits for step k+1 of sweep
     // s-1): the time is set by the latency of one step, which co-resident CTAs stretch.
@@ -971,9 +1419,20 @@ int band_to_tridiag(gep_handle_t h, int M, const double* C, int ldc, int b, doub
     a.M = M; a.b = b; a.ldab = ldab; a.Q = Q; a.AB = AB; a.prog = prog; a.q2 = q2; a.st = h->d_status;
     a.wait_ns = h->wait_limit_ns;
     a.drop_sweep = h->fault_drop_sweep;
+    if (fixed) {
+      GEP_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long), h->stream));
+      k_band_rowsum<<<(M + 255) / 256, 256, 0, h->stream>>>(M, b, AB, ldab, mx, h->d_status);
+      GEP_CHECK(check_launch(h));
+      k_band_fix<<<std::min(M, 4 * h->sm_count), 256, 0, h->stream>>>(M, AB, ldab, mx, h->d_status);
+      GEP_CHECK(check_launch(h));
+    }
     void* args[] = {&a};
-    GEP_CUDA(cudaLaunchCooperativeKernel((void*)k_bulge, dim3(grid), dim3(256), args, smem, h->stream));
+    GEP_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, smem, h->stream));
     GEP_CHECK(check_launch(h));
+    if (fixed) {
+      k_band_diag_fix<<<(M + 255) / 256, 256, 0, h->stream>>>(M, AB, ldab, mx, d, e, h->d_status);
+      return check_launch(h);
+    }
   }
   k_band_diag<<<(M + 255) / 256, 256, 0, h->stream>>>(M, AB, ldab, d, e, h->d_status);
   return check_launch(h);
