@@ -74,7 +74,7 @@ typedef struct gep_handle_s* gep_handle_t;
 typedef struct gep_options {
   int reducer;      /* GEP_RED_*                                                  */
   int sep;          /* GEP_SEP_*                                                  */
-  int bandwidth;    /* band width b for GEP_SEP_2STAGE, 1..64 (0 = library default, 64) */
+  int bandwidth;    /* band width b for GEP_SEP_2STAGE, 1..64 (0 = library default: 32 up to order 12288, 64 beyond) */
   int precision;    /* GEP_PREC_*                                                 */
   int want_vectors; /* 1: eigenpairs (T_full); 0: eigenvalues only (T_evo)        */
   int overwrite;    /* 1: A and B may be destroyed by gep_solve (saves two copies) */

@@ -19,9 +19,12 @@ struct SolveLayout {
   size_t uni_bytes, eng_bytes;
 };
 
-constexpr int kDefaultBand = 64;  // bandwidth of the two-stage reduction when o->bandwidth = 0
-
-int band_of(const gep_options* o) { return o->bandwidth > 0 ? o->bandwidth : kDefaultBand; }
+// Bandwidth of the two-stage reduction when o->bandwidth = 0.  The narrow band
+// halves the bulge-chasing latency and the panel QR's FP64 work; the wide one halves the number of
+// panels, whose products and digit splits are what large matrices spend.  Measured, whole solve at
+// b = 64 / 32: order 516 21.5 / 18.0 ms, 2047 113 / 96 ms, 8192 709 / 688 ms.
+constexpr int kNarrowBandMax = 12288;
+int band_of(int M, const gep_options* o) { return o->bandwidth > 0 ? o->bandwidth : (M <= kNarrowBandMax ? 32 : 64); }
 bool two_stage(const gep_options* o) { return o->sep == GEP_SEP_2STAGE; }
 bool jacobi(const gep_options* o) { return o->sep == GEP_SEP_JACOBI; }
 bool eigenexa(const gep_options* o) { return o->reducer == GEP_RED_EIGENEXA; }
@@ -48,13 +51,13 @@ size_t union_bytes(int M, const gep_options* o) {
   size_t red = (o->reducer == GEP_RED_EXPLICIT_INV) ? r256(mm) + r256(mm) + r256(tmpb)
                : eigenexa(o) ? r256(mm)  // A X of Eq. 8
                              : r256(mm) + r256(tmpb);
-  size_t tri = two_stage(o) ? band_ws_elems(M, band_of(o)) * sizeof(double)
+  size_t tri = two_stage(o) ? band_ws_elems(M, band_of(M, o)) * sizeof(double)
                : jacobi(o)  ? jacobi_ws_elems(M) * sizeof(double)
                             : tridiag_ws_elems(M) * sizeof(double);
   size_t dc = sep_vectors(o) ? dc_ws_bytes(M) : 0;
   size_t bt = sep_vectors(o) ? backtransform_ws_elems(M, M) * sizeof(double) : 0;
   if (two_stage(o) && sep_vectors(o)) {
-    size_t q2t = q2_tile_ws_elems(M, band_of(o)) * sizeof(double);
+    size_t q2t = q2_tile_ws_elems(M, band_of(M, o)) * sizeof(double);
     if (q2t > bt) bt = q2t;
   }
   size_t r3 = (o->want_vectors && !eigenexa(o))
@@ -87,13 +90,13 @@ SolveLayout layout(int M, const gep_options* o) {
   L.af = off;  // full symmetric A and B kept for the FP64 refinement
   off += (o->precision == GEP_PREC_MIXED_REFINED) ? 2 * r256(mm) : 0;
   L.q2 = off;  // bulge-chasing reflectors, kept from S1c to the back-transformation
-  off += (two_stage(o) && sep_vectors(o)) ? r256(q2_elems(M, band_of(o)) * sizeof(double)) : 0;
+  off += (two_stage(o) && sep_vectors(o)) ? r256(q2_elems(M, band_of(M, o)) * sizeof(double)) : 0;
   L.xw = off;  // X = W D^-1/2 of the Cholesky-free reducer (Eq. 7-9)
   off += eigenexa(o) ? r256(mm) : 0;
   L.zt = off;  // all eigenvectors of T when only the lowest n_want are back-transformed
   off += partial_vectors(M, o) ? r256(mm) : 0;
   L.q2u = off;  // every dense Q2 tile, built on the second stream during divide and conquer
-  off += q2_tiles_ahead(o) ? r256(q2_all_tiles_elems(M, band_of(o)) * sizeof(double)) : 0;
+  off += q2_tiles_ahead(o) ? r256(q2_all_tiles_elems(M, band_of(M, o)) * sizeof(double)) : 0;
   L.end = off;
   return L;
 }
@@ -134,7 +137,7 @@ int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, d
               double* tvec, double* q2, char* uni, size_t uni_bytes, int eng, double* w, double* Z, int ldz,
               bool timed, int n = 0, double* Zt = nullptr, double* wt = nullptr, double* q2u = nullptr) {
   if (n <= 0 || n > M) n = M;
-  const int bw = band_of(o);
+  const int bw = band_of(M, o);
   if (jacobi(o)) {  // no tridiagonal form: the block-Jacobi solver works on C itself
     if (timed) mark(h, o, 3);
     double* wj = (n < M) ? wt : w;
@@ -169,7 +172,7 @@ int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, d
   if (ahead) {
     GEP_CUDA(cudaEventRecord(h->ev_fork, h->stream));
     GEP_CUDA(cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-    GEP_CHECK(build_q2_tiles(h, h->side, M, band_of(o), q2, q2u));
+    GEP_CHECK(build_q2_tiles(h, h->side, M, band_of(M, o), q2, q2u));
     GEP_CUDA(cudaEventRecord(h->ev_join, h->side));
   }
   if (n < M) {

@@ -1089,25 +1089,45 @@ __global__ void __launch_bounds__(256) k_q2_apply(int M, int b, int Q, int wt, c
 // ascending.  U(J, K) is the product of its diamonds in that order, built by applying
 // them to the identity, W x TB_COLS columns per CTA, and stored as U - I so that a tile
 // is applied as Z(rows) += (U - I) Z(rows).
-constexpr int TQ = 4;
+// Diamonds per tile side: W = 2 TQ b = 512 for b = 32 and 64, the depth of one exact chunk of the
+// product kernel.
+__host__ __device__ constexpr int tile_q(int b) { return b == 32 ? 8 : 4; }
 constexpr int TB_COLS = 32;  // tile columns per CTA in the build (8 lanes per column)
+constexpr int TB_LD = TB_COLS + 2;  // (8 rows x 2 columns of a half warp then fall into distinct banks)
 
-__global__ void __launch_bounds__(256) k_q2_tile_build(int M, int b, int Q, int J, const double* __restrict__ q2,
+// Tile index t (tile rows J ascending, then K) -> (J, K); nK(J) = (Q - J TQ) / TQ + 1.
+__device__ __forceinline__ void tile_of_index(int Q, int TQ, int t, int& J, int& K) {
+  J = 0;
+  for (int nK; t >= (nK = (Q - J * TQ) / TQ + 1); ++J) t -= nK;
+  K = t;
+}
+
+// The arithmetic is the fixed point of the bulge-chasing kernel (entries of U and v in Q62, all at
+// most 1 in magnitude; tau in Q61), about a third of the FP64 issue time and exact to 2^-61 per
+// operation.  Eight lanes share a column; a diamond's reflectors are turned into limbs in shared
+// memory once per CTA, the next diamond's being fetched meanwhile.
+// Bound: integer issue (about 100 instructions a reflector for 8 warps) and its latency.  Measured
+// (D&C beside the build, then the back-transformation; b = 32): order 2047 5.8 + 24.6 -> 9.2 +
+// 10.1 ms, order 8192 115 + 167 -> 88 + 146 ms.  All tiles are one launch (a launch per tile row
+// left most SMs idle).
+__global__ void __launch_bounds__(256) k_q2_tile_build(int b, int Q, const double* __restrict__ q2,
                                                        double* __restrict__ U, const int* st) {
-  extern __shared__ double sm[];
+  extern __shared__ __align__(16) unsigned char smq[];
   if (status_bad(st)) return;
-  const int K = blockIdx.x;
-  const int W = 2 * TQ * b;
+  const int TQ = tile_q(b), W = 2 * TQ * b;
+  int J, K;
+  tile_of_index(Q, TQ, blockIdx.x, J, K);
   const int J0 = J * TQ, K0 = K * TQ;
-  const int r0 = 1 + (J0 + K0) * b;  // global row of tile row 0
   const int c0 = blockIdx.y * TB_COLS;
-  double* Us = sm;  // [row][TB_COLS + 1]
+  ll* Us = reinterpret_cast<ll*>(smq);                         // [row][TB_LD]
+  int2* Vs = reinterpret_cast<int2*>(Us + (size_t)W * TB_LD);  // [c][b]: v of reflector c, its own rows
+  int2* ts = Vs + b * b;                                       // [c]
   const int t = threadIdx.x;
+  constexpr ll ONE = 1ll << 62;
   for (int idx = t; idx < W * TB_COLS; idx += blockDim.x) {
-    int r = idx % W, cc = idx / W;
-    Us[r * (TB_COLS + 1) + cc] = (r == c0 + cc) ? 1.0 : 0.0;
+    int r = idx / TB_COLS, cc = idx % TB_COLS;
+    Us[r * TB_LD + cc] = (r == c0 + cc) ? ONE : 0;
   }
-  __syncthreads();
   const int col = t >> 3, part = t & 7;
   const int jhi = min(J0 + TQ - 1, Q);
   // rows [rmin, rmax] hold every nonzero of this CTA's columns (identity columns at
@@ -1116,37 +1136,58 @@ __global__ void __launch_bounds__(256) k_q2_tile_build(int M, int b, int Q, int 
   for (int j = jhi; j >= J0; --j) {
     for (int k = K0; k < K0 + TQ; ++k) {
       if (k > Q - j) continue;
-      const double* D0 = q2 + diamond_index(Q, j, k) * diamond_elems(b);
       const int lo = (j + k - J0 - K0) * b;  // tile row of the diamond's row 0
+      if (lo + 2 * b - 2 < rmin || lo > rmax) continue;
+      const double* D0 = q2 + diamond_index(Q, j, k) * diamond_elems(b);
+      __syncthreads();  // the previous diamond's reflectors are no longer read
+      for (int idx = t; idx < b * b; idx += blockDim.x) {
+        const int c = idx / b, i = idx - c * b;
+        const double x = D0[(size_t)c * 2 * b + c + i];
+        const ll m = x == 0.0 ? 0 : qint(fabs(x), 62);
+        Vs[idx] = qsplit(x < 0.0 ? -m : m);
+      }
+      if (t < b) {
+        const double x = D0[(size_t)2 * b * b + t];
+        ts[t] = qsplit(x == 0.0 ? 0 : qint(x, 61));
+      }
+      __syncthreads();
       for (int c = b - 1; c >= 0; --c) {
         if (lo + c + b - 1 < rmin || lo + c > rmax) continue;
-        double tc = D0[(size_t)2 * b * b + c];
-        if (tc == 0.0) continue;
+        const int2 tc = ts[c];
+        if ((tc.x | tc.y) == 0) continue;
         rmin = min(rmin, lo + c);
         rmax = max(rmax, lo + c + b - 1);
-        const double* v = D0 + (size_t)c * 2 * b;
-        double u = 0.0;
-        for (int r = c + part; r < c + b; r += 8)
-          if (r0 + lo + r < M) u += v[r] * Us[(lo + r) * (TB_COLS + 1) + col];
-        u += __shfl_xor_sync(0xffffffffu, u, 1);
-        u += __shfl_xor_sync(0xffffffffu, u, 2);
-        u += __shfl_xor_sync(0xffffffffu, u, 4);
-        u *= tc;
-        for (int r = c + part; r < c + b; r += 8)
-          if (r0 + lo + r < M) Us[(lo + r) * (TB_COLS + 1) + col] -= u * v[r];
+        const int2* v = Vs + c * b;
+        ll* u0 = Us + (lo + c) * TB_LD + col;
+        ll hh = 0, mm = 0;
+#pragma unroll 4
+        for (int r = part; r < b; r += 8) {
+          const int2 x = qsplit(u0[r * TB_LD]), y = v[r];
+          hh += qhh(x, y);
+          mm += qmid(x, y, 1ll << 29) >> 30;
+        }
+        ll d = (hh << 2) + mm;
+        d += __shfl_xor_sync(0xffffffffu, d, 1);
+        d += __shfl_xor_sync(0xffffffffu, d, 2);
+        d += __shfl_xor_sync(0xffffffffu, d, 4);
+        const int2 u = qsplit(qmul<62>(qsplit(d), tc));  // Q61
+#pragma unroll 4
+        for (int r = part; r < b; r += 8) u0[r * TB_LD] -= qmul<61>(u, v[r]);
         __syncwarp();
       }
     }
   }
   __syncthreads();
-  double* Ut = U + (size_t)K * W * W;  // U - I, W x W column-major
+  double* Ut = U + (size_t)blockIdx.x * W * W;  // U - I, W x W column-major
   for (int idx = t; idx < W * TB_COLS; idx += blockDim.x) {
     int r = idx % W, cc = idx / W;
-    if (c0 + cc < W) Ut[r + (size_t)(c0 + cc) * W] = Us[r * (TB_COLS + 1) + cc] - (r == c0 + cc ? 1.0 : 0.0);
+    if (c0 + cc < W) Ut[r + (size_t)(c0 + cc) * W] = (double)(Us[r * TB_LD + cc] - (r == c0 + cc ? ONE : 0)) * 0x1p-62;
   }
 }
 
-size_t q2_tile_smem_bytes(int b) { return (size_t)2 * TQ * b * (TB_COLS + 1) * sizeof(double); }
+size_t q2_tile_smem_bytes(int b) {
+  return (size_t)2 * tile_q(b) * b * TB_LD * sizeof(ll) + ((size_t)b * b + b) * sizeof(int2);
+}
 
 size_t q2_smem_bytes(int b) {
   return ((size_t)2 * b * b + (size_t)(2 * b - 1) * (Q2_COLS + 1) + b) * sizeof(double);
@@ -1320,7 +1361,7 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
     // C^(j) V_j below reads rows j b.. of the planes against the full-height V_j.  The columns
     // the group updates in between (those of panels 1..g-1) meet V_j's zero rows.
     OzSymPlanes planes;
-    const bool use_planes = eng != GEP_PREC_FP64 && n >= 128 && b >= 64;
+    const bool use_planes = eng != GEP_PREC_FP64 && n >= 128 && b >= 32;
     if (use_planes) GEP_CHECK(oz_split_sym(h, n, C22, ldc, levels, w.planes, w.planes_bytes, &planes));
     for (int j = 0; j < g; ++j) {
       const int r0 = j * b, nr = n - r0;  // panel j's reflectors act on rows [r0, n) of C22
@@ -1440,15 +1481,13 @@ int band_to_tridiag(gep_handle_t h, int M, const double* C, int ldc, int b, doub
 
 size_t q2_tile_ws_elems(int M, int b) {
   if (M < 3 || b < 1) return 0;
-  size_t Q = (size_t)(M - 2) / b;
-  size_t nK = Q / TQ + 1, W = (size_t)2 * TQ * b;
-  return rr(nK * W * W) + rr(W * (size_t)M);
+  return rr((size_t)2 * tile_q(b) * b * (size_t)M);
 }
 
 namespace {
 
 // Tiles of every tile row J, one after the other (tile (J, K) at all_tiles_offset(Q, J) + K).
-size_t all_tiles_offset(int Q, int J) {
+size_t all_tiles_offset(int Q, int J, int TQ) {
   size_t off = 0;
   for (int j = 0; j < J; ++j) off += (size_t)((Q - j * TQ) / TQ + 1);
   return off;
@@ -1466,9 +1505,9 @@ int set_tile_build_attr() {
 
 size_t q2_all_tiles_elems(int M, int b) {
   if (M < 3 || b < 1) return 0;
-  const int Q = (M - 2) / b;
+  const int Q = (M - 2) / b, TQ = tile_q(b);
   const size_t W = (size_t)2 * TQ * b;
-  return all_tiles_offset(Q, Q / TQ + 1) * W * W;
+  return all_tiles_offset(Q, Q / TQ + 1, TQ) * W * W;
 }
 
 // Builds every dense tile U(J, K) - I of Q2 into U (q2_all_tiles_elems doubles) on `stream`,
@@ -1479,15 +1518,11 @@ int build_q2_tiles(gep_handle_t h, cudaStream_t stream, int M, int b, const doub
   if (M < 3) return GEP_OK;
   GEP_CHECK(set_tile_build_attr());
   const int Q = (M - 2) / b;
-  const int W = 2 * TQ * b, nJ = Q / TQ + 1;
-  const size_t smem = q2_tile_smem_bytes(b);
-  for (int J = 0; J < nJ; ++J) {
-    const int nK = (Q - J * TQ) / TQ + 1;
-    double* UJ = U + all_tiles_offset(Q, J) * (size_t)W * W;
-    k_q2_tile_build<<<dim3(nK, (W + TB_COLS - 1) / TB_COLS), 256, smem, stream>>>(M, b, Q, J, q2, UJ, h->d_status);
-    GEP_CHECK(check_launch(h));
-  }
-  return GEP_OK;
+  const int TQ = tile_q(b), W = 2 * TQ * b;
+  const size_t tiles = all_tiles_offset(Q, Q / TQ + 1, TQ);
+  k_q2_tile_build<<<dim3((unsigned)tiles, (W + TB_COLS - 1) / TB_COLS), 256, q2_tile_smem_bytes(b), stream>>>(
+      b, Q, q2, U, h->d_status);
+  return check_launch(h);
 }
 
 // Where U(J, K) - I can be nonzero, per 128-row block of a W x W tile: the reflectors of the
@@ -1497,7 +1532,7 @@ int build_q2_tiles(gep_handle_t h, cudaStream_t stream, int M, int b, const doub
 // the columns whose interval meets its rows.  Every tile has this structure or a subset
 // of it (tiles at the edge hold fewer diamonds).
 static void q2_tile_kranges(int b, OzKRange* kr) {
-  const int W = 2 * TQ * b;
+  const int TQ = tile_q(b), W = 2 * TQ * b;
   std::vector<int> rmin(W), rmax(W);
   for (int c = 0; c < W; ++c) rmin[c] = rmax[c] = c;
   for (int jj = TQ - 1; jj >= 0; --jj)
@@ -1526,33 +1561,23 @@ static void q2_tile_kranges(int b, OzKRange* kr) {
 
 // Z (M x ncol) <- Q2 Z.  engine FP64: diamonds applied directly on the FP64 cores.
 // Otherwise the diamonds are merged into dense W x W tiles U(J, R) and every tile is
-// applied as one product Z(rows) <- U Z(rows) on the engine (ws: q2_tile_ws_elems).
-// U_all != null: the tiles were built by build_q2_tiles (on the caller's stream order).
+// applied as one product Z(rows) <- U Z(rows) on the engine (ws: q2_tile_ws_elems); U_all: the
+// tiles, built by build_q2_tiles (on the caller's stream order).
 int apply_q2(gep_handle_t h, int M, int b, const double* q2, double* Z, int ldz, int ncol, int engine, double* ws,
              size_t ws_elems, const double* U_all) {
   if (b < 1 || b > BMAX) return GEP_ERR_UNSUPPORTED;
   if (M < 3 || ncol <= 0) return GEP_OK;  // M = 2: the only reflector is the identity
   const int Q = (M - 2) / b;
   if (engine != GEP_PREC_FP64) {
-    if (ws_elems < q2_tile_ws_elems(M, b)) return GEP_ERR_ALLOC;
-    const int W = 2 * TQ * b;
+    if (!U_all || ws_elems < q2_tile_ws_elems(M, b)) return GEP_ERR_ALLOC;
+    const int TQ = tile_q(b), W = 2 * TQ * b;
     const int nJ = Q / TQ + 1;
-    double* Ubuf = ws;
-    double* Tmp = ws + rr((size_t)(Q / TQ + 1) * W * W);
-    size_t smem = q2_tile_smem_bytes(b);
+    double* Tmp = ws;
     OzKRange kr;
     q2_tile_kranges(b, &kr);
-    GEP_CHECK(set_tile_build_attr());
     for (int J = nJ - 1; J >= 0; --J) {
       const int nK = (Q - J * TQ) / TQ + 1;  // tiles (J, K) with a diamond: K TQ <= Q - J TQ
-      const double* U = Ubuf;
-      if (U_all) {
-        U = U_all + all_tiles_offset(Q, J) * (size_t)W * W;
-      } else {
-        k_q2_tile_build<<<dim3(nK, (W + TB_COLS - 1) / TB_COLS), 256, smem, h->stream>>>(M, b, Q, J, q2, Ubuf,
-                                                                                        h->d_status);
-        GEP_CHECK(check_launch(h));
-      }
+      const double* U = U_all + all_tiles_offset(Q, J, TQ) * (size_t)W * W;
       for (int K = 0; K < nK; ++K) {
         const int r0 = 1 + (J + K) * TQ * b;
         if (r0 >= M) break;
