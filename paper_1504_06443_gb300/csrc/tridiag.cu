@@ -14,6 +14,8 @@
 // second kernel adds them in a fixed order.
 #include <math.h>
 
+#include <type_traits>
+
 #include "gep_internal.cuh"
 
 namespace gep {
@@ -26,6 +28,8 @@ constexpr int DCH = 128;    // panel dot-product rows per CTA
 
 struct TWs {
   double *Vp, *W, *y, *Pd, *Pt, *part, *part2, *WV, *tq;
+  double *P, *vav, *xbuf;  // the one-launch panel: tile partial sums, v^T A v parts, next column
+  int* bar;
   float2* S2;  // float-pair copy of the trailing matrix (lower triangle) for the SYMVs
   int M, nblk, maxch, ndch;
 };
@@ -480,6 +484,382 @@ __global__ void __launch_bounds__(256) k_w_finish(int n, int nblk, const double*
   }
 }
 
+// ---- one panel of the reduction in one cooperative launch (trailing order <= TRD_COOP_MAX)
+//
+// Six launches per column (about 10 us each, mostly launch gaps and single-CTA reductions) made
+// the small and ordinary orders launch-bound.  Here the trailing matrix, which a panel does not
+// change, is cut into TS x TS tiles of its lower triangle that stay in the shared memory of the G
+// CTAs for all columns of the panel, and a column costs two grid barriers:
+//   A: every CTA reads the column x, forms the reflector v for itself, multiplies its tiles
+//      (row and column partial sums to P), its share of t1 = W^T v, t2 = V^T v (whole dots, one
+//      CTA each) and its part of v^T A v;                                           [barrier]
+//   B: every CTA sums P for the rows it owns, w = tau (A v - V t1 - W t2) + alpha v with
+//      alpha from v^T A v - 2 t1.t2 (so that no third barrier is needed for w^T v), then the same
+//      rows of the next column, x = C(:, c+1) - V W(c+1,:)^T - W V(c+1,:)^T; the row c+1 of W is
+//      formed by every CTA for itself.                                              [barrier]
+// Bound: the two barriers (1.2 us each on 152 SMs) and the latency of the reductions between
+// them; native FP64 tiles also by FP64 issue (two FMAs per element).  Measured per column (six
+// launches before): order 500 FP64 69 -> 12.8 us, order 1501 float pairs 72 -> 18 us, order 64
+// 58 -> 20 us.
+constexpr int TRD_COOP_MAX = 4096;  // vs and the tiles fit shared memory; beyond, the SYMV is bound by HBM anyway
+constexpr int TRD_T = 256;          // threads
+constexpr int LPR = 16;             // lanes per owned row
+
+struct TrdArgs {
+  int M, j0, nbp, nt, nb, tiles, nres, slots, rpc, ldc;
+  double *C, *d, *e, *tau, *Vp, *W, *P, *t, *vav, *xbuf;
+  int *bar, *st;
+};
+
+// Tile element a (any of the three storage forms) times a vector entry, accumulated.
+struct AccD {
+  double s = 0.0;
+  __device__ void add(double a, double v) { s = fma(a, v, s); }
+  __device__ double get() const { return s; }
+};
+struct AccF {
+  ff s = {0.f, 0.f};
+  __device__ void add(float2 a, float2 v) { ff_madd(s, a.x, a.y, v.x, v.y); }
+  __device__ void add(float a, float2 v) { ff_madd(s, a, 0.f, v.x, v.y); }
+  __device__ double get() const { return (double)s.h + (double)s.l; }
+};
+template <class T> struct TrdForm;
+template <> struct TrdForm<double> { typedef double Vec; typedef AccD Acc; };
+template <> struct TrdForm<float2> { typedef float2 Vec; typedef AccF Acc; };
+template <> struct TrdForm<float> { typedef float2 Vec; typedef AccF Acc; };
+__device__ __forceinline__ void trd_put(double& p, double x) { p = x; }
+__device__ __forceinline__ void trd_put(float2& p, double x) { ff s = ff_split(x); p = make_float2(s.h, s.l); }
+__device__ __forceinline__ void trd_put(float& p, double x) { p = ff_split(x).h; }
+
+__device__ __forceinline__ unsigned long long trd_clock() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Grid barrier number ep (1, 2, ...): bounded; false when it gave up or an error is recorded.
+__device__ bool trd_barrier(int* bar, int ep, int* st, int* ok_s) {
+  __syncthreads();
+  if (gridDim.x == 1) return true;
+  if (threadIdx.x == 0) {
+    const int target = ep * gridDim.x;
+    int v, ok = 1;
+    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned long long t0 = 0;
+    for (int it = 0;; ++it) {
+      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v >= target) break;
+      if ((it & 31) == 31) {
+        if (*(volatile int*)(st + 1) != 0) { ok = 0; break; }
+        const unsigned long long now = trd_clock();
+        if (t0 == 0) t0 = now;
+        if (now - t0 > 4000000000ull) {
+          atomicExch(st + 1, GEP_ERR_TIMEOUT);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    *ok_s = ok;
+  }
+  __syncthreads();
+  return *ok_s != 0;
+}
+
+__host__ __device__ __forceinline__ size_t trd_align(size_t x) { return (x + 15) & ~(size_t)15; }
+template <class T, int TS>
+size_t trd_smem_bytes(int nt, int rpc, int slots) {
+  return trd_align((size_t)slots * TS * (TS + 1) * sizeof(T)) + trd_align((size_t)(nt + TS) * sizeof(double)) +
+         2 * (size_t)rpc * (NBT + 1) * sizeof(double);
+}
+
+template <class T, int TS>
+__global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
+  typedef typename TrdForm<T>::Vec Vec;
+  typedef typename TrdForm<T>::Acc Acc;
+  constexpr int NQ = TRD_T / TS, CQ = TS / NQ;  // column groups of a tile, columns of a group
+  extern __shared__ __align__(16) unsigned char smt[];
+  T* tile_s = reinterpret_cast<T*>(smt);
+  double* vs = reinterpret_cast<double*>(smt + trd_align((size_t)a.slots * TS * (TS + 1) * sizeof(T)));
+  double* Vr = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(vs) + trd_align((size_t)(a.nt + TS) * sizeof(double)));
+  double* Wr = Vr + (size_t)a.rpc * (NBT + 1);
+  __shared__ Acc redd[NQ][TS], redt[NQ][TS];
+  __shared__ Vec vI[TS], vJ[TS];
+  __shared__ double red[32], tq[2 * NBT], v0[NBT], w0[NBT], sc[4];
+  __shared__ int ok_s;
+  if (status_bad(a.st)) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, k = blockIdx.x, G = gridDim.x;
+  const int nt = a.nt, nb = a.nb, j0 = a.j0, M = a.M;
+  const int row0 = k * a.rpc, nrow = max(0, min(a.rpc, nt - row0));  // rows [row0, row0 + nrow) of the panel's frame
+  // tile index -> (I, J), I >= J, row by row
+  auto tile_ij = [&](int t, int& I, int& J) {
+    I = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+    while ((I + 1) * (I + 2) / 2 <= t) ++I;
+    while (I * (I + 1) / 2 > t) --I;
+    J = t - I * (I + 1) / 2;
+  };
+  auto elem = [&](int I, int J, int r, int c) -> double {  // element (r, c) of tile (I, J), symmetric on the diagonal
+    int lr = I * TS + r, lc = J * TS + c;
+    if (lr >= nt || lc >= nt) return 0.0;
+    if (lr < lc) { const int q = lr; lr = lc; lc = q; }
+    return a.C[GEP_IX(j0 + lr, j0 + lc, a.ldc)];
+  };
+  auto load_tile = [&](int I, int J, T* ts) {
+    for (int idx = tid; idx < TS * TS; idx += TRD_T) trd_put(ts[(idx / TS) * (TS + 1) + idx % TS], elem(I, J, idx % TS, idx / TS));
+  };
+  for (int s = 0; s < a.nres; ++s) {
+    const int t = k + s * G;
+    if (t >= a.tiles) break;
+    int I, J;
+    tile_ij(t, I, J);
+    load_tile(I, J, tile_s + (size_t)s * TS * (TS + 1));
+  }
+  for (int l = tid; l < nt + TS; l += TRD_T) vs[l] = 0.0;
+  for (int lr = tid; lr < nrow; lr += TRD_T) __stcg(a.xbuf + row0 + lr, a.C[GEP_IX(j0 + row0 + lr, j0, a.ldc)]);
+  int ep = 0;
+  // (also: every tile is loaded before the first reflector is stored over its column)
+  if (!trd_barrier(a.bar, ++ep, a.st, &ok_s)) return;
+  for (int i = 0; i < a.nbp; ++i) {
+    const int c = j0 + i;
+    const double* xsrc = a.xbuf + (size_t)(i & 1) * M;
+    if (c == M - 1) {
+      if (k == 0 && tid == 0) a.d[c] = __ldcg(xsrc + i);
+      return;
+    }
+    // ---- A: reflector
+    __syncthreads();
+    double s2 = 0.0;
+    for (int l = i + 2 + tid; l < nt; l += TRD_T) {
+      const double x = __ldcg(xsrc + l);
+      vs[l] = x;
+      s2 = fma(x, x, s2);
+    }
+    double alpha = 0.0, dg = 0.0;
+    if (tid == 0) {
+      alpha = __ldcg(xsrc + i + 1);
+      dg = __ldcg(xsrc + i);
+    }
+    s2 = warp_sum(s2);
+    if (lane == 0) red[warp] = s2;
+    __syncthreads();
+    if (tid == 0) {
+      double s = 0.0;
+#pragma unroll
+      for (int q = 0; q < TRD_T / 32; ++q) s += red[q];
+      double tv = 0.0, beta = alpha, scal = 0.0;
+      if (s != 0.0) {
+        const double nrm = sqrt(fma(alpha, alpha, s));
+        beta = alpha >= 0.0 ? -nrm : nrm;
+        scal = 1.0 / (alpha - beta);
+        tv = (beta - alpha) / beta;
+      }
+      sc[0] = tv;
+      sc[1] = scal;
+      sc[2] = beta;
+      if (k == 0) {
+        a.d[c] = dg;
+        a.e[c] = beta;
+        a.tau[c] = tv;
+      }
+    }
+    __syncthreads();
+    const double tv = sc[0], scal = sc[1];
+    for (int l = i + 2 + tid; l < nt; l += TRD_T) vs[l] *= scal;
+    if (tid == 0) {
+      vs[i + 1] = 1.0;
+      vs[i] = 0.0;
+    }
+    __syncthreads();
+    for (int lr = tid; lr < nrow; lr += TRD_T) {
+      const int l = row0 + lr;
+      const double v = vs[l];
+      Vr[lr * (NBT + 1) + i] = v;
+      a.Vp[GEP_IX(j0 + l, i, M)] = v;
+      if (l <= i) {
+        Wr[lr * (NBT + 1) + i] = 0.0;
+        a.W[GEP_IX(j0 + l, i, M)] = 0.0;
+      } else {
+        a.C[GEP_IX(j0 + l, c, a.ldc)] = l == i + 1 ? sc[2] : v;
+      }
+    }
+    // ---- A: partial products of this CTA's tiles
+    double vav = 0.0;
+    for (int s = 0, t = k; t < a.tiles; ++s, t += G) {
+      int I, J;
+      tile_ij(t, I, J);
+      if ((I + 1) * TS - 1 <= i) continue;  // (all its rows are done)
+      T* ts = tile_s + (size_t)min(s, a.nres) * TS * (TS + 1);
+      // tiles that do not fit are brought in again for every column (columns already overwritten
+      // by reflectors meet zeros of v)
+      if (s >= a.nres) load_tile(I, J, ts);
+      if (tid < TS) trd_put(vJ[tid], vs[J * TS + tid]);
+      else if (tid < 2 * TS) trd_put(vI[tid - TS], vs[I * TS + tid - TS]);
+      __syncthreads();
+      const int p = tid % TS, q = tid / TS;
+      Acc dr, tr;
+#pragma unroll
+      for (int u = 0; u < CQ; ++u) dr.add(ts[(q * CQ + u) * (TS + 1) + p], vJ[q * CQ + u]);
+      if (I != J) {
+#pragma unroll
+        for (int u = 0; u < CQ; ++u) tr.add(ts[p * (TS + 1) + q * CQ + u], vI[q * CQ + u]);
+      }
+      redd[q][p] = dr;
+      redt[q][p] = tr;
+      __syncthreads();
+      if (tid < 2 * TS) {
+        const bool direct = tid < TS;
+        const int r = direct ? tid : tid - TS;
+        double s0 = 0.0;
+#pragma unroll
+        for (int u = 0; u < NQ; ++u) s0 += direct ? redd[u][r].get() : redt[u][r].get();
+        const int l = (direct ? I : J) * TS + r;
+        if (l < nt && (direct || I != J)) {
+          __stcg(a.P + (size_t)(direct ? J : I) * nt + l, s0);
+          if (direct) vav = fma(s0 * (I == J ? 1.0 : 2.0), vs[l], vav);
+        }
+      }
+    }
+    // ---- A: t1 = W^T v (q < i), t2 = V^T v (q >= i)
+    auto colq = [&](int q) { return (q < i ? a.W + (size_t)q * M : a.Vp + (size_t)(q - i) * M) + j0; };
+    if (2 * i <= 2 * G) {  // at most two dots a CTA: the whole CTA on each
+      for (int q = k; q < 2 * i; q += G) {
+        const double* col = colq(q);
+        double s = 0.0;
+        for (int l = i + 1 + tid; l < nt; l += TRD_T) s = fma(__ldcg(col + l), vs[l], s);
+        s = warp_sum(s);
+        __syncthreads();
+        if (lane == 0) red[warp] = s;
+        __syncthreads();
+        if (tid == 0) {
+          double z = 0.0;
+#pragma unroll
+          for (int u = 0; u < TRD_T / 32; ++u) z += red[u];
+          __stcg(a.t + q, z);
+        }
+      }
+    } else {
+      for (int q = k + warp * G; q < 2 * i; q += G * (TRD_T / 32)) {
+        const double* col = colq(q);
+        double s = 0.0;
+        for (int l = i + 1 + lane; l < nt; l += 32) s = fma(__ldcg(col + l), vs[l], s);
+        s = warp_sum(s);
+        if (lane == 0) __stcg(a.t + q, s);
+      }
+    }
+    vav = warp_sum(vav);  // (threads beyond 2 TS hold zeros)
+    __syncthreads();
+    if (lane == 0) red[warp] = vav;
+    __syncthreads();
+    if (tid == 0) {
+      double z = 0.0;
+#pragma unroll
+      for (int u = 0; u < TRD_T / 32; ++u) z += red[u];
+      __stcg(a.vav + k, z);
+    }
+    if (!trd_barrier(a.bar, ++ep, a.st, &ok_s)) return;
+    // ---- B: w on the owned rows and on row i + 1
+    if (tid < 2 * i) tq[tid] = __ldcg(a.t + tid);
+    if (tid >= TRD_T - NBT && tid - (TRD_T - NBT) < i) {
+      const int q = tid - (TRD_T - NBT);
+      v0[q] = __ldcg(a.Vp + GEP_IX(c + 1, q, M));
+      w0[q] = __ldcg(a.W + GEP_IX(c + 1, q, M));
+    }
+    double z = 0.0;
+    for (int u = tid; u < G; u += TRD_T) z += __ldcg(a.vav + u);
+    __syncthreads();
+    if (tid < i) z -= 2.0 * tq[tid] * tq[i + tid];
+    z = warp_sum(z);
+    if (lane == 0) red[warp] = z;
+    __syncthreads();
+    if (tid == 0) {
+      double s = 0.0;
+#pragma unroll
+      for (int u = 0; u < TRD_T / 32; ++u) s += red[u];
+      sc[3] = -0.5 * tv * (tv * s);
+    }
+    __syncthreads();
+    const double al2 = sc[3];
+    const bool next = i + 1 < a.nbp;
+    const int sub = tid % LPR, grp = tid / LPR;
+    constexpr int GR = TRD_T / LPR - 1;  // owned rows per pass; the last group forms row i + 1
+    for (int b0 = 0; b0 == 0 || b0 < nrow; b0 += GR) {
+      const bool first = grp == GR;
+      const int lr = b0 + grp, l = first ? i + 1 : row0 + lr;
+      const bool act = first ? b0 == 0 : (lr < nrow && l > i);
+      double s = 0.0;
+      if (act) {
+        const double* Vq = first ? v0 : Vr + lr * (NBT + 1);
+        const double* Wq = first ? w0 : Wr + lr * (NBT + 1);
+        for (int q = sub; q < nb; q += LPR) s += __ldcg(a.P + (size_t)q * nt + l);
+        for (int q = sub; q < i; q += LPR) s -= fma(Vq[q], tq[q], Wq[q] * tq[i + q]);
+      }
+      for (int o = LPR / 2; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (act && sub == 0) {
+        const double wv = fma(tv, s, al2 * vs[l]);
+        if (first) {
+          v0[i] = 1.0;
+          w0[i] = wv;
+        } else {
+          Wr[lr * (NBT + 1) + i] = wv;
+          a.W[GEP_IX(j0 + l, i, M)] = wv;
+        }
+      }
+    }
+    if (!next) break;
+    __syncthreads();
+    // ---- B: the owned rows of the next column
+    double* xdst = a.xbuf + (size_t)((i + 1) & 1) * M;
+    for (int b0 = 0; b0 < nrow; b0 += GR + 1) {
+      const int lr = b0 + grp, l = row0 + lr;
+      const bool act = lr < nrow && l > i;
+      double s = 0.0;
+      if (act)
+        for (int q = sub; q <= i; q += LPR) s = fma(Vr[lr * (NBT + 1) + q], w0[q], fma(Wr[lr * (NBT + 1) + q], v0[q], s));
+      for (int o = LPR / 2; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (act && sub == 0) __stcg(xdst + l, a.C[GEP_IX(j0 + l, c + 1, a.ldc)] - s);
+    }
+    if (!trd_barrier(a.bar, ++ep, a.st, &ok_s)) return;
+  }
+}
+
+// Launch of one panel: tile size, CTAs and resident tiles for the trailing order nt.
+template <class T, int TS>
+int trd_panel_launch(gep_handle_t h, TrdArgs a) {
+  a.nb = (a.nt + TS - 1) / TS;
+  a.tiles = a.nb * (a.nb + 1) / 2;
+  // float pairs: two tiles a CTA (a second tile costs less than a wider barrier); FP64 tiles: one
+  int G = a.tiles <= 3 ? 1 : std::is_same<T, double>::value ? a.tiles : (a.tiles + 1) / 2;
+  if (G > h->sm_count) G = h->sm_count;
+  a.rpc = (a.nt + G - 1) / G;
+  const int per = (a.tiles + G - 1) / G;
+  a.nres = per;
+  const size_t cap = (size_t)200 << 10;  // 227 KB less the static arrays
+  int slots = per;
+  while (slots > 1 && trd_smem_bytes<T, TS>(a.nt, a.rpc, slots) > cap) --slots;
+  if (slots < per) a.nres = slots - 1;  // the last slot takes the tiles that do not stay
+  a.slots = slots;
+  const size_t smem = trd_smem_bytes<T, TS>(a.nt, a.rpc, slots);
+  if (smem > cap) return GEP_ERR_UNSUPPORTED;
+  static unsigned long long devices = 0;
+  if (first_use_on_device(devices))
+    GEP_CUDA(cudaFuncSetAttribute(k_trd_panel<T, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
+  GEP_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(int), h->stream));
+  void* args[] = {&a};
+  GEP_CUDA(cudaLaunchCooperativeKernel((void*)k_trd_panel<T, TS>, dim3(G), dim3(TRD_T), args, smem, h->stream));
+  return check_launch(h);
+}
+
+template <class T>
+int trd_panel(gep_handle_t h, const TrdArgs& a) {
+  return a.nt >= 768 ? trd_panel_launch<T, 64>(h, a) : trd_panel_launch<T, 32>(h, a);
+}
+
+// Partial sums of the one-launch panel: one row of nt values per tile row.
+size_t trd_p_elems(int M) {
+  const size_t m = M < TRD_COOP_MAX ? M : TRD_COOP_MAX;
+  return m < 768 ? m * ((m + 31) / 32) : m * ((m + 63) / 64) + 768 * 24;
+}
+
 TWs carve(double* ws, int M) {
   TWs t;
   t.M = M;
@@ -496,8 +876,12 @@ TWs carve(double* ws, int M) {
   t.part = take((size_t)t.ndch * 2 * NBT);
   t.part2 = take((size_t)(M + 255) / 256 + 1);
   t.WV = take((size_t)M * 2 * NBT);
-  t.S2 = (float2*)take((size_t)M * M);
+  t.S2 = (float2*)take(M > TRD_COOP_MAX ? (size_t)M * M : 0);
   t.tq = take((size_t)2 * NBT);
+  t.P = take(trd_p_elems(M));
+  t.vav = take(1024);
+  t.xbuf = take((size_t)2 * M);
+  t.bar = (int*)take(32);
   return t;
 }
 
@@ -507,7 +891,8 @@ size_t tridiag_ws_elems(int M) {
   size_t nblk = (M + SW - 1) / SW, maxch = (M + SCH - 1) / SCH, ndch = (M + DCH - 1) / DCH;
   auto r = [](size_t n) { return (n + 31) & ~(size_t)31; };
   return r((size_t)M * NBT) * 2 + r(M) + r(nblk * M) + r(nblk * maxch * SW) + r(ndch * 2 * NBT) +
-         r((M + 255) / 256 + 1) + r((size_t)M * 2 * NBT) + r((size_t)M * M) + r(2 * NBT);
+         r((M + 255) / 256 + 1) + r((size_t)M * 2 * NBT) + r(M > TRD_COOP_MAX ? (size_t)M * M : 0) + r(2 * NBT) +
+         r(trd_p_elems(M)) + r(1024) + r((size_t)2 * M) + r(32);
 }
 
 int tridiag_1stage(gep_handle_t h, int M, double* C, int ldc, double* d, double* e, double* tau,
@@ -526,7 +911,15 @@ int tridiag_1stage(gep_handle_t h, int M, double* C, int ldc, double* d, double*
   for (int j0 = 0; j0 < M; j0 += NBT) {
     int nbp = min(NBT, M - j0);
     int done = 0;
-    if (pairs && M - j0 > 1) {
+    const bool coop = M - j0 <= TRD_COOP_MAX;
+    if (coop) {
+      TrdArgs a;
+      a.M = M; a.j0 = j0; a.nbp = nbp; a.nt = M - j0; a.ldc = ldc;
+      a.C = C; a.d = d; a.e = e; a.tau = tau; a.Vp = t.Vp; a.W = t.W; a.P = t.P; a.t = t.tq; a.vav = t.vav;
+      a.xbuf = t.xbuf; a.bar = t.bar; a.st = h->d_status;
+      GEP_CHECK(single ? trd_panel<float>(h, a) : pairs ? trd_panel<float2>(h, a) : trd_panel<double>(h, a));
+      done = j0 + nbp >= M;
+    } else if (pairs) {
       int nt = M - j0;
       dim3 g((nt + 255) / 256, nt < 65535 ? nt : 65535);
       if (single)
@@ -535,7 +928,7 @@ int tridiag_1stage(gep_handle_t h, int M, double* C, int ldc, double* d, double*
         k_to_ff<float2><<<g, 256, 0, s>>>(nt, C + GEP_IX(j0, j0, ldc), ldc, t.S2 + GEP_IX(j0, j0, M), M, st);
       GEP_CHECK(check_launch(h));
     }
-    for (int i = 0; i < nbp; ++i) {
+    for (int i = 0; i < (coop ? 0 : nbp); ++i) {
       int c = j0 + i;
       // (columns i > 0 of the panel were already updated by the previous column's k_w_finish)
       if (c == M - 1) {
