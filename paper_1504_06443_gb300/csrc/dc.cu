@@ -772,32 +772,169 @@ __global__ void k_gersh(int M, const double* __restrict__ d, const double* __res
   }
 }
 
-// Sturm count: eigenvalues of T strictly below x (signs of the LDL^T pivots of T - xI).
-__device__ int sturm(int M, const double* __restrict__ d, const double* __restrict__ e, double x) {
+// Sturm count: eigenvalues of T strictly below x, the sign changes of the leading minors
+//     p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1}
+// of T - xI with T scaled by a power of two to norm at most 1: three FP64 instructions a row
+// instead of a division (565 clocks) in the chain of pivots; the same rounding errors per row,
+// so the same backward error.  A zero minor counts as a sign change (the pivot of -0), and the
+// pair is scaled up again, exactly, before it can underflow (one row grows it at most 3-fold).
+// PRE: d and e hold the scaled diagonal and the squares of the scaled off-diagonal.
+struct SturmState {
+  double p = 1.0, pp = 0.0;
   int cnt = 0;
-  double q = 1.0;
-  for (int i = 0; i < M; ++i) {
-    double off = (i > 0) ? e[i - 1] * e[i - 1] / q : 0.0;
-    q = (d[i] - x) - off;
-    if (q == 0.0) q = -0x1p-1000;
-    cnt += (q < 0.0);
+};
+
+// One row, with every special case.
+__device__ __forceinline__ void sturm_row(SturmState& s, double t, double e2) {
+  double pn = fma(t, s.p, -(e2 * s.pp));
+  const int hp = __double2hiint(s.p);
+  int hn = __double2hiint(pn);
+  if (((hn & 0x7fffffff) | __double2loint(pn)) == 0) {  // zero: a tiny value of the other sign
+    pn = __hiloint2double((~hp & 0x80000000) | ((hp & 0x7ff00000) - (200 << 20)), 0);
+    hn = __double2hiint(pn);
   }
-  return cnt;
+  s.cnt += (unsigned)(hn ^ hp) >> 31;
+  s.pp = s.p;
+  s.p = pn;
+  const int E = hn & 0x7ff00000;
+  if (E < 0x3ff00000 - (300 << 20) || E > 0x3ff00000 + (300 << 20)) {
+    const double f = E > 0x3ff00000 ? 0x1p-300 : (E == 0 ? 0x1p600 : 0x1p300);
+    s.p *= f;
+    s.pp *= f;
+  }
 }
 
-// w[k], k < n: the (k+1)-th smallest eigenvalue of T (order M) by bisection on Sturm counts.
-__global__ void k_bisect(int n, int M, const double* __restrict__ d, const double* __restrict__ e,
-                         const double* __restrict__ gb, double* __restrict__ w, const int* st) {
-  if (status_bad(st)) return;
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  double a = gb[0], b = gb[1];
-  for (int it = 0; it < 200; ++it) {
-    double mid = 0.5 * (a + b);
-    if (mid <= a || mid >= b) break;
-    if (sturm(M, d, e, mid) > k) b = mid; else a = mid;
+// Rows are taken 32 at a time, their data spread over the lanes (the next 32 are on the way), and
+// in blocks of 8 without any check but the smallest exponent met: a block that met one below
+// 2^-400 (or a zero) is done again row by row.  Every lane of the warp calls this together.
+template <bool PRE>
+__device__ int sturm(int M, const double* __restrict__ d, const double* __restrict__ e, double x, double sc) {
+  const int lane = threadIdx.x & 31;
+  SturmState s;
+  auto row = [&](int i, double& dv, double& ev) {
+    dv = i < M ? d[i] : 0.0;
+    ev = i > 0 && i < M ? e[i - 1] : 0.0;
+    if (!PRE) {
+      dv *= sc;
+      ev *= sc;
+      ev *= ev;
+    }
+  };
+  double dn, en;
+  row(lane, dn, en);
+  for (int i0 = 0; i0 < M; i0 += 32) {
+    const double dv = dn, ev = en;
+    row(i0 + 32 + lane, dn, en);
+#pragma unroll
+    for (int b = 0; b < 32; b += 8) {
+      const SturmState s0 = s;
+      unsigned emin = 0xffffffffu;
+      if (i0 + b + 8 <= M) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const double t = __shfl_sync(0xffffffffu, dv, b + u) - x, e2 = __shfl_sync(0xffffffffu, ev, b + u);
+          const double pn = fma(t, s.p, -(e2 * s.pp));
+          const int hn = __double2hiint(pn);
+          s.cnt += (unsigned)(hn ^ __double2hiint(s.p)) >> 31;
+          emin = min(emin, (unsigned)hn & 0x7ff00000u);
+          s.pp = s.p;
+          s.p = pn;
+        }
+        // (8 rows grow the pair at most 2^13-fold: no block overflows from 2^300)
+        const int E = __double2hiint(s.p) & 0x7ff00000;
+        if (E > 0x3ff00000 + (300 << 20)) {
+          s.p *= 0x1p-300;
+          s.pp *= 0x1p-300;
+        }
+      } else {
+        emin = 0;
+      }
+      if (__any_sync(0xffffffffu, emin < 0x3ff00000u - (400u << 20))) {
+        s = s0;
+        for (int u = 0; u < 8 && i0 + b + u < M; ++u)
+          sturm_row(s, __shfl_sync(0xffffffffu, dv, b + u) - x, __shfl_sync(0xffffffffu, ev, b + u));
+      }
+    }
   }
-  w[k] = 0.5 * (a + b);
+  return s.cnt;
+}
+
+// d and e scaled to norm at most 1 (a power of two), e squared.
+__device__ __forceinline__ double bisect_scale(const double* gb) {
+  const int E = (int)((__double_as_longlong(fmax(fabs(gb[0]), fabs(gb[1]))) >> 52) & 0x7ff);
+  const int k = max(1, min(2046, 2045 - E));  // 2^(1022 - E): norm into [1/2, 1)
+  return __longlong_as_double((long long)k << 52);
+}
+__global__ void k_bisect_prep(int M, const double* __restrict__ d, const double* __restrict__ e,
+                              const double* __restrict__ gb, double* __restrict__ ds, double* __restrict__ e2,
+                              const int* st) {
+  if (status_bad(st)) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= M) return;
+  const double sc = bisect_scale(gb);
+  ds[i] = d[i] * sc;
+  const double es = i + 1 < M ? e[i] * sc : 0.0;
+  e2[i] = es * es;
+}
+
+// w[k], k < n: the (k+1)-th smallest eigenvalue of T (order M) by multisection on Sturm counts:
+// a group of K lanes evaluates K interior points of the bracket at once (log2(K + 1) bits a
+// count), K chosen so that every SM's four schedulers have a warp.  The first brackets come from
+// the counts of a uniform grid (k_bisect_grid).
+template <bool PRE>
+__global__ void __launch_bounds__(32) k_bisect(int n, int M, int K, const double* __restrict__ d,
+                                               const double* __restrict__ e, const double* __restrict__ gb,
+                                               const int* __restrict__ grid_cnt, int ngrid,
+                                               double* __restrict__ w, const int* st) {
+  if (status_bad(st)) return;
+  const int lane = threadIdx.x, sub = lane % K, per = 32 / K;
+  const int k = blockIdx.x * per + lane / K;
+  const double sc = bisect_scale(gb);
+  double a = gb[0] * sc, b = gb[1] * sc;
+  const bool live = k < n;
+  if (live && ngrid > 0) {  // the grid cell that holds eigenvalue k: counts ascend along the grid
+    int lo = 0, hi = ngrid;  // first grid point with a count above k
+    while (lo < hi) {
+      const int m = (lo + hi) >> 1;
+      if (grid_cnt[m] > k) hi = m; else lo = m + 1;
+    }
+    const double h = (b - a) / (ngrid + 1), a0 = a, b0 = b;
+    if (lo < ngrid) b = fma(h, lo + 1.0, a0);
+    if (lo > 0) a = fma(h, (double)lo, a0);
+    if (!(b <= b0)) b = b0;
+  }
+  const unsigned gmask = K == 32 ? 0xffffffffu : ((1u << K) - 1u) << (lane / K * K);
+  for (int it = 0; it < 200; ++it) {
+    const double mid = 0.5 * (a + b);
+    const bool done = !live || mid <= a || mid >= b;
+    if (__all_sync(0xffffffffu, done)) break;
+    double x = K == 1 ? mid : fma((b - a) / (K + 1), sub + 1.0, a);
+    if (x <= a || x >= b) x = mid;
+    const bool above = sturm<PRE>(M, d, e, x, sc) > k;
+    const unsigned m = __ballot_sync(0xffffffffu, above) & gmask;
+    const int first = m ? __ffs(m) - 1 : -1;  // lowest point above eigenvalue k
+    const double xb = __shfl_sync(0xffffffffu, x, first < 0 ? lane : first);
+    const int below = first < 0 ? (lane / K * K + K - 1) : first - 1;
+    const double xa = __shfl_sync(0xffffffffu, x, below < 0 ? 0 : below);
+    if (!done) {
+      if (first >= 0) b = xb;
+      if (below >= lane / K * K) a = fmax(a, xa);
+      if (a > b) a = b;
+    }
+  }
+  if (live && sub == 0) w[k] = (0.5 * (a + b)) / sc;
+}
+
+// Sturm counts at ngrid points of a uniform grid inside the Gershgorin interval.
+template <bool PRE>
+__global__ void __launch_bounds__(32) k_bisect_grid(int M, const double* __restrict__ d, const double* __restrict__ e,
+                                                    const double* __restrict__ gb, int* __restrict__ cnt, int ngrid,
+                                                    const int* st) {
+  if (status_bad(st)) return;
+  const int g = blockIdx.x * 32 + threadIdx.x;
+  const double sc = bisect_scale(gb), a = gb[0] * sc, b = gb[1] * sc, h = (b - a) / (ngrid + 1);
+  const int c = sturm<PRE>(M, d, e, fma(h, g + 1.0, a), sc);
+  if (g < ngrid) cnt[g] = c;
 }
 
 }  // namespace
@@ -809,7 +946,27 @@ int tridiag_eig_bisect(gep_handle_t h, int M, const double* d, const double* e, 
   double* gb = (double*)(h->d_status + 8);  // two doubles of the handle's status block
   k_gersh<<<1, 1024, 0, h->stream>>>(M, d, e, gb);
   GEP_CHECK(check_launch(h));
-  k_bisect<<<(n + 127) / 128, 128, 0, h->stream>>>(n, M, d, e, gb, w, h->d_status);
+  // four warps an SM (one a scheduler) are free of charge: their lanes share the eigenvalues
+  const int lanes = 4 * 32 * h->sm_count;
+  int K = 1;
+  while (K < 32 && (long long)2 * K * n <= lanes) K *= 2;
+  const int blocks = (n + 32 / K - 1) / (32 / K);
+  // scratch of the split FP64 products: scaled diagonal, squared off-diagonal, grid counts
+  const size_t need = 2 * (size_t)M + (lanes + 1) / 2;
+  if (h->d_splitk && need <= SPLITK_DOUBLES) {
+    double *ds = h->d_splitk, *e2 = ds + M;
+    int* cnt = (int*)(e2 + M);
+    const int ng = n > 64 ? lanes : 0;
+    k_bisect_prep<<<(M + 255) / 256, 256, 0, h->stream>>>(M, d, e, gb, ds, e2, h->d_status);
+    GEP_CHECK(check_launch(h));
+    if (ng) {
+      k_bisect_grid<true><<<lanes / 32, 32, 0, h->stream>>>(M, ds, e2, gb, cnt, ng, h->d_status);
+      GEP_CHECK(check_launch(h));
+    }
+    k_bisect<true><<<blocks, 32, 0, h->stream>>>(n, M, K, ds, e2, gb, cnt, ng, w, h->d_status);
+    return check_launch(h);
+  }
+  k_bisect<false><<<blocks, 32, 0, h->stream>>>(n, M, K, d, e, gb, nullptr, 0, w, h->d_status);
   return check_launch(h);
 }
 

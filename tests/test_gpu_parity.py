@@ -330,3 +330,40 @@ def test_dc_leaf_and_level_edges(gep, oracle_lib, name, d, e):
     assert np.max(np.abs(wh - w_ref)) <= 64 * M * EPS * nT
     assert np.max(np.abs(Zh.T @ Zh - np.eye(M))) <= 64 * M * EPS
     assert np.max(np.abs(T @ Zh - Zh * wh[None, :])) <= 64 * M * EPS * nT
+
+
+def _bisection_cases():
+    rng = np.random.default_rng(21)
+    cases = []
+    for M in (1, 2, 5, 63, 65, 300, 1300):
+        cases.append((f"random{M}", rng.standard_normal(M), rng.standard_normal(M - 1)))
+    n = 200
+    i = np.arange(n)
+    cases.append(("diagonal", 10.0 ** rng.uniform(-9, 3, n) * rng.choice([-1, 1], n), np.zeros(n - 1)))
+    cases.append(("zero", np.zeros(n), np.zeros(n - 1)))
+    cases.append(("zero_pivots", np.zeros(n), np.ones(n - 1)))                       # minors that vanish
+    cases.append(("singular", np.where(i % 2, 2.0, 0.0), np.where(i[:-1] % 2, 0.0, 1e-8)))
+    cases.append(("tiny", rng.standard_normal(n) * 1e-290, rng.standard_normal(n - 1) * 1e-290))
+    cases.append(("huge", rng.standard_normal(n) * 1e290, rng.standard_normal(n - 1) * 1e290))
+    cases.append(("steep", 10.0 ** (-i * 1.2), 10.0 ** (-i[:-1] * 1.2 - 0.6)))        # underflowing products
+    cases.append(("weak", rng.standard_normal(n), np.where(rng.random(n - 1) < 0.5, 1e-170, 1e-9)))
+    cases.append(("equal", np.full(n, 7.0), np.full(n - 1, 1e-15)))
+    return cases
+
+
+# Multisection on division-free Sturm counts: each count is exact for a matrix within a few eps of T,
+# so an eigenvalue is within a few eps of the norm (the oracle's own bound is the same).
+@pytest.mark.parametrize("name,d,e", _bisection_cases(), ids=lambda x: x if isinstance(x, str) else "")
+def test_bisection_vs_oracle(gep, oracle_lib, name, d, e):
+    # the oracle squares e as it stands: it is given T scaled by an exact power of two
+    top = max(np.max(np.abs(d), initial=0.0), np.max(np.abs(e), initial=0.0))
+    k = int(np.frexp(top)[1]) if top > 0 else 0
+    ref = np.ldexp(oracle_lib.bisect(np.ldexp(d, -k), np.ldexp(e, -k)), k)
+    nT = max(np.max(np.abs(ref)), 1e-300)
+    w, Z, info = gep.tridiag_eig(dev(d), dev(e), want_vectors=False)
+    assert info == 0 and Z is None
+    wh = host(w)
+    assert np.all(np.diff(wh) >= -16 * EPS * nT)
+    assert np.max(np.abs(wh - ref)) <= 64 * EPS * nT
+    if name == "diagonal":
+        assert np.max(np.abs(wh - np.sort(d)) / np.abs(np.sort(d))) <= 4 * EPS
