@@ -283,6 +283,246 @@ __global__ void __launch_bounds__(PQ_ROWS) k_pqr_coop(int n, int nb, int rp, dou
 
 size_t pqr_coop_smem_bytes(int rp, int nb) { return (size_t)rp * (nb + 1) * sizeof(double); }
 
+// ---- panel QR of at most 32 columns, registers only, with its T factor
+//
+// One cooperative launch: warp w of a CTA holds RPW consecutive rows of the panel, lane j column j,
+// so that a column's update and the next column's dot products are one FMA each per row of a
+// warp (an FP64 instruction holds a scheduler 64 clocks whatever its lanes do) and the entries
+// of the pivot column reach the lanes by shuffle.  Per column one grid barrier carries the
+// partial dots of the next pivot column with all columns: those to its right give w = v^T P, those
+// to its left the Gram entries v_q^T v of the T factor, which a ninth warp of CTA 0 accumulates
+// beside the others.  The results go where the two-sided update reads them: P (R and the
+// reflectors), both group buffers of V at full height (zero rows above), T.
+//
+// Bound: the barrier (1.2 us), the partial sums (G / 8 adds a thread) and the scalars' chain.
+// Rows per CTA balance row work against partial sums: 304 RPW + 2.4 n / RPW clocks, least at
+// RPW = sqrt(n / 127).  Measured per panel of 32 columns with everything up to W (before: QR, V, Gram
+// product, T, four copies and four products in 14 launches): order 2047 460 -> 305 us, S1b 29.8 ->
+// 19.6 ms; order 8192 224 -> 184 ms.
+constexpr int PQN = 32;        // columns, one per lane
+constexpr int PQW = 8;         // row warps
+struct PanelArgs {
+  int n, nb, ldp, r0, ldv;  // r0: zero rows above the panel in Va, Vb
+  double *P, *tau, *part, *prow, *Va, *Vb, *T;
+  int *bar, *st;
+};
+
+template <int RPW>
+__global__ void __launch_bounds__(32 * (PQW + 1)) k_panel_qr(PanelArgs a) {
+  constexpr int ROWS = PQW * RPW;
+  __shared__ double tile[PQN][ROWS + 1];
+  __shared__ double red[PQW][PQN], hv[PQN], cv[PQN], gb[2][PQN], ts[2];
+  __shared__ double Ts[PQN][PQN + 1];
+  __shared__ int ok_s;
+  if (status_bad(a.st)) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, blk = blockIdx.x, G = gridDim.x;
+  const int n = a.n, nb = a.nb, rb = blk * ROWS;
+  const int nref = n < nb ? n : nb;
+  const bool worker = warp < PQW;
+  auto work_sync = [&]() { asm volatile("bar.sync 1, %0;" ::"n"(32 * PQW) : "memory"); };
+  for (int idx = tid; idx < ROWS * PQN; idx += blockDim.x) {
+    const int r = idx % ROWS, j = idx / ROWS;
+    tile[j][r] = rb + r < n && j < nb ? a.P[rb + r + (size_t)j * a.ldp] : 0.0;
+  }
+  for (int idx = tid; idx < PQN * (PQN + 1); idx += blockDim.x) (&Ts[0][0])[idx] = 0.0;
+  for (int idx = blk * blockDim.x + tid; idx < a.r0 * nb; idx += G * blockDim.x) {
+    const size_t o = (size_t)(idx / a.r0) * a.ldv + idx % a.r0;
+    a.Va[o] = 0.0;
+    a.Vb[o] = 0.0;
+  }
+  __syncthreads();
+  double x[RPW];
+  const int row0 = rb + warp * RPW;
+#pragma unroll
+  for (int u = 0; u < RPW; ++u) x[u] = worker ? tile[lane][warp * RPW + u] : 0.0;
+  for (int c = -1; c < nref; ++c) {
+    double *pin = a.part + (size_t)(c & 1) * G * PQN, *pout = a.part + (size_t)((c + 1) & 1) * G * PQN;
+    double *rin = a.prow + (c & 1) * PQN, *rout = a.prow + ((c + 1) & 1) * PQN;
+    if (c >= 0) {
+      if (worker) {
+        double s0 = 0.0, s1 = 0.0;
+        int g = warp;
+        for (; g + 3 * PQW < G; g += 4 * PQW) {
+          const double p0 = __ldcg(pin + (size_t)g * PQN + lane), p1 = __ldcg(pin + (size_t)(g + PQW) * PQN + lane);
+          const double p2 = __ldcg(pin + (size_t)(g + 2 * PQW) * PQN + lane), p3 = __ldcg(pin + (size_t)(g + 3 * PQW) * PQN + lane);
+          s0 += p0; s1 += p1; s0 += p2; s1 += p3;
+        }
+        for (; g < G; g += PQW) s0 += __ldcg(pin + (size_t)g * PQN + lane);
+        red[warp][lane] = s0 + s1;
+        const double pr = warp == 0 ? __ldcg(rin + lane) : 0.0;
+        work_sync();
+        if (warp == 0) {
+          double s = ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane])) +
+                     ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
+          const double xn2 = __shfl_sync(0xffffffffu, s, c), alpha = __shfl_sync(0xffffffffu, pr, c);
+          double tt = 0.0, sl = 0.0, be = alpha;
+          if (xn2 > 0.0) {
+            const double n2 = fma(alpha, alpha, xn2);
+            const double ri = rsqrt(n2);
+            be = -copysign(n2 * ri, alpha);
+            sl = 1.0 / (alpha - be);
+            tt = fma(fabs(alpha), ri, 1.0);
+          }
+          const double wj = fma(sl, s, pr);  // v^T P(:, j); for j < c the Gram entry v_j^T v
+          gb[c & 1][lane] = wj;
+          cv[lane] = lane > c ? -(tt * wj) : 0.0;               // pivot row: P(c, j) -= tau w_j
+          hv[lane] = lane > c ? -(sl * (tt * wj)) : (lane == c ? sl : 0.0);  // rows below: += P(r, c) h_j
+          if (lane == 0) {
+            ts[0] = tt;
+            ts[1] = be;
+            if (blk == 0) a.tau[c] = tt;
+          }
+        }
+      }
+      __syncthreads();
+      if (worker) {
+        const double h = hv[lane];
+#pragma unroll
+        for (int u = 0; u < RPW; ++u) {
+          const int r = row0 + u;
+          if (r > c) {
+            const double xc = __shfl_sync(0xffffffffu, x[u], c);
+            x[u] = fma(xc, h, lane == c ? 0.0 : x[u]);
+          } else if (r == c) {
+            x[u] = lane == c ? ts[1] : x[u] + cv[lane];
+          }
+        }
+      } else if (blk == 0) {  // column c of T: T(0:c, c) = -tau T(0:c, 0:c) G(0:c, c)
+        const double tt = ts[0];
+        double s = 0.0;
+        for (int q = 0; q < c; ++q) s = fma(Ts[lane][q], gb[c & 1][q], s);
+        Ts[lane][c] = lane < c ? -tt * s : (lane == c ? tt : 0.0);
+        __syncwarp();
+      }
+    }
+    const int nc = c + 1;
+    if (nc >= nref) break;
+    if (worker) {
+      double s = 0.0;
+#pragma unroll
+      for (int u = 0; u < RPW; ++u) {
+        const int r = row0 + u;
+        if (r > nc) s = fma(__shfl_sync(0xffffffffu, x[u], nc), x[u], s);
+        else if (r == nc) __stcg(rout + lane, x[u]);
+      }
+      red[warp][lane] = s;
+      work_sync();
+      if (warp == 0) {
+        s = ((red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane])) +
+            ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
+        __stcg(pout + (size_t)blk * PQN + lane, s);
+        __syncwarp();
+        if (lane == 0) {
+          int ok = 1;
+          if (G > 1) {
+            asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(a.bar) : "memory");
+            const int target = (nc + 1) * G;
+            unsigned long long t0 = 0;
+            for (int it = 0; ld_acquire(a.bar) < target; ++it) {
+              if ((it & 31) != 31) continue;
+              if (*(volatile int*)(a.st + 1) != 0) { ok = 0; break; }
+              const unsigned long long now = gclock();
+              if (t0 == 0) t0 = now;
+              if (now - t0 > 4000000000ull) {
+                atomicExch(a.st + 1, GEP_ERR_TIMEOUT);
+                ok = 0;
+                break;
+              }
+            }
+          }
+          ok_s = ok;
+        }
+      }
+    }
+    __syncthreads();
+    if (!ok_s) return;
+  }
+  __syncthreads();
+  if (worker)
+#pragma unroll
+    for (int u = 0; u < RPW; ++u) tile[lane][warp * RPW + u] = x[u];
+  __syncthreads();
+  for (int idx = tid; idx < ROWS * nb; idx += blockDim.x) {
+    const int lr = idx % ROWS, j = idx / ROWS, r = rb + lr;
+    if (r >= n) continue;
+    const double p = tile[j][lr], v = r > j ? p : (r == j ? 1.0 : 0.0);
+    a.P[r + (size_t)j * a.ldp] = p;
+    const size_t o = (size_t)j * a.ldv + a.r0 + r;
+    a.Va[o] = v;
+    a.Vb[o] = v;
+  }
+  if (blk == 0)
+    for (int idx = tid; idx < nb * nb; idx += blockDim.x) a.T[idx] = Ts[idx % nb][idx / nb];
+}
+
+// W = (Y - V M) T with Y = C22 V (n x nb), M = T^T S / 2, S = V^T Y: the companion of V in the
+// two-sided update, written to both group buffers at full height.  Lane j owns column j, a warp a
+// row at a time; M is formed by every CTA for itself (a b^3 / 2 product: cheaper than a launch).
+__global__ void __launch_bounds__(256) k_panel_w(int n, int nb, const double* __restrict__ V, int ldv,
+                                                 const double* __restrict__ Y, const double* __restrict__ T,
+                                                 const double* __restrict__ S, double* __restrict__ Wa,
+                                                 double* __restrict__ Wb, int r0, const int* st) {
+  __shared__ double Tm[PQN][PQN + 1], Sm[PQN][PQN + 1], Mm[PQN][PQN + 1];
+  __shared__ double yt[PQN][33], vt[PQN][33];
+  if (status_bad(st)) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int idx = blockIdx.x * blockDim.x + tid; idx < r0 * nb; idx += gridDim.x * blockDim.x) {
+    const size_t o = (size_t)(idx / r0) * ldv + idx % r0;
+    Wa[o] = 0.0;
+    Wb[o] = 0.0;
+  }
+  for (int idx = tid; idx < PQN * PQN; idx += 256) {
+    const int i = idx & 31, j = idx >> 5;
+    const bool in = i < nb && j < nb;
+    Tm[i][j] = in && i <= j ? T[i + j * nb] : 0.0;
+    Sm[i][j] = in ? S[i + j * nb] : 0.0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = warp; i < PQN; i += 8) {
+    double s = 0.0;
+    for (int q = 0; q <= i; ++q) s = fma(Tm[q][i], Sm[q][lane], s);
+    Mm[i][lane] = 0.5 * s;
+  }
+  for (int b0 = blockIdx.x * 32; b0 < n; b0 += gridDim.x * 32) {
+    __syncthreads();
+    for (int idx = tid; idx < 32 * nb; idx += 256) {
+      const int r = b0 + (idx & 31), j = idx >> 5;
+      yt[j][idx & 31] = r < n ? Y[r + (size_t)j * n] : 0.0;
+      vt[j][idx & 31] = r < n ? V[r + (size_t)j * ldv] : 0.0;
+    }
+    __syncthreads();
+    double y[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) y[u] = lane < nb ? yt[lane][warp * 4 + u] : 0.0;
+#pragma unroll 4
+    for (int q = 0; q < nb; ++q) {
+      const double m = Mm[q][lane];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) y[u] = fma(-vt[q][warp * 4 + u], m, y[u]);
+    }
+    double w[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+    for (int q = 0; q < nb; ++q) {
+      const double t = Tm[q][lane];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) w[u] = fma(__shfl_sync(0xffffffffu, y[u], q), t, w[u]);
+    }
+    __syncthreads();
+    if (lane < nb)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) yt[lane][warp * 4 + u] = w[u];
+    __syncthreads();
+    for (int idx = tid; idx < 32 * nb; idx += 256) {
+      const int r = b0 + (idx & 31), j = idx >> 5;
+      if (r >= n) continue;
+      const size_t o = (size_t)j * ldv + r0 + r;
+      Wa[o] = yt[j][idx & 31];
+      Wb[o] = yt[j][idx & 31];
+    }
+  }
+}
+
 // V (n x nb, ld n): unit lower trapezoidal factor of the panel QR stored in P.
 __global__ void k_panel_v(int n, int nb, const double* __restrict__ P, int ldp, double* __restrict__ V,
                           const int* st) {
@@ -1292,6 +1532,41 @@ int panel_factor(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, 
   return larft_rec(h, b, w.GV, b, tau, w.T, b, w.Tt);
 }
 
+// k_panel_qr's launch (b <= 32): V_j into Va and Vb (ld ldv, r0 zero rows first), T into w.T.
+// Returns GEP_ERR_UNSUPPORTED when the grid cannot be resident or its partial sums do not fit.
+template <int RPW>
+int panel_qr_launch(gep_handle_t h, const PanelArgs& a, long long part_elems) {
+  const int G = (a.n + PQW * RPW - 1) / (PQW * RPW);
+  static int per_sm_of[64];
+  static unsigned long long devices = 0;
+  int dev = 0;
+  GEP_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64) return GEP_ERR_UNSUPPORTED;
+  if (first_use_on_device(devices))
+    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_of[dev], k_panel_qr<RPW>, 32 * (PQW + 1), 0));
+  if ((long long)G > (long long)per_sm_of[dev] * h->sm_count || 2LL * G * PQN > part_elems) return GEP_ERR_UNSUPPORTED;
+  GEP_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(int), h->stream));
+  PanelArgs aa = a;
+  void* args[] = {&aa};
+  GEP_CUDA(cudaLaunchCooperativeKernel((void*)k_panel_qr<RPW>, dim3(G), dim3(32 * (PQW + 1)), args, 0, h->stream));
+  return check_launch(h);
+}
+
+int panel_qr(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, const BandWs& w, double* Va, double* Vb,
+             int r0, int ldv) {
+  PanelArgs a;
+  a.n = n; a.nb = b; a.ldp = ldp; a.r0 = r0; a.ldv = ldv;
+  a.P = P; a.tau = tau; a.part = w.part0; a.prow = w.prow0; a.Va = Va; a.Vb = Vb; a.T = w.T;
+  a.bar = w.bar; a.st = h->d_status;
+  const long long cap = 2 * w.gcap * BMAX;  // part0 and part1 together
+  const int rows = n <= 127 * 2 ? 1 : n <= 127 * 8 ? 2 : n <= 127 * 32 ? 4 : n <= 127 * 128 ? 8 : 16;
+  if (rows == 1) return panel_qr_launch<1>(h, a, cap);
+  if (rows == 2) return panel_qr_launch<2>(h, a, cap);
+  if (rows == 4) return panel_qr_launch<4>(h, a, cap);
+  if (rows == 8) return panel_qr_launch<8>(h, a, cap);
+  return panel_qr_launch<16>(h, a, cap);
+}
+
 // W = X - V (T^T V^T X) / 2 with X = CV T (CV = C22 V, n x b): the two-sided update of
 // the trailing matrix is then C22 - W V^T - V W^T.
 int panel_w(gep_handle_t h, int n, int b, const double* V, const double* CV, double* W, const BandWs& w, int eng) {
@@ -1366,10 +1641,9 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
     for (int j = 0; j < g; ++j) {
       const int r0 = j * b, nr = n - r0;  // panel j's reflectors act on rows [r0, n) of C22
       double* Vj;
-      if (j == 0) {
-        GEP_CHECK(panel_factor(h, n, b, P, ldc, tau1 + pb, w, w.V, eng));
-        Vj = w.V;
-      } else {
+      int ldv = nr;
+      double* Pj = P;
+      if (j > 0) {
         // panel j = C22 columns [(j-1) b, j b), rows [(j-1) b, n): the pending updates of
         // panels 0..j-1 first (its diagonal block on the lower triangle only), then its QR
         const int c0 = r0 - b;
@@ -1377,30 +1651,52 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
         GEP_CHECK(dgemm(h, 'N', 'T', 'L', b, b, 2 * j * b, -1.0, w.WV + c0, n, w.VW + c0, n, 1.0, Dj, ldc, eng));
         GEP_CHECK(dgemm(h, 'N', 'T', 'F', nr, b, 2 * j * b, -1.0, w.WV + r0, n, w.VW + c0, n, 1.0, Dj + b, ldc,
                         eng));
-        GEP_CHECK(panel_factor(h, nr, b, Dj + b, ldc, tau1 + pb + r0, w, w.V1, eng));
+        Pj = Dj + b;
+      }
+      int rc = GEP_ERR_UNSUPPORTED;
+      if (b <= PQN && h->pqr_rows == 0) rc = panel_qr(h, nr, b, Pj, ldc, tau1 + pb + r0, w, wv(2 * j + 1), vw(2 * j), r0, n);
+      const bool narrow = rc != GEP_ERR_UNSUPPORTED;  // V_j is in the group buffers
+      if (narrow) {
+        GEP_CHECK(rc);
+        Vj = vw(2 * j) + r0;
+        ldv = n;
+      } else if (j == 0) {
+        GEP_CHECK(panel_factor(h, n, b, P, ldc, tau1 + pb, w, w.V, eng));
+        Vj = w.V;
+      } else {
+        GEP_CHECK(panel_factor(h, nr, b, Pj, ldc, tau1 + pb + r0, w, w.V1, eng));
         Vj = w.V1;
       }
       // V_j at full height into both group buffers (zero rows above r0)
-      if (r0 > 0) {
+      if (!narrow && r0 > 0) {
         GEP_CHECK(set_matrix(h, r0, b, 0.0, 0.0, wv(2 * j + 1), n));
         GEP_CHECK(set_matrix(h, r0, b, 0.0, 0.0, vw(2 * j), n));
         GEP_CHECK(set_matrix(h, r0, b, 0.0, 0.0, wv(2 * j), n));
         GEP_CHECK(set_matrix(h, r0, b, 0.0, 0.0, vw(2 * j + 1), n));
       }
-      GEP_CHECK(copy_matrix(h, nr, b, Vj, nr, wv(2 * j + 1) + r0, n));
-      GEP_CHECK(copy_matrix(h, nr, b, Vj, nr, vw(2 * j) + r0, n));
+      if (!narrow) {
+        GEP_CHECK(copy_matrix(h, nr, b, Vj, nr, wv(2 * j + 1) + r0, n));
+        GEP_CHECK(copy_matrix(h, nr, b, Vj, nr, vw(2 * j) + r0, n));
+      }
       // C^(j) V_j = C22(r0:, r0:) V_j - sum_{i<j} (W_i V_i^T + V_i W_i^T)(r0:, r0:) V_j
       if (use_planes && nr >= 128) {
         GEP_CHECK(dgemm_oz_sym_planes(h, planes, r0, b, 1.0, vw(2 * j), n, 0.0, w.CV, nr));
       } else {
-        GEP_CHECK(dgemm(h, 'S', 'N', 'F', nr, b, nr, 1.0, C22 + r0 + (size_t)r0 * ldc, ldc, Vj, nr, 0.0, w.CV, nr,
+        GEP_CHECK(dgemm(h, 'S', 'N', 'F', nr, b, nr, 1.0, C22 + r0 + (size_t)r0 * ldc, ldc, Vj, ldv, 0.0, w.CV, nr,
                         eng));
       }
       if (j > 0) {
         // Zs = [V_0 W_0 .. V_{j-1} W_{j-1}](r0:)^T V_j, CV -= [W_0 V_0 ..](r0:) Zs
-        GEP_CHECK(dgemm(h, 'T', 'N', 'F', 2 * j * b, b, nr, 1.0, w.VW + r0, n, Vj, nr, 0.0, w.Zs, 2 * j * b, eng));
+        GEP_CHECK(dgemm(h, 'T', 'N', 'F', 2 * j * b, b, nr, 1.0, w.VW + r0, n, Vj, ldv, 0.0, w.Zs, 2 * j * b, eng));
         GEP_CHECK(dgemm(h, 'N', 'N', 'F', nr, b, 2 * j * b, -1.0, w.WV + r0, n, w.Zs, 2 * j * b, 1.0, w.CV, nr,
                         eng));
+      }
+      if (narrow) {
+        GEP_CHECK(dgemm_f64(h, 'T', 'N', 'F', b, b, nr, 1.0, Vj, ldv, w.CV, nr, 0.0, w.Pm, b));  // V^T C22 V
+        k_panel_w<<<std::min((nr + 31) / 32, 2 * h->sm_count), 256, 0, h->stream>>>(
+            nr, b, Vj, ldv, w.CV, w.T, w.Pm, wv(2 * j), vw(2 * j + 1), r0, h->d_status);
+        GEP_CHECK(check_launch(h));
+        continue;
       }
       GEP_CHECK(panel_w(h, nr, b, Vj, w.CV, w.W1, w, eng));
       GEP_CHECK(copy_matrix(h, nr, b, w.W1, nr, wv(2 * j) + r0, n));
