@@ -66,7 +66,7 @@ __device__ __forceinline__ int scale_exp(int m, int xbit) { return m ? m - 1022 
 // largest biased exponent field of the K panel (raw); scale_exp turns it into the scale.
 //
 // raw[r] = max over the K panel of exp_field(X(r, kk)), X(r,kk) = X[r*sr + kk*sk], for an
-// operand whose K is strided (consecutive rows contiguous): block (256 rows, one 128-deep
+// operand whose K is strided (consecutive rows contiguous): block (256 rows, one 32-deep
 // slab of K), atomicMax into raw (zero on entry), so that short-and-wide panels spread over
 // many CTAs.
 __global__ void k_rowexp_slab(int R, int K, const double* __restrict__ X, long long sr, long long sk,
@@ -74,8 +74,9 @@ __global__ void k_rowexp_slab(int R, int K, const double* __restrict__ X, long l
   if (status_bad(st)) return;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
-  const int k0 = blockIdx.y * 128, k1 = min(K, k0 + 128);
+  const int k0 = blockIdx.y * 32, k1 = min(K, k0 + 32);
   int m = 0;
+#pragma unroll 8
   for (int kk = k0; kk < k1; ++kk) m = max(m, exp_field(X[r * sr + kk * sk]));
   if (m) atomicMax(raw + r, m);
 }
@@ -253,6 +254,42 @@ __global__ void __launch_bounds__(256) k_split_row_blk(int R, int K, int Kpad, c
 #pragma unroll
     for (int u = 0; u < 4; ++u) v[u] = (k0 + u < K) ? x[k0 + u] : 0.0;
     split4_store(v, k0, K, e, S, (size_t)r * Kpad + k0, plane, out);
+  }
+}
+
+// The same for an operand whose K is strided (consecutive rows contiguous) and at most FUSE_K deep:
+// one CTA stages ROWS rows with their whole K panel in shared memory, so that the exponent pass,
+// its zeroing memset and the transposing split are one launch that reads the operand once
+// (2000 x 64 and 128 x 128: the three launches took about 20 us, this one 5 us).
+constexpr int FUSE_K = 512;
+template <int ROWS>
+__global__ void __launch_bounds__(256) k_split_cols(int R, int K, int Kpad, const double* __restrict__ X, long long sk,
+                                                    int* __restrict__ e_out, int S, int xbit,
+                                                    unsigned short* __restrict__ out, const int* st) {
+  extern __shared__ double t[];  // [kk][ROWS + 1]
+  __shared__ int mx[ROWS];
+  if (status_bad(st)) return;
+  const int r0 = blockIdx.x * ROWS, tx = threadIdx.x % ROWS, ty = threadIdx.x / ROWS;
+  constexpr int TY = 256 / ROWS, LD = ROWS + 1;
+  if (threadIdx.x < ROWS) mx[threadIdx.x] = 0;
+  const int r = min(r0 + tx, R - 1);
+  int m = 0;
+#pragma unroll 8
+  for (int kk = ty; kk < Kpad; kk += TY) {
+    const double v = kk < K ? X[r + kk * sk] : 0.0;
+    t[kk * LD + tx] = v;
+    m = max(m, exp_field(v));
+  }
+  __syncthreads();
+  atomicMax(&mx[tx], m);
+  __syncthreads();
+  if (threadIdx.x < ROWS && r0 + (int)threadIdx.x < R) e_out[r0 + threadIdx.x] = mx[threadIdx.x];
+  const int q4 = Kpad / 4;
+  for (int idx = threadIdx.x; idx < ROWS * q4; idx += 256) {
+    const int q = idx / q4, c4 = (idx - q * q4) * 4;
+    if (r0 + q >= R) break;
+    double x[4] = {t[c4 * LD + q], t[(c4 + 1) * LD + q], t[(c4 + 2) * LD + q], t[(c4 + 3) * LD + q]};
+    split4_store(x, c4, K, scale_exp(mx[q], xbit), S, (size_t)(r0 + q) * Kpad + c4, (size_t)R * Kpad, out);
   }
 }
 
@@ -437,66 +474,34 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, float* v) {
   else tmem_ld32(taddr, v);
 }
 
-// T = hi * 2^D + lo as a 128-bit two's-complement integer (0 <= D < 64), returned
-// as the double nearest to T * 2^adj (round to nearest even), built with integer
-// operations only: the FP64 pipe of this part is ~60x slower than its integer ALUs.
-// Falls back to FP64 arithmetic when the result would be subnormal or overflow.
-__device__ __forceinline__ double fixed_to_double(long long hi, long long lo, int D, int adj) {
-  unsigned long long tl, th;
-  if (D == 0) {
-    tl = (unsigned long long)hi + (unsigned long long)lo;
-    unsigned long long c = tl < (unsigned long long)hi ? 1ull : 0ull;
-    th = (unsigned long long)(hi >> 63) + (unsigned long long)(lo >> 63) + c;
-  } else {
-    unsigned long long a = (unsigned long long)hi << D;
-    unsigned long long ah = (unsigned long long)(hi >> (64 - D));
-    tl = a + (unsigned long long)lo;
-    unsigned long long c = tl < a ? 1ull : 0ull;
-    th = ah + (unsigned long long)(lo >> 63) + c;
+// Bits of the double nearest to (hi 2^D + lo) 2^adj (0 <= D < 64; the bits beyond the 64 leading
+// ones are dropped before rounding half up: an error of 2^-11 of half a unit), built with integer
+// operations only: an FP64 instruction holds a scheduler 64 clocks, an FP64 compare included, so
+// the whole epilogue has none but the addition of beta C.  With the fused split: 128^3 47 -> 28 us,
+// 2000 x 2000 x 64 101 -> 54 us, 512 x 8192 x 512 180 -> 156 us, 4096^3 3107 -> 3067 us.
+__device__ __forceinline__ long long fixed_to_bits(long long hi, long long lo, int D, int adj) {
+  long long A = hi + (lo >> D);                                          // T = A 2^D + B 2^(D - 64)
+  unsigned long long B = D ? (unsigned long long)lo << (64 - D) : 0ull;  // the low D bits, left-aligned
+  const long long neg = A >> 63;
+  A = (A ^ neg) + (neg != 0 && B == 0 ? 1 : 0);  // magnitude
+  B = (B ^ (unsigned long long)neg) - (unsigned long long)neg;
+  int e = 63 + D + adj;
+  if (A == 0) {  // all of the value lies in B
+    if (B == 0) return 0;
+    A = (long long)(B >> 1);
+    B <<= 63;
+    e -= 63;
+    if (A == 0) { A = 1; B = 0; }
   }
-  unsigned long long sign = th >> 63;
-  if (sign) {  // magnitude of the 128-bit value
-    tl = ~tl + 1ull;
-    th = ~th + (tl == 0ull ? 1ull : 0ull);
+  const int lz = __clzll(A);  // 1 .. 63
+  const unsigned long long m = ((unsigned long long)A << lz) | (B >> (64 - lz));
+  const unsigned long long q = (m >> 11) + ((m >> 10) & 1ull);
+  const int ex = e - lz + 1023;
+  if (ex <= 0 || ex >= 2046) {  // outside the normal range: let FP64 arithmetic handle it
+    const double v = ldexp((double)q, e - lz - 52);
+    return __double_as_longlong(neg ? -v : v);
   }
-  if ((th | tl) == 0ull) return 0.0;
-  int p;  // position of the leading one
-  if (th) p = 127 - __clzll((long long)th);
-  else p = 63 - __clzll((long long)tl);
-  unsigned long long m;
-  if (p <= 52) {
-    m = tl << (52 - p);
-  } else {
-    int sh = p - 52;  // 1 .. 75
-    unsigned long long rem_hi, rem_lo, half_hi, half_lo;
-    if (sh < 64) {
-      m = (tl >> sh) | (sh ? (th << (64 - sh)) : 0ull);
-      rem_lo = tl & ((1ull << sh) - 1ull);
-      rem_hi = 0ull;
-      half_lo = 1ull << (sh - 1);
-      half_hi = 0ull;
-    } else {
-      int s2 = sh - 64;
-      m = th >> s2;
-      rem_lo = tl;
-      rem_hi = s2 ? (th & ((1ull << s2) - 1ull)) : 0ull;
-      if (s2 == 0) { half_hi = 0ull; half_lo = 1ull << 63; }
-      else { half_hi = 1ull << (s2 - 1); half_lo = 0ull; }
-    }
-    bool gt = (rem_hi > half_hi) || (rem_hi == half_hi && rem_lo > half_lo);
-    bool eq = (rem_hi == half_hi) && (rem_lo == half_lo);
-    if (gt || (eq && (m & 1ull))) {
-      ++m;
-      if (m >> 53) { m >>= 1; ++p; }
-    }
-  }
-  int ex = p + adj + 1023;
-  if (ex <= 0 || ex >= 2047) {  // outside the normal range: let FP64 arithmetic handle it
-    double v = ldexp((double)(m & ((1ull << 53) - 1ull)), p - 52 + adj);
-    return sign ? -v : v;
-  }
-  unsigned long long bits = (sign << 63) | ((unsigned long long)ex << 52) | (m & ((1ull << 52) - 1ull));
-  return __longlong_as_double((long long)bits);
+  return (long long)(((unsigned long long)(ex - 1) << 52) + q) | (neg & (1ll << 63));
 }
 
 constexpr int GROUP_M = 8;  // row tiles per group of the tile order (L2 reuse of the A planes)
@@ -511,6 +516,7 @@ struct OzArgs {
   const int* ea;
   const int* eb;
   double alpha, beta;
+  int amode, bmode;  // alpha: 1 or -1 (0: another value); beta: 0 or 1 (2: another value)
   double* C;
   int ldc;
   int* st;
@@ -717,16 +723,36 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
       const bool two = LMAX >= 5;  // a second (low) accumulator is in use
       const int D = two ? 7 * LMAX - 28 : 0;
       const int base_adj = ea - (two ? 7 * LMAX : 28);
-      const double alpha = p.alpha, beta = p.beta;
+      const int amode = p.amode, bmode = p.bmode;
+      const long long flip = amode < 0 ? 1ll << 63 : 0ll;
+      double* cp = p.C + (size_t)row + (size_t)(tn + cg * CPW) * p.ldc;
+      constexpr int CG = 4;  // columns whose loads of C are in flight together, one group ahead
+      double cv[CG], cn[CG];
+      auto fetch = [&](int g) {
 #pragma unroll
-      for (int j = 0; j < CPW; ++j) {
-        int col = tn + cg * CPW + j;
-        if (col >= p.n || (p.lower && row < col)) continue;
-        double v = fixed_to_double(hi[j], two ? lo[j] : 0ll, D, base_adj + scale_exp(p.eb[col], p.xbit));
-        double* cp = p.C + (size_t)row + (size_t)col * p.ldc;
-        double out = (alpha == 1.0) ? v : (alpha == -1.0 ? -v : alpha * v);
-        if (beta != 0.0) out = fma(beta, *cp, out);
-        *cp = out;
+        for (int j = 0; j < CG; ++j) {
+          const int col = tn + cg * CPW + g + j;
+          cn[j] = (col < p.n && !(p.lower && row < col)) ? cp[(size_t)(g + j) * p.ldc] : 0.0;
+        }
+      };
+      if (bmode != 0) fetch(0);
+#pragma unroll
+      for (int g = 0; g < CPW; g += CG) {
+#pragma unroll
+        for (int j = 0; j < CG; ++j) cv[j] = cn[j];
+        if (bmode != 0 && g + CG < CPW) fetch(g + CG);
+#pragma unroll
+        for (int j = 0; j < CG; ++j) {
+          const int col = tn + cg * CPW + g + j;
+          if (col >= p.n || (p.lower && row < col)) continue;
+          const long long bits =
+              fixed_to_bits(hi[g + j], two ? lo[g + j] : 0ll, D, base_adj + scale_exp(p.eb[col], p.xbit));
+          double out = __longlong_as_double(bits ^ flip);
+          if (amode == 0) out *= p.alpha;
+          if (bmode == 1) out += cv[j];
+          else if (bmode == 2) out = fma(p.beta, cv[j], out);
+          cp[(size_t)(g + j) * p.ldc] = out;
+        }
       }
     }
     }
@@ -798,6 +824,30 @@ int split_rows(gep_handle_t h, int R, int K, int Kpad, const double* X, long lon
   return check_launch(h);
 }
 
+// Exponent pass and split of an operand with strided K.
+int split_cols(gep_handle_t h, int R, int K, int Kpad, const double* X, long long sr, long long sk, int* e, int S,
+               int xbit, unsigned short* out) {
+  if (sr == 1 && Kpad <= FUSE_K) {
+    static unsigned long long devices = 0;
+    if (first_use_on_device(devices)) {
+      GEP_CUDA(cudaFuncSetAttribute(k_split_cols<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 9 * 8));
+      GEP_CUDA(cudaFuncSetAttribute(k_split_cols<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 33 * 8));
+    }
+    // 8 rows a CTA while that fills the GPU at most a few times over (a row segment is 64 bytes),
+    // else 32
+    if (R <= 32 * h->sm_count)
+      k_split_cols<8><<<(R + 7) / 8, 256, (size_t)Kpad * 9 * 8, h->stream>>>(R, K, Kpad, X, sk, e, S, xbit, out, h->d_status);
+    else
+      k_split_cols<32><<<(R + 31) / 32, 256, (size_t)Kpad * 33 * 8, h->stream>>>(R, K, Kpad, X, sk, e, S, xbit, out, h->d_status);
+    return check_launch(h);
+  }
+  GEP_CUDA(cudaMemsetAsync(e, 0, sizeof(int) * (size_t)R, h->stream));
+  k_rowexp_slab<<<dim3((R + 255) / 256, (K + 31) / 32), 256, 0, h->stream>>>(R, K, X, sr, sk, e, h->d_status);
+  GEP_CHECK(check_launch(h));
+  k_split<<<dim3(Kpad / 32, (R + 31) / 32), 256, 0, h->stream>>>(R, K, Kpad, X, sr, sk, e, S, xbit, out, h->d_status);
+  return check_launch(h);
+}
+
 // Product-kernel launch for one K panel (kc deep, planes padded to a.kpad): dynamic shared
 // memory attribute, optional per-launch timing, template dispatch on the plane/level counts.
 int oz_launch(gep_handle_t h, const CUtensorMap& mA, const CUtensorMap& mB, const OzArgs& a, int kc) {
@@ -837,7 +887,9 @@ int oz_launch(gep_handle_t h, const CUtensorMap& mA, const CUtensorMap& mB, cons
 void oz_args_init(OzArgs& a, int m, int n, int kpad, int S, int levels, int lower, int xbit, const int* ea,
                   const int* eb, double alpha, double beta, double* C, int ldc, int* st) {
   a.m = m; a.n = n; a.kpad = kpad; a.S = S; a.lmax = levels; a.lower = lower; a.xbit = xbit;
-  a.ea = ea; a.eb = eb; a.alpha = alpha; a.beta = beta; a.C = C; a.ldc = ldc; a.st = st;
+  a.ea = ea; a.eb = eb; a.alpha = alpha; a.beta = beta;
+  a.amode = alpha == 1.0 ? 1 : alpha == -1.0 ? -1 : 0;
+  a.bmode = beta == 0.0 ? 0 : beta == 1.0 ? 1 : 2; a.C = C; a.ldc = ldc; a.st = st;
   a.gx = (m + TM - 1) / TM;
   a.gy = (n + TN - 1) / TN;
   a.ntiles = a.gx * a.gy;
@@ -954,8 +1006,6 @@ int dgemm_oz(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, d
     int* eb = ea + m;
     const double* Ap = A + (size_t)kb * ska;
     const double* Bp = B + (size_t)kb * skb;
-    // operands whose K is contiguous take the fused exponent-and-split kernel; the others
-    // (K strided) an exponent pass down the rows, then the tile-transposing split
     if (SA) {
       GEP_CUDA(cudaMemsetAsync(ea, 0, sizeof(int) * (size_t)m, h->stream));
       k_rowexp_sym_row<<<dim3((m + 255) / 256, (kc + 63) / 64), 256, 0, h->stream>>>(m, kb, kc, A, lda, ea,
@@ -969,24 +1019,12 @@ int dgemm_oz(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, d
     } else if (ska == 1) {
       GEP_CHECK(split_rows(h, m, kc, kpad, Ap, sra, ea, S, xbit, As));
     } else {
-      GEP_CUDA(cudaMemsetAsync(ea, 0, sizeof(int) * (size_t)m, h->stream));
-      k_rowexp_slab<<<dim3((m + 255) / 256, (kc + 127) / 128), 256, 0, h->stream>>>(m, kc, Ap, sra, ska, ea,
-                                                                                   h->d_status);
-      GEP_CHECK(check_launch(h));
-      k_split<<<dim3(kpad / 32, (m + 31) / 32), 256, 0, h->stream>>>(m, kc, kpad, Ap, sra, ska, ea, S, xbit, As,
-                                                                     h->d_status);
-      GEP_CHECK(check_launch(h));
+      GEP_CHECK(split_cols(h, m, kc, kpad, Ap, sra, ska, ea, S, xbit, As));
     }
     if (skb == 1) {
       GEP_CHECK(split_rows(h, n, kc, kpad, Bp, srb, eb, S, xbit, Bs));
     } else {
-      GEP_CUDA(cudaMemsetAsync(eb, 0, sizeof(int) * (size_t)n, h->stream));
-      k_rowexp_slab<<<dim3((n + 255) / 256, (kc + 127) / 128), 256, 0, h->stream>>>(n, kc, Bp, srb, skb, eb,
-                                                                                   h->d_status);
-      GEP_CHECK(check_launch(h));
-      k_split<<<dim3(kpad / 32, (n + 31) / 32), 256, 0, h->stream>>>(n, kc, kpad, Bp, srb, skb, eb, S, xbit, Bs,
-                                                                     h->d_status);
-      GEP_CHECK(check_launch(h));
+      GEP_CHECK(split_cols(h, n, kc, kpad, Bp, srb, skb, eb, S, xbit, Bs));
     }
     CUtensorMap mA, mB;
     GEP_CHECK(encode_map(&mA, As, kpad, m, S, TM));
