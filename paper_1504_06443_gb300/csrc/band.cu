@@ -1882,7 +1882,7 @@ int apply_q2(gep_handle_t h, int M, int b, const double* q2, double* Z, int ldz,
         // one K panel of the split-BF16 engine: all of Z(rows) is split into digit planes
         // before its product kernel writes C, so the update may run in place
         const size_t one_panel = (size_t)16 * (Wc + ncol) * ((Wc + 31) / 32 * 32) + (size_t)4 * (Wc + ncol) + 4096;
-        if (Wc >= 128 && ncol >= 64 && Wc <= 4096 && one_panel <= h->eng_bytes) {
+        if (product_on_tensor_cores(h, 'F', Wc, ncol, Wc, engine) && Wc <= 4096 && one_panel <= h->eng_bytes) {
           GEP_CHECK(dgemm(h, 'N', 'N', 'F', Wc, ncol, Wc, 1.0, Ut, W, Z + r0, ldz, 1.0, Z + r0, ldz, engine, &kr));
         } else {  // Z(rows) += (U - I) copy(Z(rows))
           GEP_CHECK(copy_matrix(h, Wc, ncol, Z + r0, ldz, Tmp, Wc));

@@ -296,14 +296,29 @@ int dgemm_f64(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, 
   return check_launch(h);
 }
 
+// The faster engine for a product on the tensor-core precisions, by the measured costs of both
+// (us, launches included; checked against 14 shapes from 128^3 to 4096^3, within a fifth):
+//   FP64 units:    8 + mnk / 0.525e6
+//   split-BF16:    20 for the digit splits and launches, per wave of 128 x 64 tiles 4 (epilogue)
+//                  + 0.047 k (36 plane products; 0.01 k with 3 planes), and the operands' digits
+//                  (24 bytes an element at 5 TB/s).
+// So 128^3 (10.5 / 28 us) and 128 x 128 x 2048 stay on the FP64 units, 256^3 (35 / 35 us) and
+// 127 x 1024 x 1024 (234 / 60 us) go to the tensor cores.
+bool product_on_tensor_cores(gep_handle_t h, char uplo, int m, int n, int k, int engine) {
+  if (engine == GEP_PREC_FP64 || m < 32 || n < 16 || k < 16) return false;
+  const double half = (uplo == 'L' || uplo == 'l') ? 0.5 : 1.0;
+  const double tiles = half * ((m + 127) / 128) * ((n + 63) / 64);
+  const double waves = tiles <= h->sm_count ? 1.0 : tiles / h->sm_count;
+  const double oz = 20.0 + waves * (4.0 + (engine == GEP_PREC_FP64_EMULATED ? 0.047 : 0.01) * k) +
+                    5e-6 * ((double)m + n) * k;
+  const double f64 = 8.0 + half * (double)m * n * k * (1e-6 / 0.525);
+  return oz < f64;
+}
+
 int dgemm(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha,
           const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
           int engine, const OzKRange* kr) {
-  // Products too small to fill 128 x 64 tensor-core tiles stay on the FP64 FMA kernel, and
-  // so do outputs of one or two tiles with a long K (split K over many CTAs there).
-  bool big = m >= 128 && n >= 64 && k >= 16;
-  const long long oz_tiles = (long long)((m + 127) / 128) * ((n + 63) / 64);
-  if (big && oz_tiles <= 2 && k >= 2048) big = false;
+  const bool big = product_on_tensor_cores(h, uplo, m, n, k, engine);
   if (engine == GEP_PREC_FP64_EMULATED && big)
     return dgemm_oz(h, ta, tb, uplo, m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, 9, kr);
   if (engine == GEP_PREC_MIXED_REFINED && big)

@@ -131,6 +131,8 @@ struct OzKRange {
 int dgemm(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha,
           const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
           int engine, const OzKRange* kr = nullptr);
+// Whether dgemm takes the split-BF16 engine for this product (gemm_f64.cu).
+bool product_on_tensor_cores(gep_handle_t h, char uplo, int m, int n, int k, int engine);
 int dgemm_f64(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha,
               const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc);
 int dgemm_oz(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha,

@@ -104,3 +104,35 @@ def test_symmetric_lower_operand(gep, engine, m, n):
     bound = 1e-14 * (np.abs(S) @ np.abs(B)) + 1e-300
     assert np.all(np.isfinite(out))
     assert np.all(np.abs(out - ref) <= bound * (4 if engine == "fp64" else 1) + 4 * m * 2.0 ** -52 * (np.abs(S) @ np.abs(B)) * (engine == "fp64"))
+
+
+# Shapes on both sides of the engine rule (FP64 units or tensor cores), fewer than 128 rows or 64
+# columns on the tensor cores, strided and contiguous K up to and beyond the fused split's depth,
+# every alpha / beta form of the epilogue.  Bound: that of the other FP64-accurate products.
+@pytest.mark.parametrize("m,n,k", [(128, 128, 128), (257, 255, 256), (33, 1100, 1050), (1000, 17, 1500),
+                                   (90, 700, 512), (700, 90, 513), (2100, 40, 600), (127, 1024, 1024)])
+@pytest.mark.parametrize("ta,tb,alpha,beta", [("N", "N", 1.0, 0.0), ("T", "N", -1.0, 1.0), ("N", "T", 0.75, 1.0),
+                                              ("T", "T", -1.0, -0.5)])
+def test_engine_rule_shapes(gep, m, n, k, ta, tb, alpha, beta):
+    rng = np.random.default_rng(m + 3 * n + k)
+    A = rng.standard_normal((k, m) if ta == "T" else (m, k)) * np.exp(rng.uniform(-8, 8))
+    B = rng.standard_normal((n, k) if tb == "T" else (k, n))
+    A[0] = 0.0
+    C = rng.standard_normal((m, n))
+    At, Bt = (A.T if ta == "T" else A), (B.T if tb == "T" else B)
+    out = host(gep.dgemm(dev(A), dev(B), ta, tb, alpha=alpha, beta=beta, C=dev(C), engine="fp64_emulated"))
+    ref = alpha * (At @ Bt) + beta * C
+    row = np.max(np.abs(At), axis=1, keepdims=True) * np.max(np.abs(Bt), axis=0, keepdims=True)
+    bound = 2 * k * 2.0 ** -52 * (row + np.abs(At) @ np.abs(Bt) / k) + 4 * 2.0 ** -52 * np.abs(beta * C)
+    assert np.all(np.abs(out - ref) <= bound + 1e-300)
+
+
+def test_negative_and_exact_results(gep):
+    """Small integers: every product is exact, signs and zeros included."""
+    rng = np.random.default_rng(0)
+    A = rng.integers(-3, 4, (300, 280)).astype(float)
+    B = rng.integers(-3, 4, (280, 310)).astype(float)
+    out = host(gep.dgemm(dev(A), dev(B), engine="fp64_emulated"))
+    assert np.array_equal(out, A @ B)
+    out = host(gep.dgemm(dev(A * 2.0 ** -40), dev(B * 2.0 ** 30), alpha=-1.0, engine="fp64_emulated"))
+    assert np.array_equal(out, -(A @ B) * 2.0 ** -10)
