@@ -782,11 +782,17 @@ __device__ __forceinline__ ll qwarp_sum(ll v) {
   const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 40));
   return ((ll)hi << 40) + ((ll)mi << 20) + lo;
 }
-// The double nearest below in magnitude of a positive integer (its 53 leading bits).
+// The double nearest to a non-negative integer (half up: truncation would lengthen every
+// reflector by the same sign, a growth of the spectrum by 2^-59 a sweep).
 __device__ __forceinline__ double qdouble(unsigned long long x) {
   if (x == 0) return 0.0;
   const int lz = __clzll((ll)x);
-  return __longlong_as_double((ll)(((unsigned long long)(1085 - lz) << 52) + ((x << lz) >> 11)));
+  const unsigned long long y = x << lz;
+  return __longlong_as_double((ll)(((unsigned long long)(1085 - lz) << 52) + (y >> 11) + ((y >> 10) & 1ull)));
+}
+// a^2 2^-63, the low limb's square (never negative, so not a rounding error) included.
+__device__ __forceinline__ ll qsquare(int2 a) {
+  return (qhh(a, a) << 1) + (qmid(a, a, (1ll << 30) + (((ll)a.x * a.x) >> 32)) >> 31);
 }
 // x 2^e as an integer, for a positive normal x with x 2^e < 2^63 (rounded half up).
 __device__ __forceinline__ ll qint(double x, int e) {
@@ -989,7 +995,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
           const ll z = up >= 0 ? x[r] << up : x[r] >> -up;
           if (r == 0) x00 = z;
           xs[r] = qsplit(z);
-          if (lane + 32 * r > 0) s2 += qmul<63>(xs[r], xs[r]);
+          if (lane + 32 * r > 0) s2 += qsquare(xs[r]);
         }
         s2 = qwarp_sum(s2);
         const ll alpha_q = __shfl_sync(0xffffffffu, x[0], 0), xa = __shfl_sync(0xffffffffu, x00, 0);

@@ -98,3 +98,22 @@ def test_reflectors_give_an_orthogonal_basis(gep, b):
     n = np.max(np.abs(np.linalg.eigvalsh(C)))
     assert np.max(np.abs(Z.T @ Z - np.eye(M))) <= 200 * M * EPS
     assert np.max(np.abs(Z.T @ C @ Z - T)) <= 200 * M * EPS * n
+
+
+@pytest.mark.parametrize("b", [32, 64])
+def test_no_drift_of_the_spectrum(gep, b):
+    """A reflector that is longer or shorter than it should be by the same sign every time scales the
+    whole spectrum, a little more with every sweep.  Random rounding leaves 2 to 3 eps of the norm
+    per eigenvalue at this order; 6 eps (root mean square) would be a drift of 2^-60 a sweep."""
+    import torch
+    M = 2000
+    g = torch.Generator(device="cuda").manual_seed(b)
+    Q, _ = torch.linalg.qr(torch.randn(M, M, generator=g, dtype=torch.float64, device="cuda"))
+    lam = torch.linspace(-20.0, 20.0, M, dtype=torch.float64, device="cuda")
+    C = (Q * lam) @ Q.t()
+    C = 0.5 * (C + C.t())
+    w, _, info = gep.solve(C, torch.eye(M, dtype=torch.float64, device="cuda"), sep="2stage", bandwidth=b,
+                           precision="fp64_emulated", want_vectors=False)
+    assert info == 0
+    ref = torch.linalg.eigvalsh(C)
+    assert float((w - ref).norm() / ref.norm()) <= 6 * EPS
