@@ -847,6 +847,13 @@ struct BatchPlan {
 
 int small_limit(const gep_options* o) { return o->batch_small < SMALL_MAX ? o->batch_small : SMALL_MAX; }
 
+// Time of one staged solve of order M on its stream, in ms (measured: order 64 2.1, 256 5.7, 516 12,
+// 1024 25, 2047 60): the balance of the streams.
+double staged_ms(int M) { return 1.0 + 0.02 * M + 3e-9 * (double)M * M * M; }
+// Time of the one-CTA solver (cyclic Jacobi, about 12 M^3 FP64 operations on one SM): 53 ms at
+// order 128.  Up to two pencils an SM run at once.
+double one_cta_ms(int M) { return 53.0 / (128.0 * 128.0 * 128.0) * M * M * M; }
+
 // Options of pencil i: opts[i] when given, else o with precision[i] (when given).
 gep_options pencil_opts(const gep_options* o, const int* prec, const gep_options* opts, int i) {
   if (opts) return opts[i];
@@ -873,6 +880,19 @@ int make_plan(gep_handle_t h, int count, const int* M, const gep_options* o, con
     while (b >= 0 && M[order[b]] < M[t]) { order[b + 1] = order[b]; --b; }
     order[b + 1] = t;
   }
+  // Of the pencils that may take the one-CTA solver, those keep it whose time there (all run at
+  // once) is below what the small pencils together cost on the streams: a few pencils of order
+  // 128 (53 ms in one CTA, 3.2 ms staged) go to the streams, hundreds of them stay.
+  double on_streams = 0.0;
+  int nsm = 0;
+  for (int i = 0; i < count; ++i)
+    if (small_of[i]) {
+      on_streams += staged_ms(M[i]);
+      ++nsm;
+    }
+  const double batches = nsm > 2 * h->sm_count ? (double)nsm / (2 * h->sm_count) : 1.0;
+  for (int i = 0; i < count; ++i)
+    if (small_of[i] && batches * one_cta_ms(M[i]) > on_streams / nstreams) small_of[i] = false;
   p->nsmall = 0;
   for (int a = 0; a < count; ++a)
     if (small_of[order[a]]) p->small_order[p->nsmall++] = order[a];
@@ -890,7 +910,7 @@ int make_plan(gep_handle_t h, int count, const int* M, const gep_options* o, con
     for (int s = 1; s < p->ns; ++s)
       if (load[s] < load[best]) best = s;
     p->assign[i] = best;
-    load[best] += (double)M[i] * M[i] * M[i];
+    load[best] += staged_ms(M[i]);
     const gep_options oi = pencil_opts(o, prec, opts, i);
     size_t need = layout(M[i], &oi).end;
     if (need > p->need[best]) p->need[best] = need;
