@@ -1535,7 +1535,7 @@ int panel_factor(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, 
   k_panel_v<<<dim3((n + 255) / 256, b), 256, 0, h->stream>>>(n, b, P, ldp, V, h->d_status);
   GEP_CHECK(check_launch(h));
   GEP_CHECK(dgemm(h, 'T', 'N', 'F', b, b, n, 1.0, V, n, V, n, 0.0, w.GV, b, eng));
-  return larft_rec(h, b, w.GV, b, tau, w.T, b, w.Tt);
+  return larft_rec(h, b, w.GV, b, tau, w.T, b, w.Tt, GEP_PREC_FP64);
 }
 
 // k_panel_qr's launch (b <= 32): V_j into Va and Vb (ld ldv, r0 zero rows first), T into w.T.

@@ -195,7 +195,7 @@ int backtransform_q(gep_handle_t h, int M, int ncol, const double* C, int ldc, c
                     double* Z, int ldz, double* ws, size_t ws_elems, int engine, int off = 1);
 // T (nb x nb, upper) of the block reflector whose Gram matrix is G = V^T V (backtrans.cu).
 int larft_rec(gep_handle_t h, int nb, const double* G, int ldg, const double* tau, double* T, int ldt,
-              double* tmp);
+              double* tmp, int engine);
 // two-stage SEP path (band.cu)
 size_t q2_elems(int M, int b);
 size_t band_ws_elems(int M, int b);
