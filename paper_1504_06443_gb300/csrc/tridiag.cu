@@ -499,8 +499,8 @@ __global__ void __launch_bounds__(256) k_w_finish(int n, int nblk, const double*
 //      formed by every CTA for itself.                                              [barrier]
 // Bound: the two barriers (1.2 us each on 152 SMs) and the latency of the reductions between
 // them; native FP64 tiles also by FP64 issue (two FMAs per element).  Measured per column (six
-// launches before): order 500 FP64 69 -> 12.8 us, order 1501 float pairs 72 -> 18 us, order 64
-// 58 -> 20 us.
+// launches before): order 500 FP64 69 -> 11.3 us, order 1501 float pairs 72 -> 13.6 us, order 64
+// 58 -> 9.9 us.
 constexpr int TRD_COOP_MAX = 4096;  // vs and the tiles fit shared memory; beyond, the SYMV is bound by HBM anyway
 constexpr int TRD_T = 256;          // threads
 constexpr int LPR = 16;             // lanes per owned row
@@ -515,12 +515,14 @@ struct TrdArgs {
 struct AccD {
   double s = 0.0;
   __device__ void add(double a, double v) { s = fma(a, v, s); }
+  __device__ void join(const AccD& o) { s += o.s; }
   __device__ double get() const { return s; }
 };
 struct AccF {
   ff s = {0.f, 0.f};
   __device__ void add(float2 a, float2 v) { ff_madd(s, a.x, a.y, v.x, v.y); }
   __device__ void add(float a, float2 v) { ff_madd(s, a, 0.f, v.x, v.y); }
+  __device__ void join(const AccF& o) { ff_add_acc(s, o.s); }
   __device__ double get() const { return (double)s.h + (double)s.l; }
 };
 template <class T> struct TrdForm;
@@ -535,6 +537,14 @@ __device__ __forceinline__ unsigned long long trd_clock() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+
+// Sum of red[0..7] in every lane of a warp.
+__device__ __forceinline__ double red8(const double* red, int lane) {
+  double s = red[lane & 7];
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  return s + __shfl_xor_sync(0xffffffffu, s, 4);
 }
 
 // Grid barrier number ep (1, 2, ...): bounded; false when it gave up or an error is recorded.
@@ -641,25 +651,29 @@ __global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
     }
     s2 = warp_sum(s2);
     if (lane == 0) red[warp] = s2;
-    __syncthreads();
     if (tid == 0) {
-      double s = 0.0;
-#pragma unroll
-      for (int q = 0; q < TRD_T / 32; ++q) s += red[q];
-      double tv = 0.0, beta = alpha, scal = 0.0;
-      if (s != 0.0) {
-        const double nrm = sqrt(fma(alpha, alpha, s));
-        beta = alpha >= 0.0 ? -nrm : nrm;
-        scal = 1.0 / (alpha - beta);
-        tv = (beta - alpha) / beta;
+      sc[2] = alpha;
+      sc[3] = dg;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      const double al = sc[2], ss = red8(red, lane);
+      double tvv = 0.0, beta = al, sl = 0.0;
+      if (ss != 0.0) {
+        const double n2 = fma(al, al, ss), ri = rsqrt(n2), nrm = n2 * ri;
+        beta = al >= 0.0 ? -nrm : nrm;
+        sl = 1.0 / (al - beta);
+        tvv = fma(fabs(al), ri, 1.0);
       }
-      sc[0] = tv;
-      sc[1] = scal;
-      sc[2] = beta;
-      if (k == 0) {
-        a.d[c] = dg;
-        a.e[c] = beta;
-        a.tau[c] = tv;
+      if (lane == 0) {
+        sc[0] = tvv;
+        sc[1] = sl;
+        if (k == 0) {
+          a.d[c] = sc[3];
+          a.e[c] = beta;
+          a.tau[c] = tvv;
+        }
+        sc[2] = beta;
       }
     }
     __syncthreads();
@@ -709,9 +723,11 @@ __global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
       if (tid < 2 * TS) {
         const bool direct = tid < TS;
         const int r = direct ? tid : tid - TS;
-        double s0 = 0.0;
+        // (float pairs are joined as such: a conversion to FP64 and an FP64 add cost 64 clocks each)
+        Acc s4 = direct ? redd[0][r] : redt[0][r];
 #pragma unroll
-        for (int u = 0; u < NQ; ++u) s0 += direct ? redd[u][r].get() : redt[u][r].get();
+        for (int u = 1; u < NQ; ++u) s4.join(direct ? redd[u][r] : redt[u][r]);
+        const double s0 = s4.get();
         const int l = (direct ? I : J) * TS + r;
         if (l < nt && (direct || I != J)) {
           __stcg(a.P + (size_t)(direct ? J : I) * nt + l, s0);
@@ -721,22 +737,33 @@ __global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
     }
     // ---- A: t1 = W^T v (q < i), t2 = V^T v (q >= i)
     auto colq = [&](int q) { return (q < i ? a.W + (size_t)q * M : a.Vp + (size_t)(q - i) * M) + j0; };
-    if (2 * i <= 2 * G) {  // at most two dots a CTA: the whole CTA on each
-      for (int q = k; q < 2 * i; q += G) {
-        const double* col = colq(q);
+    const bool whole = i <= G;  // at most two dots a CTA: the whole CTA on each, v^T A v beside the first
+    if (whole) {
+      int q = k;
+      do {
         double s = 0.0;
-        for (int l = i + 1 + tid; l < nt; l += TRD_T) s = fma(__ldcg(col + l), vs[l], s);
-        s = warp_sum(s);
-        __syncthreads();
-        if (lane == 0) red[warp] = s;
-        __syncthreads();
-        if (tid == 0) {
-          double z = 0.0;
-#pragma unroll
-          for (int u = 0; u < TRD_T / 32; ++u) z += red[u];
-          __stcg(a.t + q, z);
+        if (q < 2 * i) {
+          const double* col = colq(q);
+          for (int l = i + 1 + tid; l < nt; l += TRD_T) s = fma(__ldcg(col + l), vs[l], s);
         }
-      }
+        for (int o = 16; o; o >>= 1) {
+          s += __shfl_xor_sync(0xffffffffu, s, o);
+          vav += __shfl_xor_sync(0xffffffffu, vav, o);
+        }
+        __syncthreads();
+        if (lane == 0) {
+          red[warp] = s;
+          red[8 + warp] = vav;
+        }
+        __syncthreads();
+        if (warp == 0) {
+          const double z = red8(red + (lane & 8), lane);  // lanes 0..7: the dot, 8..15: v^T A v
+          if (lane == 0 && q < 2 * i) __stcg(a.t + q, z);
+          if (lane == 8 && q == k) __stcg(a.vav + k, z);
+        }
+        vav = 0.0;
+        q += G;
+      } while (q < 2 * i);
     } else {
       for (int q = k + warp * G; q < 2 * i; q += G * (TRD_T / 32)) {
         const double* col = colq(q);
@@ -745,16 +772,14 @@ __global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
         s = warp_sum(s);
         if (lane == 0) __stcg(a.t + q, s);
       }
-    }
-    vav = warp_sum(vav);  // (threads beyond 2 TS hold zeros)
-    __syncthreads();
-    if (lane == 0) red[warp] = vav;
-    __syncthreads();
-    if (tid == 0) {
-      double z = 0.0;
-#pragma unroll
-      for (int u = 0; u < TRD_T / 32; ++u) z += red[u];
-      __stcg(a.vav + k, z);
+      vav = warp_sum(vav);  // (threads beyond 2 TS hold zeros)
+      __syncthreads();
+      if (lane == 0) red[warp] = vav;
+      __syncthreads();
+      if (warp == 0) {
+        const double z = red8(red, lane);
+        if (lane == 0) __stcg(a.vav + k, z);
+      }
     }
     if (!trd_barrier(a.bar, ++ep, a.st, &ok_s)) return;
     // ---- B: w on the owned rows and on row i + 1
@@ -764,18 +789,12 @@ __global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
       v0[q] = __ldcg(a.Vp + GEP_IX(c + 1, q, M));
       w0[q] = __ldcg(a.W + GEP_IX(c + 1, q, M));
     }
-    double z = 0.0;
-    for (int u = tid; u < G; u += TRD_T) z += __ldcg(a.vav + u);
-    __syncthreads();
-    if (tid < i) z -= 2.0 * tq[tid] * tq[i + tid];
-    z = warp_sum(z);
-    if (lane == 0) red[warp] = z;
-    __syncthreads();
-    if (tid == 0) {
-      double s = 0.0;
-#pragma unroll
-      for (int u = 0; u < TRD_T / 32; ++u) s += red[u];
-      sc[3] = -0.5 * tv * (tv * s);
+    if (warp == 3) {  // v^T A v - 2 t1.t2, by a warp that loads nothing else
+      double z = 0.0;
+      for (int u = lane; u < G; u += 32) z += __ldcg(a.vav + u);
+      for (int q = lane; q < i; q += 32) z = fma(-2.0 * __ldcg(a.t + q), __ldcg(a.t + i + q), z);
+      z = warp_sum(z);
+      if (lane == 0) sc[3] = -0.5 * tv * (tv * z);
     }
     __syncthreads();
     const double al2 = sc[3];
@@ -791,7 +810,7 @@ __global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
         const double* Vq = first ? v0 : Vr + lr * (NBT + 1);
         const double* Wq = first ? w0 : Wr + lr * (NBT + 1);
         for (int q = sub; q < nb; q += LPR) s += __ldcg(a.P + (size_t)q * nt + l);
-        for (int q = sub; q < i; q += LPR) s -= fma(Vq[q], tq[q], Wq[q] * tq[i + q]);
+        for (int q = sub; q < i; q += LPR) s = fma(-Vq[q], tq[q], fma(-Wq[q], tq[i + q], s));
       }
       for (int o = LPR / 2; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (act && sub == 0) {
@@ -827,8 +846,10 @@ template <class T, int TS>
 int trd_panel_launch(gep_handle_t h, TrdArgs a) {
   a.nb = (a.nt + TS - 1) / TS;
   a.tiles = a.nb * (a.nb + 1) / 2;
-  // float pairs: two tiles a CTA (a second tile costs less than a wider barrier); FP64 tiles: one
-  int G = a.tiles <= 3 ? 1 : std::is_same<T, double>::value ? a.tiles : (a.tiles + 1) / 2;
+  // float pairs: two tiles a CTA (a second tile costs less than a wider barrier); FP64 tiles: one;
+  // and at most 15 owned rows (one pass of phase B)
+  int G = std::is_same<T, double>::value ? a.tiles : (a.tiles + 1) / 2;
+  if (G < (a.nt + 14) / 15) G = (a.nt + 14) / 15;
   if (G > h->sm_count) G = h->sm_count;
   a.rpc = (a.nt + G - 1) / G;
   const int per = (a.tiles + G - 1) / G;
