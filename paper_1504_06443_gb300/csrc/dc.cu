@@ -28,7 +28,7 @@
 namespace gep {
 namespace {
 
-constexpr int LEAF = 16;
+constexpr int LEAF = 8;
 constexpr int FP64_WIDTH = 256;  // merges up to this order form their products in FP64, one launch a level
 constexpr double EPS = 0x1p-53;
 
@@ -133,7 +133,8 @@ __global__ void k_tear(int M, const double* __restrict__ d, const double* __rest
 // same for one lane as for 32), the split test is one ballot.  The leaf is scaled by a power of
 // two so that a rotation needs one rsqrt instead of a hypot and two divisions.  Sorted
 // ascending and written to Z/D at the end.  With leaves of 32 rows, hypot and divisions in
-// lane 0 this kernel took 2.46 ms; now 0.33 ms.
+// lane 0 this kernel took 2.46 ms, with 16 rows 0.33 ms; at 8 the extra level of merges costs less than
+// the leaves save (D&C of order 64 0.48 -> 0.35 ms, 2047 8.6 -> 6.6 ms).
 __global__ void __launch_bounds__(32) k_leaf(int M, const double* __restrict__ dd, const double* __restrict__ e,
                                              double* __restrict__ D, double* __restrict__ Z, int ldz, int* st) {
   __shared__ double Zs[LEAF][33];

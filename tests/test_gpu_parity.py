@@ -303,12 +303,12 @@ def test_dgemm_fp64_symmetric_operand_split_depth(gep):
 
 
 def _dc_edge_cases():
-    """Orders at the edges of the leaves (16) and of the merge levels, with and without a ragged or
+    """Orders at the edges of the leaves and of the merge levels, with and without a ragged or
     unmerged tail, each with rotations in chains (equal and nearly equal eigenvalues of the halves)
     and with negligible couplings."""
     rng = np.random.default_rng(11)
     cases = []
-    for M in (15, 16, 17, 47, 48, 49, 127, 129, 255, 256, 258, 511, 520, 770):
+    for M in (7, 8, 9, 15, 16, 17, 24, 25, 47, 48, 49, 127, 129, 255, 256, 258, 511, 520, 770):
         cases.append((f"random{M}", rng.standard_normal(M), rng.standard_normal(M - 1)))
         cases.append((f"equal{M}", np.full(M, -3.0), np.full(M - 1, 1e-12)))
         d = np.round(rng.standard_normal(M) * 2)
