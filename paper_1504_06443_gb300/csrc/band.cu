@@ -40,7 +40,8 @@ namespace {
 constexpr int BMAX = 64;      // largest bandwidth
 constexpr int BULGE_CTAS_PER_SM = 1;  // resident bulge-chasing CTAs per SM
 constexpr int BAND_GROUP = 4;  // panels per group of the full -> band reduction (trailing update depth 2 G b)
-constexpr int BAND_GROUP_MIN_N = 8192;  // trailing order from which groups of BAND_GROUP are used
+constexpr int BAND_GROUP_MIN_N = 8192;  // trailing order from which groups of BAND_GROUP are used (b = 64; half of
+                                        // it at b <= 32: order 8192 S1b 130 -> 123 ms, order 4000 no gain)
 constexpr int PQ_ROWS = 256;  // panel rows per CTA in the panel QR (one per thread)
 constexpr int PQ_CH = 16;     // columns per reduction chunk in the panel QR
 
@@ -1461,7 +1462,8 @@ size_t band_ws_elems(int M, int b) {
   // + the digit planes of the trailing matrix (shared by the C22 products of a panel group)
   size_t reduce = 2 * rr(G * BMAX) + 2 * rr(BMAX) + rr(32) + 4 * rr((size_t)M * b) +
                   2 * rr((size_t)M * 2 * BAND_GROUP * b) + 5 * rr((size_t)2 * b * b) +
-                  rr((size_t)2 * BAND_GROUP * b * b) + rr(oz_sym_planes_bytes(M, 9) / sizeof(double) + 1);
+                  rr((size_t)2 * BAND_GROUP * b * b) + rr(oz_sym_planes_bytes(M, 9) / sizeof(double) + 1) +
+                  rr(oz_sym_part_elems(M, b));
   size_t chase = rr((size_t)2 * b * M) + rr((size_t)M) + rr(1);  // band, progress counters, norm bound
   return reduce > chase ? reduce : chase;
 }
@@ -1477,6 +1479,8 @@ struct BandWs {
   double *GV, *T, *Tt, *Pm, *Ym, *Zs;
   void* planes;        // digit planes of C22
   size_t planes_bytes;
+  double* parts;       // partial products of C22 V
+  size_t part_elems;
 };
 
 // QR of the n x b panel P (ld ldp): reflectors stay in P, tau[0..b), explicit V (n x b,
@@ -1623,6 +1627,8 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
   w.Zs = take((size_t)2 * BAND_GROUP * b * b);
   w.planes_bytes = oz_sym_planes_bytes(M, 9);
   w.planes = take(w.planes_bytes / sizeof(double) + 1);
+  w.part_elems = oz_sym_part_elems(M, b);
+  w.parts = take(w.part_elems);
   const int levels = eng == GEP_PREC_MIXED_REFINED ? 4 : 9;
   for (int pb = 0; M - pb - b >= 2;) {
     const int n = M - pb - b;
@@ -1630,7 +1636,7 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
     // reflectors act on rows [j b, n), which needs n - j b >= 2
     // (groups pay where the trailing matrix is large; below that pairs, whose two C22 products
     // need no cross-panel corrections beyond one pair of small products)
-    const int gmin = h->band_group_min >= 0 ? h->band_group_min : BAND_GROUP_MIN_N;
+    const int gmin = h->band_group_min >= 0 ? h->band_group_min : (b <= 32 ? BAND_GROUP_MIN_N / 2 : BAND_GROUP_MIN_N);
     const int g = std::min(n >= gmin ? BAND_GROUP : 2, (n - 2) / b + 1);
     double* P = C + (pb + b) + (size_t)pb * ldc;
     double* C22 = C + (pb + b) + (size_t)(pb + b) * ldc;
@@ -1686,7 +1692,7 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
       }
       // C^(j) V_j = C22(r0:, r0:) V_j - sum_{i<j} (W_i V_i^T + V_i W_i^T)(r0:, r0:) V_j
       if (use_planes && nr >= 128) {
-        GEP_CHECK(dgemm_oz_sym_planes(h, planes, r0, b, 1.0, vw(2 * j), n, 0.0, w.CV, nr));
+        GEP_CHECK(dgemm_oz_sym_planes(h, planes, r0, b, 1.0, vw(2 * j), n, 0.0, w.CV, nr, w.parts, w.part_elems));
       } else {
         GEP_CHECK(dgemm(h, 'S', 'N', 'F', nr, b, nr, 1.0, C22 + r0 + (size_t)r0 * ldc, ldc, Vj, ldv, 0.0, w.CV, nr,
                         eng));

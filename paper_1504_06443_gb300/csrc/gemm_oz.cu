@@ -40,9 +40,10 @@ namespace {
 
 constexpr int TM = 128, TN = 64, TK = 32, KCH = 512, STAGES = 2, MAXS = 8;
 // warp 0 issues the TMA loads, warp 1 the MMAs; EPI_WARPS warps drain the accumulators
-// (four per 32-lane quarter of TMEM, each with CPW of the tile's TN columns): the drain
+// (four per 32-lane quarter of TMEM, each with a quarter of the tile's columns): the drain
 // stalls the MMAs, and more warps per scheduler hide its TMEM-load and conversion latency
-constexpr int EPI_WARPS = 16, CPW = TN / (EPI_WARPS / 4);
+constexpr int EPI_WARPS = 16;
+constexpr int TNS = 32;  // tile columns of the skinny form (products with the symmetric planes)
 constexpr int NTHREADS = 64 + 32 * EPI_WARPS;
 constexpr int KP_MAX = 4096;  // K panel per launch (integer accumulators sized for <= 16 chunks)
 
@@ -230,14 +231,19 @@ __global__ void __launch_bounds__(256) k_split_rows(int R, int K, int Kpad, cons
 
 // The same for few rows (fewer than can fill the GPU one warp per row): one CTA per row,
 // the exponent pass reduced over the CTA.
-__global__ void __launch_bounds__(256) k_split_row_blk(int R, int K, int Kpad, const double* __restrict__ X,
+// blockIdx.y: K panel of KP columns (the planes of all panels share rows of ldk elements; the panels'
+// exponents follow each other).
+__global__ void __launch_bounds__(256) k_split_row_blk(int R, int Ktot, int ldk, int KP, const double* __restrict__ X,
                                                        long long sr, int* __restrict__ e_out, int S, int xbit,
                                                        unsigned short* __restrict__ out, const int* st) {
   __shared__ int red[8];
   if (status_bad(st)) return;
-  const int r = blockIdx.x;
+  const int r = blockIdx.x, kb = blockIdx.y * KP;
   if (r >= R) return;
-  const double* x = X + (size_t)r * sr;
+  const int K = min(KP, Ktot - kb), Kpad = min(KP, ldk - kb);
+  const double* x = X + (size_t)r * sr + kb;
+  e_out += (size_t)blockIdx.y * R;
+  out += kb;
   int m = 0;
   for (int kk = threadIdx.x; kk < K; kk += 256) m = max(m, exp_field(x[kk]));
   for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -248,12 +254,12 @@ __global__ void __launch_bounds__(256) k_split_row_blk(int R, int K, int Kpad, c
   for (int w = 1; w < 8; ++w) m = max(m, red[w]);
   const int e = scale_exp(m, xbit);
   if (threadIdx.x == 0) e_out[r] = m;
-  const size_t plane = (size_t)R * Kpad;
+  const size_t plane = (size_t)R * ldk;
   for (int k0 = 4 * threadIdx.x; k0 < Kpad; k0 += 1024) {
     double v[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) v[u] = (k0 + u < K) ? x[k0 + u] : 0.0;
-    split4_store(v, k0, K, e, S, (size_t)r * Kpad + k0, plane, out);
+    split4_store(v, k0, K, e, S, (size_t)r * ldk + k0, plane, out);
   }
 }
 
@@ -322,7 +328,7 @@ __global__ void k_rowexp_sym_col(int R, int kb, int kc, const double* __restrict
   }
 }
 
-__global__ void __launch_bounds__(256) k_split_sym(int R, int K, int Kpad, int kb, const double* __restrict__ C,
+__global__ void __launch_bounds__(256) k_split_sym(int R, int K, int ldk, int koff, int kb, const double* __restrict__ C,
                                                    long long ldc, const int* __restrict__ e, int S, int xbit,
                                                    unsigned short* __restrict__ out, const int* st) {
   __shared__ double t[32][33];
@@ -347,7 +353,7 @@ __global__ void __launch_bounds__(256) k_split_sym(int R, int K, int Kpad, int k
     const int r = r0 + q;
     if (r < R) {
       double x[4] = {t[q][c4], t[q][c4 + 1], t[q][c4 + 2], t[q][c4 + 3]};
-      split4_store(x, k0 + c4, K, scale_exp(e[r], xbit), S, (size_t)r * Kpad + k0 + c4, (size_t)R * Kpad, out);
+      split4_store(x, k0 + c4, K, scale_exp(e[r], xbit), S, (size_t)r * ldk + koff + k0 + c4, (size_t)R * ldk, out);
     }
   }
 }
@@ -468,9 +474,20 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 template <int N>
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, float* v) {
-  if constexpr (N == 16) tmem_ld16(taddr, v);
+  if constexpr (N == 8) tmem_ld8(taddr, v);
+  else if constexpr (N == 16) tmem_ld16(taddr, v);
   else tmem_ld32(taddr, v);
 }
 
@@ -513,6 +530,11 @@ struct OzArgs {
   // (op(A) is exactly zero elsewhere in its rows); other row tiles run all of them
   int kr_n;
   short kr_lo[OZ_KR_MAX], kr_hi[OZ_KR_MAX];
+  // skinny form: spp > 0 splits every K panel of OZ_SYM_KP among spp CTAs per tile; part z writes its
+  // partial product to C + z zstride, with the exponents of its panel at ea + panel eastr, eb + panel ebstr
+  int spp;
+  long long zstride;
+  int eastr, ebstr;
   const int* ea;
   const int* eb;
   double alpha, beta;
@@ -525,9 +547,11 @@ struct OzArgs {
 // SC, LC > 0 fix the plane and level counts at compile time (the two settings the
 // solver uses): the MMA sequence of a k-step is then straight-line code whose
 // descriptors are a per-stage base plus constants.  SC = LC = 0 reads them from p.
-template <int SC, int LC>
+template <int SC, int LC, int TNC = TN>
 __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__ CUtensorMap tmA,
                                                           const __grid_constant__ CUtensorMap tmB, OzArgs p) {
+  constexpr int TN = TNC, CPW = TN / (EPI_WARPS / 4), PG = 256 / TN;  // PG planes per MMA (N = 256)
+  constexpr bool SKINNY = TN == TNS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[2 * STAGES + 3];
   __shared__ uint32_t tmem_slot;
@@ -542,7 +566,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
   // numbered in groups of GROUP_M row tiles, row fastest inside a group: the tiles that run
   // at the same time cover a near-square block of C (8 rows x ~19 columns on 152 SMs), so
   // their A and B planes are read from DRAM about once and then hit in L2.
+  const int per_z = p.gx * p.gy;
   auto tile_rc = [&](int t, int& tm, int& tn) {
+    if constexpr (SKINNY) t %= per_z;
     const int per_group = GROUP_M * p.gy;
     const int first = (t / per_group) * GROUP_M;
     const int gm = min(p.gx - first, GROUP_M);
@@ -565,9 +591,17 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
   const int nsteps = p.kpad / TK;
   const int nlev = LMAX - 1;  // levels 2..LMAX
   // the k-steps [s0, s1) of the tile whose first row is tm (every role takes the same)
-  auto tile_steps = [&](int tm, int& s0, int& s1) {
+  auto tile_steps = [&](int t, int tm, int& s0, int& s1) {
     s0 = 0;
     s1 = nsteps;
+    if constexpr (SKINNY) {  // part z of its K panel
+      constexpr int SP = OZ_SYM_KP / TK;
+      const int z = t / per_z, pn = z / p.spp, q = z - pn * p.spp;
+      const int np = min(SP, nsteps - pn * SP), c = (np + p.spp - 1) / p.spp;
+      s0 = pn * SP + min(np, q * c);
+      s1 = pn * SP + min(np, q * c + c);
+      return;
+    }
     const int r = tm / TM;
     if (r < p.kr_n) {
       s0 = kr_lo[r];
@@ -614,7 +648,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
       for (int i = 0, t; ok && (t = tile_of(i)) < p.ntiles; ++i) {
         int tm, tn, s0, s1;
         if (!tile_rc(t, tm, tn)) continue;
-        tile_steps(tm, s0, s1);
+        tile_steps(t, tm, s0, s1);
         for (int step = s0; step < s1 && ok; ++step, ++g) {
           int sidx = g % STAGES;
           uint32_t ph = (uint32_t)(g / STAGES) & 1u;
@@ -637,7 +671,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
       for (int i = 0, t; ok && (t = tile_of(i)) < p.ntiles; ++i) {
       int tm, tn, s0, s1;
       if (!tile_rc(t, tm, tn)) continue;
-      tile_steps(tm, s0, s1);
+      tile_steps(t, tm, s0, s1);
       const int nch = (s1 - s0 + SPC - 1) / SPC;
       int step = s0;
       for (int c = 0; c < nch && ok; ++c, ++gc) {
@@ -662,9 +696,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
               // descriptor start field = byte address / 16: offsets add to it directly
               const uint64_t adesc = a0 + (uint64_t)((((s - 1) * TM * TK * 2) + kk * 32) >> 4);
 #pragma unroll
-              for (int t0 = 1; t0 <= MAXS; t0 += 4) {
+              for (int t0 = 1; t0 <= MAXS; t0 += PG) {
                 if (t0 > tmax) break;
-                const int nt = min(4, tmax - t0 + 1);
+                const int nt = min(PG, tmax - t0 + 1);
                 const uint64_t bdesc = b0 + (uint64_t)((((t0 - 1) * TN * TK * 2) + kk * 32) >> 4);
                 const uint32_t col = (uint32_t)(s + t0 - 2) * TN;
                 const uint32_t acc = (sic == 0 && kk == 0 && s == 1) ? 0u : 1u;
@@ -689,7 +723,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
     for (int i = 0, t; ok && (t = tile_of(i)) < p.ntiles; ++i) {
     int tm, tn, s0, s1;
     if (!tile_rc(t, tm, tn)) continue;
-    tile_steps(tm, s0, s1);
+    tile_steps(t, tm, s0, s1);
     const int nch = (s1 - s0 + SPC - 1) / SPC;
     const int row = tm + q * 32 + lane;
     long long hi[CPW], lo[CPW];
@@ -719,13 +753,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
       if (lane == 0) mbar_arrive(bar_acce);
     }
     if (ok && row < p.m) {
-      const int ea = scale_exp(p.ea[row], p.xbit);
+      const int zi = SKINNY ? t / per_z : 0, pz = SKINNY ? zi / p.spp : 0;
+      const int* ebp = p.eb + (size_t)pz * p.ebstr;
+      const int ea = scale_exp(p.ea[(size_t)pz * p.eastr + row], p.xbit);
       const bool two = LMAX >= 5;  // a second (low) accumulator is in use
       const int D = two ? 7 * LMAX - 28 : 0;
       const int base_adj = ea - (two ? 7 * LMAX : 28);
       const int amode = p.amode, bmode = p.bmode;
       const long long flip = amode < 0 ? 1ll << 63 : 0ll;
-      double* cp = p.C + (size_t)row + (size_t)(tn + cg * CPW) * p.ldc;
+      double* cp = p.C + (SKINNY ? (size_t)zi * p.zstride : 0) + (size_t)row + (size_t)(tn + cg * CPW) * p.ldc;
       constexpr int CG = 4;  // columns whose loads of C are in flight together, one group ahead
       double cv[CG], cn[CG];
       auto fetch = [&](int g) {
@@ -746,7 +782,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
           const int col = tn + cg * CPW + g + j;
           if (col >= p.n || (p.lower && row < col)) continue;
           const long long bits =
-              fixed_to_bits(hi[g + j], two ? lo[g + j] : 0ll, D, base_adj + scale_exp(p.eb[col], p.xbit));
+              fixed_to_bits(hi[g + j], two ? lo[g + j] : 0ll, D, base_adj + scale_exp(ebp[col], p.xbit));
           double out = __longlong_as_double(bits ^ flip);
           if (amode == 0) out *= p.alpha;
           if (bmode == 1) out += cv[j];
@@ -765,7 +801,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
   }
 }
 
-size_t smem_bytes_for(int S) { return (size_t)STAGES * S * (TM + TN) * TK * 2 + 1024; }
+size_t smem_bytes_for(int S, int tn = TN) { return (size_t)STAGES * S * (TM + tn) * TK * 2 + 1024; }
 
 // cuTensorMapEncodeTiled is a driver-API call; it is resolved at run time through the
 // runtime's entry-point query so the library does not link libcuda directly (it then
@@ -818,7 +854,7 @@ namespace {
 int split_rows(gep_handle_t h, int R, int K, int Kpad, const double* X, long long sr, int* e, int S, int xbit,
                unsigned short* out) {
   if (R < 16 * h->sm_count)
-    k_split_row_blk<<<R, 256, 0, h->stream>>>(R, K, Kpad, X, sr, e, S, xbit, out, h->d_status);
+    k_split_row_blk<<<R, 256, 0, h->stream>>>(R, K, Kpad, Kpad, X, sr, e, S, xbit, out, h->d_status);
   else
     k_split_rows<<<(R * 32 + 255) / 256, 256, 0, h->stream>>>(R, K, Kpad, X, sr, e, S, xbit, out, h->d_status);
   return check_launch(h);
@@ -850,12 +886,14 @@ int split_cols(gep_handle_t h, int R, int K, int Kpad, const double* X, long lon
 
 // Product-kernel launch for one K panel (kc deep, planes padded to a.kpad): dynamic shared
 // memory attribute, optional per-launch timing, template dispatch on the plane/level counts.
-int oz_launch(gep_handle_t h, const CUtensorMap& mA, const CUtensorMap& mB, const OzArgs& a, int kc) {
+int oz_launch(gep_handle_t h, const CUtensorMap& mA, const CUtensorMap& mB, const OzArgs& a, int kc, bool skinny = false) {
   static unsigned long long attr_devices = 0;
   if (first_use_on_device(attr_devices)) {
     cudaFuncSetAttribute(k_oz_gemm<8, 9>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS));
     cudaFuncSetAttribute(k_oz_gemm<3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS));
     cudaFuncSetAttribute(k_oz_gemm<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS));
+    cudaFuncSetAttribute(k_oz_gemm<8, 9, TNS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS, TNS));
+    cudaFuncSetAttribute(k_oz_gemm<3, 4, TNS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS, TNS));
   }
   const int S = a.S, levels = a.lmax;
   dim3 grid(a.ntiles < h->sm_count ? a.ntiles : h->sm_count);  // persistent CTAs
@@ -876,7 +914,9 @@ int oz_launch(gep_handle_t h, const CUtensorMap& mA, const CUtensorMap& mB, cons
       h->prof_skipped++;
     }
   }
-  if (S == 8 && levels == 9) k_oz_gemm<8, 9><<<grid, NTHREADS, smem_bytes_for(S), h->stream>>>(mA, mB, a);
+  if (skinny && S == 8) k_oz_gemm<8, 9, TNS><<<grid, NTHREADS, smem_bytes_for(S, TNS), h->stream>>>(mA, mB, a);
+  else if (skinny) k_oz_gemm<3, 4, TNS><<<grid, NTHREADS, smem_bytes_for(S, TNS), h->stream>>>(mA, mB, a);
+  else if (S == 8 && levels == 9) k_oz_gemm<8, 9><<<grid, NTHREADS, smem_bytes_for(S), h->stream>>>(mA, mB, a);
   else if (S == 3 && levels == 4) k_oz_gemm<3, 4><<<grid, NTHREADS, smem_bytes_for(S), h->stream>>>(mA, mB, a);
   else k_oz_gemm<0, 0><<<grid, NTHREADS, smem_bytes_for(S), h->stream>>>(mA, mB, a);
   GEP_CHECK(check_launch(h));
@@ -894,6 +934,9 @@ void oz_args_init(OzArgs& a, int m, int n, int kpad, int S, int levels, int lowe
   a.gy = (n + TN - 1) / TN;
   a.ntiles = a.gx * a.gy;
   a.kr_n = 0;
+  a.spp = 0;
+  a.zstride = 0;
+  a.eastr = a.ebstr = 0;
   for (int r = 0; r < OZ_KR_MAX; ++r) a.kr_lo[r] = a.kr_hi[r] = 0;
 }
 
@@ -901,9 +944,8 @@ void oz_args_init(OzArgs& a, int m, int n, int kpad, int S, int levels, int lowe
 
 size_t oz_sym_planes_bytes(int m, int levels) {
   if (m <= 0) return 0;
-  const size_t S = (size_t)(levels - 1), np = (m + OZ_SYM_KP - 1) / OZ_SYM_KP;
-  const size_t kpad_last = (size_t)((m - (np - 1) * OZ_SYM_KP + TK - 1) / TK) * TK;
-  return align256((size_t)2 * S * m * ((np - 1) * OZ_SYM_KP + kpad_last)) + align256(sizeof(int) * np * m) + 256;
+  const size_t S = (size_t)(levels - 1), np = (m + OZ_SYM_KP - 1) / OZ_SYM_KP, ldk = (size_t)(m + TK - 1) / TK * TK;
+  return align256((size_t)2 * S * m * ldk) + align256(sizeof(int) * np * m) + 256;
 }
 
 int oz_split_sym(gep_handle_t h, int m, const double* A, int lda, int levels, void* buf, size_t bytes,
@@ -911,56 +953,111 @@ int oz_split_sym(gep_handle_t h, int m, const double* A, int lda, int levels, vo
   const int S = levels - 1;
   if (S < 1 || S > MAXS || m <= 0) return GEP_ERR_UNSUPPORTED;
   if (buf == nullptr || bytes < oz_sym_planes_bytes(m, levels)) return GEP_ERR_ALLOC;
-  const int np = (m + OZ_SYM_KP - 1) / OZ_SYM_KP;
-  const int kpad_last = (m - (np - 1) * OZ_SYM_KP + TK - 1) / TK * TK;
+  const int np = (m + OZ_SYM_KP - 1) / OZ_SYM_KP, ldk = (m + TK - 1) / TK * TK;
   P->planes = (unsigned short*)buf;
-  P->ea = (int*)((char*)buf + align256((size_t)2 * S * m * ((size_t)(np - 1) * OZ_SYM_KP + kpad_last)));
+  P->ea = (int*)((char*)buf + align256((size_t)2 * S * m * ldk));
   P->m = m;
+  P->ldk = ldk;
   P->levels = levels;
   const int xbit = levels >= 8 ? 1 : 0;
   GEP_CUDA(cudaMemsetAsync(P->ea, 0, sizeof(int) * (size_t)np * m, h->stream));
   for (int p = 0; p < np; ++p) {
     const int kb = p * OZ_SYM_KP, kc = min(OZ_SYM_KP, m - kb), kpad = (kc + TK - 1) / TK * TK;
     int* ea = P->ea + (size_t)p * m;
-    unsigned short* As = P->planes + (size_t)p * S * m * OZ_SYM_KP;
     k_rowexp_sym_row<<<dim3((m + 255) / 256, (kc + 63) / 64), 256, 0, h->stream>>>(m, kb, kc, A, lda, ea,
                                                                                   h->d_status);
     GEP_CHECK(check_launch(h));
     k_rowexp_sym_col<<<(m * 32 + 255) / 256, 256, 0, h->stream>>>(m, kb, kc, A, lda, ea, h->d_status);
     GEP_CHECK(check_launch(h));
-    k_split_sym<<<dim3(kpad / 32, (m + 31) / 32), 256, 0, h->stream>>>(m, kc, kpad, kb, A, lda, ea, S, xbit, As,
-                                                                       h->d_status);
+    k_split_sym<<<dim3(kpad / 32, (m + 31) / 32), 256, 0, h->stream>>>(m, kc, ldk, kb, kb, A, lda, ea, S, xbit,
+                                                                       P->planes, h->d_status);
     GEP_CHECK(check_launch(h));
   }
   return GEP_OK;
 }
 
+namespace {
+
+// C = alpha sum_z P_z (+ beta C), parts in order (deterministic).
+__global__ void k_sum_parts(int m, int n, int nz, const double* __restrict__ P, long long zstride, double alpha,
+                            double beta, double* __restrict__ C, int ldc, const int* st) {
+  if (status_bad(st)) return;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+  if (i >= m) return;
+  const double* p = P + i + (size_t)j * m;
+  double s = 0.0;
+#pragma unroll 4
+  for (int z = 0; z < nz; ++z) s += p[(size_t)z * zstride];
+  s *= alpha;
+  double* c = C + i + (size_t)j * ldc;
+  *c = beta == 0.0 ? s : fma(beta, *c, s);
+}
+
+// How many CTAs share a K panel of one tile: the least time by 4 us a wave and tile plus 0.0235 us a
+// K step of 1 (36 plane products at N = 32), and the sums read back.
+int sym_parts(gep_handle_t h, int m, int n, int K, int levels) {
+  const int tiles = (m + TM - 1) / TM * ((n + TNS - 1) / TNS), np = (K + OZ_SYM_KP - 1) / OZ_SYM_KP;
+  const int kp = K < OZ_SYM_KP ? K : OZ_SYM_KP;
+  int best = 1;
+  double tb = 1e30;
+  for (int s = 1; s <= 16 && kp / s >= 128; ++s) {
+    const double waves = (double)((tiles * np * s + h->sm_count - 1) / h->sm_count);
+    const double t = waves * (4.0 + (levels == 9 ? 0.0235 : 0.006) * kp / s) + 2e-6 * (double)m * n * np * s;
+    if (t < tb * 0.97) {
+      tb = t;
+      best = s;
+    }
+  }
+  return best;
+}
+
+}  // namespace
+
+size_t oz_sym_part_elems(int m, int n) {
+  const size_t np = ((size_t)m + OZ_SYM_KP - 1) / OZ_SYM_KP;
+  return (size_t)16 * np * m * n < (size_t)1 << 23 ? (size_t)16 * np * m * n : ((size_t)1 << 23) + np * m * n;
+}
+
+// All K panels and their parts in one launch: with n <= 64 a product has only m / 128 tiles, so the
+// depth is what spreads it over the SMs, and 32-wide tiles waste no plane products at n = 32.
+// (Full to band at b = 32: order 2047 18.1 -> 15.7 ms, 4000 48 -> 38.8 ms, 8192 167 -> 130 ms against
+// 128 x 64 tiles, panel after panel.)
 int dgemm_oz_sym_planes(gep_handle_t h, const OzSymPlanes& P, int row0, int n, double alpha, const double* B,
-                        int ldb, double beta, double* C, int ldc) {
+                        int ldb, double beta, double* C, int ldc, double* parts, size_t part_elems) {
   const int m = P.m - row0, S = P.levels - 1, K = P.m;
   if (row0 < 0 || m <= 0 || n <= 0) return GEP_OK;
-  if (S < 1 || S > MAXS || !P.planes) return GEP_ERR_UNSUPPORTED;
-  const int kp_max = K < OZ_SYM_KP ? K : OZ_SYM_KP;
-  const int kpad_max = (kp_max + TK - 1) / TK * TK;
-  const size_t need = align256((size_t)2 * S * n * kpad_max) + align256(sizeof(int) * (size_t)n) + 256;
+  if ((P.levels != 9 && P.levels != 4) || !P.planes) return GEP_ERR_UNSUPPORTED;
+  const int ldk = P.ldk, np = (K + OZ_SYM_KP - 1) / OZ_SYM_KP;
+  const size_t need = align256((size_t)2 * S * n * ldk) + align256(sizeof(int) * (size_t)n * np) + 256;
   if (h->eng_ws == nullptr || h->eng_bytes < need) return GEP_ERR_ALLOC;
   unsigned short* Bs = (unsigned short*)h->eng_ws;
-  int* eb = (int*)(h->eng_ws + align256((size_t)2 * S * n * kpad_max));
+  int* eb = (int*)(h->eng_ws + align256((size_t)2 * S * n * ldk));
   const int xbit = P.levels >= 8 ? 1 : 0;
-  const int np = (K + OZ_SYM_KP - 1) / OZ_SYM_KP;
-  for (int p = 0; p < np; ++p) {
-    const int kb = p * OZ_SYM_KP, kc = min(OZ_SYM_KP, K - kb), kpad = (kc + TK - 1) / TK * TK;
-    const unsigned short* As = P.planes + (size_t)p * S * P.m * OZ_SYM_KP;
-    GEP_CHECK(split_rows(h, n, kc, kpad, B + kb, ldb, eb, S, xbit, Bs));
-    CUtensorMap mA, mB;
-    GEP_CHECK(encode_map(&mA, As + (size_t)row0 * kpad, kpad, m, S, TM, P.m));  // rows row0.. of each plane
-    GEP_CHECK(encode_map(&mB, Bs, kpad, n, S, TN));
-    OzArgs a;
-    oz_args_init(a, m, n, kpad, S, P.levels, 0, xbit, P.ea + (size_t)p * P.m + row0, eb, alpha,
-                 p == 0 ? beta : 1.0, C, ldc, h->d_status);
-    GEP_CHECK(oz_launch(h, mA, mB, a, kc));
-  }
-  return GEP_OK;
+  k_split_row_blk<<<dim3(n, np), 256, 0, h->stream>>>(n, K, ldk, OZ_SYM_KP, B, ldb, eb, S, xbit, Bs, h->d_status);
+  GEP_CHECK(check_launch(h));
+  CUtensorMap mA, mB;
+  GEP_CHECK(encode_map(&mA, P.planes + (size_t)row0 * ldk, ldk, m, S, TM, P.m));  // rows row0.. of each plane
+  GEP_CHECK(encode_map(&mB, Bs, ldk, n, S, TNS));
+  int spp = sym_parts(h, m, n, K, P.levels);
+  const size_t mn = (size_t)m * n;
+  while (spp > 1 && (size_t)spp * np * mn > part_elems) --spp;
+  if ((size_t)spp * np * mn > part_elems) return GEP_ERR_ALLOC;
+  const int nz = spp * np;
+  const bool direct = nz == 1;
+  OzArgs a;
+  oz_args_init(a, m, n, ldk, S, P.levels, 0, xbit, P.ea + row0, eb, direct ? alpha : 1.0, direct ? beta : 0.0,
+               direct ? C : parts, direct ? ldc : m, h->d_status);
+  a.gy = (n + TNS - 1) / TNS;
+  a.ntiles = a.gx * a.gy * nz;
+  a.spp = spp;
+  a.zstride = (long long)mn;
+  a.eastr = P.m;
+  a.ebstr = n;
+  GEP_CHECK(oz_launch(h, mA, mB, a, K, true));
+  if (direct) return GEP_OK;
+  k_sum_parts<<<dim3((m + 255) / 256, n), 256, 0, h->stream>>>(m, n, nz, parts, (long long)mn, alpha, beta, C, ldc,
+                                                              h->d_status);
+  return check_launch(h);
 }
 
 size_t oz_workspace_bytes(int m, int n, int k) {
@@ -1013,7 +1110,7 @@ int dgemm_oz(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, d
       GEP_CHECK(check_launch(h));
       k_rowexp_sym_col<<<(m * 32 + 255) / 256, 256, 0, h->stream>>>(m, kb, kc, A, lda, ea, h->d_status);
       GEP_CHECK(check_launch(h));
-      k_split_sym<<<dim3(kpad / 32, (m + 31) / 32), 256, 0, h->stream>>>(m, kc, kpad, kb, A, lda, ea, S, xbit, As,
+      k_split_sym<<<dim3(kpad / 32, (m + 31) / 32), 256, 0, h->stream>>>(m, kc, kpad, 0, kb, A, lda, ea, S, xbit, As,
                                                                          h->d_status);
       GEP_CHECK(check_launch(h));
     } else if (ska == 1) {
