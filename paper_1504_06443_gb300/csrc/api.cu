@@ -10,7 +10,7 @@ using namespace gep;
 
 namespace {
 
-constexpr int NB = 128;  // diagonal block order of the triangular kernels (tri.cu)
+constexpr int NB = TRI_NB;  // diagonal block order of the triangular solves (tri.cu)
 
 bool handle_ok(gep_handle_t h) { return h != nullptr && h->magic == 0x6e70; }
 

@@ -172,6 +172,7 @@ int scale_cols_rsqrt_checked(gep_handle_t h, int m, int n, const double* d, doub
 int scan_nonfinite(gep_handle_t h, int M, const double* A, int lda);  // lower triangle
 
 // ---- triangular building blocks (tri.cu) ----
+constexpr int TRI_NB = 256;  // order of the inverted diagonal blocks
 // Inverts every nb x nb diagonal block of the lower triangular L into invD
 // (block b at invD + b*nb*nb, column-major nb x nb, lower; ragged last block padded
 // with identity).

@@ -51,13 +51,13 @@ __device__ void tri_inv_smem(double* S, double* tmp, int r) {
 
 // Writes the r x r lower inverse from shared memory into an NB x NB block (identity
 // padding for r < NB, zero strict upper triangle).
-__device__ void store_inv(const double* S, int r, double* out) {
+__device__ void store_inv(const double* S, int r, double* out, int ldo) {
   for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {
     int i = idx % NB, j = idx / NB;
     double v;
     if (i < r && j < r) v = (i >= j) ? S[i + j * NB] : 0.0;
     else v = (i == j) ? 1.0 : 0.0;
-    out[idx] = v;
+    out[i + j * ldo] = v;
   }
 }
 
@@ -107,7 +107,8 @@ __device__ __forceinline__ bool row_wait(uint32_t bar, int* st) {
 }
 
 __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_diag(int r, double* B, int ldb,
-                                                                                   double* invD, int kb, int* st) {
+                                                                                   double* invD, int ldi, int kb,
+                                                                                   int* st) {
   extern __shared__ __align__(16) unsigned char smraw[];
   PotrfShared& sh = *reinterpret_cast<PotrfShared*>(smraw);
   constexpr int U = NB / 32;
@@ -207,7 +208,7 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_di
   for (int u = 0; u < U; ++u) {
     const int c = lane + 32 * u;
     if (i < r && c <= i) B[GEP_IX(i, c, ldb)] = c == i ? sh.sq[i] : sh.f[w][c] * sh.sq[c];
-    invD[i + c * NB] = c < i ? x[u] * ri : (c == i ? ri : 0.0);
+    invD[i + c * ldi] = c < i ? x[u] * ri : (c == i ? ri : 0.0);
   }
 }
 
@@ -225,7 +226,9 @@ __global__ void __launch_bounds__(256) k_inv_diag(int M, const double* L, int ld
     S[i + j * NB] = (i >= j) ? L[GEP_IX(kb + i, kb + j, ldl)] : 0.0;
   }
   tri_inv_smem(S, tmp, r);
-  store_inv(S, r, invD + (size_t)b * NB * NB);
+  // block b is the upper or lower diagonal half of an inverse block of TRI_NB
+  constexpr int Q = TRI_NB / NB;
+  store_inv(S, r, invD + (size_t)(b / Q) * TRI_NB * TRI_NB + GEP_IX(b % Q * NB, b % Q * NB, TRI_NB), TRI_NB);
 }
 
 constexpr size_t kSmemDiag = (size_t)NB * NB * sizeof(double) + NB * sizeof(double);
@@ -243,30 +246,52 @@ int set_smem_attr() {
 
 size_t trsm_tmp_elems(int M, int n, int nb) { (void)M; return (size_t)nb * (size_t)(n > 0 ? n : 1); }
 
+namespace {
+
+// X21 = -X22 L21 X11 of a block of order n > NB whose diagonal halves are inverted in X (ld
+// TRI_NB), and the zero above it; tmp holds NB x NB.
+int inv_merge(gep_handle_t h, int n, const double* L21, int ldl, double* X, double* tmp, int engine) {
+  const int n1 = NB, n2 = n - NB;
+  GEP_CHECK(set_matrix(h, n1, n2, 0.0, 0.0, X + GEP_IX(0, n1, TRI_NB), TRI_NB));
+  GEP_CHECK(dgemm(h, 'N', 'N', 'F', n2, n1, n1, 1.0, L21, ldl, X, TRI_NB, 0.0, tmp, n2, engine));
+  return dgemm(h, 'N', 'N', 'F', n2, n1, n2, -1.0, X + GEP_IX(n1, n1, TRI_NB), TRI_NB, tmp, n2, 0.0, X + n1, TRI_NB,
+               engine);
+}
+
+}  // namespace
+
 int tri_inv_diag_blocks(gep_handle_t h, int M, const double* L, int ldl, double* invD, int nb) {
-  if (nb != NB) return GEP_ERR_UNSUPPORTED;
+  if (nb != TRI_NB) return GEP_ERR_UNSUPPORTED;
   if (M <= 0) return GEP_OK;
   set_smem_attr();
   int nblk = (M + NB - 1) / NB;
   k_inv_diag<<<nblk, 256, kSmemDiag, h->stream>>>(M, L, ldl, invD, h->d_status);
-  return check_launch(h);
+  GEP_CHECK(check_launch(h));
+  double* tmp = invD + (size_t)((M + TRI_NB - 1) / TRI_NB) * TRI_NB * TRI_NB;
+  for (int o = 0; o + NB < M; o += TRI_NB)
+    GEP_CHECK(inv_merge(h, M - o < TRI_NB ? M - o : TRI_NB, L + GEP_IX(o + NB, o, ldl), ldl,
+                        invD + (size_t)(o / TRI_NB) * TRI_NB * TRI_NB, tmp, GEP_PREC_FP64));
+  return GEP_OK;
 }
 
 // All triangular solves and the Cholesky factorisation below recurse on halves whose
-// split points are multiples of NB, down to the NB x NB diagonal blocks (leaf o covers
-// rows o .. o+NB-1 and uses invD block o/NB).  The off-diagonal work is then a few
+// split points are multiples of TRI_NB, down to the diagonal blocks of TRI_NB = 256 (leaf o covers
+// rows o .. o+TRI_NB-1 and uses invD block o/TRI_NB; a block's factor and inverse come from two
+// halves of NB).  With leaves of NB = 128 the solves took twice as many products, most of them
+// 25 to 60 us of launches and splits (order 2047: reduction 7.0 -> 4.3 ms, back-substitution 1.25 ->
+// 0.76 ms; order 8192: 47 -> 34 and 16.7 -> 15 ms).  The off-diagonal work is then a few
 // products with a long inner dimension (n/2, n/4, ...), which the tensor-core engine
 // runs near its best rate, instead of many rank-NB updates.
 namespace {
 
-int split_nb(int n) { return ((n / NB + 1) / 2) * NB; }
+int split_nb(int n) { return ((n / TRI_NB + 1) / 2) * TRI_NB; }
 
 // rows [o, o+n) of X (X points at row o) := L(o:o+n, o:o+n)^-1 X
 int lln_rec(gep_handle_t h, int o, int n, int ncol, const double* L, int ldl, const double* invD, double* X, int ldx,
             double* tmp, int engine) {
-  if (n <= NB) {
-    const double* Dk = invD + (size_t)(o / NB) * NB * NB;
-    GEP_CHECK(dgemm(h, 'N', 'N', 'F', n, ncol, n, 1.0, Dk, NB, X, ldx, 0.0, tmp, n, engine));
+  if (n <= TRI_NB) {
+    const double* Dk = invD + (size_t)(o / TRI_NB) * TRI_NB * TRI_NB;
+    GEP_CHECK(dgemm(h, 'N', 'N', 'F', n, ncol, n, 1.0, Dk, TRI_NB, X, ldx, 0.0, tmp, n, engine));
     return copy_matrix(h, n, ncol, tmp, n, X, ldx);
   }
   int n1 = split_nb(n), n2 = n - n1;
@@ -279,9 +304,9 @@ int lln_rec(gep_handle_t h, int o, int n, int ncol, const double* L, int ldl, co
 // rows [o, o+n) of X := L(o:o+n, o:o+n)^-T X
 int llt_rec(gep_handle_t h, int o, int n, int ncol, const double* L, int ldl, const double* invD, double* X, int ldx,
             double* tmp, int engine) {
-  if (n <= NB) {
-    const double* Dk = invD + (size_t)(o / NB) * NB * NB;
-    GEP_CHECK(dgemm(h, 'T', 'N', 'F', n, ncol, n, 1.0, Dk, NB, X, ldx, 0.0, tmp, n, engine));
+  if (n <= TRI_NB) {
+    const double* Dk = invD + (size_t)(o / TRI_NB) * TRI_NB * TRI_NB;
+    GEP_CHECK(dgemm(h, 'T', 'N', 'F', n, ncol, n, 1.0, Dk, TRI_NB, X, ldx, 0.0, tmp, n, engine));
     return copy_matrix(h, n, ncol, tmp, n, X, ldx);
   }
   int n1 = split_nb(n), n2 = n - n1;
@@ -294,9 +319,9 @@ int llt_rec(gep_handle_t h, int o, int n, int ncol, const double* L, int ldl, co
 // X (m x n, columns o .. o+n of the factor) := X L(o:o+n, o:o+n)^-T
 int rlt_rec(gep_handle_t h, int o, int n, int m, const double* L, int ldl, const double* invD, double* X, int ldx,
             double* tmp, int engine) {
-  if (n <= NB) {
-    const double* Dk = invD + (size_t)(o / NB) * NB * NB;
-    GEP_CHECK(dgemm(h, 'N', 'T', 'F', m, n, n, 1.0, X, ldx, Dk, NB, 0.0, tmp, m, engine));
+  if (n <= TRI_NB) {
+    const double* Dk = invD + (size_t)(o / TRI_NB) * TRI_NB * TRI_NB;
+    GEP_CHECK(dgemm(h, 'N', 'T', 'F', m, n, n, 1.0, X, ldx, Dk, TRI_NB, 0.0, tmp, m, engine));
     return copy_matrix(h, m, n, tmp, m, X, ldx);
   }
   int n1 = split_nb(n), n2 = n - n1;
@@ -308,10 +333,23 @@ int rlt_rec(gep_handle_t h, int o, int n, int m, const double* L, int ldl, const
 
 // Eq. 4 on the diagonal block (o, o) of order n; B points at the full matrix.
 int potrf_rec(gep_handle_t h, int o, int n, double* B, int ldb, double* invD, double* tmp, int engine) {
-  if (n <= NB) {
-    k_potrf_diag<<<PC, 32 * PW, sizeof(PotrfShared), h->stream>>>(n, B + GEP_IX(o, o, ldb), ldb, invD + (size_t)(o / NB) * NB * NB, o,
-                                                   h->d_status);
-    return check_launch(h);
+  if (n <= TRI_NB) {
+    double* X = invD + (size_t)(o / TRI_NB) * TRI_NB * TRI_NB;
+    const int n1 = n < NB ? n : NB, n2 = n - n1;
+    auto leaf = [&](int at, int r) {
+      k_potrf_diag<<<PC, 32 * PW, sizeof(PotrfShared), h->stream>>>(r, B + GEP_IX(o + at, o + at, ldb), ldb,
+                                                                    X + GEP_IX(at, at, TRI_NB), TRI_NB, o + at, h->d_status);
+      return check_launch(h);
+    };
+    GEP_CHECK(leaf(0, n1));
+    if (n2 == 0) return GEP_OK;
+    double* L21 = B + GEP_IX(o + n1, o, ldb);
+    GEP_CHECK(dgemm(h, 'N', 'T', 'F', n2, n1, n1, 1.0, L21, ldb, X, TRI_NB, 0.0, tmp, n2, engine));  // A21 L11^-T
+    GEP_CHECK(copy_matrix(h, n2, n1, tmp, n2, L21, ldb));
+    GEP_CHECK(dgemm(h, 'N', 'T', 'L', n2, n2, n1, -1.0, L21, ldb, L21, ldb, 1.0, B + GEP_IX(o + n1, o + n1, ldb), ldb,
+                    engine));
+    GEP_CHECK(leaf(n1, n2));
+    return inv_merge(h, n, L21, ldb, X, tmp, engine);
   }
   int n1 = split_nb(n), n2 = n - n1;
   GEP_CHECK(potrf_rec(h, o, n1, B, ldb, invD, tmp, engine));
@@ -327,7 +365,7 @@ int potrf_rec(gep_handle_t h, int o, int n, double* B, int ldb, double* invD, do
 // X := L^-1 X (forward substitution); tmp holds max(NB x n) doubles.
 int trsm_lln(gep_handle_t h, int M, int n, const double* L, int ldl, const double* invD, int nb,
              double* X, int ldx, double* tmp, int engine) {
-  if (nb != NB) return GEP_ERR_UNSUPPORTED;
+  if (nb != TRI_NB) return GEP_ERR_UNSUPPORTED;
   if (M <= 0 || n <= 0) return GEP_OK;
   return lln_rec(h, 0, M, n, L, ldl, invD, X, ldx, tmp, engine);
 }
@@ -335,7 +373,7 @@ int trsm_lln(gep_handle_t h, int M, int n, const double* L, int ldl, const doubl
 // X := L^-T X (backward substitution with the upper triangular L^T).
 int trsm_llt(gep_handle_t h, int M, int n, const double* L, int ldl, const double* invD, int nb,
              double* X, int ldx, double* tmp, int engine) {
-  if (nb != NB) return GEP_ERR_UNSUPPORTED;
+  if (nb != TRI_NB) return GEP_ERR_UNSUPPORTED;
   if (M <= 0 || n <= 0) return GEP_OK;
   return llt_rec(h, 0, M, n, L, ldl, invD, X, ldx, tmp, engine);
 }
@@ -346,8 +384,8 @@ int trsm_llt(gep_handle_t h, int M, int n, const double* L, int ldl, const doubl
 int cholesky(gep_handle_t h, int M, double* B, int ldb, double* invD, int engine) {
   if (M <= 0) return GEP_OK;
   set_smem_attr();
-  int nblk = (M + NB - 1) / NB;
-  double* tmp = invD + (size_t)nblk * NB * NB;
+  int nblk = (M + TRI_NB - 1) / TRI_NB;
+  double* tmp = invD + (size_t)nblk * TRI_NB * TRI_NB;
   return potrf_rec(h, 0, M, B, ldb, invD, tmp, engine);
 }
 
@@ -366,8 +404,8 @@ int reduce_twosided(gep_handle_t h, int M, double* A, int lda, const double* L, 
                     const double* invD, double* X, double* tmp, int engine) {
   if (M <= 0) return GEP_OK;
   // panel width: a multiple of NB (the triangular recursions split at multiples of NB)
-  int nbp = (M / 8) / NB * NB;
-  if (nbp < NB) nbp = NB;
+  int nbp = (M / 8) / TRI_NB * TRI_NB;
+  if (nbp < TRI_NB) nbp = TRI_NB;
   if (nbp > 1024) nbp = 1024;
   for (int k = 0; k < M; k += nbp) {
     const int nb = (M - k) < nbp ? (M - k) : nbp, n2 = M - k - nb;
@@ -410,7 +448,7 @@ int reduce_explicit_inv(gep_handle_t h, int M, double* A, int lda, double* L, in
   double* T = tmp;                    // M x M
   double* tmp_small = tmp + (size_t)M * M;  // NB x M
   GEP_CHECK(set_matrix(h, M, M, 0.0, 1.0, X, M));
-  GEP_CHECK(trsm_lln(h, M, M, L, ldl, invD, NB, X, M, tmp_small, engine));  // X = R = L^-1
+  GEP_CHECK(trsm_lln(h, M, M, L, ldl, invD, TRI_NB, X, M, tmp_small, engine));  // X = R = L^-1
   GEP_CHECK(symmetrize_lower(h, M, A, lda));
   GEP_CHECK(dgemm(h, 'N', 'N', 'F', M, M, M, 1.0, X, M, A, lda, 0.0, T, M, engine));   // T = R A
   GEP_CHECK(dgemm(h, 'N', 'T', 'L', M, M, M, 1.0, T, M, X, M, 0.0, A, lda, engine));   // C = T R^T
