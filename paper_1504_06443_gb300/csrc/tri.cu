@@ -403,10 +403,16 @@ int cholesky(gep_handle_t h, int M, double* B, int ldb, double* invD, int engine
 int reduce_twosided(gep_handle_t h, int M, double* A, int lda, const double* L, int ldl,
                     const double* invD, double* X, double* tmp, int engine) {
   if (M <= 0) return GEP_OK;
-  // panel width: a multiple of NB (the triangular recursions split at multiples of NB)
-  int nbp = (M / 8) / TRI_NB * TRI_NB;
+  // Panel width: a multiple of NB (the triangular recursions split at multiples of NB), half the
+  // matrix up to 2048.  Every panel is a chain of some twenty launches that depend on one another,
+  // and its rank-2 nb update splits its operands anew; wide panels have fewer chains and give the
+  // tensor engine deep products.  R2 at 1501 / 2047 / 3000 / 4000 / 6000 / 8192: with M / 8 up to
+  // 1024 2.4 / 4.2 / 8.6 / 15.1 / 23.1 / 33.5 ms, with M / 3 up to 2048 2.4 / 3.0 / 5.3 / 7.9 /
+  // 15.9 / 29.3 ms, so 1.8 / 2.8 / 4.7 / 7.6 / 14.8 / 29.2 ms; up to 4096 order 6000 takes 15.7 ms.
+  // [A21 L21] and its twin need 4 (M - nb) nb <= M^2 numbers of X for every nb.
+  int nbp = (M / 2) / TRI_NB * TRI_NB;
   if (nbp < TRI_NB) nbp = TRI_NB;
-  if (nbp > 1024) nbp = 1024;
+  if (nbp > 2048) nbp = 2048;
   for (int k = 0; k < M; k += nbp) {
     const int nb = (M - k) < nbp ? (M - k) : nbp, n2 = M - k - nb;
     double* A11 = A + GEP_IX(k, k, lda);
