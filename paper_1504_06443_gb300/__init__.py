@@ -603,7 +603,11 @@ def dgemm(A, B, transa="N", transb="N", alpha=1.0, beta=0.0, C=None, uplo="F", e
     Ac, Bc = colmajor(A), colmajor(B)
     Cc = colmajor(C.clone()) if C is not None else torch.zeros((n, m), dtype=torch.float64, device=A.device).t()
     kp = min(max(k, 1), 4096)
-    h.ensure_workspace(8 * (m + n) * (kp + 32) * 2 + 4 * (m + n) + 8192)
+    need = 8 * (m + n) * (kp + 32) * 2 + 4 * (m + n) + 8192
+    if k >= 512 and engine == "fp64_emulated":  # residue products in full K panels, 2048 columns at a time
+        nb = min(n, 2048) + 256
+        need = max(need, 32 * (m + nb) * (kp + 64) + 16 * m * nb + 4 * (m + nb) + 8192)
+    h.ensure_workspace(need)
     _check(h.lib.gep_dgemm(h.h, transa.encode(), transb.encode(), uplo.encode(), m, n, k, float(alpha), _ptr(Ac),
                            _ld(Ac), _ptr(Bc), _ld(Bc), float(beta), _ptr(Cc), _ld(Cc), _PRECS[engine]), "gep_dgemm")
     return Cc

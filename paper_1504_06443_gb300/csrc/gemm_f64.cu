@@ -303,7 +303,7 @@ int dgemm_f64(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, 
 //                  + 0.047 k (36 plane products; 0.01 k with 3 planes), and the operands' digits
 //                  (24 bytes an element at 5 TB/s).
 // So 128^3 (10.5 / 28 us) and 128 x 128 x 2048 stay on the FP64 units, 256^3 (35 / 35 us) and
-// 127 x 1024 x 1024 (234 / 60 us) go to the tensor cores.
+// 127 x 1024 x 1024 (234 / 60 us) go to the tensor cores (deep ones in the form of gemm_res.cu).
 bool product_on_tensor_cores(gep_handle_t h, char uplo, int m, int n, int k, int engine) {
   if (engine == GEP_PREC_FP64 || m < 32 || n < 16 || k < 16) return false;
   const double half = (uplo == 'L' || uplo == 'l') ? 0.5 : 1.0;

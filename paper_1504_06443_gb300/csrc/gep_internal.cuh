@@ -135,6 +135,12 @@ int dgemm(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, doub
 bool product_on_tensor_cores(gep_handle_t h, char uplo, int m, int n, int k, int engine);
 int dgemm_f64(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha,
               const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc);
+// The same product through residues (gemm_res.cu): where it is the faster form, and the product itself
+// (GEP_ERR_ALLOC / GEP_ERR_UNSUPPORTED before any work if the scratch is too small or C overlaps an operand).
+bool res_product_wins(gep_handle_t h, char uplo, int m, int n, int k);
+size_t res_workspace_bytes(int m, int n, int k);
+int dgemm_res(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha, const double* A,
+              int lda, const double* B, int ldb, double beta, double* C, int ldc);
 int dgemm_oz(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha,
              const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
              int levels, const OzKRange* kr = nullptr);
