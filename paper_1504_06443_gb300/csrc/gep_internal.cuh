@@ -197,6 +197,9 @@ int reduce_twosided(gep_handle_t h, int M, double* A, int lda, const double* L, 
                     const double* invD, double* X, double* tmp, int engine);
 int reduce_explicit_inv(gep_handle_t h, int M, double* A, int lda, double* L, int ldl,
                         const double* invD, double* X, double* tmp, int engine);
+// Small trailing matrices of it in one cluster (tridiag_cluster.cu).
+bool tridiag_cluster_takes(int n);
+int tridiag_cluster(gep_handle_t h, int n, double* C, int ldc, double* d, double* e, double* tau);
 int tridiag_1stage(gep_handle_t h, int M, double* C, int ldc, double* d, double* e, double* tau,
                    double* ws, size_t ws_elems, int engine);
 size_t tridiag_ws_elems(int M);

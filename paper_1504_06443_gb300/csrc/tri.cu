@@ -92,18 +92,24 @@ struct PotrfShared {
 
 __device__ __forceinline__ uint32_t cta_shared(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Bounded wait for a published row (about a second); on expiry records the timeout.
+// Bounded wait (two seconds) for a published row; on expiry records the timeout.
 __device__ __forceinline__ bool row_wait(uint32_t bar, int* st) {
-  for (int it = 0; it < (1 << 22); ++it) {
+  unsigned long long t0 = 0, now;
+  for (int it = 0;; ++it) {
     uint32_t ok;
     asm volatile(
         "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0; selp.u32 %0, 1, 0, p; }"
         : "=r"(ok) : "r"(bar) : "memory");
     if (ok) return true;
-    if ((it & 1023) == 1023 && *(volatile int*)(st + 1) != 0) return false;
+    if ((it & 15) != 15) continue;
+    if (*(volatile int*)(st + 1) != 0) return false;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    if (t0 == 0) t0 = now;
+    if (now - t0 > 2000000000ull) {
+      atomicExch(st + 1, GEP_ERR_TIMEOUT);
+      return false;
+    }
   }
-  atomicExch(st + 1, GEP_ERR_TIMEOUT);
-  return false;
 }
 
 __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_diag(int r, double* B, int ldb,

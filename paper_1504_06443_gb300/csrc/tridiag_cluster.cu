@@ -1,0 +1,355 @@
+// Tridiagonalisation of small matrices, and of the last columns of large ones, in one launch of one cluster.
+//
+// The trailing matrix (order n <= 512) stays in the registers of 4 to 16 CTAs for the whole
+// reduction: CTA k holds the rows l = k mod CL, a warp one or two of them, lane and slot the
+// columns 32 t + lane, both triangles.  A column then costs one exchange instead of two grid barriers:
+//   every CTA knows column i (thread l holds x_l) and forms the reflector for itself;
+//   every warp applies the update of the step before to its rows (while warp 0 forms the
+//   reflector's scalars), multiplies them with v and pushes y_l = (A v)_l together with its
+//   element of column i + 1 to all CTAs (st.async, counted by an mbarrier of each);
+//   every CTA forms w = tau y - (tau / 2) (tau y^T v) v and column i + 1 - v w_1 - w v_1 for itself.
+// Unblocked: three products an element and column.  In FP64 they would take 3 n^2 / 32 clocks on 16
+// SMs, more than everything else from n = 150 on, so the matrix is held in fixed point, as in the
+// bulge chasing: C = q 2^-sh with the largest absolute row sum (a bound on the 2-norm, which no
+// similarity changes) in (2^60, 2^61], v in Q62 with v_1 = 1, tau in Q61; ||w|| <= 2 ||C||.  Products
+// are rounded to 2^-62 of the bound; only a reflector's scalars are FP64.
+//
+// Bound: the chain of a column (two warp and CTA reductions, the scalars, the push: 2.8 us) and from
+// n = 260 on the integer products (6 us a column in all at n = 512).  S1 of the cooperative panels -> here:
+// order 64 0.62 -> 0.18 ms, 128 1.28 -> 0.37, 256 2.74 -> 0.80, 500 5.67 -> 2.45, the last 512 columns of
+// 1501 6 -> 2.5.  Beyond 512 rows the registers of 16 SMs are full.
+#include <cooperative_groups.h>
+
+#include "fixed.cuh"
+#include "gep_internal.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace gep {
+namespace {
+
+constexpr int TRC_MAX = 512, TRC_WARPS = 16, TRC_THREADS = 32 * TRC_WARPS, TRC_CL = 16;
+
+struct TrcArgs {
+  int n, ldc;
+  double *C, *d, *e, *tau;  // C: element (0, 0) of the trailing matrix; d, e, tau: of its first column
+  int* st;
+};
+
+struct TrcShared {
+  int2 v[2][TRC_MAX], w[TRC_MAX];
+  longlong2 recv[2][TRC_MAX];  // y_l, element (l, i + 1)
+  longlong2 ack[TRC_CL];
+  unsigned long long bar[2];
+  ll xmax[TRC_CL], xa, tauq, zs[TRC_WARPS], tops[TRC_WARPS], mids[TRC_WARPS];
+  int2 mq;
+  int lzs[TRC_WARPS], zero;
+  double tau, beta;
+};
+
+__device__ __forceinline__ uint32_t trc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Sum over the warp of 44-bit non-negative numbers.
+__device__ __forceinline__ ll sum44(ll v) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x3FFFFFu);
+  const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 22));
+  return ((ll)hi << 22) + lo;
+}
+
+// x 2^sh rounded to an integer, from the bits of x (finite; |x| 2^sh < 2^62).
+__device__ __forceinline__ ll trc_fix(ll bits, int sh) {
+  const int E = (int)((bits >> 52) & 0x7FF);
+  if (E == 0) return 0;
+  const ll m = (bits & 0xFFFFFFFFFFFFFll) | (1ll << 52);
+  const int s = E - 1075 + sh;
+  const ll q = s >= 0 ? m << s : (s > -54 ? (m + (1ll << (-s - 1))) >> -s : 0);
+  return bits < 0 ? -q : q;
+}
+
+// v 2^-62 as a double.
+__device__ __forceinline__ double trc_unit(ll v) {
+  if (v == 0) return 0.0;
+  const double m = qdouble((unsigned long long)(v < 0 ? -v : v));
+  return __longlong_as_double((__double_as_longlong(m) - (62ll << 52)) | (v & (1ll << 63)));
+}
+
+// Largest value over the CTAs of the cluster (not below 0).
+__device__ ll trc_cluster_max(cg::cluster_group& cl, TrcShared& sh, ll v) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int o = 16; o; o >>= 1) {
+    const ll q = __shfl_xor_sync(0xffffffffu, v, o);
+    v = q > v ? q : v;
+  }
+  if (lane == 0) sh.zs[warp] = v;
+  __syncthreads();
+  if (threadIdx.x < cl.num_blocks()) {
+    ll m = 0;
+    for (int q = 0; q < TRC_WARPS; ++q) m = sh.zs[q] > m ? sh.zs[q] : m;
+    cl.map_shared_rank(sh.xmax, threadIdx.x)[cl.block_rank()] = m;
+  }
+  cl.sync();
+  ll m = 0;
+  for (int q = 0; q < (int)cl.num_blocks(); ++q) m = sh.xmax[q] > m ? sh.xmax[q] : m;
+  cl.sync();
+  return m;
+}
+
+// Bounded wait (two seconds) for the pushes of a column.
+__device__ bool trc_wait(uint32_t bar, uint32_t parity, int* st) {
+  unsigned long long t0 = 0, now;
+  for (int it = 0;; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
+    if ((it & 15) != 15) continue;
+    if (*(volatile int*)(st + 1) != 0) return false;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    if (t0 == 0) t0 = now;
+    if (now - t0 > 2000000000ull) {
+      atomicExch(st + 1, GEP_ERR_TIMEOUT);
+      return false;
+    }
+  }
+}
+
+// RPW rows a warp, NT slots of 32 columns: n <= 32 NT and n <= 16 RPW CL.
+template <int RPW, int NT>
+__global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
+  __shared__ TrcShared sh;
+  cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), k = (int)cl.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = p.n, l = tid;
+  const bool bad = status_bad(p.st);  // (every thread of the cluster passes through the same barriers)
+  if (tid == 0)
+    for (int b = 0; b < 2; ++b)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(trc_smem(&sh.bar[b])) : "memory");
+  if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  for (int j = tid; j < TRC_MAX; j += TRC_THREADS) sh.v[0][j] = sh.v[1][j] = sh.w[j] = make_int2(0, 0);
+
+  // rows as bits of doubles; their largest exponent
+  ll a[RPW][NT];
+  int em = 0;
+#pragma unroll
+  for (int u = 0; u < RPW; ++u) {
+    const int r = (warp + TRC_WARPS * u) * CL + k;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const int j = 32 * t + lane;
+      a[u][t] = r < n && j < n ? __double_as_longlong(p.C[GEP_IX(r > j ? r : j, r > j ? j : r, p.ldc)]) : 0;
+      em = max(em, (int)((a[u][t] >> 52) & 0x7FF));
+    }
+  }
+  const int emax = (int)trc_cluster_max(cl, sh, em);
+  const bool finite = emax < 0x7FF;
+  // row sums with every element below 2^53, then the shift that puts the largest into (2^60, 2^61]
+  const int sh0 = 1075 - emax;
+  ll rs = 0;
+#pragma unroll
+  for (int u = 0; u < RPW; ++u) {
+    ll s = 0;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const ll q = trc_fix(a[u][t] & ~(1ll << 63), sh0);
+      s += q;
+    }
+    s = qwarp_sum(s);
+    rs = s > rs ? s : rs;
+  }
+  rs = trc_cluster_max(cl, sh, rs);
+  const int scale = sh0 + (rs > 0 ? __clzll(rs) - 3 : 0);
+#pragma unroll
+  for (int u = 0; u < RPW; ++u)
+#pragma unroll
+    for (int t = 0; t < NT; ++t) a[u][t] = trc_fix(a[u][t], scale);
+  ll x = l < n ? trc_fix(__double_as_longlong(p.C[l]), scale) : 0;
+  cl.sync();  // every element is read before the first reflector is stored
+
+  // two words to the same place in CTA q, counted by its barrier
+  auto push = [&](longlong2* slot, int buf, int q, ll y, ll el) {
+    uint32_t rd, rb;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(trc_smem(slot)), "r"(q));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(trc_smem(&sh.bar[buf])), "r"(q));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(rd),
+                 "l"(y), "l"(el), "r"(rb) : "memory");
+  };
+  const int cols = bad ? 0 : n;
+  for (int i = 0; i < cols; ++i) {
+    const int buf = i & 1;
+    const bool act = l > i && l < n;
+    if (l == i && k == 0) p.d[i] = finite ? scale2((double)x, -scale) : NAN;
+    if (i == n - 1) break;
+    if (tid == 0)
+      asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(trc_smem(&sh.bar[buf])),
+                   "r"(16 * max(n - 1 - i, CL)) : "memory");
+    // ---- norm of x(i + 2 ..), x scaled up until its largest entry fills [2^61, 2^62)
+    {
+      const unsigned lz = act ? (unsigned)__clzll(x < 0 ? ~x : x) : 64u;
+      const unsigned m = __reduce_min_sync(0xffffffffu, lz);
+      if (lane == 0) sh.lzs[warp] = (int)m;
+      if (l == i + 1) sh.xa = x;
+    }
+    __syncthreads();
+    const int up = max(0, min((int)__reduce_min_sync(0xffffffffu, (unsigned)sh.lzs[lane & (TRC_WARPS - 1)]), 62) - 2);
+    const ll z = act ? x << up : 0;
+    {
+      const unsigned long long az = l > i + 1 ? (unsigned long long)(z < 0 ? -z : z) : 0ull;
+      const unsigned long long hi = __umul64hi(az, az), lo = az * az;  // squares in two parts: 2^86 and 2^48
+      const ll top = sum44((ll)(hi >> 22)), mid = sum44((ll)(((hi << 16) | (lo >> 48)) & 0x3FFFFFFFFFull));
+      if (lane == 0) {
+        sh.tops[warp] = top;
+        sh.mids[warp] = mid;
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      ll top = sum44(lane < TRC_WARPS ? sh.tops[lane] : 0);
+      const ll mid = sum44(lane < TRC_WARPS ? sh.mids[lane] : 0);
+      top += mid >> 38;
+      const ll low = mid & 0x3FFFFFFFFFll, xa = sh.xa;
+      if (lane == 0) {
+        if ((top | low) != 0) {
+          const int sft = top ? min(__clzll(top) - 1, 38) : 38;
+          const double s2 = qdouble((unsigned long long)((top << sft) + (low >> (38 - sft)))) *
+                            __longlong_as_double((ll)(1023 + 86 - sft) << 52);
+          const ll za = xa << up;
+          const double al = qdouble((unsigned long long)(za < 0 ? -za : za)), n2 = fma(al, al, s2);
+          const double ri = qrsqrt(n2), nrm = n2 * ri;
+          const ll m = qint(qrcp(al + nrm), 123);
+          const double tau = fma(al, ri, 1.0);
+          sh.mq = qsplit(za < 0 ? -m : m);
+          sh.tauq = qint(tau, 61);
+          sh.zero = 0;
+          sh.tau = tau;
+          sh.beta = scale2(za < 0 ? nrm : -nrm, -(up + scale));
+        } else {
+          sh.zero = 1;
+          sh.tauq = 0;
+          sh.tau = 0.0;
+          sh.beta = scale2((double)xa, -scale);
+        }
+      }
+    }
+    // ---- the update of the step before
+    if (i > 0) {
+#pragma unroll
+      for (int u = 0; u < RPW; ++u) {
+        const int r = (warp + TRC_WARPS * u) * CL + k;
+        if (r > i && r < n) {
+          const int2 vr = sh.v[buf ^ 1][r], wr = sh.w[r];
+#pragma unroll
+          for (int t = 0; t < NT; ++t) {
+            if (32 * t + 31 <= i) continue;
+            const int j = 32 * t + lane;
+            const int2 vj = sh.v[buf ^ 1][j], wj = sh.w[j];
+            a[u][t] -= ((qhh(vr, wj) + qhh(wr, vj)) << 2) + ((qmid(vr, wj, 1ll << 29) >> 30) + (qmid(wr, vj, 1ll << 29) >> 30));
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // ---- v
+    const int2 tq = qsplit(sh.tauq);
+    ll v = 0;
+    if (act && !sh.zero) v = l == i + 1 ? 1ll << 62 : qmul<61>(qsplit(z), sh.mq);
+    const int2 vl = qsplit(v);
+    sh.v[buf][l] = vl;
+    if (act && l % CL == k) p.C[GEP_IX(l, i, p.ldc)] = !finite ? NAN : l == i + 1 ? sh.beta : trc_unit(v);
+    if (k == 0 && tid == 0) {
+      p.e[i] = finite ? sh.beta : NAN;
+      p.tau[i] = finite ? sh.tau : NAN;
+    }
+    __syncthreads();
+    // ---- y = A v on this warp's rows, pushed to every CTA with the element of column i + 1
+    ll yr[RPW], nx[RPW];
+#pragma unroll
+    for (int u = 0; u < RPW; ++u) {
+      const int r = (warp + TRC_WARPS * u) * CL + k;
+      yr[u] = nx[u] = 0;
+      if (r > i && r < n) {
+        ll hh = 0, mm = 0, c1 = 0;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+          c1 |= a[u][t] & (t == ((i + 1) >> 5) ? -1ll : 0ll);
+          if (32 * t + 31 <= i) continue;
+          const int2 q = qsplit(a[u][t]), vj = sh.v[buf][32 * t + lane];
+          hh += qhh(q, vj);
+          mm += qmid(q, vj, 1ll << 29) >> 30;
+        }
+        yr[u] = qwarp_sum((hh << 2) + mm);
+        nx[u] = __shfl_sync(0xffffffffu, c1, (i + 1) & 31);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < RPW; ++u) {
+      const int r = (warp + TRC_WARPS * u) * CL + k;
+      if (r > i && r < n && lane < CL) {
+        push(&sh.recv[buf][r], buf, lane, yr[u], nx[u]);
+      }
+    }
+    // A CTA whose rows are all done still reports every column: the others may be one column ahead of
+    // it, as the two buffers allow, and not more.
+    if (n - 1 - i < CL && warp == 0 && lane < CL) {
+      const int first = i + 1 + (k - (i + 1) % CL + CL) % CL;  // its next row
+      if (first >= n) push(&sh.ack[k], buf, lane, 0, 0);
+    }
+    const bool ok = trc_wait(trc_smem(&sh.bar[buf]), (uint32_t)(i >> 1) & 1u, p.st);
+    // ---- w and column i + 1
+    const ll y = act ? sh.recv[buf][l].x : 0, raw = act ? sh.recv[buf][l].y : 0;
+    const ll pl = qmul<61>(qsplit(y), tq);
+    {
+      const ll s = qwarp_sum(qmul<62>(qsplit(pl), vl));
+      if (lane == 0) sh.zs[warp] = s;
+    }
+    const ll p1 = qmul<61>(qsplit(sh.recv[buf][i + 1].x), tq);
+    if (!__syncthreads_and(ok)) break;
+    const ll dot = qwarp_sum(lane < TRC_WARPS ? sh.zs[lane] : 0);
+    const int2 al = qsplit(qmul<62>(qsplit(dot), tq));
+    const ll w = pl - qmul<62>(al, vl);
+    const ll w1 = p1 - qjoin(al);
+    sh.w[l] = qsplit(act ? w : 0);
+    x = act ? raw - qmul<62>(vl, qsplit(sh.zero ? 0 : w1)) - w : 0;
+  }
+  cl.sync();  // no CTA leaves while another may still push to it
+}
+
+template <int RPW, int NT>
+int trc_launch(gep_handle_t h, const TrcArgs& a, int cl) {
+  static unsigned long long devices = 0;
+  if (first_use_on_device(devices))
+    GEP_CUDA(cudaFuncSetAttribute((const void*)k_trd_cluster<RPW, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cl);
+  cfg.blockDim = dim3(TRC_THREADS);
+  cfg.stream = h->stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cl;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  GEP_CUDA(cudaLaunchKernelEx(&cfg, k_trd_cluster<RPW, NT>, a));
+  return check_launch(h);
+}
+
+}  // namespace
+
+// Whether tridiag_cluster takes a trailing matrix of order n.
+bool tridiag_cluster_takes(int n) { return n <= TRC_MAX; }
+
+// Reduces the n x n symmetric matrix in the lower triangle of C to tridiagonal form: d, e, tau and the
+// reflectors below the subdiagonal, as tridiag_1stage stores them.
+int tridiag_cluster(gep_handle_t h, int n, double* C, int ldc, double* d, double* e, double* tau) {
+  if (n <= 0) return GEP_OK;
+  if (n > TRC_MAX) return GEP_ERR_UNSUPPORTED;
+  TrcArgs a;
+  a.n = n; a.ldc = ldc; a.C = C; a.d = d; a.e = e; a.tau = tau; a.st = h->d_status;
+  // 16 rows a CTA: a warp each
+  if (n <= 64) return trc_launch<1, 2>(h, a, n <= 16 ? 1 : n <= 32 ? 2 : 4);
+  if (n <= 128) return trc_launch<1, 4>(h, a, 8);
+  if (n <= 256) return trc_launch<1, 8>(h, a, 16);
+  return trc_launch<2, 16>(h, a, 16);
+}
+
+}  // namespace gep
