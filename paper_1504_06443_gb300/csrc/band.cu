@@ -742,9 +742,9 @@ __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
 // at most 2^61; reflectors have v in Q62 (|v_i| <= 1 by construction), tau in Q61.  The norms
 // in play (v^T v <= 2, tau |v| <= 2, w = tau C v - ... at most 2 |C|) keep every intermediate
 // below 2^63.  A product drops only the low x low limb: its error is about half a unit, 2^-62
-// of the row-sum bound, where an FP64 operation rounds its result at 2^-54.  Only a
-// reflector's scalars (norm, reciprocal, tau, beta) are FP64, from the column scaled up to
-// full width.  An FP64 instruction holds a scheduler for 64 clocks on this part; the three
+// of the row-sum bound, where an FP64 operation rounds its result at 2^-54; every term is rounded by
+// itself (a constant for the floors of a sum would leave noise in rows beyond the matrix and turn
+// zeros into 2^-57).  A reflector's scalars come from exact squares (q_reflector).  An FP64 instruction holds a scheduler for 64 clocks on this part; the three
 // 32 x 32 -> 64 multiply-adds of a fixed-point product and their shifts take about 20.
 //
 // Schedule.  A sweep's reflectors form a chain of their own: x of step k + 1 is column 0 of
@@ -769,7 +769,6 @@ struct BulgeShared {
   ll redU[N / BC][N], redD[N / BC][N];
   int2 yv[2][N], vp[2][N], vc[2][N];  // split into limbs
   ll sc[2][2];                        // tau (Q61), beta
-  double taud[2];
   unsigned long long full_y[2], full_v[2], empty[2];
   int abort_a[2], abort_u[2];
 };
@@ -887,7 +886,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
           if (R > 1 && w >= G / R) vsel = v[R - 1];  // the half of v that holds this warp's columns
           ll hh[R], mm[R];
 #pragma unroll
-          for (int r = 0; r < R; ++r) { hh[r] = 0; mm[r] = C / 2; }  // (C / 2: the floors of C shifts)
+          for (int r = 0; r < R; ++r) { hh[r] = 0; mm[r] = 0; }
 #pragma unroll
           for (int q = 0; q < C; ++q) {
             int2 vq;
@@ -897,7 +896,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
             for (int r = 0; r < R; ++r) {
               const int2 bb = qsplit(b[r][q]);
               hh[r] += qhh(bb, vq);
-              mm[r] += qmid(bb, vq, 0) >> 30;
+              mm[r] += qmid(bb, vq, 1ll << 29) >> 30;
             }
           }
 #pragma unroll
@@ -926,42 +925,25 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
             for (int q = 0; q < C; ++q) sh.Bs[buf][w * C + q][lane + 32 * r] = b[r][q];
         }
         mb_arrive(&sh.full_y[buf]);
-        // reflector of x, formed by every finder warp for itself: x scaled up so that its largest
-        // entry fills [2^59, 2^60), squares in units of 2^63 (2^-55 of the largest or finer)
-        int lz = 64;
-#pragma unroll
-        for (int r = 0; r < R; ++r) lz = min(lz, __clzll(x[r] < 0 ? ~x[r] : x[r]));
-        const int up = min((int)__reduce_min_sync(0xffffffffu, (unsigned)lz), 62) - 4;  // may be negative
-        ll s2 = 0;
-        int2 xs[R];
-        ll x00 = 0;
+        // reflector of x, formed by every finder warp for itself, from the exact sum of the squares:
+        // entries far below alpha must not vanish in it
+        unsigned sq[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          const ll z = up >= 0 ? x[r] << up : x[r] >> -up;
-          if (r == 0) x00 = z;
-          xs[r] = qsplit(z);
-          if (lane + 32 * r > 0) s2 += qsquare(xs[r]);
+          const unsigned long long ax = lane + 32 * r > 0 ? (unsigned long long)(x[r] < 0 ? -x[r] : x[r]) : 0ull;
+          add_square(sq, ax);
         }
-        s2 = qwarp_sum(s2);
-        const ll alpha_q = __shfl_sync(0xffffffffu, x[0], 0), xa = __shfl_sync(0xffffffffu, x00, 0);
-        ll beq = alpha_q, tauq = 0;
-        double tau = 0.0;
-        if (s2 > 0) {
-          // be = -sign(alpha) |x|, v = x / (alpha - be), tau = 1 + |alpha| / |x|
-          const double al = qdouble(xa < 0 ? -xa : xa), n2 = fma(al, al, qdouble(s2) * 0x1p63);
-          const double ri = qrsqrt(n2), nrm = n2 * ri;
-          const ll m = qint(qrcp(al + nrm), 121);
-          const int2 mq = qsplit(xa < 0 ? -m : m);
+        const Sum128 s2 = warp_squares(sq);
+        const ll alpha_q = __shfl_sync(0xffffffffu, x[0], 0);
+        QReflector o;
+        o.m = o.tq = 0;
+        o.beta = alpha_q;
+        o.up = 0;
+        if ((s2.lo | s2.hi) != 0) o = q_reflector(alpha_q, s2);
+        const int2 mq = qsplit(o.m);
 #pragma unroll
-          for (int r = 0; r < R; ++r) v[r] = qsplit(qmul<59>(xs[r], mq));
-          tau = fma(al, ri, 1.0);
-          tauq = qint(tau, 61);
-          beq = qint(nrm, -up);
-          if (xa >= 0) beq = -beq;
-        } else {
-#pragma unroll
-          for (int r = 0; r < R; ++r) v[r] = make_int2(0, 0);
-        }
+        for (int r = 0; r < R; ++r) v[r] = qsplit(qmul<61>(qsplit(x[r] << o.up), mq));
+        const ll beq = o.beta, tauq = o.tq;
         taup = qsplit(tauq);
         if (lane == 0) v[0] = make_int2(0, 1 << 30);
         if (w == 0) {
@@ -970,7 +952,6 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
           if (lane == 0) {
             sh.sc[buf][0] = tauq;
             sh.sc[buf][1] = beq;
-            sh.taud[buf] = tau;
             AB[k == 0 ? 1 + (size_t)s * LD : N + (size_t)stp * LD] = beq;
           }
           mb_arrive(&sh.full_v[buf]);
@@ -1005,7 +986,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
 #pragma unroll
           for (int r = 0; r < R; ++r) {
             zh[r] = 0;
-            zm[r] = C / 2;  // the floors of C shifts
+            zm[r] = 0;
           }
 #pragma unroll
           for (int q = 0; q < C; ++q) {
@@ -1014,7 +995,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
             for (int r = 0; r < R; ++r) {
               const int2 bb = qsplit(b[r][q]);
               zh[r] += qhh(bb, vq);
-              zm[r] += qmid(bb, vq, 0) >> 30;
+              zm[r] += qmid(bb, vq, 1ll << 29) >> 30;
             }
           }
 #pragma unroll
@@ -1059,7 +1040,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
           for (int r = 0; r < R; ++r)
             if (lane + 32 * r < len)
               D0[(c + lane + 32 * r) + (size_t)c * 2 * N] = (double)qjoin(sh.vc[buf][lane + 32 * r]) * 0x1p-62;
-          if (lane == 0) D0[(size_t)2 * N * N + c] = sh.taud[buf];
+          if (lane == 0) D0[(size_t)2 * N * N + c] = qscaled(sh.sc[buf][0], 61);
         }
         mb_arrive(&sh.empty[buf]);
         group_sync<4, 2 * G>();  // the stores of both groups precede the release
@@ -1108,7 +1089,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
         for (int r = 0; r < R; ++r) {
           vr[r] = sh.vc[buf][lane + 32 * r];
           hh[r] = 0;
-          mm[r] = C / 2;
+          mm[r] = 0;
         }
 #pragma unroll
         for (int q = 0; q < C; ++q) {
@@ -1117,7 +1098,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
           for (int r = 0; r < R; ++r) {
             const int2 dd = qsplit(sh.Ds[u * C + q][lane + 32 * r]);
             hh[r] += qhh(dd, vq);
-            mm[r] += qmid(dd, vq, 0) >> 30;
+            mm[r] += qmid(dd, vq, 1ll << 29) >> 30;
           }
         }
 #pragma unroll

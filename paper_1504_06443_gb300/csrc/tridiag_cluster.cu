@@ -12,7 +12,7 @@
 // SMs, more than everything else from n = 150 on, so the matrix is held in fixed point, as in the
 // bulge chasing: C = q 2^-sh with the largest absolute row sum (a bound on the 2-norm, which no
 // similarity changes) in (2^60, 2^61], v in Q62 with v_1 = 1, tau in Q61; ||w|| <= 2 ||C||.  Products
-// are rounded to 2^-62 of the bound; only a reflector's scalars are FP64.
+// are rounded to 2^-62 of the bound, squares and their sums are exact.
 //
 // Bound: the chain of a column (two warp and CTA reductions, the scalars, the push: 2.8 us) and from
 // n = 260 on the integer products (6 us a column in all at n = 512).  S1 of the cooperative panels -> here:
@@ -41,37 +41,14 @@ struct TrcShared {
   longlong2 recv[2][TRC_MAX];  // y_l, element (l, i + 1)
   longlong2 ack[TRC_CL];
   unsigned long long bar[2];
-  ll xmax[TRC_CL], xa, tauq, zs[TRC_WARPS], tops[TRC_WARPS], mids[TRC_WARPS];
+  ll xmax[TRC_CL], xa, tauq, zs[TRC_WARPS];
+  ll d[TRC_MAX], e[TRC_MAX], tau[TRC_MAX];  // results, turned into doubles at the end
+  unsigned sq[TRC_WARPS][6];                // sums of squares in six parts
   int2 mq;
-  int lzs[TRC_WARPS], zero;
-  double tau, beta;
+  int up, zero;
 };
 
 __device__ __forceinline__ uint32_t trc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Sum over the warp of 44-bit non-negative numbers.
-__device__ __forceinline__ ll sum44(ll v) {
-  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x3FFFFFu);
-  const unsigned hi = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 22));
-  return ((ll)hi << 22) + lo;
-}
-
-// x 2^sh rounded to an integer, from the bits of x (finite; |x| 2^sh < 2^62).
-__device__ __forceinline__ ll trc_fix(ll bits, int sh) {
-  const int E = (int)((bits >> 52) & 0x7FF);
-  if (E == 0) return 0;
-  const ll m = (bits & 0xFFFFFFFFFFFFFll) | (1ll << 52);
-  const int s = E - 1075 + sh;
-  const ll q = s >= 0 ? m << s : (s > -54 ? (m + (1ll << (-s - 1))) >> -s : 0);
-  return bits < 0 ? -q : q;
-}
-
-// v 2^-62 as a double.
-__device__ __forceinline__ double trc_unit(ll v) {
-  if (v == 0) return 0.0;
-  const double m = qdouble((unsigned long long)(v < 0 ? -v : v));
-  return __longlong_as_double((__double_as_longlong(m) - (62ll << 52)) | (v & (1ll << 63)));
-}
 
 // Largest value over the CTAs of the cluster (not below 0).
 __device__ ll trc_cluster_max(cg::cluster_group& cl, TrcShared& sh, ll v) {
@@ -151,7 +128,7 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
     ll s = 0;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
-      const ll q = trc_fix(a[u][t] & ~(1ll << 63), sh0);
+      const ll q = qfix(a[u][t] & ~(1ll << 63), sh0);
       s += q;
     }
     s = qwarp_sum(s);
@@ -162,8 +139,8 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
 #pragma unroll
   for (int u = 0; u < RPW; ++u)
 #pragma unroll
-    for (int t = 0; t < NT; ++t) a[u][t] = trc_fix(a[u][t], scale);
-  ll x = l < n ? trc_fix(__double_as_longlong(p.C[l]), scale) : 0;
+    for (int t = 0; t < NT; ++t) a[u][t] = qfix(a[u][t], scale);
+  ll x = l < n ? qfix(__double_as_longlong(p.C[l]), scale) : 0;
   cl.sync();  // every element is read before the first reflector is stored
 
   // two words to the same place in CTA q, counted by its barrier
@@ -178,57 +155,43 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
   for (int i = 0; i < cols; ++i) {
     const int buf = i & 1;
     const bool act = l > i && l < n;
-    if (l == i && k == 0) p.d[i] = finite ? scale2((double)x, -scale) : NAN;
+    if (l == i) sh.d[i] = x;
     if (i == n - 1) break;
     if (tid == 0)
       asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(trc_smem(&sh.bar[buf])),
                    "r"(16 * max(n - 1 - i, CL)) : "memory");
-    // ---- norm of x(i + 2 ..), x scaled up until its largest entry fills [2^61, 2^62)
+    // ---- norm of x(i + 2 ..): from the exact squares
     {
-      const unsigned lz = act ? (unsigned)__clzll(x < 0 ? ~x : x) : 64u;
-      const unsigned m = __reduce_min_sync(0xffffffffu, lz);
-      if (lane == 0) sh.lzs[warp] = (int)m;
+      const unsigned long long ax = act && l > i + 1 ? (unsigned long long)(x < 0 ? -x : x) : 0ull;
+      unsigned q[6] = {0, 0, 0, 0, 0, 0};
+      add_square(q, ax);
+#pragma unroll
+      for (int u = 0; u < 6; ++u) q[u] = __reduce_add_sync(0xffffffffu, q[u]);
+      if (lane == 0)
+#pragma unroll
+        for (int u = 0; u < 6; ++u) sh.sq[warp][u] = q[u];
       if (l == i + 1) sh.xa = x;
     }
     __syncthreads();
-    const int up = max(0, min((int)__reduce_min_sync(0xffffffffu, (unsigned)sh.lzs[lane & (TRC_WARPS - 1)]), 62) - 2);
-    const ll z = act ? x << up : 0;
-    {
-      const unsigned long long az = l > i + 1 ? (unsigned long long)(z < 0 ? -z : z) : 0ull;
-      const unsigned long long hi = __umul64hi(az, az), lo = az * az;  // squares in two parts: 2^86 and 2^48
-      const ll top = sum44((ll)(hi >> 22)), mid = sum44((ll)(((hi << 16) | (lo >> 48)) & 0x3FFFFFFFFFull));
-      if (lane == 0) {
-        sh.tops[warp] = top;
-        sh.mids[warp] = mid;
-      }
-    }
-    __syncthreads();
     if (warp == 0) {
-      ll top = sum44(lane < TRC_WARPS ? sh.tops[lane] : 0);
-      const ll mid = sum44(lane < TRC_WARPS ? sh.mids[lane] : 0);
-      top += mid >> 38;
-      const ll low = mid & 0x3FFFFFFFFFll, xa = sh.xa;
+      unsigned q[6];
+#pragma unroll
+      for (int u = 0; u < 6; ++u) q[u] = lane < TRC_WARPS ? sh.sq[lane][u] : 0u;
+      const Sum128 S = warp_squares(q);
+      const ll xa = sh.xa;
+      QReflector o;
+      o.m = o.tq = 0;
+      o.beta = xa;
+      o.up = 0;
+      const bool nz = (S.lo | S.hi) != 0;
+      if (nz) o = q_reflector(xa, S);
       if (lane == 0) {
-        if ((top | low) != 0) {
-          const int sft = top ? min(__clzll(top) - 1, 38) : 38;
-          const double s2 = qdouble((unsigned long long)((top << sft) + (low >> (38 - sft)))) *
-                            __longlong_as_double((ll)(1023 + 86 - sft) << 52);
-          const ll za = xa << up;
-          const double al = qdouble((unsigned long long)(za < 0 ? -za : za)), n2 = fma(al, al, s2);
-          const double ri = qrsqrt(n2), nrm = n2 * ri;
-          const ll m = qint(qrcp(al + nrm), 123);
-          const double tau = fma(al, ri, 1.0);
-          sh.mq = qsplit(za < 0 ? -m : m);
-          sh.tauq = qint(tau, 61);
-          sh.zero = 0;
-          sh.tau = tau;
-          sh.beta = scale2(za < 0 ? nrm : -nrm, -(up + scale));
-        } else {
-          sh.zero = 1;
-          sh.tauq = 0;
-          sh.tau = 0.0;
-          sh.beta = scale2((double)xa, -scale);
-        }
+        sh.mq = qsplit(o.m);
+        sh.tauq = o.tq;
+        sh.up = o.up;
+        sh.zero = !nz;
+        sh.e[i] = o.beta;
+        sh.tau[i] = o.tq;
       }
     }
     // ---- the update of the step before
@@ -252,14 +215,9 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
     // ---- v
     const int2 tq = qsplit(sh.tauq);
     ll v = 0;
-    if (act && !sh.zero) v = l == i + 1 ? 1ll << 62 : qmul<61>(qsplit(z), sh.mq);
+    if (act && !sh.zero) v = l == i + 1 ? 1ll << 62 : qmul<61>(qsplit(x << sh.up), sh.mq);
     const int2 vl = qsplit(v);
     sh.v[buf][l] = vl;
-    if (act && l % CL == k) p.C[GEP_IX(l, i, p.ldc)] = !finite ? NAN : l == i + 1 ? sh.beta : trc_unit(v);
-    if (k == 0 && tid == 0) {
-      p.e[i] = finite ? sh.beta : NAN;
-      p.tau[i] = finite ? sh.tau : NAN;
-    }
     __syncthreads();
     // ---- y = A v on this warp's rows, pushed to every CTA with the element of column i + 1
     ll yr[RPW], nx[RPW];
@@ -294,6 +252,8 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
       const int first = i + 1 + (k - (i + 1) % CL + CL) % CL;  // its next row
       if (first >= n) push(&sh.ack[k], buf, lane, 0, 0);
     }
+    if (act && l % CL == k)  // (while the others push)
+      p.C[GEP_IX(l, i, p.ldc)] = !finite ? NAN : l == i + 1 ? scale2(qscaled(sh.e[i], 0), -scale) : qscaled(v, 62);
     const bool ok = trc_wait(trc_smem(&sh.bar[buf]), (uint32_t)(i >> 1) & 1u, p.st);
     // ---- w and column i + 1
     const ll y = act ? sh.recv[buf][l].x : 0, raw = act ? sh.recv[buf][l].y : 0;
@@ -310,6 +270,14 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
     const ll w1 = p1 - qjoin(al);
     sh.w[l] = qsplit(act ? w : 0);
     x = act ? raw - qmul<62>(vl, qsplit(sh.zero ? 0 : w1)) - w : 0;
+  }
+  __syncthreads();
+  if (k == 0 && l < cols) {
+    p.d[l] = finite ? scale2(qscaled(sh.d[l], 0), -scale) : NAN;
+    if (l + 1 < n) {
+      p.e[l] = finite ? scale2(qscaled(sh.e[l], 0), -scale) : NAN;
+      p.tau[l] = finite ? qscaled(sh.tau[l], 61) : NAN;
+    }
   }
   cl.sync();  // no CTA leaves while another may still push to it
 }

@@ -117,3 +117,38 @@ def test_no_drift_of_the_spectrum(gep, b):
     assert info == 0
     ref = torch.linalg.eigvalsh(C)
     assert float((w - ref).norm() / ref.norm()) <= 6 * EPS
+
+
+@pytest.mark.parametrize("b", [32, 64])
+@pytest.mark.parametrize("M", [200, 400])
+@pytest.mark.parametrize("decay", [20.0, 60.0])
+def test_graded_reflectors_stay_orthogonal(gep, M, b, decay):
+    """Columns far below the norm bound: the reflectors are formed from a few units of the fixed point, and
+    those at the end of the matrix must not see rows beyond it."""
+    import torch
+    rng = np.random.default_rng(b)
+    S = rng.standard_normal((M, M))
+    s = np.exp(-np.linspace(0, decay, M))
+    C = dev((S + S.T) * np.outer(s, s))
+    d, e, tau1, q2, Cr = gep.tridiag_2stage(C, b=b)
+    eye = torch.eye(M, dtype=torch.float64, device="cuda")
+    Q = gep.sep_backtransform_2stage(Cr, tau1, q2, b, eye)
+    T = torch.diag(d) + torch.diag(e, 1) + torch.diag(e, -1)
+    assert float((Q.t() @ Q - eye).abs().max()) <= 200 * M * EPS
+    assert float((Q.t() @ C @ Q - T).abs().max()) <= 200 * M * EPS * float(torch.linalg.matrix_norm(C, 2))
+
+
+@pytest.mark.parametrize("b", [32, 64])
+@pytest.mark.parametrize("eps", [1e-6, 1e-9, 1e-12])
+def test_nearly_tridiagonal(gep, b, eps):
+    """Entries far below alpha are annihilated, not dropped."""
+    M = 200
+    rng = np.random.default_rng(b)
+    S = rng.standard_normal((M, M))
+    S = S + S.T
+    i = np.arange(M)
+    C = np.where(np.abs(i[:, None] - i[None, :]) <= 1, S, S * eps)
+    w = np.linalg.eigvalsh(C)
+    d, e, _, _, _ = gep.tridiag_2stage(dev(C), b=b)
+    T = np.diag(d.cpu().numpy()) + np.diag(e.cpu().numpy(), 1) + np.diag(e.cpu().numpy(), -1)
+    assert np.max(np.abs(np.linalg.eigvalsh(T) - w)) <= 200 * M * EPS * np.max(np.abs(w))
