@@ -285,7 +285,8 @@ __global__ void __launch_bounds__(PQ_ROWS) k_pqr_coop(int n, int nb, int rp, dou
 
 size_t pqr_coop_smem_bytes(int rp, int nb) { return (size_t)rp * (nb + 1) * sizeof(double); }
 
-// ---- panel QR of at most 32 columns, registers only, with its T factor
+// ---- panel QR of at most 32 columns, registers only, with its T factor (panels of more than 2048 rows;
+// panel_cluster.cu takes the shorter ones)
 //
 // One cooperative launch: warp w of a CTA holds RPW consecutive rows of the panel, lane j column j,
 // so that a column's update and the next column's dot products are one FMA each per row of a
@@ -1485,14 +1486,13 @@ int panel_qr_launch(gep_handle_t h, const PanelArgs& a, long long part_elems) {
 
 int panel_qr(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, const BandWs& w, double* Va, double* Vb,
              int r0, int ldv) {
+  if (panel_qr_cluster_takes(n, b)) return panel_qr_cluster(h, n, b, P, ldp, tau, Va, Vb, r0, ldv, w.T);
   PanelArgs a;
   a.n = n; a.nb = b; a.ldp = ldp; a.r0 = r0; a.ldv = ldv;
   a.P = P; a.tau = tau; a.part = w.part0; a.prow = w.prow0; a.Va = Va; a.Vb = Vb; a.T = w.T;
   a.bar = w.bar; a.st = h->d_status;
   const long long cap = 2 * w.gcap * BMAX;  // part0 and part1 together
-  const int rows = n <= 127 * 2 ? 1 : n <= 127 * 8 ? 2 : n <= 127 * 32 ? 4 : n <= 127 * 128 ? 8 : 16;
-  if (rows == 1) return panel_qr_launch<1>(h, a, cap);
-  if (rows == 2) return panel_qr_launch<2>(h, a, cap);
+  const int rows = n <= 127 * 32 ? 4 : n <= 127 * 128 ? 8 : 16;
   if (rows == 4) return panel_qr_launch<4>(h, a, cap);
   if (rows == 8) return panel_qr_launch<8>(h, a, cap);
   return panel_qr_launch<16>(h, a, cap);

@@ -197,6 +197,10 @@ int reduce_twosided(gep_handle_t h, int M, double* A, int lda, const double* L, 
                     const double* invD, double* X, double* tmp, int engine);
 int reduce_explicit_inv(gep_handle_t h, int M, double* A, int lda, double* L, int ldl,
                         const double* invD, double* X, double* tmp, int engine);
+// QR of a panel of at most 32 columns with its T factor in one cluster (panel_cluster.cu).
+bool panel_qr_cluster_takes(int n, int nb);
+int panel_qr_cluster(gep_handle_t h, int n, int nb, double* P, int ldp, double* tau, double* Va, double* Vb, int r0,
+                     int ldv, double* T);
 // Small trailing matrices of it in one cluster (tridiag_cluster.cu).
 bool tridiag_cluster_takes(int n);
 int tridiag_cluster(gep_handle_t h, int n, double* C, int ldc, double* d, double* e, double* tau);
