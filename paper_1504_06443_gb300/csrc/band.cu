@@ -459,14 +459,18 @@ __global__ void __launch_bounds__(32 * (PQW + 1)) k_panel_qr(PanelArgs a) {
 }
 
 // W = (Y - V M) T with Y = C22 V (n x nb), M = T^T S / 2, S = V^T Y: the companion of V in the
-// two-sided update, written to both group buffers at full height.  Lane j owns column j, a warp a
-// row at a time; M is formed by every CTA for itself (a b^3 / 2 product: cheaper than a launch).
+// two-sided update, written to both group buffers at full height.  Lane j owns column j, a warp U
+// rows; M is formed by every CTA for itself (a b^3 / 2 product: cheaper than a launch).
+// Bound: FP64 issue, 2 U + 4 products of 32 FMAs a warp: U = 4 takes 29 us whatever n, so few rows go to
+// more CTAs: U = 1 15 us, U = 2 20 us.
+template <int U>
 __global__ void __launch_bounds__(256) k_panel_w(int n, int nb, const double* __restrict__ V, int ldv,
                                                  const double* __restrict__ Y, const double* __restrict__ T,
                                                  const double* __restrict__ S, double* __restrict__ Wa,
                                                  double* __restrict__ Wb, int r0, const int* st) {
   __shared__ double Tm[PQN][PQN + 1], Sm[PQN][PQN + 1], Mm[PQN][PQN + 1];
-  __shared__ double yt[PQN][33], vt[PQN][33];
+  constexpr int ROWS = 8 * U;
+  __shared__ double yt[PQN][ROWS + 1], vt[PQN][ROWS + 1];
   if (status_bad(st)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int idx = blockIdx.x * blockDim.x + tid; idx < r0 * nb; idx += gridDim.x * blockDim.x) {
@@ -487,41 +491,43 @@ __global__ void __launch_bounds__(256) k_panel_w(int n, int nb, const double* __
     for (int q = 0; q <= i; ++q) s = fma(Tm[q][i], Sm[q][lane], s);
     Mm[i][lane] = 0.5 * s;
   }
-  for (int b0 = blockIdx.x * 32; b0 < n; b0 += gridDim.x * 32) {
+  for (int b0 = blockIdx.x * ROWS; b0 < n; b0 += gridDim.x * ROWS) {
     __syncthreads();
-    for (int idx = tid; idx < 32 * nb; idx += 256) {
-      const int r = b0 + (idx & 31), j = idx >> 5;
-      yt[j][idx & 31] = r < n ? Y[r + (size_t)j * n] : 0.0;
-      vt[j][idx & 31] = r < n ? V[r + (size_t)j * ldv] : 0.0;
+    for (int idx = tid; idx < ROWS * nb; idx += 256) {
+      const int r = b0 + idx % ROWS, j = idx / ROWS;
+      yt[j][idx % ROWS] = r < n ? Y[r + (size_t)j * n] : 0.0;
+      vt[j][idx % ROWS] = r < n ? V[r + (size_t)j * ldv] : 0.0;
     }
     __syncthreads();
-    double y[4];
+    double y[U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) y[u] = lane < nb ? yt[lane][warp * 4 + u] : 0.0;
+    for (int u = 0; u < U; ++u) y[u] = lane < nb ? yt[lane][warp * U + u] : 0.0;
 #pragma unroll 4
     for (int q = 0; q < nb; ++q) {
       const double m = Mm[q][lane];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) y[u] = fma(-vt[q][warp * 4 + u], m, y[u]);
+      for (int u = 0; u < U; ++u) y[u] = fma(-vt[q][warp * U + u], m, y[u]);
     }
-    double w[4] = {0.0, 0.0, 0.0, 0.0};
+    double w[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) w[u] = 0.0;
 #pragma unroll 4
     for (int q = 0; q < nb; ++q) {
       const double t = Tm[q][lane];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) w[u] = fma(__shfl_sync(0xffffffffu, y[u], q), t, w[u]);
+      for (int u = 0; u < U; ++u) w[u] = fma(__shfl_sync(0xffffffffu, y[u], q), t, w[u]);
     }
     __syncthreads();
     if (lane < nb)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) yt[lane][warp * 4 + u] = w[u];
+      for (int u = 0; u < U; ++u) yt[lane][warp * U + u] = w[u];
     __syncthreads();
-    for (int idx = tid; idx < 32 * nb; idx += 256) {
-      const int r = b0 + (idx & 31), j = idx >> 5;
+    for (int idx = tid; idx < ROWS * nb; idx += 256) {
+      const int r = b0 + idx % ROWS, j = idx / ROWS;
       if (r >= n) continue;
       const size_t o = (size_t)j * ldv + r0 + r;
-      Wa[o] = yt[j][idx & 31];
-      Wb[o] = yt[j][idx & 31];
+      Wa[o] = yt[j][idx % ROWS];
+      Wb[o] = yt[j][idx % ROWS];
     }
   }
 }
@@ -1626,7 +1632,9 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
       }
       if (narrow) {
         GEP_CHECK(dgemm_f64(h, 'T', 'N', 'F', b, b, nr, 1.0, Vj, ldv, w.CV, nr, 0.0, w.Pm, b));  // V^T C22 V
-        k_panel_w<<<std::min((nr + 31) / 32, 2 * h->sm_count), 256, 0, h->stream>>>(
+        const auto kernel = nr <= 8 * h->sm_count ? k_panel_w<1> : nr <= 16 * h->sm_count ? k_panel_w<2> : k_panel_w<4>;
+        const int rows = nr <= 8 * h->sm_count ? 8 : nr <= 16 * h->sm_count ? 16 : 32;
+        kernel<<<std::min((nr + rows - 1) / rows, 2 * h->sm_count), 256, 0, h->stream>>>(
             nr, b, Vj, ldv, w.CV, w.T, w.Pm, wv(2 * j), vw(2 * j + 1), r0, h->d_status);
         GEP_CHECK(check_launch(h));
         continue;
