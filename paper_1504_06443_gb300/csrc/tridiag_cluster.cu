@@ -11,12 +11,14 @@
 // Unblocked: three products an element and column.  In FP64 they would take 3 n^2 / 32 clocks on 16
 // SMs, more than everything else from n = 150 on, so the matrix is held in fixed point, as in the
 // bulge chasing: C = q 2^-sh with the largest absolute row sum (a bound on the 2-norm, which no
-// similarity changes) in (2^60, 2^61], v in Q62 with v_1 = 1, tau in Q61; ||w|| <= 2 ||C||.  Products
-// are rounded to 2^-62 of the bound, squares and their sums are exact.
+// similarity changes) in (2^60, 2^61], v in Q62 with v_1 = 1, tau in Q61; ||w|| <= 2 ||C||.  A dense
+// matrix of order 500 has entries of about 52 bits in it, so sums are kept ten bits longer than their
+// result and an update rounds once (a rounding per product made the vectors of order 500 2.2 times as
+// far off as FP64 panels); squares and their sums are exact.
 //
-// Bound: the chain of a column (two warp and CTA reductions, the scalars, the push: 2.8 us) and from
-// n = 260 on the integer products (6 us a column in all at n = 512).  S1 of the cooperative panels -> here:
-// order 64 0.62 -> 0.18 ms, 128 1.28 -> 0.37, 256 2.74 -> 0.80, 500 5.67 -> 2.45, the last 512 columns of
+// Bound: the chain of a column (two warp and CTA reductions, the scalars, the push: 2.2 us) and from
+// n = 260 on the integer products (7 us a column in all at n = 512).  S1 of the cooperative panels -> here:
+// order 64 0.62 -> 0.14 ms, 128 1.28 -> 0.29, 256 2.74 -> 0.67, 500 5.67 -> 2.4, the last 512 columns of
 // 1501 6 -> 2.5.  Beyond 512 rows the registers of 16 SMs are full.
 #include <cooperative_groups.h>
 
@@ -206,7 +208,8 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
             if (32 * t + 31 <= i) continue;
             const int j = 32 * t + lane;
             const int2 vj = sh.v[buf ^ 1][j], wj = sh.w[j];
-            a[u][t] -= ((qhh(vr, wj) + qhh(wr, vj)) << 2) + ((qmid(vr, wj, 1ll << 29) >> 30) + (qmid(wr, vj, 1ll << 29) >> 30));
+            // (one rounding; with v_r^2 + v_j^2 <= 1 beside v_1 the four middle products stay below 2^63)
+            a[u][t] -= ((qhh(vr, wj) + qhh(wr, vj)) << 2) + (qmid(vr, wj, qmid(wr, vj, 1ll << 29)) >> 30);
           }
         }
       }
@@ -233,9 +236,9 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
           if (32 * t + 31 <= i) continue;
           const int2 q = qsplit(a[u][t]), vj = sh.v[buf][32 * t + lane];
           hh += qhh(q, vj);
-          mm += qmid(q, vj, 1ll << 29) >> 30;
+          mm += qmid(q, vj, (((ll)q.x * vj.x) >> 32) + (1ll << 19)) >> 20;  // 10 bits more than a unit
         }
-        yr[u] = qwarp_sum((hh << 2) + mm);
+        yr[u] = qwarp_sum((hh << 2) + ((mm + 512) >> 10));
         nx[u] = __shfl_sync(0xffffffffu, c1, (i + 1) & 31);
       }
     }
