@@ -1796,6 +1796,95 @@ static void q2_tile_kranges(int b, OzKRange* kr) {
   }
 }
 
+namespace {
+
+// ---- larger Q2 tiles
+//
+// Four tiles (2J + a, 2K + b) of order w make one of order 2 w (the same staircase with twice the
+// step): U = T01 T00 T11 T10, T_ab at rows (a + b) w / 2.  With U = I + V and the overlaps of w / 2 rows,
+//   VA = V10 + V11 + V11(:, :w/2) V10(w/2:, :),  VB = V00 + V01 + V01(:, :w/2) V00(w/2:, :),
+//   V = VA + VB + VB(:, w/2:3w/2) VA(w/2:3w/2, :).
+// A tile twice as large costs the same flops a row of Z but half the passes over it (digits or residues
+// of Z, C in and out), and from order 1024 on the products go through residues.  Order 8192: S3 102 -> 75 ms.
+
+// VA and VB of tiles z: their placed parts (tiles of a row follow each other; nA, nB of them).
+__global__ void __launch_bounds__(256) k_q2_place(int w, const double* __restrict__ rowA, int nA,
+                                                  const double* __restrict__ rowB, int nB, double* __restrict__ VA,
+                                                  double* __restrict__ VB, const int* st) {
+  if (status_bad(st)) return;
+  const int z = blockIdx.z, c = blockIdx.y, r = blockIdx.x * 256 + threadIdx.x, h = w / 2;
+  if (r >= 2 * w) return;
+  const size_t ww = (size_t)w * w, o = (size_t)z * 4 * ww + r + (size_t)c * 2 * w;
+  auto el = [&](const double* row, int n, int t, int off) {
+    const int i = r - off, j = c - off;
+    return t < n && i >= 0 && i < w && j >= 0 && j < w ? row[t * ww + i + (size_t)j * w] : 0.0;
+  };
+  VA[o] = el(rowB, nB, 2 * z, h) + el(rowB, nB, 2 * z + 1, w);
+  VB[o] = el(rowA, nA, 2 * z, 0) + el(rowA, nA, 2 * z + 1, h);
+}
+
+__global__ void __launch_bounds__(256) k_q2_sum(size_t n, const double* __restrict__ VA, const double* __restrict__ VB,
+                                                double* __restrict__ V, const int* st) {
+  if (status_bad(st)) return;
+  for (size_t i = blockIdx.x * (size_t)256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) V[i] = VA[i] + VB[i];
+}
+
+// dst: the (nA + 1) / 2 tiles of order 2 w that the tiles of rows 2J (rowA) and 2J + 1 (rowB) make.
+int merge_q2_tiles(gep_handle_t h, int w, const double* rowA, int nA, const double* rowB, int nB, double* VA,
+                   double* VB, double* dst) {
+  const int count = (nA + 1) / 2, hw = w / 2, ld = 2 * w;
+  const long long ww = (long long)w * w;
+  k_q2_place<<<dim3((2 * w + 255) / 256, 2 * w, count), 256, 0, h->stream>>>(w, rowA, nA, rowB, nB, VA, VB, h->d_status);
+  GEP_CHECK(check_launch(h));
+  if (nB >= 2)
+    GEP_CHECK(dgemm_oz_batched(h, w, w, hw, rowB + ww, w, 2 * ww, rowB + hw, w, 2 * ww, VA + w + (size_t)hw * ld, ld,
+                               4 * ww, nB / 2));
+  if (nA >= 2)
+    GEP_CHECK(dgemm_oz_batched(h, w, w, hw, rowA + ww, w, 2 * ww, rowA + hw, w, 2 * ww, VB + hw, ld, 4 * ww, nA / 2));
+  k_q2_sum<<<8 * h->sm_count, 256, 0, h->stream>>>((size_t)count * 4 * ww, VA, VB, dst, h->d_status);
+  GEP_CHECK(check_launch(h));
+  if (nB >= 1)
+    GEP_CHECK(dgemm_oz_batched(h, 3 * hw, 3 * hw, w, VB + (size_t)hw * ld, ld, 4 * ww, VA + hw + (size_t)hw * ld, ld,
+                               4 * ww, dst + (size_t)hw * ld, ld, 4 * ww, (nB + 1) / 2));
+  return GEP_OK;
+}
+
+// Tiles of level L (order W 2^L) out of the tiles of level 0.
+struct Q2Levels {
+  gep_handle_t h;
+  int Q, TQ, W;
+  const double* U;
+  int nJ(int L) const { return ((Q / TQ + 1) + (1 << L) - 1) >> L; }
+  int nK(int L, int J) const {
+    if (L == 0) return J * TQ <= Q ? (Q - J * TQ) / TQ + 1 : 0;
+    return (nK(L - 1, 2 * J) + 1) / 2;
+  }
+  size_t tile(int L) const { return (size_t)W * W << (2 * L); }
+  // doubles that tiles(L, ..., cnt) takes from its buffer
+  size_t need(int L, int cnt) const { return L == 0 ? 0 : 3 * cnt * tile(L) + 2 * need(L - 1, 2 * cnt); }
+  // *out: tiles K0 .. K0 + cnt - 1 of row J (those that exist, following each other); buf: need(L, cnt)
+  int tiles(int L, int J, int K0, int cnt, double* buf, const double** out, int* have) const {
+    *have = std::max(0, std::min(cnt, nK(L, J) - K0));
+    if (L == 0) {
+      *out = U + (all_tiles_offset(Q, J, TQ) + K0) * tile(0);
+      return GEP_OK;
+    }
+    double* dst = buf;
+    double* VA = dst + cnt * tile(L);
+    double* VB = VA + cnt * tile(L);
+    double* bA = VB + cnt * tile(L);
+    double* bB = bA + need(L - 1, 2 * cnt);
+    const double *rA = nullptr, *rB = nullptr;
+    int nA = 0, nB = 0;
+    GEP_CHECK(tiles(L - 1, 2 * J, 2 * K0, 2 * cnt, bA, &rA, &nA));
+    if (nK(L - 1, 2 * J + 1) > 2 * K0) GEP_CHECK(tiles(L - 1, 2 * J + 1, 2 * K0, 2 * cnt, bB, &rB, &nB));
+    *out = dst;
+    return nA > 0 ? merge_q2_tiles(h, W << (L - 1), rA, nA, rB, nB, VA, VB, dst) : GEP_OK;
+  }
+};
+
+}  // namespace
+
 // Z (M x ncol) <- Q2 Z.  engine FP64: diamonds applied directly on the FP64 cores.
 // Otherwise the diamonds are merged into dense W x W tiles U(J, R) and every tile is
 // applied as one product Z(rows) <- U Z(rows) on the engine (ws: q2_tile_ws_elems); U_all: the
@@ -1808,26 +1897,49 @@ int apply_q2(gep_handle_t h, int M, int b, const double* q2, double* Z, int ldz,
   if (engine != GEP_PREC_FP64) {
     if (!U_all || ws_elems < q2_tile_ws_elems(M, b)) return GEP_ERR_ALLOC;
     const int TQ = tile_q(b), W = 2 * TQ * b;
-    const int nJ = Q / TQ + 1;
+    // Levels of merging, where the tiles suit the batched products and the scratch holds them (narrow Z does
+    // not pay for the merging).  S3 with 0 / 1 / 2 levels: order 2047 3.82 / 3.86 / 3.86 ms, 3000 9.5 / 8.2 / 8.2,
+    // 4000 16.8 / 14.5 / 16.7, 6000 46.5 / 39.2 / 38.8, 8192 102 / 81 / 75, 16384 (b = 64) 651 / 531 / 451; a third
+    // level gains nothing (467 at 16384).
+    Q2Levels lv{h, Q, TQ, W, U_all};
+    int L = engine == GEP_PREC_FP64_EMULATED && W % 256 == 0 && ncol >= 2048 ? (M >= 6000 ? 2 : M >= 2560 ? 1 : 0) : 0;
+    // (beside the tiles: a copy of up to 256 rows of Z, and one K panel of digits for products in place)
+    const size_t rest = (size_t)256 * ncol;
+    auto fits = [&](int l, int c) {
+      const size_t w = (size_t)W << l;
+      return w <= 2048 && lv.need(l, c) + rest <= ws_elems && 16 * (w + ncol) * w + 4 * (w + ncol) + 4096 <= h->eng_bytes;
+    };
+    while (L > 0 && !fits(L, 1)) --L;
+    int chunk = 1;
+    while (L > 0 && chunk < 8 && fits(L, 2 * chunk)) chunk *= 2;
+    const int WL = W << L;
     double* Tmp = ws;
     OzKRange kr;
     q2_tile_kranges(b, &kr);
-    for (int J = nJ - 1; J >= 0; --J) {
-      const int nK = (Q - J * TQ) / TQ + 1;  // tiles (J, K) with a diamond: K TQ <= Q - J TQ
-      const double* U = U_all + all_tiles_offset(Q, J, TQ) * (size_t)W * W;
+    for (int J = lv.nJ(L) - 1; J >= 0; --J) {
+      const int nK = lv.nK(L, J);  // tiles (J, K) with a diamond
+      const double* row = nullptr;
+      int first = 0, have = 0;
       for (int K = 0; K < nK; ++K) {
-        const int r0 = 1 + (J + K) * TQ * b;
+        const int r0 = 1 + (J + K) * (WL / 2);
         if (r0 >= M) break;
-        const int Wc = (M - r0) < W ? (M - r0) : W;
-        const double* Ut = U + (size_t)K * W * W;
+        if (K >= first + have) {
+          first = K;
+          GEP_CHECK(lv.tiles(L, J, K, L ? chunk : nK, ws, &row, &have));
+        }
+        const int Wc = (M - r0) < WL ? (M - r0) : WL;
+        const double* Ut = row + (size_t)(K - first) * WL * WL;
         // one K panel of the split-BF16 engine: all of Z(rows) is split into digit planes
         // before its product kernel writes C, so the update may run in place
         const size_t one_panel = (size_t)16 * (Wc + ncol) * ((Wc + 31) / 32 * 32) + (size_t)4 * (Wc + ncol) + 4096;
         if (product_on_tensor_cores(h, 'F', Wc, ncol, Wc, engine) && Wc <= 4096 && one_panel <= h->eng_bytes) {
-          GEP_CHECK(dgemm(h, 'N', 'N', 'F', Wc, ncol, Wc, 1.0, Ut, W, Z + r0, ldz, 1.0, Z + r0, ldz, engine, &kr));
+          GEP_CHECK(dgemm(h, 'N', 'N', 'F', Wc, ncol, Wc, 1.0, Ut, WL, Z + r0, ldz, 1.0, Z + r0, ldz, engine,
+                          L ? nullptr : &kr));
         } else {  // Z(rows) += (U - I) copy(Z(rows))
-          GEP_CHECK(copy_matrix(h, Wc, ncol, Z + r0, ldz, Tmp, Wc));
-          GEP_CHECK(dgemm(h, 'N', 'N', 'F', Wc, ncol, Wc, 1.0, Ut, W, Tmp, Wc, 1.0, Z + r0, ldz, engine, &kr));
+          double* T = L ? ws + lv.need(L, chunk) : Tmp;
+          if (L && lv.need(L, chunk) + (size_t)Wc * ncol > ws_elems) return GEP_ERR_ALLOC;
+          GEP_CHECK(copy_matrix(h, Wc, ncol, Z + r0, ldz, T, Wc));
+          GEP_CHECK(dgemm(h, 'N', 'N', 'F', Wc, ncol, Wc, 1.0, Ut, WL, T, Wc, 1.0, Z + r0, ldz, engine, L ? nullptr : &kr));
         }
       }
     }

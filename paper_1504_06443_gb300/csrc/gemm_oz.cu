@@ -202,16 +202,16 @@ __global__ void __launch_bounds__(256) k_split_rows(int R, int K, int Kpad, cons
 // The same for few rows (fewer than can fill the GPU one warp per row): one CTA per row,
 // the exponent pass reduced over the CTA.
 // blockIdx.y: K panel of KP columns (the planes of all panels share rows of ldk elements; the panels'
-// exponents follow each other).
+// exponents follow each other).  Row r is row r mod zrows of operand r / zrows of a batch, xz apart.
 __global__ void __launch_bounds__(256) k_split_row_blk(int R, int Ktot, int ldk, int KP, const double* __restrict__ X,
-                                                       long long sr, int* __restrict__ e_out, int S, int xbit,
+                                                       long long sr, int zrows, long long xz, int* __restrict__ e_out, int S, int xbit,
                                                        unsigned short* __restrict__ out, const int* st) {
   __shared__ int red[8];
   if (status_bad(st)) return;
   const int r = blockIdx.x, kb = blockIdx.y * KP;
   if (r >= R) return;
   const int K = min(KP, Ktot - kb), Kpad = min(KP, ldk - kb);
-  const double* x = X + (size_t)r * sr + kb;
+  const double* x = X + (r / zrows) * xz + (r % zrows) * sr + kb;
   e_out += (size_t)blockIdx.y * R;
   out += kb;
   int m = 0;
@@ -236,16 +236,21 @@ __global__ void __launch_bounds__(256) k_split_row_blk(int R, int Ktot, int ldk,
 // The same for an operand whose K is strided (consecutive rows contiguous) and at most FUSE_K deep:
 // one CTA stages ROWS rows with their whole K panel in shared memory, so that the exponent pass,
 // its zeroing memset and the transposing split are one launch that reads the operand once
-// (2000 x 64 and 128 x 128: the three launches took about 20 us, this one 5 us).
+// (2000 x 64 and 128 x 128: the three launches took about 20 us, this one 5 us).  blockIdx.y: operand of a
+// batch, xz apart; their planes and exponents follow each other row by row.
 constexpr int FUSE_K = 512;
 template <int ROWS>
 __global__ void __launch_bounds__(256) k_split_cols(int R, int K, int Kpad, const double* __restrict__ X, long long sk,
-                                                    int* __restrict__ e_out, int S, int xbit,
+                                                    long long xz, int* __restrict__ e_out, int S, int xbit,
                                                     unsigned short* __restrict__ out, const int* st) {
   extern __shared__ double t[];  // [kk][ROWS + 1]
   __shared__ int mx[ROWS];
   if (status_bad(st)) return;
   const int r0 = blockIdx.x * ROWS, tx = threadIdx.x % ROWS, ty = threadIdx.x / ROWS;
+  const size_t plane = (size_t)R * gridDim.y * Kpad;
+  X += blockIdx.y * xz;
+  e_out += (size_t)blockIdx.y * R;
+  out += (size_t)blockIdx.y * R * Kpad;
   constexpr int TY = 256 / ROWS, LD = ROWS + 1;
   if (threadIdx.x < ROWS) mx[threadIdx.x] = 0;
   const int r = min(r0 + tx, R - 1);
@@ -265,7 +270,7 @@ __global__ void __launch_bounds__(256) k_split_cols(int R, int K, int Kpad, cons
     const int q = idx / q4, c4 = (idx - q * q4) * 4;
     if (r0 + q >= R) break;
     double x[4] = {t[c4 * LD + q], t[(c4 + 1) * LD + q], t[(c4 + 2) * LD + q], t[(c4 + 3) * LD + q]};
-    split4_store(x, c4, K, scale_exp(mx[q], xbit), S, (size_t)(r0 + q) * Kpad + c4, (size_t)R * Kpad, out);
+    split4_store(x, c4, K, scale_exp(mx[q], xbit), S, (size_t)(r0 + q) * Kpad + c4, plane, out);
   }
 }
 
@@ -342,6 +347,7 @@ struct OzArgs {
   int spp;
   long long zstride;
   int eastr, ebstr;
+  int zper;  // > 0: a batch, zper tiles a product; operand rows and exponents follow each other, C zstride apart
   const int* ea;
   const int* eb;
   double alpha, beta;
@@ -376,6 +382,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
   const int per_z = p.gx * p.gy;
   auto tile_rc = [&](int t, int& tm, int& tn) {
     if constexpr (SKINNY) t %= per_z;
+    else if (p.zper) t %= p.zper;
     const int per_group = GROUP_M * p.gy;
     const int first = (t / per_group) * GROUP_M;
     const int gm = min(p.gx - first, GROUP_M);
@@ -456,6 +463,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
         int tm, tn, s0, s1;
         if (!tile_rc(t, tm, tn)) continue;
         tile_steps(t, tm, s0, s1);
+        const int zb = !SKINNY && p.zper ? t / p.zper : 0;
         for (int step = s0; step < s1 && ok; ++step, ++g) {
           int sidx = g % STAGES;
           uint32_t ph = (uint32_t)(g / STAGES) & 1u;
@@ -463,8 +471,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
           if (!ok) break;
           uint32_t dst = smem_u32(smem + (size_t)sidx * stage_bytes);
           mbar_expect_tx(bar_full + 8 * sidx, stage_bytes);
-          tma_load_3d(dst, &tmA, step * TK, tm, 0, bar_full + 8 * sidx);
-          tma_load_3d(dst + a_bytes, &tmB, step * TK, tn, 0, bar_full + 8 * sidx);
+          tma_load_3d(dst, &tmA, step * TK, zb * p.m + tm, 0, bar_full + 8 * sidx);
+          tma_load_3d(dst + a_bytes, &tmB, step * TK, zb * p.n + tn, 0, bar_full + 8 * sidx);
         }
       }
       // make sure every copy this thread started has landed before the CTA retires
@@ -561,14 +569,15 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
     }
     if (ok && row < p.m) {
       const int zi = SKINNY ? t / per_z : 0, pz = SKINNY ? zi / p.spp : 0;
-      const int* ebp = p.eb + (size_t)pz * p.ebstr;
-      const int ea = scale_exp(p.ea[(size_t)pz * p.eastr + row], p.xbit);
+      const int zb = !SKINNY && p.zper ? t / p.zper : 0;
+      const int* ebp = p.eb + (size_t)pz * p.ebstr + (size_t)zb * p.n;
+      const int ea = scale_exp(p.ea[(size_t)pz * p.eastr + (size_t)zb * p.m + row], p.xbit);
       const bool two = LMAX >= 5;  // a second (low) accumulator is in use
       const int D = two ? 7 * LMAX - 28 : 0;
       const int base_adj = ea - (two ? 7 * LMAX : 28);
       const int amode = p.amode, bmode = p.bmode;
       const long long flip = amode < 0 ? 1ll << 63 : 0ll;
-      double* cp = p.C + (SKINNY ? (size_t)zi * p.zstride : 0) + (size_t)row + (size_t)(tn + cg * CPW) * p.ldc;
+      double* cp = p.C + (SKINNY ? (size_t)zi : (size_t)zb) * p.zstride + (size_t)row + (size_t)(tn + cg * CPW) * p.ldc;
       constexpr int CG = 4;  // columns whose loads of C are in flight together, one group ahead
       double cv[CG], cn[CG];
       auto fetch = [&](int g) {
@@ -642,7 +651,7 @@ namespace {
 int split_rows(gep_handle_t h, int R, int K, int Kpad, const double* X, long long sr, int* e, int S, int xbit,
                unsigned short* out) {
   if (R < 16 * h->sm_count)
-    k_split_row_blk<<<R, 256, 0, h->stream>>>(R, K, Kpad, Kpad, X, sr, e, S, xbit, out, h->d_status);
+    k_split_row_blk<<<R, 256, 0, h->stream>>>(R, K, Kpad, Kpad, X, sr, R, 0, e, S, xbit, out, h->d_status);
   else
     k_split_rows<<<(R * 32 + 255) / 256, 256, 0, h->stream>>>(R, K, Kpad, X, sr, e, S, xbit, out, h->d_status);
   return check_launch(h);
@@ -660,9 +669,9 @@ int split_cols(gep_handle_t h, int R, int K, int Kpad, const double* X, long lon
     // 8 rows a CTA while that fills the GPU at most a few times over (a row segment is 64 bytes),
     // else 32
     if (R <= 32 * h->sm_count)
-      k_split_cols<8><<<(R + 7) / 8, 256, (size_t)Kpad * 9 * 8, h->stream>>>(R, K, Kpad, X, sk, e, S, xbit, out, h->d_status);
+      k_split_cols<8><<<(R + 7) / 8, 256, (size_t)Kpad * 9 * 8, h->stream>>>(R, K, Kpad, X, sk, 0, e, S, xbit, out, h->d_status);
     else
-      k_split_cols<32><<<(R + 31) / 32, 256, (size_t)Kpad * 33 * 8, h->stream>>>(R, K, Kpad, X, sk, e, S, xbit, out, h->d_status);
+      k_split_cols<32><<<(R + 31) / 32, 256, (size_t)Kpad * 33 * 8, h->stream>>>(R, K, Kpad, X, sk, 0, e, S, xbit, out, h->d_status);
     return check_launch(h);
   }
   GEP_CUDA(cudaMemsetAsync(e, 0, sizeof(int) * (size_t)R, h->stream));
@@ -723,6 +732,7 @@ void oz_args_init(OzArgs& a, int m, int n, int kpad, int S, int levels, int lowe
   a.ntiles = a.gx * a.gy;
   a.kr_n = 0;
   a.spp = 0;
+  a.zper = 0;
   a.zstride = 0;
   a.eastr = a.ebstr = 0;
   for (int r = 0; r < OZ_KR_MAX; ++r) a.kr_lo[r] = a.kr_hi[r] = 0;
@@ -821,7 +831,7 @@ int dgemm_oz_sym_planes(gep_handle_t h, const OzSymPlanes& P, int row0, int n, d
   unsigned short* Bs = (unsigned short*)h->eng_ws;
   int* eb = (int*)(h->eng_ws + align256((size_t)2 * S * n * ldk));
   const int xbit = P.levels >= 8 ? 1 : 0;
-  k_split_row_blk<<<dim3(n, np), 256, 0, h->stream>>>(n, K, ldk, OZ_SYM_KP, B, ldb, eb, S, xbit, Bs, h->d_status);
+  k_split_row_blk<<<dim3(n, np), 256, 0, h->stream>>>(n, K, ldk, OZ_SYM_KP, B, ldb, n, 0, eb, S, xbit, Bs, h->d_status);
   GEP_CHECK(check_launch(h));
   CUtensorMap mA, mB;
   GEP_CHECK(encode_map(&mA, P.planes + (size_t)row0 * ldk, ldk, m, S, TM, P.m));  // rows row0.. of each plane
@@ -846,6 +856,46 @@ int dgemm_oz_sym_planes(gep_handle_t h, const OzSymPlanes& P, int row0, int n, d
   k_sum_parts<<<dim3((m + 255) / 256, n), 256, 0, h->stream>>>(m, n, nz, parts, (long long)mn, alpha, beta, C, ldc,
                                                               h->d_status);
   return check_launch(h);
+}
+
+// C_z += A_z B_z for z < count, operands sa, sb, sc apart: one split of each side and one product launch for
+// all of them.  m a multiple of 128, n of 64 and k of 32, so that no tile or step meets two products.
+int dgemm_oz_batched(gep_handle_t h, int m, int n, int k, const double* A, int lda, long long sa, const double* B,
+                     int ldb, long long sb, double* C, int ldc, long long sc, int count) {
+  if (m % TM || n % TN || k % TK) return GEP_ERR_UNSUPPORTED;
+  constexpr int S = 8;
+  for (int kb = 0; kb < k; kb += FUSE_K) {
+    const int kc = min(FUSE_K, k - kb);
+    const size_t per = align256((size_t)2 * S * (m + n) * kc) + align256((size_t)4 * (m + n));
+    const int fit = h->eng_ws ? (int)std::min<size_t>(h->eng_bytes / (per + 1024), 1 << 12) : 0;
+    if (fit < 1) return GEP_ERR_ALLOC;
+    for (int z0 = 0; z0 < count; z0 += fit) {
+      const int nz = min(fit, count - z0);
+      unsigned short* As = (unsigned short*)h->eng_ws;
+      unsigned short* Bs = As + align256((size_t)2 * S * m * nz * kc) / 2;
+      int* ea = (int*)(Bs + align256((size_t)2 * S * n * nz * kc) / 2);
+      int* eb = ea + (size_t)m * nz;
+      static unsigned long long devices = 0;
+      if (first_use_on_device(devices))
+        GEP_CUDA(cudaFuncSetAttribute(k_split_cols<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 33 * 8));
+      k_split_cols<32><<<dim3((m + 31) / 32, nz), 256, (size_t)kc * 33 * 8, h->stream>>>(
+          m, kc, kc, A + z0 * sa + (size_t)kb * lda, lda, sa, ea, S, 1, As, h->d_status);
+      GEP_CHECK(check_launch(h));
+      k_split_row_blk<<<n * nz, 256, 0, h->stream>>>(n * nz, kc, kc, kc, B + z0 * sb + kb, ldb, n, sb, eb, S, 1, Bs,
+                                                     h->d_status);
+      GEP_CHECK(check_launch(h));
+      CUtensorMap mA, mB;
+      GEP_CHECK(encode_map(&mA, As, kc, m * nz, S, TM));
+      GEP_CHECK(encode_map(&mB, Bs, kc, n * nz, S, TN));
+      OzArgs a;
+      oz_args_init(a, m, n, kc, S, 9, 0, 1, ea, eb, 1.0, 1.0, C + z0 * sc, ldc, h->d_status);
+      a.zper = a.gx * a.gy;
+      a.ntiles = a.zper * nz;
+      a.zstride = sc;
+      GEP_CHECK(oz_launch(h, mA, mB, a, kc));
+    }
+  }
+  return GEP_OK;
 }
 
 size_t oz_workspace_bytes(int m, int n, int k) {

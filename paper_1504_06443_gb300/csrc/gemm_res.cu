@@ -644,7 +644,10 @@ int dgemm_res(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, 
   const long long sra = TA ? lda : 1, ska = TA ? 1 : lda, srb = TB ? 1 : ldb, skb = TB ? ldb : 1;
   const ResPlan pl = res_plan(m, n, k, h->eng_ws ? h->eng_bytes : 0);
   if (pl.kp == 0) return GEP_ERR_ALLOC;
-  if (overlap(A, lda, TA ? k : m, TA ? m : k, C, ldc, m, n) || overlap(B, ldb, TB ? n : k, TB ? k : n, C, ldc, m, n))
+  // C <- C + A C: in one K panel, a column block of B is split before its block of C is written
+  const bool in_place = B == C && ldb == ldc && !TB && m == k && pl.kp >= k;
+  if (overlap(A, lda, TA ? k : m, TA ? m : k, C, ldc, m, n) ||
+      (!in_place && overlap(B, ldb, TB ? n : k, TB ? k : n, C, ldc, m, n)))
     return GEP_ERR_UNSUPPORTED;
   static unsigned long long attr_devices = 0;
   if (first_use_on_device(attr_devices))

@@ -135,6 +135,9 @@ int dgemm(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, doub
 bool product_on_tensor_cores(gep_handle_t h, char uplo, int m, int n, int k, int engine);
 int dgemm_f64(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, double alpha,
               const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc);
+// C_z += A_z B_z for a batch of equal products (split-BF16, FP64 setting).
+int dgemm_oz_batched(gep_handle_t h, int m, int n, int k, const double* A, int lda, long long sa, const double* B,
+                     int ldb, long long sb, double* C, int ldc, long long sc, int count);
 // The same product through residues (gemm_res.cu): where it is the faster form, and the product itself
 // (GEP_ERR_ALLOC / GEP_ERR_UNSUPPORTED before any work if the scratch is too small or C overlaps an operand).
 bool res_product_wins(gep_handle_t h, char uplo, int m, int n, int k);
