@@ -44,7 +44,7 @@ def parse():
                    help="SEP solver: 1-stage tridiagonalisation, full->band->tridiagonal, or block Jacobi")
     p.add_argument("--n-want", type=int, default=0,
                    help="only the lowest n eigenpairs (0: all; the occupied states are n = M/2)")
-    p.add_argument("--bandwidth", type=int, default=0, help="band width of --sep 2stage (0: library default, 32 up to order 12288 and 64 beyond)")
+    p.add_argument("--bandwidth", type=int, default=0, help="band width of --sep 2stage (0: library default, 32 up to order 20480 and 64 beyond)")
     p.add_argument("--values-only", action="store_true", help="eigenvalues only (T_evo of the paper's benchmark)")
     p.add_argument("--cpu-sample-M", type=int, nargs="+", default=[1024, 2048, 3072],
                    help="orders of the oracle solves the c M^3 fit of the CPU baseline is taken over")
@@ -794,7 +794,7 @@ def main():
     t_kernel_ms = prof["ms"] / covered_steps if covered_steps else None
     achieved = (prof["tensor_flops"] / (prof["ms"] * 1e-3) / 1e12) if prof["ms"] > 0 else None
     peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops"))
-    roof = {"bound": "tensor", "kernel": "k_oz_gemm (split-BF16 tcgen05 product)",
+    roof = {"bound": "tensor", "kernel": "k_oz_gemm and k_res_gemm (BF16 tcgen05 plane products)",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": (achieved / peak) if achieved else None,
             "traffic": product_traffic(prof),
@@ -805,7 +805,7 @@ def main():
             "launches_per_step": per_step_products, "steps_covered": covered_steps,
             "share_of_step": (t_kernel_ms / ms) if t_kernel_ms else None}
 
-    bw = (a.bandwidth or (32 if a.M <= 12288 else 64)) if a.sep == "2stage" else 0
+    bw = (a.bandwidth or (32 if a.M <= 20480 else 64)) if a.sep == "2stage" else 0
     stage_roof = stage_rooflines(M, stages, band_ms, vectors, a.sep, bw, peak, f64pk, reducer=a.reducer, n=n)
 
     # the CPU baseline is the oracle's full solve (all eigenpairs), the default workflow's work
@@ -827,7 +827,7 @@ def main():
                 "config": {"workload": f"tight-binding GEP M={M} ({M // 4} atoms x 4 sp orbitals), " + what,
                            "n_want": a.n_want,
                            "M": M, "seed": a.seed, "reducer": a.reducer, "sep": a.sep,
-                           "bandwidth": (a.bandwidth or (32 if a.M <= 12288 else 64)) if a.sep == "2stage" else None,
+                           "bandwidth": (a.bandwidth or (32 if a.M <= 20480 else 64)) if a.sep == "2stage" else None,
                            "precision": a.precision, "parallelism": "replicas" if world > 1 else "single",
                            "l2": (f"inputs larger than L2 ({8.0 * M * M / 1e9:.2f} GB per matrix, L2 129 MB)"
                                   if 8.0 * M * M > 129e6 else

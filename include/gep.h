@@ -74,7 +74,7 @@ typedef struct gep_handle_s* gep_handle_t;
 typedef struct gep_options {
   int reducer;      /* GEP_RED_*                                                  */
   int sep;          /* GEP_SEP_*                                                  */
-  int bandwidth;    /* band width b for GEP_SEP_2STAGE, 1..64 (0 = library default: 32 up to order 12288, 64 beyond) */
+  int bandwidth;    /* band width b for GEP_SEP_2STAGE, 1..64 (0 = library default: 32 up to order 20480, 64 beyond) */
   int precision;    /* GEP_PREC_*                                                 */
   int want_vectors; /* 1: eigenpairs (T_full); 0: eigenvalues only (T_evo)        */
   int overwrite;    /* 1: A and B may be destroyed by gep_solve (saves two copies) */
@@ -90,7 +90,8 @@ typedef struct gep_options {
   int batch_small;  /* gep_solve_batched only: pencils of order <= batch_small (at most 128) are
                        each solved whole by one CTA (Cholesky, C = L^-1 A L^-T, cyclic Jacobi,
                        Y = L^-T Q, all FP64), all of them in one persistent launch that takes
-                       them from a device work queue, largest order first; 0 = none. */
+                       them from a device work queue, largest order first, where that is
+                       the faster route (many pencils, or small ones); 0 = none. */
 } gep_options;
 
 /* Fills *o with the defaults: TWOSIDED, 1STAGE, b = 0, FP64, vectors, no overwrite, no timers.
@@ -218,8 +219,9 @@ int gep_adjoint(gep_handle_t h, int M, int n_occ, const double* w, const double*
 
 /* ---- batched solves (many independent pencils of uneven order) -------------------
  * Solves count pencils (A_i, B_i) of order M[i] with the workflow of gep_solve; host
- * arrays of device pointers.  Pencils of order <= o->batch_small go to one persistent
- * launch on the handle's stream (one CTA per pencil, see gep_options).  The others are
+ * arrays of device pointers.  Pencils of order <= o->batch_small may go to one persistent
+ * launch on the handle's stream (one CTA per pencil, see gep_options), where its time is
+ * below their share of the streams'.  The others are
  * spread over nstreams (1..64) concurrent child streams (largest M^3 first, each to the
  * least loaded stream), forked from and joined back into the handle's stream with events,
  * so the whole call can be captured into one CUDA graph (call it once outside capture

@@ -22,8 +22,8 @@ struct SolveLayout {
 // Bandwidth of the two-stage reduction when o->bandwidth = 0.  The narrow band
 // halves the bulge-chasing latency and the panel QR's FP64 work; the wide one halves the number of
 // panels, whose products and digit splits are what large matrices spend.  Measured, whole solve at
-// b = 64 / 32: order 516 21.5 / 18.0 ms, 2047 113 / 96 ms, 8192 709 / 688 ms.
-constexpr int kNarrowBandMax = 12288;
+// b = 64 / 32: order 8192 485 / 408 ms, 12288 1061 / 968 ms, 16384 1912 / 1845 ms, 32768 8.90 / 9.25 s.
+constexpr int kNarrowBandMax = 20480;
 int band_of(int M, const gep_options* o) { return o->bandwidth > 0 ? o->bandwidth : (M <= kNarrowBandMax ? 32 : 64); }
 bool two_stage(const gep_options* o) { return o->sep == GEP_SEP_2STAGE; }
 bool jacobi(const gep_options* o) { return o->sep == GEP_SEP_JACOBI; }
@@ -847,9 +847,9 @@ struct BatchPlan {
 
 int small_limit(const gep_options* o) { return o->batch_small < SMALL_MAX ? o->batch_small : SMALL_MAX; }
 
-// Time of one staged solve of order M on its stream, in ms (measured: order 64 2.1, 256 5.7, 516 12,
-// 1024 25, 2047 60): the balance of the streams.
-double staged_ms(int M) { return 1.0 + 0.02 * M + 3e-9 * (double)M * M * M; }
+// Time of one staged solve of order M on its stream, in ms (measured: order 64 0.8, 128 1.2, 256 2.1,
+// 516 6 to 8.5, 1024 17, 2047 43): the balance of the streams.
+double staged_ms(int M) { return 0.4 + 0.006 * M + 9e-6 * (double)M * M; }
 // Time of the one-CTA solver (cyclic Jacobi, about 12 M^3 FP64 operations on one SM): 53 ms at
 // order 128.  Up to two pencils an SM run at once.
 double one_cta_ms(int M) { return 53.0 / (128.0 * 128.0 * 128.0) * M * M * M; }
@@ -882,7 +882,7 @@ int make_plan(gep_handle_t h, int count, const int* M, const gep_options* o, con
   }
   // Of the pencils that may take the one-CTA solver, those keep it whose time there (all run at
   // once) is below what the small pencils together cost on the streams: a few pencils of order
-  // 128 (53 ms in one CTA, 3.2 ms staged) go to the streams, hundreds of them stay.
+  // 128 (53 ms in one CTA, 1.2 ms staged) go to the streams, many small ones stay.
   double on_streams = 0.0;
   int nsm = 0;
   for (int i = 0; i < count; ++i)
