@@ -1189,8 +1189,9 @@ __global__ void k_band_diag_fix(int M, const double* __restrict__ AB, int ldab, 
   const int i = blockIdx.x * blockDim.x + threadIdx.x, sh = band_shift(mx);
   if (i >= M) return;
   const ll* q = reinterpret_cast<const ll*>(AB);
-  d[i] = scale2((double)q[(size_t)i * ldab], -sh);
-  if (i + 1 < M) e[i] = scale2((double)q[1 + (size_t)i * ldab], -sh);
+  const bool finite = (*mx >> 52) < 0x7FF;  // an integer cannot carry a NaN or an infinity of the band
+  d[i] = finite ? scale2((double)q[(size_t)i * ldab], -sh) : NAN;
+  if (i + 1 < M) e[i] = finite ? scale2((double)q[1 + (size_t)i * ldab], -sh) : NAN;
 }
 
 __global__ void k_band_diag(int M, const double* __restrict__ AB, int ldab, double* __restrict__ d,
@@ -1492,7 +1493,10 @@ int panel_qr_launch(gep_handle_t h, const PanelArgs& a, long long part_elems) {
 
 int panel_qr(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, const BandWs& w, double* Va, double* Vb,
              int r0, int ldv) {
-  if (panel_qr_cluster_takes(n, b)) return panel_qr_cluster(h, n, b, P, ldp, tau, Va, Vb, r0, ldv, w.T);
+  if (panel_qr_cluster_takes(n, b)) {
+    const int rc = panel_qr_cluster(h, n, b, P, ldp, tau, Va, Vb, r0, ldv, w.T);
+    if (rc != GEP_ERR_UNSUPPORTED) return rc;
+  }
   PanelArgs a;
   a.n = n; a.nb = b; a.ldp = ldp; a.r0 = r0; a.ldv = ldv;
   a.P = P; a.tau = tau; a.part = w.part0; a.prow = w.prow0; a.Va = Va; a.Vb = Vb; a.T = w.T;

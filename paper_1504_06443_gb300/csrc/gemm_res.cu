@@ -616,7 +616,7 @@ bool overlap(const double* X, int ldx, int rx, int cx, const double* C, int ldc,
 // The faster of the two forms of a product on the tensor cores, by their measured costs (us):
 //   digit planes:  40 for launches and splits, 4 + 0.05 k per wave of 128 x 64 tiles, the operands' digits;
 //   residues:      60, 2 + 0.0053 k per wave of (256 x 256 tile, modulus) on the pairs of CTAs, 9 ps an
-//                  operand element (its 40 bytes) and 9 ps an output (16 bytes in, C, the CRT).
+//                  operand element (its 40 bytes) and 9 ps an output and K panel (16 bytes in, C, the CRT).
 // Digits / residues: 512^3 76 / 74, 1024 x 1024 x 512 77 / 97, 4096 x 256 x 1024 133 / 146,
 // 4096 x 4096 x 512 476 / 471, 1024^3 120 / 120, 8192 x 512 x 1024 322 / 260, 2048^3 510 / 328, 256 x 256 x 4096
 // 267 / 110, 4096^3 3130 / 1657, lower triangle 8192 x 8192 x 2048 3674 / 2026.
@@ -628,7 +628,8 @@ bool res_product_wins(gep_handle_t h, char uplo, int m, int n, int k) {
   double res_tiles = (double)((m + RM - 1) / RM) * ((n + RN - 1) / RN);
   if (lower) res_tiles = 0.5 * (res_tiles + (n + RN - 1) / RN);
   const double digits = 40.0 + ceil(digit_tiles / h->sm_count) * (4.0 + 0.05 * k) + 5e-6 * op;
-  const double residues = 60.0 + ceil(NMOD * res_tiles / (h->sm_count / 2)) * (2.0 + 0.0053 * k) + 9e-6 * (op + mn);
+  const double residues = 60.0 + ceil(NMOD * res_tiles / (h->sm_count / 2)) * (2.0 + 0.0053 * k) +
+                          9e-6 * (op + mn * ((k + RKP_MAX - 1) / RKP_MAX));
   return residues < 0.97 * digits;
 }
 

@@ -89,6 +89,35 @@ inline bool first_use_on_device(unsigned long long& mask) {
   return true;
 }
 
+// Whether a cluster of this size of the kernel can be resident at all (asked once per device: `known` and
+// `yes` are bit masks of devices, one pair per call site).
+inline bool cluster_fits(const void* kernel, int cluster, int threads, size_t smem, unsigned long long& known,
+                         unsigned long long& yes) {
+  int d = 0;
+  if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return false;
+  const unsigned long long bit = 1ull << d;
+  if (!(known & bit)) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    if (n > 0) yes |= bit;
+    known |= bit;
+  }
+  return (yes & bit) != 0;
+}
+
 inline int check_launch(gep_handle_t h) {
   h->launches++;
   cudaError_t e = cudaGetLastError();

@@ -312,6 +312,8 @@ int qr_launch(gep_handle_t h, const QrArgs& a) {
     GEP_CUDA(cudaFuncSetAttribute(k_panel_qr_cluster<RPW>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     GEP_CUDA(cudaFuncSetAttribute(k_panel_qr_cluster<RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   }
+  static unsigned long long known = 0, yes = 0;
+  if (!cluster_fits((const void*)k_panel_qr_cluster<RPW>, QC, QTHREADS, smem, known, yes)) return GEP_ERR_UNSUPPORTED;
   k_panel_qr_cluster<RPW><<<QC, QTHREADS, smem, h->stream>>>(a);
   return check_launch(h);
 }
@@ -322,7 +324,7 @@ int qr_launch(gep_handle_t h, const QrArgs& a) {
 bool panel_qr_cluster_takes(int n, int nb) { return nb <= QN && n <= QC * QW * 8; }
 
 // QR of the n x nb panel P (ld ldp): R and the reflectors in P, tau, V at full height (r0 zero rows first, ld
-// ldv) in Va and Vb, T (nb x nb).
+// ldv) in Va and Vb, T (nb x nb).  GEP_ERR_UNSUPPORTED before any work where the cluster cannot be resident.
 int panel_qr_cluster(gep_handle_t h, int n, int nb, double* P, int ldp, double* tau, double* Va, double* Vb, int r0,
                      int ldv, double* T) {
   if (!panel_qr_cluster_takes(n, nb)) return GEP_ERR_UNSUPPORTED;

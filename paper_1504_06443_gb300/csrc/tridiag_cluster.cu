@@ -290,6 +290,9 @@ int trc_launch(gep_handle_t h, const TrcArgs& a, int cl) {
   static unsigned long long devices = 0;
   if (first_use_on_device(devices))
     GEP_CUDA(cudaFuncSetAttribute((const void*)k_trd_cluster<RPW, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  static unsigned long long known = 0, yes = 0;  // (one cluster size per instance but the smallest)
+  if (!cluster_fits((const void*)k_trd_cluster<RPW, NT>, NT == 2 ? 4 : cl, TRC_THREADS, 0, known, yes))
+    return GEP_ERR_UNSUPPORTED;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cl);
   cfg.blockDim = dim3(TRC_THREADS);
@@ -310,7 +313,8 @@ int trc_launch(gep_handle_t h, const TrcArgs& a, int cl) {
 bool tridiag_cluster_takes(int n) { return n <= TRC_MAX; }
 
 // Reduces the n x n symmetric matrix in the lower triangle of C to tridiagonal form: d, e, tau and the
-// reflectors below the subdiagonal, as tridiag_1stage stores them.
+// reflectors below the subdiagonal, as tridiag_1stage stores them.  GEP_ERR_UNSUPPORTED before any work
+// where the cluster cannot be resident.
 int tridiag_cluster(gep_handle_t h, int n, double* C, int ldc, double* d, double* e, double* tau) {
   if (n <= 0) return GEP_OK;
   if (n > TRC_MAX) return GEP_ERR_UNSUPPORTED;

@@ -152,3 +152,19 @@ def test_nearly_tridiagonal(gep, b, eps):
     d, e, _, _, _ = gep.tridiag_2stage(dev(C), b=b)
     T = np.diag(d.cpu().numpy()) + np.diag(e.cpu().numpy(), 1) + np.diag(e.cpu().numpy(), -1)
     assert np.max(np.abs(np.linalg.eigvalsh(T) - w)) <= 200 * M * EPS * np.max(np.abs(w))
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("route", ["1stage", "1stage_large", "b32", "b64"])
+def test_nonfinite_shows_in_the_result(gep, route, bad):
+    """The stage entry points take any matrix: a NaN or an infinity comes out as NaN, not as numbers."""
+    M = 700 if route == "1stage_large" else 150
+    rng = np.random.default_rng(1)
+    C = rng.standard_normal((M, M))
+    C = C + C.T
+    C[M - 20, M - 30] = C[M - 30, M - 20] = bad
+    if route.startswith("1stage"):
+        d, e = gep.tridiag_1stage(dev(C))[:2]
+    else:
+        d, e = gep.tridiag_2stage(dev(C), b=int(route[1:]))[:2]
+    assert np.isnan(d.cpu().numpy()).any()
