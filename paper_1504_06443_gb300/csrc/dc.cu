@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(32) k_leaf(int M, const double* __restrict__ d
 #pragma unroll
   for (int c = 0; c < LEAF; ++c) Zs[c][lane] = (lane == c) ? 1.0 : 0.0;
   __syncwarp();
-  int bad = 0;
+  int bad = mx == 0x7FF;  // a NaN or an infinity: the merges order finite numbers only
   for (int l = 0; l < n && !bad; ++l) {
     for (int iter = 0;; ++iter) {
       bool small = true;

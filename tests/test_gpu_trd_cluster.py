@@ -84,3 +84,16 @@ def test_many_at_once(gep):
             assert all(torch.equal(w[4 * q], w[4 * q + u]) for u in range(1, 4))
         ref = ref or w
         assert all(torch.equal(a, b) for a, b in zip(ref, w))
+
+
+@pytest.mark.parametrize("M", [9, 17, 40])
+def test_nonfinite_tridiagonal_is_a_failure(gep, M):
+    """A NaN or an infinity in the last entry, alone in its leaf for M = 9 and 17: reported, not ordered."""
+    import torch
+    h = gep.Handle()  # (the status stays with the handle until its next reset)
+    for bad in (float("nan"), float("inf")):
+        d = torch.linspace(0, 1, M, dtype=torch.float64, device="cuda")
+        e = torch.full((M - 1,), 0.25, dtype=torch.float64, device="cuda")
+        d[M - 1] = bad
+        assert gep.tridiag_eig(d, e, handle=h)[2] != 0
+    h.close()
