@@ -124,7 +124,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
     const int r = idx % ROWS, j = idx / ROWS;
     tile[j * (ROWS + 1) + r] = rb + r < n && j < nb ? p.P[rb + r + (size_t)j * p.ldp] : 0.0;
   }
-  __syncthreads();
+  cl.sync();  // every CTA of the cluster runs, its barriers are initialised: its shared memory may be reached
   ll a[RPW];
   int em = 0;
 #pragma unroll

@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
       em = max(em, (int)((a[u][t] >> 52) & 0x7FF));
     }
   }
+  cl.sync();  // every CTA of the cluster runs, its barriers are initialised: its shared memory may be reached
   const int emax = (int)trc_cluster_max(cl, sh, em);
   const bool finite = emax < 0x7FF;
   // row sums with every element below 2^53, then the shift that puts the largest into (2^60, 2^61]

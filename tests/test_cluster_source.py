@@ -1,0 +1,63 @@
+"""Rules of thread-block clusters, checked in the text of the kernels (no GPU).
+
+Shared memory of another CTA of a cluster may be accessed only once that CTA is known to run, which a
+cluster barrier gives and co-scheduling alone does not.
+"""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1504_06443_gb300", "csrc")
+REMOTE = re.compile(r"map_shared_rank|\bmapa\.")
+BARRIER = re.compile(r"\bcl\.sync\(\)|barrier\.cluster\.wait")
+
+
+def functions(text):
+    """[(name, body, is_kernel)] of the device functions and kernels of a source, comments taken out."""
+    text = re.sub(r"//[^\n]*", "", text)
+    text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
+    out = []
+    for m in re.finditer(r"__(global|device)__[^;{]*?(\w+)\s*\([^{;]*\)\s*\{", text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[i], 0)
+            i += 1
+        name = m.group(2)
+        if m.group(1) == "global":  # the name before the parameter list (attributes come before it)
+            name = re.findall(r"(\w+)\s*\(", m.group(0))[-1]
+        out.append((name, text[m.end():i], m.group(1) == "global"))
+    return out
+
+
+def first_events(body, helpers, depth=0):
+    """The remote accesses and cluster barriers of a body in program order, helpers expanded in place."""
+    pats = [REMOTE.pattern, BARRIER.pattern] + ([r"\b(?:%s)\s*\(" % "|".join(helpers)] if helpers else [])
+    for m in re.finditer("|".join(pats), body):
+        if REMOTE.fullmatch(m.group(0)):
+            yield "remote"
+        elif BARRIER.fullmatch(m.group(0)):
+            yield "barrier"
+        elif depth < 4:
+            yield from first_events(helpers[m.group(0).rstrip("( \t")], helpers, depth + 1)
+
+
+def cluster_kernels():
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu"))):
+        fns = functions(open(path).read())
+        helpers = {n: b for n, b, k in fns if not k}
+        for name, body, kernel in fns:
+            if kernel and "remote" in list(first_events(body, helpers)):
+                yield pytest.param(body, helpers, id=f"{os.path.basename(path)}:{name}")
+
+
+def test_cluster_kernels_are_found():
+    assert {p.id for p in cluster_kernels()} >= {"tri.cu:k_potrf_diag", "gemm_res.cu:k_res_gemm",
+                                                 "tridiag_cluster.cu:k_trd_cluster",
+                                                 "panel_cluster.cu:k_panel_qr_cluster"}
+
+
+@pytest.mark.parametrize("body,helpers", list(cluster_kernels()))
+def test_no_remote_access_before_a_cluster_barrier(body, helpers):
+    assert next(first_events(body, helpers)) == "barrier"
