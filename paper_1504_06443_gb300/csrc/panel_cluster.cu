@@ -70,7 +70,7 @@ struct QrShared {
   ll beta;
   double T[QN][QN + 1];
   ll g[2][QN], tq[2];        // Gram entries of the column (Q60), tau (Q61)
-  int up, fail;
+  int up, fail;              // fail: column + 1 whose wait gave up, 0 for none
 };
 
 __device__ bool qr_wait(uint32_t bar, uint32_t parity, int* st) {
@@ -207,11 +207,11 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
           sh.up = o.up;
           sh.beta = o.beta;
           sh.tq[c & 1] = o.tq;
-          if (!ok) sh.fail = 1;
+          if (!ok) sh.fail = c + 1;
         }
       }
       all_sync();
-      if (sh.fail) break;
+      if (sh.fail == c + 1) break;  // (a warp still here may already see the next column's)
       if (worker) {
         const int2 tw = sh.tw[lane];
         const ll be = sh.beta;

@@ -61,3 +61,15 @@ def test_cluster_kernels_are_found():
 @pytest.mark.parametrize("body,helpers", list(cluster_kernels()))
 def test_no_remote_access_before_a_cluster_barrier(body, helpers):
     assert next(first_events(body, helpers)) == "barrier"
+
+
+def test_a_failed_wait_ends_the_panel_at_one_column():
+    """The warp that accumulates T meets the row warps at one barrier a column only, so it may read the flag of a
+    failed wait when warp 0 already stores the next column's.  The flag therefore names its column: were it a
+    mere truth value, the warps would leave at different columns and wait at different barriers for good."""
+    text = open(os.path.join(CSRC, "panel_cluster.cu")).read()
+    body = {n: b for n, b, _ in functions(text)}["k_panel_qr_cluster"]
+    stores = re.findall(r"sh\.fail\s*=(?!=)\s*([^;]+);", body)
+    tests = re.findall(r"if\s*\(([^()]*sh\.fail[^()]*)\)", body)
+    assert stores and tests
+    assert set(stores) == {"0", "c + 1"} and set(tests) == {"sh.fail == c + 1"}
