@@ -181,12 +181,13 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   return r;
 }
 
-// Address of the same shared variable in the pair's first CTA.
-__device__ __forceinline__ uint32_t leader_addr(uint32_t addr) {
+// Address of the same shared variable in the pair's CTA of this rank.
+__device__ __forceinline__ uint32_t pair_addr(uint32_t addr, int rank) {
   uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(addr));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
+__device__ __forceinline__ uint32_t leader_addr(uint32_t addr) { return pair_addr(addr, 0); }
 
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
@@ -221,7 +222,7 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
       : "memory");
 }
 
-// A wait for this CTA's own work in flight: a bad status does not cut it short, its limit does.
+// A wait for work in flight: a bad status does not cut it short, its limit does.
 __device__ __forceinline__ void mbar_wait_bounded(uint32_t bar, uint32_t parity, int* st) {
   unsigned long long t0 = gtimer();
   while (!mbar_try(bar, parity))
@@ -265,13 +266,14 @@ __device__ __forceinline__ void res_tile(const ResArgs& p, int t, int& tm, int& 
 // buffers, a chunk of 1024 each, and 16 warps of each CTA reduce the other buffer modulo m_i meanwhile
 // (four instructions an element and chunk; reduced fully and packed after every chunk they slowed the
 // MMAs: 16 x 4096 x 2048 x 2048 380 us, now 307).  The pair halves the shared-memory traffic of B, which bounds one
-// CTA with 128 x 256 tiles.  Waits are bounded as in k_oz_gemm.
+// CTA with 128 x 256 tiles.  Waits are bounded as in k_oz_gemm; the CTAs of a pair may give up at different
+// steps, so before they retire each learns how many steps the other has loaded and both are brought level.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(RTHREADS, 1)
     k_res_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, ResArgs p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ __align__(8) unsigned long long bars[2 * RSTAGES + 5];
   __shared__ uint32_t tmem_slot;
-  __shared__ int skip;
+  __shared__ int skip, issued;  // issued: steps whose copies this CTA has started
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_rank(), pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -283,6 +285,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(RTHREADS, 1)
 
   if (threadIdx.x == 0) {
     skip = status_bad(p.st) ? 1 : 0;
+    issued = 0;
     for (int s = 0; s < RSTAGES; ++s) {
       mbar_init(bar_full + 8 * s, 1);
       mbar_init(bar_empty + 8 * s, 1);
@@ -331,11 +334,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(RTHREADS, 1)
           tma_load_3d_pair(dst + RA_BYTES, &tmB, step * RK, tn + rank * (RN / 2), md, full);
         }
       }
-      // every copy has landed before the CTAs retire: the first CTA sees both CTAs' copies, the second
-      // waits for it at the closing barrier
-      if (rank == 0)
-        for (int s2 = (g > RSTAGES ? g - RSTAGES : 0); s2 < g; ++s2)
-          mbar_wait_bounded(bar_full + 8 * (s2 % RSTAGES), (uint32_t)(s2 / RSTAGES) & 1u, p.st);
+      issued = g;
     }
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
@@ -425,6 +424,29 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(RTHREADS, 1)
     }
   }
   tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // both counts stand, and no MMA reads the stages any more
+  // Every copy lands before the CTAs retire.  A step's barrier (the first CTA's) completes with the copies
+  // of both: where one CTA gave up earlier, the second loads what it is behind (its stages are free), the
+  // first expects what the second is ahead.
+  if (threadIdx.x == 0) {
+    const int mine = issued;
+    int other;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(other) : "r"(pair_addr(smem_u32(&issued), rank ^ 1)) : "memory");
+    if (rank == 1) {
+      for (int s = mine; s < other; ++s) {
+        const uint32_t dst = smem_u32(smem + (size_t)(s % RSTAGES) * RSTAGE_BYTES);
+        const uint32_t full = leader_addr(bar_full + 8 * (s % RSTAGES));
+        tma_load_3d_pair(dst, &tmA, 0, 0, 0, full);
+        tma_load_3d_pair(dst + RA_BYTES, &tmB, 0, 0, 0, full);
+      }
+    } else {
+      for (int s = max(mine - RSTAGES, 0); s < max(mine, other); ++s) {
+        if (s >= mine) mbar_expect_tx(bar_full + 8 * (s % RSTAGES), RSTAGE_BYTES);
+        mbar_wait_bounded(bar_full + 8 * (s % RSTAGES), (uint32_t)(s / RSTAGES) & 1u, p.st);
+      }
+    }
+  }
   __syncthreads();
   cluster_sync_all();  // no copy, MMA or arrival of the pair is in flight any more
   if (warp == 1) {

@@ -73,3 +73,52 @@ def test_a_failed_wait_ends_the_panel_at_one_column():
     tests = re.findall(r"if\s*\(([^()]*sh\.fail[^()]*)\)", body)
     assert stores and tests
     assert set(stores) == {"0", "c + 1"} and set(tests) == {"sh.fail == c + 1"}
+
+
+def test_the_copies_of_a_pair_are_waited_for():
+    """The CTAs of a pair may give up at different steps.  Between the barrier after which both step counts
+    stand and the one after which the CTAs retire, the first CTA waits for the copies of both."""
+    text = open(os.path.join(CSRC, "gemm_res.cu")).read()
+    body = {n: b for n, b, _ in functions(text)}["k_res_gemm"]
+    tail = body[body.index("issued = g;"):]
+    order = ["cluster_sync_all()", "pair_addr(smem_u32(&issued), rank ^ 1)", "mbar_expect_tx(bar_full", "mbar_wait_bounded(bar_full",
+             "cluster_sync_all()", "tcgen05.dealloc"]
+    at = 0
+    for token in order:
+        at = tail.index(token, at) + 1
+
+
+@pytest.mark.parametrize("first,second", [(f, f + a) for f in (0, 1, 5, 6, 7, 12, 40) for a in range(-6, 7) if f + a >= 0])
+def test_model_of_the_pairs_last_copies(first, second):
+    """A model of those barriers (one arrival and an expected byte count a phase): with the first CTA at `first` steps and the
+    second up to a ring ahead or behind, the closing steps leave no copy unexpected and no wait unmet."""
+    R = 6
+    done = max(min(first, second), max(first, second) - R)  # steps consumed: every older phase is complete
+    phase, arrived, tx = [0] * R, [False] * R, [0] * R
+
+    def settle(s):
+        if arrived[s] and tx[s] == 0:
+            phase[s], arrived[s] = phase[s] + 1, False
+
+    def expect(s, n):
+        assert not arrived[s]
+        arrived[s], tx[s] = True, tx[s] + n
+        settle(s)
+
+    def land(s):
+        tx[s] -= 1
+        settle(s)
+
+    for s in range(done):
+        expect(s % R, 2), land(s % R), land(s % R)
+    for s in range(done, first):
+        expect(s % R, 2), land(s % R)
+    for s in range(done, second):
+        land(s % R)
+    for s in range(second, first):  # the second CTA's missing copies
+        land(s % R)
+    for s in range(max(first - R, 0), max(first, second)):
+        if s >= first:
+            expect(s % R, 1)
+        assert phase[s % R] % 2 != (s // R) % 2, "a wait that would not end"
+    assert tx == [0] * R and not any(arrived)
