@@ -20,6 +20,7 @@
 // 4000 38.6 -> 37.0.
 #include <cooperative_groups.h>
 
+#include "cluster.cuh"
 #include "fixed.cuh"
 #include "gep_internal.cuh"
 
@@ -57,8 +58,6 @@ struct Dot128 {
   }
 };
 
-__device__ __forceinline__ uint32_t qr_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
 struct QrShared {
   Sum128 part[QW][QN + 1];   // sums of the warps (read two columns of all warps at a time)
   Sum128 recv[2][QC][QN];    // sums of the CTAs
@@ -70,27 +69,8 @@ struct QrShared {
   ll beta;
   double T[QN][QN + 1];
   ll g[2][QN], tq[2];        // Gram entries of the column (Q60), tau (Q61)
-  int up, fail;              // fail: column + 1 whose wait gave up, 0 for none
+  int up, done, fail;        // fail: column + 1 whose wait gave up, 0 for none
 };
-
-__device__ bool qr_wait(uint32_t bar, uint32_t parity, int* st) {
-  unsigned long long t0 = 0, now;
-  for (int it = 0;; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-    if ((it & 15) != 15) continue;
-    if (*(volatile int*)(st + 1) != 0) return false;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    if (t0 == 0) t0 = now;
-    if (now - t0 > 2000000000ull) {
-      atomicExch(st + 1, GEP_ERR_TIMEOUT);
-      return false;
-    }
-  }
-}
 
 // Named barriers: 1 all warps, 2 the row warps.
 __device__ __forceinline__ void all_sync() { asm volatile("bar.sync 1, %0;" ::"n"(QTHREADS) : "memory"); }
@@ -108,7 +88,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
   const bool bad = status_bad(p.st), worker = warp < QW;
   if (tid == 0) {
     for (int b = 0; b < 2; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(qr_smem(&sh.bar[b])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cta_shared(&sh.bar[b])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     sh.fail = 0;
   }
@@ -169,13 +149,33 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
   for (int u = 0; u < RPW; ++u) a[u] = qfix(a[u], scale);
   cl.sync();  // recv is read everywhere before the first push
 
+  auto expect = [&](int c) {
+    if (tid == 0)
+      asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(cta_shared(&sh.bar[c & 1])),
+                   "r"(QC * QN * 16 + QN * 8) : "memory");
+  };
+  // warp w pushes the sums of columns 2 w and 2 w + 1, one CTA a lane pair, and the owner the pivot row
+  auto push = [&](int c, Sum128 s) {
+    const int col = 2 * warp + (lane & 1);
+    uint32_t rd, rb;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(cta_shared(&sh.recv[c & 1][k][col])), "r"(lane >> 1));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(cta_shared(&sh.bar[c & 1])), "r"(lane >> 1));
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(rd),
+                 "l"(s.lo), "l"(s.hi), "r"(rb) : "memory");
+    if (c / ROWS == k) {
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(cta_shared(&sh.rrow[c & 1][col])), "r"(lane >> 1));
+      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(rd),
+                   "l"(sh.prow[col]), "r"(rb) : "memory");
+    }
+  };
   bool run = !bad;
   ll xk = 0;  // lane u: the pivot column in the warp's row u
-  for (int c = -1; run && c < nref; ++c) {
+  int c = -1;
+  for (; run && c < nref; ++c) {
     const int nc = c + 1;
     if (c >= 0) {
       if (warp == 0) {
-        const bool ok = qr_wait(qr_smem(&sh.bar[c & 1]), (uint32_t)(c >> 1) & 1u, p.st);
+        const bool ok = cluster_wait<false>(cta_shared(&sh.bar[c & 1]), (uint32_t)(c >> 1) & 1u, p.st);
         const Sum128(*rv)[QN] = sh.recv[c & 1];
         Sum128 s = rv[0][lane];
 #pragma unroll
@@ -238,9 +238,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
     }
     if (nc >= nref) break;
     if (worker) {
-      if (tid == 0)
-        asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(qr_smem(&sh.bar[nc & 1])),
-                     "r"(QC * QN * 16 + QN * 8) : "memory");
+      expect(nc);
       Dot128 d;
       xk = 0;
 #pragma unroll
@@ -256,7 +254,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
       }
       sh.part[warp][lane] = d.get();
       row_sync();
-      // warp w adds columns 2 w and 2 w + 1 over the warps and pushes them, one CTA a lane pair
+      // warp w adds columns 2 w and 2 w + 1 over the warps
       Sum128 s = sh.part[lane >> 1][2 * warp + (lane & 1)];
 #pragma unroll
       for (int o = 2; o < 32; o <<= 1) {
@@ -265,17 +263,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
         t.hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
         s = add128(s, t);
       }
-      const int col = 2 * warp + (lane & 1);
-      uint32_t rd, rb;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(qr_smem(&sh.recv[nc & 1][k][col])), "r"(lane >> 1));
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(qr_smem(&sh.bar[nc & 1])), "r"(lane >> 1));
-      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(rd),
-                   "l"(s.lo), "l"(s.hi), "r"(rb) : "memory");
-      if (nc / ROWS == k) {
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(qr_smem(&sh.rrow[nc & 1][col])), "r"(lane >> 1));
-        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(rd),
-                     "l"(sh.prow[col]), "r"(rb) : "memory");
-      }
+      push(nc, s);
     }
   }
   __syncthreads();
@@ -301,7 +289,22 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
     if (k == 0)
       for (int idx = tid; idx < nb * nb; idx += QTHREADS) p.T[idx] = sh.T[idx % nb][idx / nb];
   }
-  cl.sync();  // no CTA leaves while another may still push to it
+  // No CTA leaves before every push into its shared memory has landed.  After a timeout the CTAs may have
+  // left the loop a column apart: those behind push the columns they are behind, for their bytes.
+  const int done = c + 1;  // columns that this CTA has pushed
+  if (tid == 0) sh.done = done;
+  cl.sync();
+  const int last = __reduce_max_sync(0xffffffffu, lane < QC ? *cl.map_shared_rank(&sh.done, lane) : 0);
+  Sum128 none;
+  none.lo = none.hi = 0;
+  for (int q = max(done - 1, 0); q < last; ++q) {
+    if (q >= done && worker) {
+      expect(q);
+      push(q, none);
+    }
+    cluster_wait<true>(cta_shared(&sh.bar[q & 1]), (uint32_t)(q >> 1) & 1u, p.st);
+  }
+  cl.sync();
 }
 
 template <int RPW>

@@ -9,6 +9,7 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include "cluster.cuh"
 #include "gep_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -88,29 +89,8 @@ struct PotrfShared {
   double f[PW][NB];                // f_i of this CTA's rows
   double sq[NB], rs[NB];
   unsigned long long bar[NB];
+  unsigned pushed;                 // bit w: the row of warp w has been pushed
 };
-
-__device__ __forceinline__ uint32_t cta_shared(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// Bounded wait (two seconds) for a published row; on expiry records the timeout.
-__device__ __forceinline__ bool row_wait(uint32_t bar, int* st) {
-  unsigned long long t0 = 0, now;
-  for (int it = 0;; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok) : "r"(bar) : "memory");
-    if (ok) return true;
-    if ((it & 15) != 15) continue;
-    if (*(volatile int*)(st + 1) != 0) return false;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    if (t0 == 0) t0 = now;
-    if (now - t0 > 2000000000ull) {
-      atomicExch(st + 1, GEP_ERR_TIMEOUT);
-      return false;
-    }
-  }
-}
 
 __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_diag(int r, double* B, int ldb,
                                                                                    double* invD, int ldi, int kb,
@@ -129,6 +109,7 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_di
     asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(bar),
                  "r"(PROW * 8) : "memory");
   }
+  if (threadIdx.x == 0) sh.pushed = 0;
   double x[U];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
@@ -138,6 +119,7 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_di
   cl.sync();
   auto publish = [&](int j, double pivot) {
     const double ri = 1.0 / pivot;
+    if (lane == 0) atomicOr(&sh.pushed, 1u << w);
     const uint32_t dst = cta_shared(&sh.rows[j][lane * U]), sc = cta_shared(&sh.rows[j][NB]), bar = cta_shared(&sh.bar[j]);
 #pragma unroll
     for (int q = 0; q < PC; ++q) {
@@ -166,8 +148,8 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_di
       const int j = 32 * ju + jl;
       if (j >= last || fail) break;
       bool ok = true;
-      if (rank == (j + 1) % PC && i != j + 1) ok = row_wait(cta_shared(&sh.bar[j + 1]), st);
-      if (ok) ok = row_wait(cta_shared(&sh.bar[j]), st);
+      if (rank == (j + 1) % PC && i != j + 1) ok = cluster_wait<false>(cta_shared(&sh.bar[j + 1]), 0, st);
+      if (ok) ok = cluster_wait<false>(cta_shared(&sh.bar[j]), 0, st);
       if (!ok) { fail = -1; break; }
       const double ri = sh.rows[j][NB];  // a bad pivot is found at the end: the rows keep coming
       const double f = __shfl_sync(0xffffffffu, x[ju], jl) * ri;
@@ -184,7 +166,14 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_di
       }
     }
   }
-  cl.sync();  // every row that is to come has been pushed, and no CTA has left
+  cl.sync();  // every row that is to come has been pushed
+  // no CTA leaves before every push into its shared memory has landed (after a timeout some rows never come)
+  if (threadIdx.x < NB) {
+    const unsigned pushed = *cl.map_shared_rank(&sh.pushed, threadIdx.x % PC);
+    if (!(pushed >> (threadIdx.x / PC) & 1) || !cluster_wait<true>(cta_shared(&sh.bar[threadIdx.x]), 0, st))
+      sh.rows[threadIdx.x][NB + 1] = 0.0;  // not here: no pivot
+  }
+  cl.sync();
   if (bad) return;
   // the pivots; the first that is not positive is the leading minor reported
   __shared__ int first_bad;
@@ -193,8 +182,7 @@ __global__ void __cluster_dims__(PC, 1, 1) __launch_bounds__(32 * PW) k_potrf_di
   if (threadIdx.x < NB) {
     sh.rs[threadIdx.x] = sh.sq[threadIdx.x] = 1.0;
     if (threadIdx.x < r) {
-      // (also: no CTA leaves before every push into its shared memory has landed)
-      const double p = row_wait(cta_shared(&sh.bar[threadIdx.x]), st) ? sh.rows[threadIdx.x][NB + 1] : 0.0;
+      const double p = sh.rows[threadIdx.x][NB + 1];
       if (!(p > 0.0) || !isfinite(p)) {
         atomicMin(&first_bad, (int)threadIdx.x);
       } else {

@@ -22,6 +22,7 @@
 // 1501 6 -> 2.5.  Beyond 512 rows the registers of 16 SMs are full.
 #include <cooperative_groups.h>
 
+#include "cluster.cuh"
 #include "fixed.cuh"
 #include "gep_internal.cuh"
 
@@ -47,10 +48,8 @@ struct TrcShared {
   ll d[TRC_MAX], e[TRC_MAX], tau[TRC_MAX];  // results, turned into doubles at the end
   unsigned sq[TRC_WARPS][6];                // sums of squares in six parts
   int2 mq;
-  int up, zero;
+  int up, zero, done;
 };
-
-__device__ __forceinline__ uint32_t trc_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Largest value over the CTAs of the cluster (not below 0).
 __device__ ll trc_cluster_max(cg::cluster_group& cl, TrcShared& sh, ll v) {
@@ -73,26 +72,6 @@ __device__ ll trc_cluster_max(cg::cluster_group& cl, TrcShared& sh, ll v) {
   return m;
 }
 
-// Bounded wait (two seconds) for the pushes of a column.
-__device__ bool trc_wait(uint32_t bar, uint32_t parity, int* st) {
-  unsigned long long t0 = 0, now;
-  for (int it = 0;; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    if (ok) return true;
-    if ((it & 15) != 15) continue;
-    if (*(volatile int*)(st + 1) != 0) return false;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    if (t0 == 0) t0 = now;
-    if (now - t0 > 2000000000ull) {
-      atomicExch(st + 1, GEP_ERR_TIMEOUT);
-      return false;
-    }
-  }
-}
-
 // RPW rows a warp, NT slots of 32 columns: n <= 32 NT and n <= 16 RPW CL.
 template <int RPW, int NT>
 __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
@@ -103,7 +82,7 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
   const bool bad = status_bad(p.st);  // (every thread of the cluster passes through the same barriers)
   if (tid == 0)
     for (int b = 0; b < 2; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(trc_smem(&sh.bar[b])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cta_shared(&sh.bar[b])) : "memory");
   if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   for (int j = tid; j < TRC_MAX; j += TRC_THREADS) sh.v[0][j] = sh.v[1][j] = sh.w[j] = make_int2(0, 0);
 
@@ -149,20 +128,38 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
   // two words to the same place in CTA q, counted by its barrier
   auto push = [&](longlong2* slot, int buf, int q, ll y, ll el) {
     uint32_t rd, rb;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(trc_smem(slot)), "r"(q));
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(trc_smem(&sh.bar[buf])), "r"(q));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rd) : "r"(cta_shared(slot)), "r"(q));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(rb) : "r"(cta_shared(&sh.bar[buf])), "r"(q));
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(rd),
                  "l"(y), "l"(el), "r"(rb) : "memory");
   };
   const int cols = bad ? 0 : n;
-  for (int i = 0; i < cols; ++i) {
+  auto expect = [&](int i) {
+    if (tid == 0)
+      asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(cta_shared(&sh.bar[i & 1])),
+                   "r"(16 * max(n - 1 - i, CL)) : "memory");
+  };
+  // y and the next column's elements of this warp's rows to every CTA
+  auto push_rows = [&](int i, const ll (&y)[RPW], const ll (&el)[RPW]) {
+#pragma unroll
+    for (int u = 0; u < RPW; ++u) {
+      const int r = (warp + TRC_WARPS * u) * CL + k;
+      if (r > i && r < n && lane < CL) push(&sh.recv[i & 1][r], i & 1, lane, y[u], el[u]);
+    }
+    // A CTA whose rows are all done still reports every column: the others may be one column ahead of
+    // it, as the two buffers allow, and not more.
+    if (n - 1 - i < CL && warp == 0 && lane < CL) {
+      const int first = i + 1 + (k - (i + 1) % CL + CL) % CL;  // its next row
+      if (first >= n) push(&sh.ack[k], i & 1, lane, 0, 0);
+    }
+  };
+  int i = 0;
+  for (; i < cols; ++i) {
     const int buf = i & 1;
     const bool act = l > i && l < n;
     if (l == i) sh.d[i] = x;
     if (i == n - 1) break;
-    if (tid == 0)
-      asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(trc_smem(&sh.bar[buf])),
-                   "r"(16 * max(n - 1 - i, CL)) : "memory");
+    expect(i);
     // ---- norm of x(i + 2 ..): from the exact squares
     {
       const unsigned long long ax = act && l > i + 1 ? (unsigned long long)(x < 0 ? -x : x) : 0ull;
@@ -243,22 +240,10 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
         nx[u] = __shfl_sync(0xffffffffu, c1, (i + 1) & 31);
       }
     }
-#pragma unroll
-    for (int u = 0; u < RPW; ++u) {
-      const int r = (warp + TRC_WARPS * u) * CL + k;
-      if (r > i && r < n && lane < CL) {
-        push(&sh.recv[buf][r], buf, lane, yr[u], nx[u]);
-      }
-    }
-    // A CTA whose rows are all done still reports every column: the others may be one column ahead of
-    // it, as the two buffers allow, and not more.
-    if (n - 1 - i < CL && warp == 0 && lane < CL) {
-      const int first = i + 1 + (k - (i + 1) % CL + CL) % CL;  // its next row
-      if (first >= n) push(&sh.ack[k], buf, lane, 0, 0);
-    }
+    push_rows(i, yr, nx);
     if (act && l % CL == k)  // (while the others push)
       p.C[GEP_IX(l, i, p.ldc)] = !finite ? NAN : l == i + 1 ? scale2(qscaled(sh.e[i], 0), -scale) : qscaled(v, 62);
-    const bool ok = trc_wait(trc_smem(&sh.bar[buf]), (uint32_t)(i >> 1) & 1u, p.st);
+    const bool ok = cluster_wait<false>(cta_shared(&sh.bar[buf]), (uint32_t)(i >> 1) & 1u, p.st);
     // ---- w and column i + 1
     const ll y = act ? sh.recv[buf][l].x : 0, raw = act ? sh.recv[buf][l].y : 0;
     const ll pl = qmul<61>(qsplit(y), tq);
@@ -267,7 +252,10 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
       if (lane == 0) sh.zs[warp] = s;
     }
     const ll p1 = qmul<61>(qsplit(sh.recv[buf][i + 1].x), tq);
-    if (!__syncthreads_and(ok)) break;
+    if (!__syncthreads_and(ok)) {
+      ++i;
+      break;
+    }
     const ll dot = qwarp_sum(lane < TRC_WARPS ? sh.zs[lane] : 0);
     const int2 al = qsplit(qmul<62>(qsplit(dot), tq));
     const ll w = pl - qmul<62>(al, vl);
@@ -283,7 +271,21 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
       p.tau[l] = finite ? qscaled(sh.tau[l], 61) : NAN;
     }
   }
-  cl.sync();  // no CTA leaves while another may still push to it
+  // No CTA leaves before every push into its shared memory has landed.  After a timeout the CTAs may have
+  // left the loop a column apart: those behind push the columns they are behind, for their bytes.
+  const int done = i;  // columns that this CTA has pushed
+  if (tid == 0) sh.done = done;
+  cl.sync();
+  const int last = __reduce_max_sync(0xffffffffu, lane < CL ? *cl.map_shared_rank(&sh.done, lane) : 0);
+  const ll none[RPW] = {};
+  for (int c = max(done - 1, 0); c < last; ++c) {
+    if (c >= done) {
+      expect(c);
+      push_rows(c, none, none);
+    }
+    cluster_wait<true>(cta_shared(&sh.bar[c & 1]), (uint32_t)(c >> 1) & 1u, p.st);
+  }
+  cl.sync();
 }
 
 template <int RPW, int NT>

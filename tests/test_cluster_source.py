@@ -122,3 +122,18 @@ def test_model_of_the_pairs_last_copies(first, second):
             expect(s % R, 1)
         assert phase[s % R] % 2 != (s // R) % 2, "a wait that would not end"
     assert tx == [0] * R and not any(arrived)
+
+
+@pytest.mark.parametrize("source,kernel", [("tri.cu", "k_potrf_diag"), ("tridiag_cluster.cu", "k_trd_cluster"),
+                                           ("panel_cluster.cu", "k_panel_qr_cluster")])
+def test_pushes_have_landed_before_a_cta_leaves(source, kernel):
+    """A push (st.async) is complete only when the barrier it reports to says so.  Also after a timeout, when the main loop
+    was left early, the CTAs wait for the pushes under way between two cluster barriers, and return behind the second."""
+    text = open(os.path.join(CSRC, source)).read()
+    body = {n: b for n, b, _ in functions(text)}[kernel]
+    assert "st.async" in body
+    barriers = [m.start() for m in re.finditer(r"cl\.sync\(\)", body)]
+    drain = body.index("cluster_wait<true>")
+    assert barriers[-2] < drain < barriers[-1]
+    assert not re.search(r"\breturn\s*;", body[:barriers[-1]])
+    assert "DRAIN" in open(os.path.join(CSRC, "cluster.cuh")).read()
