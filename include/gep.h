@@ -328,7 +328,8 @@ const char* gep_status_string(int code);
  * C = alpha op(A) op(B) + beta C, op = 'N' or 'T'; transa 'S': A is symmetric (m x m,
  * k = m, transb 'N') and only its lower triangle is read.  uplo 'F' (full) or 'L' (only
  * entries i >= j of C are computed and written).  engine: GEP_PREC_FP64 (FP64 FMA)
- * or GEP_PREC_FP64_EMULATED (split-BF16 tensor cores, FP64-accurate). */
+ * or GEP_PREC_FP64_EMULATED (split-BF16 tensor cores, FP64-accurate).  On the tensor cores a row of
+ * op(A) or a column of op(B) that holds a NaN or an infinity makes its row or column of C NaN. */
 int gep_dgemm(gep_handle_t h, char transa, char transb, char uplo, int m, int n, int k, double alpha,
               const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
               int engine);

@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
       const int zi = SKINNY ? t / per_z : 0, pz = SKINNY ? zi / p.spp : 0;
       const int zb = !SKINNY && p.zper ? t / p.zper : 0;
       const int* ebp = p.eb + (size_t)pz * p.ebstr + (size_t)zb * p.n;
-      const int ea = scale_exp(p.ea[(size_t)pz * p.eastr + (size_t)zb * p.m + row], p.xbit);
+      const int ra = p.ea[(size_t)pz * p.eastr + (size_t)zb * p.m + row], ea = scale_exp(ra, p.xbit);
       const bool two = LMAX >= 5;  // a second (low) accumulator is in use
       const int D = two ? 7 * LMAX - 28 : 0;
       const int base_adj = ea - (two ? 7 * LMAX : 28);
@@ -597,8 +597,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_oz_gemm(const __grid_constant__
         for (int j = 0; j < CG; ++j) {
           const int col = tn + cg * CPW + g + j;
           if (col >= p.n || (p.lower && row < col)) continue;
-          const long long bits =
-              fixed_to_bits(hi[g + j], two ? lo[g + j] : 0ll, D, base_adj + scale_exp(ebp[col], p.xbit));
+          const int rb = ebp[col];
+          const long long bits = nonfinite(ra, rb) ? NAN_BITS : fixed_to_bits(hi[g + j], two ? lo[g + j] : 0ll, D,
+                                                                              base_adj + scale_exp(rb, p.xbit));
           double out = __longlong_as_double(bits ^ flip);
           if (amode == 0) out *= p.alpha;
           if (bmode == 1) out += cv[j];

@@ -523,7 +523,7 @@ __global__ void __launch_bounds__(256) k_res_crt(CrtArgs p) {
       t[2][g] = __byte_perm(c, d, 0x5410);
       t[3][g] = __byte_perm(c, d, 0x7632);
     }
-    const int ea = scale_exp(p.ea[row], 1) - 112 + 127;
+    const int ra = p.ea[row], ea = scale_exp(ra, 1) - 112 + 127;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const unsigned long long w0 = weight_word<0>(t[u]), w1 = weight_word<4>(t[u]) + (w0 >> 32),
@@ -534,9 +534,10 @@ __global__ void __launch_bounds__(256) k_res_crt(CrtArgs p) {
       constexpr float shift = (float)((double)(unsigned long long)(kBias >> 64) / (double)(unsigned long long)(kP >> 64));
       const int q = __float2int_rn(fmaf((float)(unsigned)(w3 >> 8), scale, -shift));
       const u128 X = sum - kBias - (u128)(unsigned)q * kP;  // modulo 2^128, signed
-      const int col = min(c0 + j4 + u, p.n - 1);
+      const int rb = p.eb[min(c0 + j4 + u, p.n - 1)];
       tile[j4 + u][i] = __longlong_as_double(
-          fixed128_to_bits((long long)(unsigned long long)(X >> 64), (unsigned long long)X, ea + scale_exp(p.eb[col], 1)));
+          nonfinite(ra, rb) ? NAN_BITS : fixed128_to_bits((long long)(unsigned long long)(X >> 64), (unsigned long long)X,
+                                                          ea + scale_exp(rb, 1)));
     }
   }
   __syncthreads();

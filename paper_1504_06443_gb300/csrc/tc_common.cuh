@@ -14,6 +14,11 @@ namespace {
 // Biased exponent field of |x| (0 for zero / subnormal).
 __device__ __forceinline__ int exp_field(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
 
+// A row of op(A) or a column of op(B) that holds a NaN or an infinity: integers cannot carry it, so the
+// epilogues store NaN wherever one of the two raw exponents of an output says so.
+__device__ __forceinline__ bool nonfinite(int raw_a, int raw_b) { return max(raw_a, raw_b) == 0x7FF; }
+constexpr long long NAN_BITS = 0x7FF8ll << 48;
+
 // Row scale exponent from the largest biased exponent m of the row: e with max |x| < 2^(e-1)
 // when xbit = 1 (for a normal x with biased exponent E, |x| < 2^(E-1022)), so that the
 // leading digit lies in [-64, 64] like the others; xbit = 0 (the FP32-grade setting, whose
