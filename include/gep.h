@@ -150,7 +150,9 @@ int gep_backtransform(gep_handle_t h, int M, int ncol, const double* B, int ldb,
  * sep_tridiag_1stage: Householder reduction C = Q T Q^T.  C (lower) is overwritten:
  *   its strictly-lower part below the subdiagonal holds the reflectors v_k (unit
  *   leading entry implied); d[M], e[M-1], tau[M-1] receive T and the reflector
- *   scalars (H_k = I - tau_k v_k v_k^T, Q = H_0 H_1 ... H_{M-2}).
+ *   scalars (H_k = I - tau_k v_k v_k^T, Q = H_0 H_1 ... H_{M-2}).  The last 512 columns are held
+ *   in 64-bit fixed point with one unit, about 2^-61 of the largest absolute row sum, where all
+ *   row sums lie within a factor of 16, and in FP64 otherwise.
  * sep_tridiag_eig: divide and conquer on (d, e).  w[M] receives the eigenvalues in
  *   ascending order; if want_vectors, Z (M x M) receives the orthonormal eigenvectors
  *   of T.  d and e are not modified.  want_vectors = 0 uses Sturm bisection.

@@ -16,6 +16,14 @@
 // result and an update rounds once (a rounding per product made the vectors of order 500 2.2 times as
 // far off as FP64 panels); squares and their sums are exact.
 //
+// One unit for the whole matrix is no coarser than FP64 only while its rows are of like size: a decoupled or
+// weakly coupled block far below the rest would lose its relative accuracy.  So where the row sums lie further
+// apart than 2^TRC_SPREAD (without the first column, which only enters the first reflector) the same columns
+// are taken in FP64, scaled by a power of two.  Order 500, two blocks: relative error of the small one's
+// eigenvalues 9.9e-15, 9.1e-15, 9.4e-15 at 1/4, 1/8, 1/10 of the other's scale in fixed point, 6.5e-15 to
+// 1.2e-14 below 1/16 in FP64; the FP64 columns take 0.46 / 0.86 / 1.8 / 5.4 ms at order 64 / 128 / 256 / 500,
+// the fixed-point ones 0.23 / 0.38 / 0.79 / 2.5 ms (whole calls).
+//
 // Bound: the chain of a column (two warp and CTA reductions, the scalars, the push: 2.2 us) and from
 // n = 260 on the integer products (7 us a column in all at n = 512).  S1 of the cooperative panels -> here:
 // order 64 0.62 -> 0.14 ms, 128 1.28 -> 0.29, 256 2.74 -> 0.67, 500 5.67 -> 2.4, the last 512 columns of
@@ -31,6 +39,7 @@ namespace cg = cooperative_groups;
 namespace gep {
 namespace {
 
+constexpr int TRC_SPREAD = 4;  // row sums further apart than 2^4: FP64
 constexpr int TRC_MAX = 512, TRC_WARPS = 16, TRC_THREADS = 32 * TRC_WARPS, TRC_CL = 16;
 
 struct TrcArgs {
@@ -44,87 +53,54 @@ struct TrcShared {
   longlong2 recv[2][TRC_MAX];  // y_l, element (l, i + 1)
   longlong2 ack[TRC_CL];
   unsigned long long bar[2];
-  ll xmax[TRC_CL], xa, tauq, zs[TRC_WARPS];
+  longlong2 mx[TRC_WARPS], xmax[TRC_CL];
+  ll xa, tauq, zs[TRC_WARPS];
   ll d[TRC_MAX], e[TRC_MAX], tau[TRC_MAX];  // results, turned into doubles at the end
   unsigned sq[TRC_WARPS][6];                // sums of squares in six parts
   int2 mq;
   int up, zero, done;
 };
 
-// Largest value over the CTAs of the cluster (not below 0).
-__device__ ll trc_cluster_max(cg::cluster_group& cl, TrcShared& sh, ll v) {
+// Largest values of two numbers over the CTAs of the cluster (not below 0).
+__device__ void trc_cluster_max(cg::cluster_group& cl, TrcShared& sh, ll& v0, ll& v1) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int o = 16; o; o >>= 1) {
-    const ll q = __shfl_xor_sync(0xffffffffu, v, o);
-    v = q > v ? q : v;
+    const ll q0 = __shfl_xor_sync(0xffffffffu, v0, o), q1 = __shfl_xor_sync(0xffffffffu, v1, o);
+    v0 = max(v0, q0);
+    v1 = max(v1, q1);
   }
-  if (lane == 0) sh.zs[warp] = v;
+  if (lane == 0) sh.mx[warp] = make_longlong2(v0, v1);
   __syncthreads();
   if (threadIdx.x < cl.num_blocks()) {
-    ll m = 0;
-    for (int q = 0; q < TRC_WARPS; ++q) m = sh.zs[q] > m ? sh.zs[q] : m;
+    longlong2 m = make_longlong2(0, 0);
+    for (int q = 0; q < TRC_WARPS; ++q) m = make_longlong2(max(m.x, sh.mx[q].x), max(m.y, sh.mx[q].y));
     cl.map_shared_rank(sh.xmax, threadIdx.x)[cl.block_rank()] = m;
   }
   cl.sync();
-  ll m = 0;
-  for (int q = 0; q < (int)cl.num_blocks(); ++q) m = sh.xmax[q] > m ? sh.xmax[q] : m;
+  v0 = v1 = 0;
+  for (int q = 0; q < (int)cl.num_blocks(); ++q) {
+    v0 = max(v0, sh.xmax[q].x);
+    v1 = max(v1, sh.xmax[q].y);
+  }
   cl.sync();
-  return m;
 }
 
-// RPW rows a warp, NT slots of 32 columns: n <= 32 NT and n <= 16 RPW CL.
-template <int RPW, int NT>
-__global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
-  __shared__ TrcShared sh;
-  cg::cluster_group cl = cg::this_cluster();
+// Entries of v and w are two limbs, or the words of a double.
+__device__ __forceinline__ double trc_dbl(int2 a) { return __hiloint2double(a.y, a.x); }
+__device__ __forceinline__ int2 trc_int2(double x) { return make_int2(__double2loint(x), __double2hiint(x)); }
+__device__ __forceinline__ double trc_dbl(ll a) { return __longlong_as_double(a); }
+__device__ __forceinline__ double trc_sum(double v) {
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The columns, in fixed point or in FP64; a, x: elements times 2^scale.
+template <bool F64, int RPW, int NT>
+__device__ __forceinline__ void trc_columns(const TrcArgs& p, TrcShared& sh, cg::cluster_group& cl, ll (&a)[RPW][NT], ll x,
+                                            int scale, bool finite, int cols) {
   const int CL = (int)cl.num_blocks(), k = (int)cl.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = p.n, l = tid;
-  const bool bad = status_bad(p.st);  // (every thread of the cluster passes through the same barriers)
-  if (tid == 0)
-    for (int b = 0; b < 2; ++b)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cta_shared(&sh.bar[b])) : "memory");
-  if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  for (int j = tid; j < TRC_MAX; j += TRC_THREADS) sh.v[0][j] = sh.v[1][j] = sh.w[j] = make_int2(0, 0);
-
-  // rows as bits of doubles; their largest exponent
-  ll a[RPW][NT];
-  int em = 0;
-#pragma unroll
-  for (int u = 0; u < RPW; ++u) {
-    const int r = (warp + TRC_WARPS * u) * CL + k;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const int j = 32 * t + lane;
-      a[u][t] = r < n && j < n ? __double_as_longlong(p.C[GEP_IX(r > j ? r : j, r > j ? j : r, p.ldc)]) : 0;
-      em = max(em, (int)((a[u][t] >> 52) & 0x7FF));
-    }
-  }
-  cl.sync();  // every CTA of the cluster runs, its barriers are initialised: its shared memory may be reached
-  const int emax = (int)trc_cluster_max(cl, sh, em);
-  const bool finite = emax < 0x7FF;
-  // row sums with every element below 2^53, then the shift that puts the largest into (2^60, 2^61]
-  const int sh0 = 1075 - emax;
-  ll rs = 0;
-#pragma unroll
-  for (int u = 0; u < RPW; ++u) {
-    ll s = 0;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      const ll q = qfix(a[u][t] & ~(1ll << 63), sh0);
-      s += q;
-    }
-    s = qwarp_sum(s);
-    rs = s > rs ? s : rs;
-  }
-  rs = trc_cluster_max(cl, sh, rs);
-  const int scale = sh0 + (rs > 0 ? __clzll(rs) - 3 : 0);
-#pragma unroll
-  for (int u = 0; u < RPW; ++u)
-#pragma unroll
-    for (int t = 0; t < NT; ++t) a[u][t] = qfix(a[u][t], scale);
-  ll x = l < n ? qfix(__double_as_longlong(p.C[l]), scale) : 0;
-  cl.sync();  // every element is read before the first reflector is stored
-
+  auto out = [&](ll q) { return scale2(F64 ? trc_dbl(q) : qscaled(q, 0), -scale); };
   // two words to the same place in CTA q, counted by its barrier
   auto push = [&](longlong2* slot, int buf, int q, ll y, ll el) {
     uint32_t rd, rb;
@@ -133,7 +109,6 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(rd),
                  "l"(y), "l"(el), "r"(rb) : "memory");
   };
-  const int cols = bad ? 0 : n;
   auto expect = [&](int i) {
     if (tid == 0)
       asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(cta_shared(&sh.bar[i & 1])),
@@ -161,7 +136,11 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
     if (i == n - 1) break;
     expect(i);
     // ---- norm of x(i + 2 ..): from the exact squares
-    {
+    if (F64) {
+      const double q = act && l > i + 1 ? trc_dbl(x) : 0.0, s2 = trc_sum(q * q);
+      if (lane == 0) sh.zs[warp] = __double_as_longlong(s2);
+      if (l == i + 1) sh.xa = x;
+    } else {
       const unsigned long long ax = act && l > i + 1 ? (unsigned long long)(x < 0 ? -x : x) : 0ull;
       unsigned q[6] = {0, 0, 0, 0, 0, 0};
       add_square(q, ax);
@@ -173,7 +152,22 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
       if (l == i + 1) sh.xa = x;
     }
     __syncthreads();
-    if (warp == 0) {
+    if (F64 && warp == 0) {
+      const double s2 = trc_sum(lane < TRC_WARPS ? trc_dbl(sh.zs[lane]) : 0.0), xa = trc_dbl(sh.xa);
+      double m = 0.0, tau = 0.0, beta = xa;
+      if (s2 != 0.0) {
+        const double n2 = fma(xa, xa, s2), ri = rsqrt(n2);
+        beta = -copysign(n2 * ri, xa);
+        m = 1.0 / (xa - beta);
+        tau = fma(fabs(xa), ri, 1.0);
+      }
+      if (lane == 0) {
+        sh.mq = trc_int2(m);
+        sh.tauq = sh.tau[i] = __double_as_longlong(tau);
+        sh.zero = s2 == 0.0;
+        sh.e[i] = __double_as_longlong(beta);
+      }
+    } else if (warp == 0) {
       unsigned q[6];
 #pragma unroll
       for (int u = 0; u < 6; ++u) q[u] = lane < TRC_WARPS ? sh.sq[lane][u] : 0u;
@@ -206,6 +200,12 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
             if (32 * t + 31 <= i) continue;
             const int j = 32 * t + lane;
             const int2 vj = sh.v[buf ^ 1][j], wj = sh.w[j];
+            if (F64) {  // (row above column first, so that both triangles round alike)
+              const double x1 = trc_dbl(r > j ? vr : wr), y1 = trc_dbl(r > j ? wj : vj);
+              const double x2 = trc_dbl(r > j ? wr : vr), y2 = trc_dbl(r > j ? vj : wj);
+              a[u][t] = __double_as_longlong(fma(-x2, y2, fma(-x1, y1, trc_dbl(a[u][t]))));
+              continue;
+            }
             // (one rounding; with v_r^2 + v_j^2 <= 1 beside v_1 the four middle products stay below 2^63)
             a[u][t] -= ((qhh(vr, wj) + qhh(wr, vj)) << 2) + (qmid(vr, wj, qmid(wr, vj, 1ll << 29)) >> 30);
           }
@@ -215,9 +215,13 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
     __syncthreads();
     // ---- v
     const int2 tq = qsplit(sh.tauq);
+    const double td = trc_dbl(sh.tauq);
     ll v = 0;
-    if (act && !sh.zero) v = l == i + 1 ? 1ll << 62 : qmul<61>(qsplit(x << sh.up), sh.mq);
-    const int2 vl = qsplit(v);
+    if (act && !sh.zero) {
+      if (F64) v = __double_as_longlong(l == i + 1 ? 1.0 : trc_dbl(x) * trc_dbl(sh.mq));
+      else v = l == i + 1 ? 1ll << 62 : qmul<61>(qsplit(x << sh.up), sh.mq);
+    }
+    const int2 vl = F64 ? trc_int2(trc_dbl(v)) : qsplit(v);
     sh.v[buf][l] = vl;
     __syncthreads();
     // ---- y = A v on this warp's rows, pushed to every CTA with the element of column i + 1
@@ -228,47 +232,57 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
       yr[u] = nx[u] = 0;
       if (r > i && r < n) {
         ll hh = 0, mm = 0, c1 = 0;
+        double yd = 0.0;
 #pragma unroll
         for (int t = 0; t < NT; ++t) {
           c1 |= a[u][t] & (t == ((i + 1) >> 5) ? -1ll : 0ll);
           if (32 * t + 31 <= i) continue;
+          if (F64) {
+            yd = fma(trc_dbl(a[u][t]), trc_dbl(sh.v[buf][32 * t + lane]), yd);
+            continue;
+          }
           const int2 q = qsplit(a[u][t]), vj = sh.v[buf][32 * t + lane];
           hh += qhh(q, vj);
           mm += qmid(q, vj, (((ll)q.x * vj.x) >> 32) + (1ll << 19)) >> 20;  // 10 bits more than a unit
         }
-        yr[u] = qwarp_sum((hh << 2) + ((mm + 512) >> 10));
+        yr[u] = F64 ? __double_as_longlong(trc_sum(yd)) : qwarp_sum((hh << 2) + ((mm + 512) >> 10));
         nx[u] = __shfl_sync(0xffffffffu, c1, (i + 1) & 31);
       }
     }
     push_rows(i, yr, nx);
     if (act && l % CL == k)  // (while the others push)
-      p.C[GEP_IX(l, i, p.ldc)] = !finite ? NAN : l == i + 1 ? scale2(qscaled(sh.e[i], 0), -scale) : qscaled(v, 62);
+      p.C[GEP_IX(l, i, p.ldc)] = !finite ? NAN : l == i + 1 ? out(sh.e[i]) : F64 ? trc_dbl(v) : qscaled(v, 62);
     const bool ok = cluster_wait<false>(cta_shared(&sh.bar[buf]), (uint32_t)(i >> 1) & 1u, p.st);
     // ---- w and column i + 1
     const ll y = act ? sh.recv[buf][l].x : 0, raw = act ? sh.recv[buf][l].y : 0;
-    const ll pl = qmul<61>(qsplit(y), tq);
+    const ll pl = F64 ? __double_as_longlong(td * trc_dbl(y)) : qmul<61>(qsplit(y), tq);
     {
-      const ll s = qwarp_sum(qmul<62>(qsplit(pl), vl));
+      const ll s = F64 ? __double_as_longlong(trc_sum(trc_dbl(pl) * trc_dbl(v))) : qwarp_sum(qmul<62>(qsplit(pl), vl));
       if (lane == 0) sh.zs[warp] = s;
     }
-    const ll p1 = qmul<61>(qsplit(sh.recv[buf][i + 1].x), tq);
+    const ll y1 = sh.recv[buf][i + 1].x;
     if (!__syncthreads_and(ok)) {
       ++i;
       break;
     }
-    const ll dot = qwarp_sum(lane < TRC_WARPS ? sh.zs[lane] : 0);
-    const int2 al = qsplit(qmul<62>(qsplit(dot), tq));
-    const ll w = pl - qmul<62>(al, vl);
-    const ll w1 = p1 - qjoin(al);
-    sh.w[l] = qsplit(act ? w : 0);
-    x = act ? raw - qmul<62>(vl, qsplit(sh.zero ? 0 : w1)) - w : 0;
+    if (F64) {
+      const double al = 0.5 * td * trc_sum(lane < TRC_WARPS ? trc_dbl(sh.zs[lane]) : 0.0);
+      const double w = fma(-al, trc_dbl(v), trc_dbl(pl)), w1 = fma(td, trc_dbl(y1), -al);
+      sh.w[l] = trc_int2(act ? w : 0.0);
+      x = act ? __double_as_longlong(fma(-trc_dbl(v), w1, trc_dbl(raw)) - w) : 0;
+    } else {
+      const int2 al = qsplit(qmul<62>(qsplit(qwarp_sum(lane < TRC_WARPS ? sh.zs[lane] : 0)), tq));
+      const ll w = pl - qmul<62>(al, vl), w1 = qmul<61>(qsplit(y1), tq) - qjoin(al);
+      sh.w[l] = qsplit(act ? w : 0);
+      x = act ? raw - qmul<62>(vl, qsplit(sh.zero ? 0 : w1)) - w : 0;
+    }
   }
   __syncthreads();
   if (k == 0 && l < cols) {
-    p.d[l] = finite ? scale2(qscaled(sh.d[l], 0), -scale) : NAN;
+    p.d[l] = finite ? out(sh.d[l]) : NAN;
     if (l + 1 < n) {
-      p.e[l] = finite ? scale2(qscaled(sh.e[l], 0), -scale) : NAN;
-      p.tau[l] = finite ? qscaled(sh.tau[l], 61) : NAN;
+      p.e[l] = finite ? out(sh.e[l]) : NAN;
+      p.tau[l] = !finite ? NAN : F64 ? trc_dbl(sh.tau[l]) : qscaled(sh.tau[l], 61);
     }
   }
   // No CTA leaves before every push into its shared memory has landed.  After a timeout the CTAs may have
@@ -286,6 +300,75 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
     cluster_wait<true>(cta_shared(&sh.bar[c & 1]), (uint32_t)(c >> 1) & 1u, p.st);
   }
   cl.sync();
+}
+
+// RPW rows a warp, NT slots of 32 columns: n <= 32 NT and n <= 16 RPW CL.
+template <int RPW, int NT>
+__global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
+  __shared__ TrcShared sh;
+  cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), k = (int)cl.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = p.n, l = tid;
+  const bool bad = status_bad(p.st);  // (every thread of the cluster passes through the same barriers)
+  if (tid == 0)
+    for (int b = 0; b < 2; ++b)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cta_shared(&sh.bar[b])) : "memory");
+  if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  for (int j = tid; j < TRC_MAX; j += TRC_THREADS) sh.v[0][j] = sh.v[1][j] = sh.w[j] = make_int2(0, 0);
+
+  // rows as bits of doubles; their largest exponent
+  ll a[RPW][NT];
+  int em = 0;
+#pragma unroll
+  for (int u = 0; u < RPW; ++u) {
+    const int r = (warp + TRC_WARPS * u) * CL + k;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const int j = 32 * t + lane;
+      a[u][t] = r < n && j < n ? __double_as_longlong(p.C[GEP_IX(r > j ? r : j, r > j ? j : r, p.ldc)]) : 0;
+      em = max(em, (int)((a[u][t] >> 52) & 0x7FF));
+    }
+  }
+  cl.sync();  // every CTA of the cluster runs, its barriers are initialised: its shared memory may be reached
+  ll emx = em, low = 0;
+  trc_cluster_max(cl, sh, emx, low);
+  const int emax = (int)emx;
+  const bool finite = emax < 0x7FF;
+  // row sums with every element below 2^53, then the shift that puts the largest into (2^60, 2^61]; and the
+  // smallest sum of a row of the matrix without its first column (of the first row: beside the diagonal)
+  const int sh0 = 1075 - emax;
+  ll rs = 0;
+  low = 0;  // 2^62 - smallest
+#pragma unroll
+  for (int u = 0; u < RPW; ++u) {
+    const int r = (warp + TRC_WARPS * u) * CL + k;
+    ll s = 0, any = 0, first = 0;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const ll m = a[u][t] & ~(1ll << 63), q = qfix(m, sh0);
+      s += q;
+      if (t == 0 && lane == 0) first = q;
+      else any |= m;
+    }
+    s = qwarp_sum(s);
+    rs = max(rs, s);
+    const ll rest = s - __shfl_sync(0xffffffffu, first, 0);
+    if (__any_sync(0xffffffffu, any != 0)) low = max(low, (1ll << 62) - rest);
+    else if (r == 0 && s > 0) low = max(low, (1ll << 62) - s);  // a decoupled first row: its diagonal
+  }
+  trc_cluster_max(cl, sh, rs, low);
+  const bool wide = finite && low > 0 && (1ll << 62) - low < rs >> TRC_SPREAD;
+  const int scale = wide ? 1023 - emax : sh0 + (rs > 0 ? __clzll(rs) - 3 : 0);
+  auto scaled = [&](double q) { return wide ? __double_as_longlong(scale2(q, scale)) : qfix(__double_as_longlong(q), scale); };
+#pragma unroll
+  for (int u = 0; u < RPW; ++u)
+#pragma unroll
+    for (int t = 0; t < NT; ++t) a[u][t] = scaled(trc_dbl(a[u][t]));
+  const ll x = l < n ? scaled(p.C[l]) : 0;
+  cl.sync();  // every element is read before the first reflector is stored
+  const int cols = bad ? 0 : n;
+  if (wide) trc_columns<true, RPW, NT>(p, sh, cl, a, x, scale, finite, cols);
+  else trc_columns<false, RPW, NT>(p, sh, cl, a, x, scale, finite, cols);
 }
 
 template <int RPW, int NT>

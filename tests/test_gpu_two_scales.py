@@ -1,0 +1,68 @@
+"""Reductions of matrices whose blocks lie on very different scales, and that are decoupled or coupled only through the
+first column: every block keeps the accuracy that it has alone (a backward error of 200 M eps of its own norm, the
+tolerance of the other stage tests), whatever arithmetic the reduction takes."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+EPS = 2.0 ** -52
+
+
+@pytest.fixture(scope="module")
+def gep():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_1504_06443_gb300 import build
+    build.build()
+    import paper_1504_06443_gb300 as g
+    g.load()
+    return g
+
+
+def _symmetric(M, seed):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    G = torch.randn(M, M, generator=g, dtype=torch.float64, device="cuda")
+    return G + G.t()
+
+
+def _blocks(M, m1, s, seed):
+    import torch
+    C = torch.zeros(M, M, dtype=torch.float64, device="cuda")
+    C[:m1, :m1] = _symmetric(m1, seed)
+    C[m1:, m1:] = s * _symmetric(M - m1, seed + 1)
+    return C
+
+
+def _backward(Q, C, T, rows):
+    """Largest entry of Q^T C Q - T on a block that Q maps into itself, over the block's norm."""
+    import torch
+    q, c, t = Q[rows, rows], C[rows, rows], T[rows, rows]
+    return float((q.t() @ c @ q - t).abs().max() / torch.linalg.matrix_norm(c, 2))
+
+
+@pytest.mark.parametrize("M,m1", [(12, 5), (40, 17), (100, 99), (128, 1), (300, 100), (500, 250), (512, 480), (700, 600)])
+@pytest.mark.parametrize("s", [0.25, 0.03, 1e-4, 1e-10, 1e-19, 1e-60, 1e8])
+def test_tridiagonal_blocks(gep, M, m1, s):
+    import torch
+    C = _blocks(M, m1, s, M)
+    d, e, tau, Cr = gep.tridiag_1stage(C)
+    Q = gep.sep_backtransform(Cr, tau, torch.eye(M, dtype=torch.float64, device="cuda"))
+    T = torch.diag(d) + torch.diag(e, 1) + torch.diag(e, -1)
+    assert float(e[m1 - 1]) == 0.0
+    assert not bool(Q[:m1, m1:].any()) and not bool(Q[m1:, :m1].any())
+    for rows in (slice(0, m1), slice(m1, M)):
+        assert _backward(Q, C, T, rows) <= 200 * M * EPS
+
+
+@pytest.mark.parametrize("M", [33, 200, 512])
+@pytest.mark.parametrize("s", [1e-3, 1e-12, 1e-25])
+def test_tridiagonal_large_first_column(gep, M, s):
+    """Only the first reflector sees the first column; what it leaves is on the scale of the rest."""
+    import torch
+    C = s * _symmetric(M, M)
+    C[0, 1:] = C[1:, 0] = torch.linspace(1, 2, M - 1, dtype=torch.float64, device="cuda")
+    d, e, tau, Cr = gep.tridiag_1stage(C)
+    Q = gep.sep_backtransform(Cr, tau, torch.eye(M, dtype=torch.float64, device="cuda"))
+    T = torch.diag(d) + torch.diag(e, 1) + torch.diag(e, -1)
+    assert _backward(Q, C, T, slice(1, M)) <= 200 * M * EPS
