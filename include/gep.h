@@ -176,6 +176,9 @@ int sep_backtransform(gep_handle_t h, int M, int ncol, const double* C, int ldc,
  *   d[M], e[M-1] receive T; q2 (device, sep_q2_elems(M, b) doubles, caller-owned;
  *   NULL when only eigenvalues are wanted) receives the bulge-chasing reflectors.
  *   C's band itself is not modified by the second stage.
+ *   With b = 32 or 64 the second stage holds the band in 64-bit fixed point with one unit, about
+ *   2^-61 of its largest absolute row sum, where all row sums lie within a factor of 16, and in
+ *   FP64 otherwise.
  * sep_backtransform_2stage: Z (M x ncol) is overwritten by Q1 (Q2 Z) using C, tau1 and
  *   q2 from sep_tridiag_2stage with the same M and b.
  * Both take their scratch from the handle workspace (size it with gep_workspace_size

@@ -560,6 +560,7 @@ struct BulgeArgs {
   int* prog;          // prog[s] = steps of sweep s completed (k_bulge_ws: see there)
   double* q2;         // diamond storage (or null)
   int* st;
+  const unsigned long long* mx;  // norm bounds (k_band_rowsum) where both arithmetics are launched, else null
   unsigned long long wait_ns;  // limit of each progress wait
   int drop_sweep;              // test hook: this sweep publishes no progress (-1: none)
 };
@@ -624,6 +625,14 @@ __device__ void two_sided(double* D, int len, const double* v, double tau, doubl
   __syncthreads();
 }
 
+// Norm bounds of the band (k_band_rowsum): mx[0] largest absolute row sum, mx[1] the complement of the
+// smallest one beside the first column (bits of doubles).  With the rows further apart than 2^4 the band stays
+// FP64: one fixed-point unit for all of it would take the relative accuracy of its small blocks.
+__device__ __forceinline__ bool band_wide(const unsigned long long* mx) {
+  const double hi = __longlong_as_double((ll)mx[0]), lo = __longlong_as_double((ll)~mx[1]);
+  return mx[1] != 0 && (mx[0] >> 52) < 0x7FF && lo < 0.0625 * hi;
+}
+
 __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
   extern __shared__ double sm[];
   double* Bm = sm;                          // BMAX x (BMAX+1), [row][col]
@@ -638,7 +647,7 @@ __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
   const int t = threadIdx.x, M = a.M, b = a.b, ldab = a.ldab;
   if (t == 0) abort_flag = 0;
   __syncthreads();
-  if (status_bad(a.st)) return;
+  if (status_bad(a.st) || (a.mx && !band_wide(a.mx))) return;
   for (int s = blockIdx.x; s <= M - 2; s += gridDim.x) {
     const int ns = bulge_steps(M, b, s);
     double taup = 0.0;
@@ -746,7 +755,7 @@ __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
 //
 // Arithmetic.  The band is held as 64-bit integers q with C = q 2^-sh, sh chosen so that the
 // largest absolute row sum of the band (a bound on its 2-norm, which no similarity changes) is
-// at most 2^61; reflectors have v in Q62 (|v_i| <= 1 by construction), tau in Q61.  The norms
+// at most 2^61 (rows too far apart for one unit: band_wide); reflectors have v in Q62 (|v_i| <= 1 by construction), tau in Q61.  The norms
 // in play (v^T v <= 2, tau |v| <= 2, w = tau C v - ... at most 2 |C|) keep every intermediate
 // below 2^63.  A product drops only the low x low limb: its error is about half a unit, 2^-62
 // of the row-sum bound, where an FP64 operation rounds its result at 2^-54; every term is rounded by
@@ -853,7 +862,7 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (status_bad(a.st)) return;
+  if (status_bad(a.st) || band_wide(a.mx)) return;
   int* progA = a.prog;
   int* progF = a.prog + M;
   int g = 0;  // steps of this CTA so far (every role counts the same)
@@ -1150,22 +1159,29 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
   }
 }
 
-// Largest absolute row sum of the band matrix (bits of a non-negative double, by atomicMax).
+// Norm bounds of the band matrix for band_wide and band_shift (mx zero on entry).
 __global__ void k_band_rowsum(int M, int b, const double* __restrict__ AB, int ldab, unsigned long long* mx,
                               const int* st) {
   if (status_bad(st)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  double s = 0.0;
+  double rest = 0.0, first = 0.0;  // first: the entry of the first column (of row 0: the diagonal)
   if (i < M) {
-    for (int o = 0; o <= b && i + o < M; ++o) s += fabs(AB[o + (size_t)i * ldab]);
-    for (int o = 1; o <= b && o <= i; ++o) s += fabs(AB[o + (size_t)(i - o) * ldab]);
+    first = i <= b ? fabs(AB[i]) : 0.0;
+    for (int o = i == 0 ? 1 : 0; o <= b && i + o < M; ++o) rest += fabs(AB[o + (size_t)i * ldab]);
+    for (int o = 1; o <= b && o < i; ++o) rest += fabs(AB[o + (size_t)(i - o) * ldab]);
   }
-  unsigned long long v = (unsigned long long)__double_as_longlong(s);
+  unsigned long long v = (unsigned long long)__double_as_longlong(rest + first);
+  if (i == 0 && rest == 0.0) rest = first;  // a decoupled first row
+  unsigned long long u = rest > 0.0 ? ~(unsigned long long)__double_as_longlong(rest) : 0;
   for (int o = 16; o; o >>= 1) {
-    const unsigned long long q = __shfl_xor_sync(0xffffffffu, v, o);
+    const unsigned long long q = __shfl_xor_sync(0xffffffffu, v, o), p = __shfl_xor_sync(0xffffffffu, u, o);
     if (q > v) v = q;
+    if (p > u) u = p;
   }
-  if ((threadIdx.x & 31) == 0 && v) atomicMax(mx, v);
+  if ((threadIdx.x & 31) == 0) {
+    if (v) atomicMax(mx, v);
+    if (u) atomicMax(mx + 1, u);
+  }
 }
 
 // sh with (largest row sum) 2^sh in (2^60, 2^61]
@@ -1175,7 +1191,7 @@ __device__ __forceinline__ int band_shift(const unsigned long long* mx) {
 }
 
 __global__ void k_band_fix(int M, double* AB, int ldab, const unsigned long long* mx, const int* st) {
-  if (status_bad(st)) return;
+  if (status_bad(st) || band_wide(mx)) return;
   const int sh = band_shift(mx);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)M * ldab; i += (size_t)gridDim.x * blockDim.x) {
     const double x = AB[i];
@@ -1188,6 +1204,11 @@ __global__ void k_band_diag_fix(int M, const double* __restrict__ AB, int ldab, 
   if (status_bad(st)) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x, sh = band_shift(mx);
   if (i >= M) return;
+  if (band_wide(mx)) {
+    d[i] = AB[(size_t)i * ldab];
+    if (i + 1 < M) e[i] = AB[1 + (size_t)i * ldab];
+    return;
+  }
   const ll* q = reinterpret_cast<const ll*>(AB);
   const bool finite = (*mx >> 52) < 0x7FF;  // an integer cannot carry a NaN or an infinity of the band
   d[i] = finite ? scale2((double)q[(size_t)i * ldab], -sh) : NAN;
@@ -1672,45 +1693,46 @@ int band_to_tridiag(gep_handle_t h, int M, const double* C, int ldc, int b, doub
     GEP_CUDA(cudaMemsetAsync(prog, 0, sizeof(int) * 2 * (size_t)M, h->stream));
     const int Q = (M - 2) / b;
     if (q2) GEP_CUDA(cudaMemsetAsync(q2, 0, q2_elems(M, b) * sizeof(double), h->stream));
-    // b = 32 and 64 take the fixed-point kernel, other widths the general one
+    // b = 32 and 64 take the fixed-point kernel unless the rows differ in scale (known on the device only: both
+    // kernels are launched and one returns at once, about 5 us), other widths the general one
     const bool fixed = b == 32 || b == 64;
     unsigned long long* mx = reinterpret_cast<unsigned long long*>(prog + rr((size_t)M) * 2);
-    const void* kern = b == 32 ? (const void*)k_bulge_ws<32> : b == 64 ? (const void*)k_bulge_ws<64> : (const void*)k_bulge;
-    const size_t smem = b == 32 ? sizeof(BulgeShared<32>) : b == 64 ? sizeof(BulgeShared<64>) : bulge_smem_bytes();
     static unsigned long long attr_devices = 0;
     if (first_use_on_device(attr_devices)) {
       GEP_CUDA(cudaFuncSetAttribute(k_bulge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bulge_smem_bytes()));
       GEP_CUDA(cudaFuncSetAttribute(k_bulge_ws<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BulgeShared<32>)));
       GEP_CUDA(cudaFuncSetAttribute(k_bulge_ws<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BulgeShared<64>)));
     }
-    int per_sm = 0;
-    const int threads = b == 32 ? bulge_threads<32>() : b == 64 ? bulge_threads<64>() : 256;
-    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
-    if (per_sm < 1) return GEP_ERR_UNSUPPORTED;
-    // The sweeps form a dependency chain (step k of sweep s waits for step k+1 of sweep
-    // s-1): the time is set by the latency of one step, which co-resident CTAs stretch.
-    if (per_sm > BULGE_CTAS_PER_SM) per_sm = BULGE_CTAS_PER_SM;
-    int grid = per_sm * h->sm_count;
-    // Sweep s starts two steps after sweep s-1 and lasts about (M - 2) / b + 1 steps, so
-    // about half that many sweeps are in flight at once: CTAs beyond that would only wait,
-    // holding SMs that concurrent solves on other streams could use.
-    const int in_flight = ((M - 2) / b + 1) / 2 + 2;
-    if (grid > in_flight) grid = in_flight;
-    if (grid > M - 1) grid = M - 1;
     BulgeArgs a;
     a.M = M; a.b = b; a.ldab = ldab; a.Q = Q; a.AB = AB; a.prog = prog; a.q2 = q2; a.st = h->d_status;
+    a.mx = fixed ? mx : nullptr;
     a.wait_ns = h->wait_limit_ns;
     a.drop_sweep = h->fault_drop_sweep;
     if (fixed) {
-      GEP_CUDA(cudaMemsetAsync(mx, 0, sizeof(unsigned long long), h->stream));
+      GEP_CUDA(cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned long long), h->stream));
       k_band_rowsum<<<(M + 255) / 256, 256, 0, h->stream>>>(M, b, AB, ldab, mx, h->d_status);
       GEP_CHECK(check_launch(h));
       k_band_fix<<<std::min(M, 4 * h->sm_count), 256, 0, h->stream>>>(M, AB, ldab, mx, h->d_status);
       GEP_CHECK(check_launch(h));
     }
-    void* args[] = {&a};
-    GEP_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, smem, h->stream));
-    GEP_CHECK(check_launch(h));
+    auto chase = [&](const void* kern, int threads, size_t smem) -> int {
+      int per_sm = 0;
+      GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+      if (per_sm < 1) return GEP_ERR_UNSUPPORTED;
+      // The sweeps form a dependency chain (step k of sweep s waits for step k+1 of sweep
+      // s-1): the time is set by the latency of one step, which co-resident CTAs stretch.
+      if (per_sm > BULGE_CTAS_PER_SM) per_sm = BULGE_CTAS_PER_SM;
+      // Sweep s starts two steps after sweep s-1 and lasts about (M - 2) / b + 1 steps, so
+      // about half that many sweeps are in flight at once: CTAs beyond that would only wait,
+      // holding SMs that concurrent solves on other streams could use.
+      const int grid = std::min({per_sm * h->sm_count, ((M - 2) / b + 1) / 2 + 2, M - 1});
+      void* args[] = {&a};
+      GEP_CUDA(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, smem, h->stream));
+      return check_launch(h);
+    };
+    if (b == 32) GEP_CHECK(chase((const void*)k_bulge_ws<32>, bulge_threads<32>(), sizeof(BulgeShared<32>)));
+    if (b == 64) GEP_CHECK(chase((const void*)k_bulge_ws<64>, bulge_threads<64>(), sizeof(BulgeShared<64>)));
+    GEP_CHECK(chase((const void*)k_bulge, 256, bulge_smem_bytes()));
     if (fixed) {
       k_band_diag_fix<<<(M + 255) / 256, 256, 0, h->stream>>>(M, AB, ldab, mx, d, e, h->d_status);
       return check_launch(h);

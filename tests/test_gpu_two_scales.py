@@ -66,3 +66,36 @@ def test_tridiagonal_large_first_column(gep, M, s):
     Q = gep.sep_backtransform(Cr, tau, torch.eye(M, dtype=torch.float64, device="cuda"))
     T = torch.diag(d) + torch.diag(e, 1) + torch.diag(e, -1)
     assert _backward(Q, C, T, slice(1, M)) <= 200 * M * EPS
+
+
+def _block_eigenvalues(C, d, e, rows):
+    """Largest error of the eigenvalues of T on a decoupled block, over the block's norm."""
+    import torch
+    t = (torch.diag(d) + torch.diag(e, 1) + torch.diag(e, -1))[rows, rows].cpu()
+    ref = torch.linalg.eigvalsh(C[rows, rows].cpu())
+    return float((torch.linalg.eigvalsh(t) - ref).abs().max() / ref.abs().max())
+
+
+@pytest.mark.parametrize("M,m1", [(90, 40), (300, 96), (700, 500)])
+@pytest.mark.parametrize("b", [20, 32, 64])
+@pytest.mark.parametrize("s", [0.25, 1e-4, 1e-10, 1e-19, 1e8])
+def test_two_stage_blocks(gep, M, m1, b, s):
+    C = _blocks(M, m1, s, M)
+    d, e, *_ = gep.tridiag_2stage(C, b)
+    assert float(e[m1 - 1]) == 0.0
+    for rows in (slice(0, m1), slice(m1, M)):
+        assert _block_eigenvalues(C, d, e, rows) <= 200 * M * EPS
+
+
+@pytest.mark.parametrize("b", [20, 32, 64])
+@pytest.mark.parametrize("s", [1e-3, 1e-12, 1e-25])
+def test_band_large_first_column(gep, b, s):
+    """A band matrix whose first column alone is large: T beyond its first row stays on the scale of the rest."""
+    import torch
+    M = 150
+    i = torch.arange(M, device="cuda")
+    C = torch.where((i[:, None] - i[None, :]).abs() <= b, s * _symmetric(M, 4), torch.zeros_like(_symmetric(M, 4)))
+    C[0, 1:b + 1] = C[1:b + 1, 0] = torch.linspace(1, 2, b, dtype=torch.float64, device="cuda")
+    d, e, *_ = gep.tridiag_2stage(C, b)
+    # the first sweep's reflector acts on rows 1.. only, so T(1:, 1:) is a similarity of C(1:, 1:)
+    assert _block_eigenvalues(C, d, e, slice(1, M)) <= 200 * M * EPS
