@@ -67,7 +67,8 @@ typedef struct gep_handle_s* gep_handle_t;
                             CUDA cores, about 8 M^3 flops per sweep.  Stage times: t[3] holds it. */
 
 /* Arithmetic of the dense contractions. */
-#define GEP_PREC_FP64 0          /* FP64 throughout                                     */
+#define GEP_PREC_FP64 0          /* FP64 throughout (reductions to tridiagonal form: FP64, or 64-bit fixed
+                                    point where the rows are of like size, see sep_tridiag_*) */
 #define GEP_PREC_FP64_EMULATED 1 /* FP64-accurate products from split-BF16 tensor cores  */
 #define GEP_PREC_MIXED_REFINED 2 /* FP32-grade split-BF16 reducer + full->band, then FP64 refinement */
 
@@ -176,9 +177,10 @@ int sep_backtransform(gep_handle_t h, int M, int ncol, const double* C, int ldc,
  *   d[M], e[M-1] receive T; q2 (device, sep_q2_elems(M, b) doubles, caller-owned;
  *   NULL when only eigenvalues are wanted) receives the bulge-chasing reflectors.
  *   C's band itself is not modified by the second stage.
- *   With b = 32 or 64 the second stage holds the band in 64-bit fixed point with one unit, about
- *   2^-61 of its largest absolute row sum, where all row sums lie within a factor of 16, and in
- *   FP64 otherwise.
+ *   With b <= 32 panels of up to 2048 rows are held in 64-bit fixed point with one unit a column,
+ *   2^-60 of its norm, and with b = 32 or 64 the second stage's band with one unit, about 2^-61 of
+ *   its largest absolute row sum, where the rows of the matrix (their largest entries; of the band
+ *   their sums) lie within a factor of 16, and in FP64 otherwise.
  * sep_backtransform_2stage: Z (M x ncol) is overwritten by Q1 (Q2 Z) using C, tau1 and
  *   q2 from sep_tridiag_2stage with the same M and b.
  * Both take their scratch from the handle workspace (size it with gep_workspace_size

@@ -162,6 +162,48 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Largest exponent field of every row of the symmetric matrix in the lower triangle of C (zero on entry), a
+// 64 x 64 tile a CTA; one pass over the triangle: order 8192 about 50 us.
+__global__ void __launch_bounds__(256) k_row_exponents(int M, const double* __restrict__ C, int ldc, int* __restrict__ ex,
+                                                       const int* st) {
+  __shared__ int row[64], col[64];
+  if (blockIdx.x < blockIdx.y || status_bad(st)) return;
+  const int t = threadIdx.x, r0 = blockIdx.x * 64, c0 = blockIdx.y * 64, r = r0 + (t & 63);
+  if (t < 64) row[t] = col[t] = 0;
+  __syncthreads();
+  int m = 0;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int q = (t >> 6) + 4 * u, c = c0 + q;
+    const int x = r < M && c <= r ? (int)((__double_as_longlong(C[r + (size_t)c * ldc]) >> 52) & 0x7FF) : 0;
+    m = max(m, x);
+    const int w = __reduce_max_sync(0xffffffffu, x);
+    if ((t & 31) == 0) atomicMax(&col[q], w);
+  }
+  atomicMax(&row[t & 63], m);
+  __syncthreads();
+  if (t < 64 && r0 + t < M) atomicMax(ex + r0 + t, row[t]);
+  else if (t >= 64 && t < 128 && c0 + t - 64 < M) atomicMax(ex + c0 + t - 64, col[t - 64]);
+}
+
+// *wide: whether the rows that are not zero lie further apart than 2^4.
+__global__ void __launch_bounds__(1024) k_row_spread(int M, const int* __restrict__ ex, int* __restrict__ wide, const int* st) {
+  __shared__ int hi, lo;
+  if (status_bad(st)) return;
+  if (threadIdx.x == 0) {
+    hi = 0;
+    lo = 0x7FF;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < M; i += 1024)
+    if (ex[i]) {
+      atomicMax(&hi, ex[i]);
+      atomicMin(&lo, ex[i]);
+    }
+  __syncthreads();
+  if (threadIdx.x == 0) *wide = hi < 0x7FF && hi - lo > 4;
+}
+
 // The whole panel QR in one cooperative launch: CTA g keeps panel rows [rp g, rp g + rp)
 // (rp = 64, 128 or 256: the per-SM FP64 rate bounds a step, so short panels take more
 // CTAs of fewer rows) in shared memory for all column steps.  Each step is k_pqr_step's
@@ -1423,7 +1465,7 @@ namespace {
 struct BandWs {
   double *part0, *part1, *prow0, *prow1;
   long long gcap;  // CTAs the partial-sum buffers hold
-  int* bar;
+  int *bar, *wide;
   double *V, *CV, *V1, *W1;
   double *WV, *VW;     // n x 2 G b: [W_0 V_0 W_1 V_1 ...] and [V_0 W_0 V_1 W_1 ...] of a panel group
   double *GV, *T, *Tt, *Pm, *Ym, *Zs;
@@ -1515,7 +1557,7 @@ int panel_qr_launch(gep_handle_t h, const PanelArgs& a, long long part_elems) {
 int panel_qr(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, const BandWs& w, double* Va, double* Vb,
              int r0, int ldv) {
   if (panel_qr_cluster_takes(n, b)) {
-    const int rc = panel_qr_cluster(h, n, b, P, ldp, tau, Va, Vb, r0, ldv, w.T);
+    const int rc = panel_qr_cluster(h, n, b, P, ldp, tau, Va, Vb, r0, ldv, w.T, w.wide);
     if (rc != GEP_ERR_UNSUPPORTED) return rc;
   }
   PanelArgs a;
@@ -1565,6 +1607,7 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
   w.prow0 = take(BMAX);
   w.prow1 = take(BMAX);
   w.bar = reinterpret_cast<int*>(take(32));
+  w.wide = w.bar + 32;
   w.V = take((size_t)M * b);
   w.CV = take((size_t)M * b);
   w.V1 = take((size_t)M * b);
@@ -1582,6 +1625,15 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
   w.part_elems = oz_sym_part_elems(M, b);
   w.parts = take(w.part_elems);
   const int levels = eng == GEP_PREC_MIXED_REFINED ? 4 : 9;
+  if (b <= PQN) {  // the arithmetic of the panels in a cluster (the exponents in V, not yet in use)
+    int* ex = reinterpret_cast<int*>(w.V);
+    GEP_CUDA(cudaMemsetAsync(ex, 0, sizeof(int) * (size_t)M, h->stream));
+    const int nt = (M + 63) / 64;
+    k_row_exponents<<<dim3(nt, nt), 256, 0, h->stream>>>(M, C, ldc, ex, h->d_status);
+    GEP_CHECK(check_launch(h));
+    k_row_spread<<<1, 1024, 0, h->stream>>>(M, ex, w.wide, h->d_status);
+    GEP_CHECK(check_launch(h));
+  }
   for (int pb = 0; M - pb - b >= 2;) {
     const int n = M - pb - b;
     // panels of this group: panel j (j >= 1) owns columns [(j-1) b, j b) of C22 and its

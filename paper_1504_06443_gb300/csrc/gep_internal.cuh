@@ -232,7 +232,7 @@ int reduce_explicit_inv(gep_handle_t h, int M, double* A, int lda, double* L, in
 // QR of a panel of at most 32 columns with its T factor in one cluster (panel_cluster.cu).
 bool panel_qr_cluster_takes(int n, int nb);
 int panel_qr_cluster(gep_handle_t h, int n, int nb, double* P, int ldp, double* tau, double* Va, double* Vb, int r0,
-                     int ldv, double* T);
+                     int ldv, double* T, const int* wide);
 // Small trailing matrices of it in one cluster (tridiag_cluster.cu).
 bool tridiag_cluster_takes(int n);
 int tridiag_cluster(gep_handle_t h, int n, double* C, int ldc, double* d, double* e, double* tau);

@@ -9,6 +9,9 @@
 // sums, so that a pivot column that has become tiny still gives an orthogonal reflector.  The
 // scalars of a reflector are formed by warp 0 of every CTA; an extra warp of CTA 0 accumulates T in FP64.
 //
+// A column's unit is fair to rows of like size only: where the rows of the matrix lie further apart than 2^4
+// (band.cu's scan) the same exchange carries FP64 numbers, columns scaled by powers of two.
+//
 // A column: every CTA pushes its sums (and the owner of the pivot row that row) to all 16
 // (st.async, counted by an mbarrier of each); warp 0 adds them up and forms the scalars and, lane by lane,
 // tau w_j; the row warps apply the reflector and form the next dots.  All CTAs push for every column, so
@@ -19,6 +22,8 @@
 // against 160, so longer panels stay there.  S1b at order 516 4.57 -> 2.68 ms, 1024 8.9 -> 5.8, 2047 15.7 -> 14.2,
 // 4000 38.6 -> 37.0.
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "cluster.cuh"
 #include "fixed.cuh"
@@ -35,8 +40,13 @@ constexpr int QTHREADS = 32 * (QW + 1);
 struct QrArgs {
   int n, nb, ldp, r0, ldv;
   double *P, *tau, *Va, *Vb, *T;
+  const int* wide;  // nonzero: FP64
   int* st;
 };
+
+__device__ __forceinline__ double qr_dbl(ll a) { return __longlong_as_double(a); }
+__device__ __forceinline__ double qr_dbl(int2 a) { return __hiloint2double(a.y, a.x); }
+__device__ __forceinline__ int2 qr_int2(double x) { return make_int2(__double2loint(x), __double2hiint(x)); }
 
 // Exact sum of products of numbers split into balanced limbs.
 struct Dot128 {
@@ -85,7 +95,7 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
   cg::cluster_group cl = cg::this_cluster();
   const int k = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = p.n, nb = p.nb, nref = n < nb ? n : nb;
-  const bool bad = status_bad(p.st), worker = warp < QW;
+  const bool bad = status_bad(p.st), worker = warp < QW, use_fp64 = *p.wide != 0;
   if (tid == 0) {
     for (int b = 0; b < 2; ++b)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cta_shared(&sh.bar[b])) : "memory");
@@ -143,10 +153,10 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
     Sum128 s = sh.recv[0][0][lane];
     for (int q = 1; q < QC; ++q) s = add128(s, sh.recv[0][q][lane]);
     const int bits = s.hi ? 128 - __clzll(s.hi) : 64 - __clzll(s.lo);  // norm^2 < 2^bits
-    scale = sh0 + 60 - (bits + 1) / 2;
+    scale = use_fp64 ? 1023 - em : sh0 + 60 - (bits + 1) / 2;
   }
 #pragma unroll
-  for (int u = 0; u < RPW; ++u) a[u] = qfix(a[u], scale);
+  for (int u = 0; u < RPW; ++u) a[u] = use_fp64 ? __double_as_longlong(scale2(qr_dbl(a[u]), scale)) : qfix(a[u], scale);
   cl.sync();  // recv is read everywhere before the first push
 
   auto expect = [&](int c) {
@@ -171,101 +181,150 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
   bool run = !bad;
   ll xk = 0;  // lane u: the pivot column in the warp's row u
   int c = -1;
-  for (; run && c < nref; ++c) {
-    const int nc = c + 1;
-    if (c >= 0) {
-      if (warp == 0) {
-        const bool ok = cluster_wait<false>(cta_shared(&sh.bar[c & 1]), (uint32_t)(c >> 1) & 1u, p.st);
-        const Sum128(*rv)[QN] = sh.recv[c & 1];
-        Sum128 s = rv[0][lane];
+  auto columns = [&](auto arithmetic) {
+    constexpr bool wide = decltype(arithmetic)::value;
+    for (; run && c < nref; ++c) {
+      const int nc = c + 1;
+      if (c >= 0) {
+        if (warp == 0) {
+          const bool ok = cluster_wait<false>(cta_shared(&sh.bar[c & 1]), (uint32_t)(c >> 1) & 1u, p.st);
+          const Sum128(*rv)[QN] = sh.recv[c & 1];
+          if (wide) {
+            double s = 0.0;
 #pragma unroll
-        for (int q = 1; q < QC; ++q) s = add128(s, rv[q][lane]);
-        const ll pr = sh.rrow[c & 1][lane];
-        const unsigned long long xlo = (unsigned long long)__shfl_sync(0xffffffffu, s.lo, c);
-        const ll xhi = __shfl_sync(0xffffffffu, s.hi, c), al_q = __shfl_sync(0xffffffffu, pr, c);
-        ll tw = 0, g = pr >> 2;
-        QReflector o;
-        o.m = o.tq = 0;
-        o.beta = al_q;
-        o.up = 0;
-        if ((xhi | (ll)xlo) != 0) {
-          Sum128 x2;
-          x2.hi = xhi;
-          x2.lo = (ll)xlo;
-          o = q_reflector(al_q, x2);
-          // to the right: w = p + S / (alpha - beta), tau w; to the left: the Gram entry, Q60.  In the unit
-          // of x 2^up the divisor is 2^123 / m, so S is taken times 2^-(61 - up).
-          const int sft = lane < c ? 63 - o.up : 61 - o.up;
-          const ll t = sft ? (ll)(((unsigned long long)s.hi << (64 - sft)) | ((unsigned long long)s.lo >> sft)) : s.lo;
-          g = (lane < c ? pr >> 2 : pr) + qmul<62>(qsplit(t), qsplit(o.m));
-          if (lane > c) tw = qmul<61>(qsplit(g), qsplit(o.tq));
+            for (int q = 0; q < QC; ++q) s += qr_dbl(rv[q][lane].lo);
+            const double pr = qr_dbl(sh.rrow[c & 1][lane]);
+            const double xn2 = __shfl_sync(0xffffffffu, s, c), alpha = __shfl_sync(0xffffffffu, pr, c);
+            double tt = 0.0, sl = 0.0, be = alpha;
+            if (xn2 > 0.0) {
+              const double n2 = fma(alpha, alpha, xn2), ri = rsqrt(n2);
+              be = -copysign(n2 * ri, alpha);
+              sl = 1.0 / (alpha - be);
+              tt = fma(fabs(alpha), ri, 1.0);
+            }
+            const double w = fma(sl, s, pr);  // v^T P(:, j); for j < c the Gram entry v_j^T v
+            sh.tw[lane] = qr_int2(lane > c ? tt * w : 0.0);
+            sh.g[c & 1][lane] = __double_as_longlong(w);
+            if (lane == 0) {
+              sh.mq = qr_int2(sl);
+              sh.beta = __double_as_longlong(be);
+              sh.tq[c & 1] = __double_as_longlong(tt);
+            }
+          } else {
+            Sum128 s = rv[0][lane];
+#pragma unroll
+            for (int q = 1; q < QC; ++q) s = add128(s, rv[q][lane]);
+            const ll pr = sh.rrow[c & 1][lane];
+            const unsigned long long xlo = (unsigned long long)__shfl_sync(0xffffffffu, s.lo, c);
+            const ll xhi = __shfl_sync(0xffffffffu, s.hi, c), al_q = __shfl_sync(0xffffffffu, pr, c);
+            ll tw = 0, g = pr >> 2;
+            QReflector o;
+            o.m = o.tq = 0;
+            o.beta = al_q;
+            o.up = 0;
+            if ((xhi | (ll)xlo) != 0) {
+              Sum128 x2;
+              x2.hi = xhi;
+              x2.lo = (ll)xlo;
+              o = q_reflector(al_q, x2);
+              // to the right: w = p + S / (alpha - beta), tau w; to the left: the Gram entry, Q60.  In the unit
+              // of x 2^up the divisor is 2^123 / m, so S is taken times 2^-(61 - up).
+              const int sft = lane < c ? 63 - o.up : 61 - o.up;
+              const ll t = sft ? (ll)(((unsigned long long)s.hi << (64 - sft)) | ((unsigned long long)s.lo >> sft)) : s.lo;
+              g = (lane < c ? pr >> 2 : pr) + qmul<62>(qsplit(t), qsplit(o.m));
+              if (lane > c) tw = qmul<61>(qsplit(g), qsplit(o.tq));
+            }
+            sh.tw[lane] = qsplit(tw);
+            sh.g[c & 1][lane] = g;
+            if (lane == 0) {
+              sh.mq = qsplit(o.m);
+              sh.up = o.up;
+              sh.beta = o.beta;
+              sh.tq[c & 1] = o.tq;
+            }
+          }
+          if (lane == 0 && !ok) sh.fail = c + 1;
         }
-        sh.tw[lane] = qsplit(tw);
-        sh.g[c & 1][lane] = g;
-        if (lane == 0) {
-          sh.mq = qsplit(o.m);
-          sh.up = o.up;
-          sh.beta = o.beta;
-          sh.tq[c & 1] = o.tq;
-          if (!ok) sh.fail = c + 1;
+        all_sync();
+        if (sh.fail == c + 1) break;  // (a warp still here may already see the next column's)
+        if (worker) {
+          const int2 tw = sh.tw[lane];
+          const ll be = sh.beta;
+          if (wide) {
+            const double vk = qr_dbl(xk) * qr_dbl(sh.mq), t = qr_dbl(tw);
+#pragma unroll
+            for (int u = 0; u < RPW; ++u) {
+              const int r = row0 + u;
+              const double v = __shfl_sync(0xffffffffu, vk, u);
+              if (r > c) a[u] = __double_as_longlong(lane == c ? v : fma(-v, t, qr_dbl(a[u])));
+              else if (r == c) a[u] = lane == c ? be : __double_as_longlong(qr_dbl(a[u]) - t);
+            }
+          } else {
+            // lane u forms v of the warp's row u
+            const int2 vk = qsplit(qmul<61>(qsplit(xk << sh.up), sh.mq));
+#pragma unroll
+            for (int u = 0; u < RPW; ++u) {
+              const int r = row0 + u;
+              int2 v;
+              v.x = __shfl_sync(0xffffffffu, vk.x, u);
+              v.y = __shfl_sync(0xffffffffu, vk.y, u);
+              if (r > c) a[u] = lane == c ? qjoin(v) : a[u] - qmul<62>(v, tw);
+              else if (r == c) a[u] = lane == c ? be : a[u] - qjoin(tw);
+            }
+          }
+        } else if (k == 0) {  // column c of T: T(0:c, c) = -tau T(0:c, 0:c) G(0:c, c)
+          const double tt = wide ? qr_dbl(sh.tq[c & 1]) : qscaled(sh.tq[c & 1], 61);
+          const double gl = lane >= c ? 0.0 : wide ? qr_dbl(sh.g[c & 1][lane]) : qscaled(sh.g[c & 1][lane], 60);
+          if (lane == 0) p.tau[c] = finite ? tt : NAN;
+          double s = 0.0;
+          for (int q = 0; q < c; ++q) s = fma(sh.T[lane][q], __shfl_sync(0xffffffffu, gl, q), s);
+          sh.T[lane][c] = lane < c ? -tt * s : (lane == c ? tt : 0.0);
+          __syncwarp();
         }
       }
-      all_sync();
-      if (sh.fail == c + 1) break;  // (a warp still here may already see the next column's)
+      if (nc >= nref) break;
       if (worker) {
-        const int2 tw = sh.tw[lane];
-        const ll be = sh.beta;
-        // lane u forms v of the warp's row u
-        const int2 vk = qsplit(qmul<61>(qsplit(xk << sh.up), sh.mq));
+        expect(nc);
+        Dot128 d;
+        double f = 0.0;
+        xk = 0;
 #pragma unroll
         for (int u = 0; u < RPW; ++u) {
           const int r = row0 + u;
-          int2 v;
-          v.x = __shfl_sync(0xffffffffu, vk.x, u);
-          v.y = __shfl_sync(0xffffffffu, vk.y, u);
-          if (r > c) a[u] = lane == c ? qjoin(v) : a[u] - qmul<62>(v, tw);
-          else if (r == c) a[u] = lane == c ? be : a[u] - qjoin(tw);
+          if (wide) {
+            const double x = __shfl_sync(0xffffffffu, qr_dbl(a[u]), nc);
+            if (lane == u) xk = r > nc ? __double_as_longlong(x) : 0;
+            if (r > nc) f = fma(x, qr_dbl(a[u]), f);
+            else if (r == nc) sh.prow[lane] = a[u];
+            continue;
+          }
+          const int2 q = qsplit(a[u]);
+          int2 x;
+          x.x = __shfl_sync(0xffffffffu, q.x, nc);
+          x.y = __shfl_sync(0xffffffffu, q.y, nc);
+          if (lane == u) xk = r > nc ? qjoin(x) : 0;
+          if (r > nc) d.add(x, q);
+          else if (r == nc) sh.prow[lane] = a[u];
         }
-      } else if (k == 0) {  // column c of T: T(0:c, c) = -tau T(0:c, 0:c) G(0:c, c)
-        const double tt = qscaled(sh.tq[c & 1], 61);
-        const double gl = lane < c ? qscaled(sh.g[c & 1][lane], 60) : 0.0;
-        if (lane == 0) p.tau[c] = finite ? tt : NAN;
-        double s = 0.0;
-        for (int q = 0; q < c; ++q) s = fma(sh.T[lane][q], __shfl_sync(0xffffffffu, gl, q), s);
-        sh.T[lane][c] = lane < c ? -tt * s : (lane == c ? tt : 0.0);
-        __syncwarp();
+        sh.part[warp][lane] = d.get();
+        if (wide) sh.part[warp][lane].lo = __double_as_longlong(f);
+        row_sync();
+        // warp w adds columns 2 w and 2 w + 1 over the warps
+        Sum128 s = sh.part[lane >> 1][2 * warp + (lane & 1)];
+#pragma unroll
+        for (int o = 2; o < 32; o <<= 1) {
+          Sum128 t;
+          t.lo = __shfl_xor_sync(0xffffffffu, s.lo, o);
+          t.hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
+          if (wide) s.lo = __double_as_longlong(qr_dbl(s.lo) + qr_dbl(t.lo));
+          else s = add128(s, t);
+        }
+        push(nc, s);
       }
     }
-    if (nc >= nref) break;
-    if (worker) {
-      expect(nc);
-      Dot128 d;
-      xk = 0;
-#pragma unroll
-      for (int u = 0; u < RPW; ++u) {
-        const int r = row0 + u;
-        const int2 q = qsplit(a[u]);
-        int2 x;
-        x.x = __shfl_sync(0xffffffffu, q.x, nc);
-        x.y = __shfl_sync(0xffffffffu, q.y, nc);
-        if (lane == u) xk = r > nc ? qjoin(x) : 0;
-        if (r > nc) d.add(x, q);
-        else if (r == nc) sh.prow[lane] = a[u];
-      }
-      sh.part[warp][lane] = d.get();
-      row_sync();
-      // warp w adds columns 2 w and 2 w + 1 over the warps
-      Sum128 s = sh.part[lane >> 1][2 * warp + (lane & 1)];
-#pragma unroll
-      for (int o = 2; o < 32; o <<= 1) {
-        Sum128 t;
-        t.lo = __shfl_xor_sync(0xffffffffu, s.lo, o);
-        t.hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
-        s = add128(s, t);
-      }
-      push(nc, s);
-    }
-  }
+  };
+  if (use_fp64) columns(std::true_type());
+  else columns(std::false_type());
   __syncthreads();
   if (!bad) {
     // R back through the column's scale, reflectors from Q62
@@ -273,7 +332,8 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
 #pragma unroll
       for (int u = 0; u < RPW; ++u) {
         const int r = row0 + u;
-        const double x = r > lane ? qscaled(a[u], 62) : scale2(qscaled(a[u], 0), -scale);
+        const double x = r > lane ? (use_fp64 ? qr_dbl(a[u]) : qscaled(a[u], 62))
+                                  : scale2(use_fp64 ? qr_dbl(a[u]) : qscaled(a[u], 0), -scale);
         tile[lane * (ROWS + 1) + warp * RPW + u] = finite ? x : NAN;
       }
     __syncthreads();
@@ -327,13 +387,13 @@ int qr_launch(gep_handle_t h, const QrArgs& a) {
 bool panel_qr_cluster_takes(int n, int nb) { return nb <= QN && n <= QC * QW * 8; }
 
 // QR of the n x nb panel P (ld ldp): R and the reflectors in P, tau, V at full height (r0 zero rows first, ld
-// ldv) in Va and Vb, T (nb x nb).  GEP_ERR_UNSUPPORTED before any work where the cluster cannot be resident.
+// ldv) in Va and Vb, T (nb x nb).  *wide (device): FP64.  GEP_ERR_UNSUPPORTED before any work where the cluster cannot be resident.
 int panel_qr_cluster(gep_handle_t h, int n, int nb, double* P, int ldp, double* tau, double* Va, double* Vb, int r0,
-                     int ldv, double* T) {
+                     int ldv, double* T, const int* wide) {
   if (!panel_qr_cluster_takes(n, nb)) return GEP_ERR_UNSUPPORTED;
   QrArgs a;
   a.n = n; a.nb = nb; a.ldp = ldp; a.r0 = r0; a.ldv = ldv;
-  a.P = P; a.tau = tau; a.Va = Va; a.Vb = Vb; a.T = T; a.st = h->d_status;
+  a.P = P; a.tau = tau; a.Va = Va; a.Vb = Vb; a.T = T; a.wide = wide; a.st = h->d_status;
   if (n <= QC * QW) return qr_launch<1>(h, a);
   if (n <= QC * QW * 2) return qr_launch<2>(h, a);
   if (n <= QC * QW * 4) return qr_launch<4>(h, a);

@@ -99,3 +99,19 @@ def test_band_large_first_column(gep, b, s):
     d, e, *_ = gep.tridiag_2stage(C, b)
     # the first sweep's reflector acts on rows 1.. only, so T(1:, 1:) is a similarity of C(1:, 1:)
     assert _block_eigenvalues(C, d, e, slice(1, M)) <= 200 * M * EPS
+
+
+@pytest.mark.parametrize("b", [8, 32])
+@pytest.mark.parametrize("M,m1", [(70, 40), (200, 100), (900, 500), (2080, 1500)])
+@pytest.mark.parametrize("s", [0.2, 1e-6, 1e-12, 1e-25])
+def test_panel_rows_of_two_scales(gep, M, m1, b, s):
+    """Rows far below the others keep their accuracy in the reflectors of a panel: LAPACK's, row by row."""
+    import torch
+    D = torch.ones(M, dtype=torch.float64, device="cuda")
+    D[m1:] = s
+    C = D[:, None] * _symmetric(M, M) * D[None, :]
+    Cr = gep.tridiag_2stage(C, b)[4]
+    V = Cr[b:, :b].cpu().tril(-1)
+    ref = torch.geqrf(C[b:, :b].cpu())[0].tril(-1)
+    scale = ref.abs().amax(1, keepdim=True)
+    assert bool(((V - ref).abs() <= 200 * M * EPS * scale).all())
