@@ -151,10 +151,12 @@ __global__ void __launch_bounds__(256) k_larft_merge(int nbt, int n1, const doub
 
 // T (nb x nb, upper) of the block reflector whose Gram matrix is G = V^T V: leaves of 64, then
 // T12 = -T1 (G12 T2) level by level, narrow levels with all their merges in one FP64 launch per
-// product, wide ones (512^3 and up: 250 us on the FP64 units) as products of the engine.  tmp: nb x nb.
+// product, wide ones (512^3 and up: 250 us on the FP64 units) as FP64-accurate products on the tensor cores unless
+// the engine is FP64 (also of the FP32-grade engine: T keeps the accuracy of G).  tmp: nb x nb.
 int larft_rec(gep_handle_t h, int nb, const double* G, int ldg, const double* tau, double* T, int ldt,
               double* tmp, int engine) {
   if (nb <= 0) return GEP_OK;
+  if (engine == GEP_PREC_MIXED_REFINED) engine = GEP_PREC_FP64_EMULATED;
   if (nb > LB) GEP_CHECK(set_matrix(h, nb, nb, 0.0, 0.0, T, ldt));
   k_larft<<<(nb + LB - 1) / LB, 256, 0, h->stream>>>(nb, G, ldg, tau, T, ldt, h->d_status);
   GEP_CHECK(check_launch(h));
