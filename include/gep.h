@@ -88,8 +88,8 @@ typedef struct gep_options {
                        T, and only the n_want wanted columns are back-transformed (Q2, Q1, Eq. 6
                        or Eq. 9 on n_want columns).  Not with GEP_PREC_MIXED_REFINED nor in
                        gep_solve_batched (GEP_ERR_UNSUPPORTED). */
-  int batch_small;  /* gep_solve_batched only: pencils of order <= batch_small (at most 128) are
-                       each solved whole by one CTA (Cholesky, C = L^-1 A L^-T, cyclic Jacobi,
+  int batch_small;  /* gep_solve_batched only: pencils of order <= batch_small (at most 128) may
+                       each be solved whole by one CTA (Cholesky, C = L^-1 A L^-T, cyclic Jacobi,
                        Y = L^-T Q, all FP64), all of them in one persistent launch that takes
                        them from a device work queue, largest order first, where that is
                        the faster route (many pencils, or small ones); 0 = none. */
@@ -244,7 +244,7 @@ int gep_solve_batched(gep_handle_t h, int count, const int* M, double* const* A,
                       double* const* Y, const gep_options* o, const int* precision, int nstreams);
 /* As gep_solve_batched / gep_solve_batched_workspace_size, with one gep_options per pencil
  * (opts[0..count), host memory): pencil i runs its own workflow (reducer, SEP solver,
- * bandwidth, precision, want_vectors; the autotuned route of its size bucket) and takes the
+ * bandwidth, precision, want_vectors; the autotuned route of its size bucket) and may take the
  * one-CTA route when M[i] <= opts[i].batch_small.  timers are ignored and n_want must be 0.
  * Returns -2 (count outside 0..4096), -3 (a null array or a negative order), -4 (opts null
  * or a negative batch_small; -8 in gep_solve_batched_opts), -5 / -9 (nstreams outside

@@ -723,7 +723,7 @@ class Autotuner:
     """Per size bucket, the fastest route of one pencil of the bucket: the FP64-accurate
     product engine (FP64 FMA tiles or split-BF16 tensor-core tiles) and the SEP reduction
     (1-stage tridiagonalisation or full -> band -> tridiagonal); and, for the pencils of
-    order <= 128, whether solving each whole in one CTA of one persistent launch
+    order <= 128, whether letting them be solved whole in one CTA of one persistent launch
     (batch_small) beats the staged workflow on concurrent streams, timed on the batch."""
 
     def __init__(self):
@@ -733,7 +733,7 @@ class Autotuner:
 
     def tune_small(self, As, Bs, nstreams=16, reps=1, precision=None):
         """Times the whole batch both ways (pencils of order <= 128 in one persistent launch of
-        one CTA each, or all of them on the streams, with the tuned routes, or with
+        one CTA each where the library's rule puts them there, or all of them on the streams, with the tuned routes, or with
         `precision` for every pencil when given) and keeps the faster: sets self.batch_small.
         The whole batch is timed because the two routes share the GPU with the larger
         pencils."""
@@ -835,7 +835,8 @@ class BatchedSolver:
     precision / sep for all); capture() records the whole batch into one CUDA graph that
     replay() launches again (inputs are read from the same device buffers each time).
     batch_small > 0 (default 128): pencils of order <= batch_small (at most 128) are solved
-    whole by one CTA each, all in one persistent launch; 0 puts every pencil on the streams.
+    whole by one CTA each, all in one persistent launch, where that is faster than the streams by
+    measured times (many pencils, or tiny ones); 0 puts every pencil on the streams.
 
     capture() refuses a batch whose eager run launched more than GRAPH_KERNEL_LIMIT kernels:
     graphs of about two million kernel nodes or more ended in a host crash inside the graph

@@ -4,6 +4,8 @@
 // enqueues kernels; no step of the method runs on the host.
 #include <string.h>
 
+#include <algorithm>
+
 #include "gep_internal.cuh"
 
 using namespace gep;
@@ -847,12 +849,12 @@ struct BatchPlan {
 
 int small_limit(const gep_options* o) { return o->batch_small < SMALL_MAX ? o->batch_small : SMALL_MAX; }
 
-// Time of one staged solve of order M on its stream, in ms (measured: order 64 0.8, 128 1.2, 256 2.1,
-// 516 6 to 8.5, 1024 17, 2047 43): the balance of the streams.
-double staged_ms(int M) { return 0.4 + 0.006 * M + 9e-6 * (double)M * M; }
-// Time of the one-CTA solver (cyclic Jacobi, about 12 M^3 FP64 operations on one SM): 53 ms at
-// order 128.  Up to two pencils an SM run at once.
-double one_cta_ms(int M) { return 53.0 / (128.0 * 128.0 * 128.0) * M * M * M; }
+// Time of one staged solve of order M on its stream, in ms (measured in a captured graph: order 2 0.09, 4 0.12,
+// 8 0.21, 12 0.28, 16 0.31, 24 0.38, 32 0.42, 40 0.54, 64 0.63, 128 1.2, 256 2.1, 516 6 to 8.5, 1024 17, 2047 43).
+double staged_ms(int M) { return std::min(0.07 + 0.016 * M, 0.28 + 0.0055 * M) + 9e-6 * (double)M * M; }
+// Time of the one-CTA solver (cyclic Jacobi on one SM; measured: order 2 0.02, 4 0.07, 8 0.16, 12 0.31, 16 0.37,
+// 20 0.65, 24 0.92, 28 1.2, 128 53).  Up to two pencils an SM run at once.
+double one_cta_ms(int M) { return (0.008 + (0.0008 + 1.86e-5 * M) * M) * M; }
 
 // Options of pencil i: opts[i] when given, else o with precision[i] (when given).
 gep_options pencil_opts(const gep_options* o, const int* prec, const gep_options* opts, int i) {
@@ -881,18 +883,22 @@ int make_plan(gep_handle_t h, int count, const int* M, const gep_options* o, con
     order[b + 1] = t;
   }
   // Of the pencils that may take the one-CTA solver, those keep it whose time there (all run at
-  // once) is below what the small pencils together cost on the streams: a few pencils of order
-  // 128 (53 ms in one CTA, 1.2 ms staged) go to the streams, many small ones stay.
-  double on_streams = 0.0;
+  // once) is below what the small pencils together take on the streams: their share of a stream, but not
+  // less than the largest of them takes alone.  One of order 8 (0.15 / 0.21 ms), 16 of order 16 on 8 streams
+  // (0.42 / 0.64) and 64 of order 24 (1.1 / 3.3) stay, 4 of order 24 on 8 streams (0.92 / 0.41), one of
+  // order 28 (1.3 / 0.40) and two of order 128 (53 / 1.2) go.
+  double on_streams = 0.0, longest = 0.0;
   int nsm = 0;
   for (int i = 0; i < count; ++i)
     if (small_of[i]) {
       on_streams += staged_ms(M[i]);
+      longest = std::max(longest, staged_ms(M[i]));
       ++nsm;
     }
   const double batches = nsm > 2 * h->sm_count ? (double)nsm / (2 * h->sm_count) : 1.0;
+  const double limit = std::max(longest, on_streams / nstreams);
   for (int i = 0; i < count; ++i)
-    if (small_of[i] && batches * one_cta_ms(M[i]) > on_streams / nstreams) small_of[i] = false;
+    if (small_of[i] && batches * one_cta_ms(M[i]) > limit) small_of[i] = false;
   p->nsmall = 0;
   for (int a = 0; a < count; ++a)
     if (small_of[order[a]]) p->small_order[p->nsmall++] = order[a];
