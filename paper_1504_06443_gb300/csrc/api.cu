@@ -935,7 +935,7 @@ int make_plan(gep_handle_t h, int count, const int* M, const gep_options* o, con
 
 int batched_workspace_size(gep_handle_t h, int count, const int* M, const gep_options* o, const int* prec,
                            const gep_options* opts, int nstreams, size_t* bytes) {
-  static BatchPlan plan;
+  static thread_local BatchPlan plan;  // (large for a stack)
   GEP_CHECK(make_plan(h, count, M, o, prec, opts, nstreams, &plan));
   *bytes = plan.total;
   return GEP_OK;
@@ -950,7 +950,7 @@ int solve_batched(gep_handle_t h, int count, const int* M, double* const* A, dou
     if (oi.n_want != 0) return GEP_ERR_UNSUPPORTED;
   }
   if (count == 0) return GEP_OK;
-  static BatchPlan plan;
+  static thread_local BatchPlan plan;  // (large for a stack)
   GEP_CHECK(make_plan(h, count, M, o, precision, opts, nstreams, &plan));
   if (h->ws == nullptr || h->ws_bytes < plan.total) return GEP_ERR_ALLOC;
   // child handles, streams and events are created once (outside any stream capture)
@@ -1040,7 +1040,7 @@ int gep_batched_info(gep_handle_t h, int* info) {
   if (!info) return -2;
   *info = 0;
   if (!h->d_batch_info || h->batch_count == 0) return GEP_OK;
-  static int st[2 * kMaxBatch];
+  static thread_local int st[2 * kMaxBatch];
   GEP_CUDA(cudaStreamSynchronize(h->stream));
   GEP_CUDA(cudaMemcpy(st, h->d_batch_info, sizeof(int) * 2 * h->batch_count, cudaMemcpyDeviceToHost));
   for (int i = 0; i < h->batch_count; ++i) {

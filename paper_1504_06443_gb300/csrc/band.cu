@@ -1483,17 +1483,14 @@ int panel_factor(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, 
   const int nref = n < b ? n : b;
   double *pin = w.part0, *pout = w.part1, *rin = w.prow0, *rout = w.prow1;
   // one cooperative launch when every CTA of the panel can be resident at once
-  static int per_sm_of[64];
-  static unsigned long long devices = 0;
-  int dev = 0;
-  GEP_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return GEP_ERR_UNSUPPORTED;
-  if (first_use_on_device(devices)) {
+  static DeviceValue resident;
+  int coop_per_sm = 0;
+  GEP_CHECK(resident.get(current_device(), &coop_per_sm, [](int* v) -> int {
     const size_t smax = pqr_coop_smem_bytes(PQ_ROWS, BMAX);
     GEP_CUDA(cudaFuncSetAttribute(k_pqr_coop, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax));
-    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_of[dev], k_pqr_coop, PQ_ROWS, smax));
-  }
-  const int coop_per_sm = per_sm_of[dev];
+    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(v, k_pqr_coop, PQ_ROWS, smax));
+    return GEP_OK;
+  }));
   // fewest rows per CTA whose grid is resident at once and fits the partial-sum buffers
   // (a test may force 64, 128 or 256 rows, or the per-column kernel with -1)
   const long long cap = (long long)coop_per_sm * h->sm_count;
@@ -1539,14 +1536,13 @@ int panel_factor(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, 
 template <int RPW>
 int panel_qr_launch(gep_handle_t h, const PanelArgs& a, long long part_elems) {
   const int G = (a.n + PQW * RPW - 1) / (PQW * RPW);
-  static int per_sm_of[64];
-  static unsigned long long devices = 0;
-  int dev = 0;
-  GEP_CUDA(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return GEP_ERR_UNSUPPORTED;
-  if (first_use_on_device(devices))
-    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_of[dev], k_panel_qr<RPW>, 32 * (PQW + 1), 0));
-  if ((long long)G > (long long)per_sm_of[dev] * h->sm_count || 2LL * G * PQN > part_elems) return GEP_ERR_UNSUPPORTED;
+  static DeviceValue resident;
+  int per_sm = 0;
+  GEP_CHECK(resident.get(current_device(), &per_sm, [](int* v) -> int {
+    GEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(v, k_panel_qr<RPW>, 32 * (PQW + 1), 0));
+    return GEP_OK;
+  }));
+  if ((long long)G > (long long)per_sm * h->sm_count || 2LL * G * PQN > part_elems) return GEP_ERR_UNSUPPORTED;
   GEP_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(int), h->stream));
   PanelArgs aa = a;
   void* args[] = {&aa};
@@ -1749,12 +1745,13 @@ int band_to_tridiag(gep_handle_t h, int M, const double* C, int ldc, int b, doub
     // kernels are launched and one returns at once, about 5 us), other widths the general one
     const bool fixed = b == 32 || b == 64;
     unsigned long long* mx = reinterpret_cast<unsigned long long*>(prog + rr((size_t)M) * 2);
-    static unsigned long long attr_devices = 0;
-    if (first_use_on_device(attr_devices)) {
+    static DeviceOnce attributes;
+    GEP_CHECK(once_per_device(attributes, []() -> int {
       GEP_CUDA(cudaFuncSetAttribute(k_bulge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bulge_smem_bytes()));
       GEP_CUDA(cudaFuncSetAttribute(k_bulge_ws<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BulgeShared<32>)));
       GEP_CUDA(cudaFuncSetAttribute(k_bulge_ws<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BulgeShared<64>)));
-    }
+      return GEP_OK;
+    }));
     BulgeArgs a;
     a.M = M; a.b = b; a.ldab = ldab; a.Q = Q; a.AB = AB; a.prog = prog; a.q2 = q2; a.st = h->d_status;
     a.mx = fixed ? mx : nullptr;
@@ -1809,11 +1806,12 @@ size_t all_tiles_offset(int Q, int J, int TQ) {
 }
 
 int set_tile_build_attr() {
-  static unsigned long long attr_devices = 0;
-  if (first_use_on_device(attr_devices))
+  static DeviceOnce attributes;
+  return once_per_device(attributes, []() -> int {
     GEP_CUDA(cudaFuncSetAttribute(k_q2_tile_build, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)q2_tile_smem_bytes(BMAX)));
-  return GEP_OK;
+    return GEP_OK;
+  });
 }
 
 }  // namespace
@@ -2024,10 +2022,11 @@ int apply_q2(gep_handle_t h, int M, int b, const double* q2, double* Z, int ldz,
     return GEP_OK;
   }
   size_t smem = q2_smem_bytes(b);
-  static unsigned long long attr_devices = 0;
-  if (first_use_on_device(attr_devices))
-    GEP_CUDA(cudaFuncSetAttribute(k_q2_apply, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)q2_smem_bytes(BMAX)));
+  static DeviceOnce attributes;
+  GEP_CHECK(once_per_device(attributes, []() -> int {
+    GEP_CUDA(cudaFuncSetAttribute(k_q2_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)q2_smem_bytes(BMAX)));
+    return GEP_OK;
+  }));
   const int slabs = (ncol + Q2_COLS - 1) / Q2_COLS;
   for (int wt = 0; wt <= 2 * Q; ++wt) {
     int kmin = wt - Q > 0 ? wt - Q : 0, kmax = wt / 2;

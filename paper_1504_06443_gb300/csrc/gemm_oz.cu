@@ -658,15 +658,20 @@ int split_rows(gep_handle_t h, int R, int K, int Kpad, const double* X, long lon
   return check_launch(h);
 }
 
+int split_cols_attr() {
+  static DeviceOnce attributes;
+  return once_per_device(attributes, []() -> int {
+    GEP_CUDA(cudaFuncSetAttribute(k_split_cols<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 9 * 8));
+    GEP_CUDA(cudaFuncSetAttribute(k_split_cols<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 33 * 8));
+    return GEP_OK;
+  });
+}
+
 // Exponent pass and split of an operand with strided K.
 int split_cols(gep_handle_t h, int R, int K, int Kpad, const double* X, long long sr, long long sk, int* e, int S,
                int xbit, unsigned short* out) {
   if (sr == 1 && Kpad <= FUSE_K) {
-    static unsigned long long devices = 0;
-    if (first_use_on_device(devices)) {
-      GEP_CUDA(cudaFuncSetAttribute(k_split_cols<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 9 * 8));
-      GEP_CUDA(cudaFuncSetAttribute(k_split_cols<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 33 * 8));
-    }
+    GEP_CHECK(split_cols_attr());
     // 8 rows a CTA while that fills the GPU at most a few times over (a row segment is 64 bytes),
     // else 32
     if (R <= 32 * h->sm_count)
@@ -685,14 +690,16 @@ int split_cols(gep_handle_t h, int R, int K, int Kpad, const double* X, long lon
 // Product-kernel launch for one K panel (kc deep, planes padded to a.kpad): dynamic shared
 // memory attribute, optional per-launch timing, template dispatch on the plane/level counts.
 int oz_launch(gep_handle_t h, const CUtensorMap& mA, const CUtensorMap& mB, const OzArgs& a, int kc, bool skinny = false) {
-  static unsigned long long attr_devices = 0;
-  if (first_use_on_device(attr_devices)) {
-    cudaFuncSetAttribute(k_oz_gemm<8, 9>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS));
-    cudaFuncSetAttribute(k_oz_gemm<3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS));
-    cudaFuncSetAttribute(k_oz_gemm<0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS));
-    cudaFuncSetAttribute(k_oz_gemm<8, 9, TNS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS, TNS));
-    cudaFuncSetAttribute(k_oz_gemm<3, 4, TNS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes_for(MAXS, TNS));
-  }
+  static DeviceOnce attributes;
+  GEP_CHECK(once_per_device(attributes, []() -> int {
+    constexpr auto limit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    GEP_CUDA(cudaFuncSetAttribute(k_oz_gemm<8, 9>, limit, (int)smem_bytes_for(MAXS)));
+    GEP_CUDA(cudaFuncSetAttribute(k_oz_gemm<3, 4>, limit, (int)smem_bytes_for(MAXS)));
+    GEP_CUDA(cudaFuncSetAttribute(k_oz_gemm<0, 0>, limit, (int)smem_bytes_for(MAXS)));
+    GEP_CUDA(cudaFuncSetAttribute((k_oz_gemm<8, 9, TNS>), limit, (int)smem_bytes_for(MAXS, TNS)));
+    GEP_CUDA(cudaFuncSetAttribute((k_oz_gemm<3, 4, TNS>), limit, (int)smem_bytes_for(MAXS, TNS)));
+    return GEP_OK;
+  }));
   const int S = a.S, levels = a.lmax;
   dim3 grid(a.ntiles < h->sm_count ? a.ntiles : h->sm_count);  // persistent CTAs
   int slot = -1;
@@ -876,9 +883,7 @@ int dgemm_oz_batched(gep_handle_t h, int m, int n, int k, const double* A, int l
       unsigned short* Bs = As + align256((size_t)2 * S * m * nz * kc) / 2;
       int* ea = (int*)(Bs + align256((size_t)2 * S * n * nz * kc) / 2);
       int* eb = ea + (size_t)m * nz;
-      static unsigned long long devices = 0;
-      if (first_use_on_device(devices))
-        GEP_CUDA(cudaFuncSetAttribute(k_split_cols<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, FUSE_K * 33 * 8));
+      GEP_CHECK(split_cols_attr());
       k_split_cols<32><<<dim3((m + 31) / 32, nz), 256, (size_t)kc * 33 * 8, h->stream>>>(
           m, kc, kc, A + z0 * sa + (size_t)kb * lda, lda, sa, ea, S, 1, As, h->d_status);
       GEP_CHECK(check_launch(h));

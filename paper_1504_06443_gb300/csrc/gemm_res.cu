@@ -673,9 +673,11 @@ int dgemm_res(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, 
   if (overlap(A, lda, TA ? k : m, TA ? m : k, C, ldc, m, n) ||
       (!in_place && overlap(B, ldb, TB ? n : k, TB ? k : n, C, ldc, m, n)))
     return GEP_ERR_UNSUPPORTED;
-  static unsigned long long attr_devices = 0;
-  if (first_use_on_device(attr_devices))
+  static DeviceOnce attributes;
+  GEP_CHECK(once_per_device(attributes, []() -> int {
     GEP_CUDA(cudaFuncSetAttribute(k_res_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RSMEM));
+    return GEP_OK;
+  }));
   const int nbw = min(pl.nb, n), ldr = (nbw + RN - 1) / RN * RN;
   char* p = h->eng_ws;
   unsigned short* As = (unsigned short*)p;

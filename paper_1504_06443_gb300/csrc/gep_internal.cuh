@@ -4,6 +4,7 @@
 #include <stdint.h>
 #include <stdio.h>
 
+#include "device_once.cuh"
 #include "gep.h"
 
 #define GEP_IX(i, j, ld) ((size_t)(i) + (size_t)(j) * (size_t)(ld))
@@ -77,47 +78,6 @@ struct Arena {
 // Counting-only arena: used by workspace queries to size the same carving.
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Kernel attributes (the dynamic shared-memory limit) belong to a device context, so
-// one-time settings are made once per device: `mask` (one per call site) records the
-// devices already done.  Returns true on the first call for the current device.
-inline bool first_use_on_device(unsigned long long& mask) {
-  int d = 0;
-  if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return true;
-  const unsigned long long bit = 1ull << d;
-  if (mask & bit) return false;
-  mask |= bit;
-  return true;
-}
-
-// Whether a cluster of this size of the kernel can be resident at all (asked once per device: `known` and
-// `yes` are bit masks of devices, one pair per call site).
-inline bool cluster_fits(const void* kernel, int cluster, int threads, size_t smem, unsigned long long& known,
-                         unsigned long long& yes) {
-  int d = 0;
-  if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return false;
-  const unsigned long long bit = 1ull << d;
-  if (!(known & bit)) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cluster);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cluster;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
-      cudaGetLastError();
-      n = 0;
-    }
-    if (n > 0) yes |= bit;
-    known |= bit;
-  }
-  return (yes & bit) != 0;
-}
-
 inline int check_launch(gep_handle_t h) {
   h->launches++;
   cudaError_t e = cudaGetLastError();
@@ -143,6 +103,42 @@ inline int check_launch(gep_handle_t h) {
       return GEP_ERR_CUDA;                                                           \
     }                                                                                \
   } while (0)
+
+// Kernel attributes (the dynamic shared-memory limit) and what can be resident belong to a device context: one
+// static of these per call site.
+inline int current_device() {
+  int d = -1;
+  return cudaGetDevice(&d) == cudaSuccess ? d : -1;
+}
+template <class F>
+int once_per_device(DeviceOnce& once, F&& f) {
+  return once.run(current_device(), f);
+}
+
+// Whether a cluster of this size of the kernel can be resident at all.
+inline bool cluster_fits(DeviceValue& known, const void* kernel, int cluster, int threads, size_t smem) {
+  int fits = 0;
+  known.get(current_device(), &fits, [&](int* v) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cluster);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    *v = n > 0;
+    return 0;
+  });
+  return fits != 0;
+}
 
 constexpr int SPLITK_TILES = 2048;          // output tiles of a product with a split depth
 constexpr int SPLITK_DOUBLES = 1 << 18;     // doubles of their partial tiles

@@ -370,13 +370,14 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
 template <int RPW>
 int qr_launch(gep_handle_t h, const QrArgs& a) {
   constexpr int smem = (int)((sizeof(QrShared) + 15) / 16 * 16 + sizeof(double) * QN * (QW * RPW + 1));
-  static unsigned long long devices = 0;
-  if (first_use_on_device(devices)) {
+  static DeviceOnce attributes;
+  GEP_CHECK(once_per_device(attributes, []() -> int {
     GEP_CUDA(cudaFuncSetAttribute(k_panel_qr_cluster<RPW>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     GEP_CUDA(cudaFuncSetAttribute(k_panel_qr_cluster<RPW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  }
-  static unsigned long long known = 0, yes = 0;
-  if (!cluster_fits((const void*)k_panel_qr_cluster<RPW>, QC, QTHREADS, smem, known, yes)) return GEP_ERR_UNSUPPORTED;
+    return GEP_OK;
+  }));
+  static DeviceValue fits;
+  if (!cluster_fits(fits, (const void*)k_panel_qr_cluster<RPW>, QC, QTHREADS, smem)) return GEP_ERR_UNSUPPORTED;
   k_panel_qr_cluster<RPW><<<QC, QTHREADS, smem, h->stream>>>(a);
   return check_launch(h);
 }

@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <math.h>
 
+#include <atomic>
+
 #include "gep_internal.cuh"
 
 namespace gep {
@@ -237,15 +239,15 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
+  static std::atomic<EncodeTiledFn> fn{nullptr};
+  if (!fn.load()) {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = (EncodeTiledFn)p;
+      fn.store((EncodeTiledFn)p);
   }
-  return fn;
+  return fn.load();
 }
 
 }  // namespace

@@ -228,12 +228,12 @@ __global__ void __launch_bounds__(256) k_inv_diag(int M, const double* L, int ld
 constexpr size_t kSmemDiag = (size_t)NB * NB * sizeof(double) + NB * sizeof(double);
 
 int set_smem_attr() {
-  static unsigned long long devices = 0;
-  if (first_use_on_device(devices)) {
-    cudaFuncSetAttribute(k_potrf_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PotrfShared));
-    cudaFuncSetAttribute(k_inv_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDiag);
-  }
-  return GEP_OK;
+  static DeviceOnce attributes;
+  return once_per_device(attributes, []() -> int {
+    GEP_CUDA(cudaFuncSetAttribute(k_potrf_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PotrfShared)));
+    GEP_CUDA(cudaFuncSetAttribute(k_inv_diag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemDiag));
+    return GEP_OK;
+  });
 }
 
 }  // namespace
@@ -257,7 +257,7 @@ int inv_merge(gep_handle_t h, int n, const double* L21, int ldl, double* X, doub
 int tri_inv_diag_blocks(gep_handle_t h, int M, const double* L, int ldl, double* invD, int nb) {
   if (nb != TRI_NB) return GEP_ERR_UNSUPPORTED;
   if (M <= 0) return GEP_OK;
-  set_smem_attr();
+  GEP_CHECK(set_smem_attr());
   int nblk = (M + NB - 1) / NB;
   k_inv_diag<<<nblk, 256, kSmemDiag, h->stream>>>(M, L, ldl, invD, h->d_status);
   GEP_CHECK(check_launch(h));
@@ -377,7 +377,7 @@ int trsm_llt(gep_handle_t h, int M, int n, const double* L, int ldl, const doubl
 // follows invD in the caller's workspace.
 int cholesky(gep_handle_t h, int M, double* B, int ldb, double* invD, int engine) {
   if (M <= 0) return GEP_OK;
-  set_smem_attr();
+  GEP_CHECK(set_smem_attr());
   int nblk = (M + TRI_NB - 1) / TRI_NB;
   double* tmp = invD + (size_t)nblk * TRI_NB * TRI_NB;
   return potrf_rec(h, 0, M, B, ldb, invD, tmp, engine);

@@ -861,9 +861,11 @@ int trd_panel_launch(gep_handle_t h, TrdArgs a) {
   a.slots = slots;
   const size_t smem = trd_smem_bytes<T, TS>(a.nt, a.rpc, slots);
   if (smem > cap) return GEP_ERR_UNSUPPORTED;
-  static unsigned long long devices = 0;
-  if (first_use_on_device(devices))
+  static DeviceOnce attributes;
+  GEP_CHECK(once_per_device(attributes, [&]() -> int {
     GEP_CUDA(cudaFuncSetAttribute(k_trd_panel<T, TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap));
+    return GEP_OK;
+  }));
   GEP_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(int), h->stream));
   void* args[] = {&a};
   GEP_CUDA(cudaLaunchCooperativeKernel((void*)k_trd_panel<T, TS>, dim3(G), dim3(TRD_T), args, smem, h->stream));

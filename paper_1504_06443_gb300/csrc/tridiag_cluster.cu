@@ -373,11 +373,13 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
 
 template <int RPW, int NT>
 int trc_launch(gep_handle_t h, const TrcArgs& a, int cl) {
-  static unsigned long long devices = 0;
-  if (first_use_on_device(devices))
+  static DeviceOnce attributes;
+  GEP_CHECK(once_per_device(attributes, []() -> int {
     GEP_CUDA(cudaFuncSetAttribute((const void*)k_trd_cluster<RPW, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  static unsigned long long known = 0, yes = 0;  // (one cluster size per instance but the smallest)
-  if (!cluster_fits((const void*)k_trd_cluster<RPW, NT>, NT == 2 ? 4 : cl, TRC_THREADS, 0, known, yes))
+    return GEP_OK;
+  }));
+  static DeviceValue fits;  // (one cluster size per instance but the smallest)
+  if (!cluster_fits(fits, (const void*)k_trd_cluster<RPW, NT>, NT == 2 ? 4 : cl, TRC_THREADS, 0))
     return GEP_ERR_UNSUPPORTED;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cl);
