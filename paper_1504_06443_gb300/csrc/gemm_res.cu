@@ -637,9 +637,14 @@ bool overlap(const double* X, int ldx, int rx, int cx, const double* C, int ldc,
 }  // namespace
 
 // The faster of the two forms of a product on the tensor cores, by their measured costs (us):
-//   digit planes:  40 for launches and splits, 4 + 0.05 k per wave of 128 x 64 tiles, the operands' digits;
-//   residues:      60, 2 + 0.0053 k per wave of (256 x 256 tile, modulus) on the pairs of CTAs, 9 ps an
-//                  operand element (its 40 bytes) and 9 ps an output and K panel (16 bytes in, C, the CRT).
+//   digit planes:  10 and 30 a K panel for launches and splits, 4 a panel + 0.05 k per wave of 128 x 64
+//                  tiles, the operands' digits;
+//   residues:      15, 10 a K panel and 35 for each of its column blocks, 0.0051 k per wave of (256 x 256 tile,
+//                  modulus) on the pairs of CTAs, 9 ps an operand element (its 40 bytes) and 13 ps an output and
+//                  K panel (16 bytes in, C, the CRT).
+// Both by the K panels and column blocks that the scratch allows.  Fitted to 40 shapes and scratches, within a tenth:
+// 1024 x 1024 x 4096 with 64 / 128 / 256 / 512 MB: digits 339 / 323 / 282 us, residues 615 / 393 / 279 / 225;
+// 4096^3 with 256 MB 3414 / 2883, 3000 x 3000 x 9000 with 128 / 256 MB 4391 / 6017 and 4290 / 3634.
 // Digits / residues: 512^3 76 / 74, 1024 x 1024 x 512 77 / 97, 4096 x 256 x 1024 133 / 146,
 // 4096 x 4096 x 512 476 / 471, 1024^3 120 / 120, 8192 x 512 x 1024 322 / 260, 2048^3 510 / 328, 256 x 256 x 4096
 // 267 / 110, 4096^3 3130 / 1657, lower triangle 8192 x 8192 x 2048 3674 / 2026.
@@ -650,9 +655,15 @@ bool res_product_wins(gep_handle_t h, char uplo, int m, int n, int k) {
   const double digit_tiles = half * ((m + 127) / 128) * ((n + 63) / 64);
   double res_tiles = (double)((m + RM - 1) / RM) * ((n + RN - 1) / RN);
   if (lower) res_tiles = 0.5 * (res_tiles + (n + RN - 1) / RN);
-  const double digits = 40.0 + ceil(digit_tiles / h->sm_count) * (4.0 + 0.05 * k) + 5e-6 * op;
-  const double residues = 60.0 + ceil(NMOD * res_tiles / (h->sm_count / 2)) * (2.0 + 0.0053 * k) +
-                          9e-6 * (op + mn * ((k + RKP_MAX - 1) / RKP_MAX));
+  const ResPlan pl = res_plan(m, n, k, h->eng_ws ? h->eng_bytes : 0);
+  if (pl.kp == 0) return false;
+  const double panels = (k + pl.kp - 1) / pl.kp, blocks = (n + pl.nb - 1) / pl.nb;
+  const double digit_k = fmin(RKP_MAX, (h->eng_bytes - 1024.0) / (16.0 * ((double)m + n))), digit_panels = ceil(k / digit_k);
+  const double digits = 10.0 + 30.0 * digit_panels +
+                        ceil(digit_tiles / h->sm_count) * (4.0 * digit_panels + 0.05 * k) + 5e-6 * op;
+  const double residues = 15.0 + panels * (10.0 + 35.0 * blocks) +
+                          blocks * ceil(NMOD * res_tiles / blocks / (h->sm_count / 2)) * 0.0051 * k + 9e-6 * op +
+                          13e-6 * mn * panels;
   return residues < 0.97 * digits;
 }
 
