@@ -289,6 +289,13 @@ int gep_set_panel_qr(gep_handle_t h, int rows);
  * path), -1 restores the default.  Returns -2 for min_order < -1. */
 int gep_set_band_group(gep_handle_t h, int min_order);
 
+/* Test hook for routes that are rarely the chosen ones.  clusters = 0 makes the kernels that need a
+ * thread-block cluster decline (tridiagonalisation of order <= 512, panel QR of up to 2048 rows), as on
+ * a device where none fits; one_cta = 1 puts every pencil of order <= batch_small of a batch on the
+ * one-CTA route, also where the streams are faster (set it before the workspace query).  (1, 0)
+ * restores the defaults.  Returns -2 / -3 for other values. */
+int gep_set_routes(gep_handle_t h, int clusters, int one_cta);
+
 /* Per-stage times (ms) of the last gep_solve with o->timers = 1:
  * t[0] Cholesky (R1), t[1] reduction (R2), t[2] tridiagonalisation (TRD/BAND),
  * t[3] tridiagonal eigensolver (D&C), t[4] Householder back-transform (BACK),

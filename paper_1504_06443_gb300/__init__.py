@@ -116,6 +116,7 @@ def load():
             "gep_solve_batched_opts": (_I, [_P, _I, _P, _P, _P, _P, _P, ctypes.POINTER(GepOptions), _I]),
             "gep_batched_info": (_I, [_P, ctypes.POINTER(_I)]),
             "gep_set_band_group": (_I, [_P, _I]),
+            "gep_set_routes": (_I, [_P, _I, _I]),
             "gep_dgemm": (_I, [_P, ctypes.c_char, ctypes.c_char, ctypes.c_char, _I, _I, _I, _D, _P, _I, _P, _I,
                                _D, _P, _I, _I]),
         }
@@ -272,6 +273,11 @@ class Handle:
         """Test hook: the trailing order from which the full -> band reduction groups panels in
         fours (0: always, -1: the library default)."""
         _check(self.lib.gep_set_band_group(self.h, int(min_order)), "gep_set_band_group")
+
+    def set_routes(self, clusters=True, one_cta=False):
+        """Test hook: clusters=False makes the cluster kernels decline (their fallbacks run), one_cta=True
+        puts every small enough pencil of a batch on the one-CTA route."""
+        _check(self.lib.gep_set_routes(self.h, int(clusters), int(one_cta)), "gep_set_routes")
 
     def stage_times(self):
         t = (_D * 7)()

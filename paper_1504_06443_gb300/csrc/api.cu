@@ -354,6 +354,15 @@ int gep_set_band_group(gep_handle_t h, int min_order) {
   return GEP_OK;
 }
 
+int gep_set_routes(gep_handle_t h, int clusters, int one_cta) {
+  if (!handle_ok(h)) return GEP_ERR_HANDLE;
+  if (clusters != 0 && clusters != 1) return -2;
+  if (one_cta != 0 && one_cta != 1) return -3;
+  h->no_clusters = !clusters;
+  h->force_one_cta = one_cta;
+  return GEP_OK;
+}
+
 long long gep_launch_count(gep_handle_t h, int reset) {
   if (!handle_ok(h)) return -1;
   long long n = h->launches;
@@ -898,7 +907,7 @@ int make_plan(gep_handle_t h, int count, const int* M, const gep_options* o, con
   const double batches = nsm > 2 * h->sm_count ? (double)nsm / (2 * h->sm_count) : 1.0;
   const double limit = std::max(longest, on_streams / nstreams);
   for (int i = 0; i < count; ++i)
-    if (small_of[i] && batches * one_cta_ms(M[i]) > limit) small_of[i] = false;
+    if (small_of[i] && !h->force_one_cta && batches * one_cta_ms(M[i]) > limit) small_of[i] = false;
   p->nsmall = 0;
   for (int a = 0; a < count; ++a)
     if (small_of[order[a]]) p->small_order[p->nsmall++] = order[a];

@@ -1552,7 +1552,7 @@ int panel_qr_launch(gep_handle_t h, const PanelArgs& a, long long part_elems) {
 
 int panel_qr(gep_handle_t h, int n, int b, double* P, int ldp, double* tau, const BandWs& w, double* Va, double* Vb,
              int r0, int ldv) {
-  if (panel_qr_cluster_takes(n, b)) {
+  if (!h->no_clusters && panel_qr_cluster_takes(n, b)) {
     const int rc = panel_qr_cluster(h, n, b, P, ldp, tau, Va, Vb, r0, ldv, w.T, w.wide);
     if (rc != GEP_ERR_UNSUPPORTED) return rc;
   }

@@ -28,6 +28,8 @@ struct gep_handle_s {
   // one-launch-per-column kernel, 0 for the automatic choice
   int pqr_rows = 0;
   int band_group_min = -1;  // trailing order from which S1b takes panels in groups of four (-1: default)
+  // test hooks: the cluster kernels decline, and every pencil that may takes the one-CTA solver
+  int no_clusters = 0, force_one_cta = 0;
   int magic = 0x6e70;
   cudaEvent_t ev[8] = {};
   cudaEvent_t ev_band = nullptr;  // between full->band and bulge chasing (two-stage, timers on)

@@ -932,7 +932,7 @@ int tridiag_1stage(gep_handle_t h, int M, double* C, int ldc, double* d, double*
   const bool single = engine == GEP_PREC_MIXED_REFINED;
   float* S1 = reinterpret_cast<float*>(t.S2);
   for (int j0 = 0; j0 < M; j0 += NBT) {
-    if (tridiag_cluster_takes(M - j0)) {
+    if (!h->no_clusters && tridiag_cluster_takes(M - j0)) {
       const int rc = tridiag_cluster(h, M - j0, C + GEP_IX(j0, j0, ldc), ldc, d + j0, e + j0, tau + j0);
       if (rc != GEP_ERR_UNSUPPORTED) return rc;
     }
