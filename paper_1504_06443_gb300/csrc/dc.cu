@@ -111,6 +111,8 @@ __device__ int block_scan(int v, int* sc, int* total) {
   return x - v + (w ? sc[w - 1] : 0);
 }
 
+__device__ __forceinline__ double pow2(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
+
 // Order-preserving integer key of a finite double (compared on the integer pipe).
 __device__ __forceinline__ long long order_key(double x) {
   const long long b = __double_as_longlong(x);
@@ -148,8 +150,7 @@ __global__ void __launch_bounds__(32) k_leaf(int M, const double* __restrict__ d
   for (int o = 16; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   // 2^(1023 - mx) and its inverse, kept inside the normal range
   const int sh = max(-1000, min(1000, 1023 - mx));
-  const double sc = __longlong_as_double((long long)(1023 + sh) << 52);
-  const double isc = __longlong_as_double((long long)(1023 - sh) << 52);
+  const double sc = pow2(sh), isc = pow2(-sh);
   if (lane < LEAF) {
     dl[lane] = dv * sc;
     el[lane] = ev * sc;
@@ -283,8 +284,8 @@ __global__ void __launch_bounds__(1024) k_prep(int M, int half, const double* __
   const int n = hi - lo, n1 = half;
   const double beta = e[mid - 1];
   const double sg = beta < 0.0 ? -1.0 : 1.0;
-  const double rho = 2.0 * fabs(beta);
-  double zmax = 0.0, dmax = 0.0;
+  double rho = 2.0 * fabs(beta);
+  double zmax = 0.0, dmax = 0.0, dall = 0.0;  // dmax: of the values that the rank-one term reaches
   for (int t = tid; t < n; t += nt) {
     double z = (t < n1) ? Z[GEP_IX(mid - 1, lo + t, ldz)] : sg * Z[GEP_IX(mid, lo + t, ldz)];
     z *= 0.70710678118654752440;
@@ -292,11 +293,22 @@ __global__ void __launch_bounds__(1024) k_prep(int M, int half, const double* __
     double dv = D[lo + t];
     w.dv[t] = dv;
     zmax = fmax(zmax, fabs(z));
-    dmax = fmax(dmax, fabs(dv));
+    dall = fmax(dall, fabs(dv));
+    if (z != 0.0) dmax = fmax(dmax, fabs(dv));
   }
   zmax = block_max(zmax, red);
   dmax = block_max(dmax, red);
-  const double tol = 8.0 * EPS * 2.0 * fmax(dmax, zmax);
+  dall = block_max(dall, red);
+  // The merge runs on numbers of order one: scaled by the power of two that brings those the rank-one term
+  // reaches into [1, 2) (values of a decoupled block of another scale only pass through).
+  auto field = [](double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); };
+  const int top = field(fmax(dmax, rho));
+  const int sh = max(-1000, min(top ? 1023 - top : 0, min(1000, 2000 - field(dall))));
+  const double f = pow2(sh);
+  rho *= f;
+  for (int t = tid; t < n; t += nt) w.dv[t] *= f;
+  __syncthreads();
+  const double tol = 8.0 * EPS * 2.0 * fmax(dmax * f, rho * zmax);
   // merge the two ascending runs [0, n1) and [n1, n), the first run's entry first on ties
   for (int x = tid; x < n; x += nt) {
     const double v = w.dv[x];
@@ -403,6 +415,7 @@ __global__ void __launch_bounds__(1024) k_prep(int M, int half, const double* __
     w.cnt[0] = k;
     w.cnt[1] = n - k;
     w.cnt[2] = snr;
+    w.cnt[3] = sh;
     w.rho[0] = rho;
   }
 }
@@ -534,6 +547,7 @@ __global__ void __launch_bounds__(256) k_zhat_order(int M, int width, double* __
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= n) return;
   const int k = w.cnt[0], nd = w.cnt[1];
+  const double isc = pow2(-w.cnt[3]);
   if (i >= k) {
     if (lane == 0) {  // after the roots that are not above it (roots first on ties)
       const int m = i - k;
@@ -544,7 +558,7 @@ __global__ void __launch_bounds__(256) k_zhat_order(int M, int width, double* __
         if (w.lam[c] <= v) a = c + 1; else b = c;
       }
       w.posd[m] = m + a;
-      D[lo + m + a] = v;
+      D[lo + m + a] = v * isc;
     }
     return;
   }
@@ -584,7 +598,7 @@ __global__ void __launch_bounds__(256) k_zhat_order(int M, int width, double* __
       if (w.dfv[q] < v) a = q + 1; else b = q;
     }
     w.posr[i] = i + a;
-    D[lo + i + a] = v;
+    D[lo + i + a] = v * isc;
   }
 }
 
