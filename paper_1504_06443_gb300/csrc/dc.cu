@@ -273,18 +273,19 @@ __device__ void sort_list(int c, double* v, double* z, int* ix, double* tv, doub
 // parallel (all set-ups of order 4096: 13.2 -> 0.23 ms).
 __global__ void __launch_bounds__(1024) k_prep(int M, int half, const double* __restrict__ e,
                                                const double* __restrict__ D, const double* __restrict__ Z,
-                                               int ldz, DcWs ws, const int* st) {
+                                               int ldz, DcWs ws, int* st) {
   __shared__ double red[32];
   __shared__ int sc[33];
   __shared__ int snr;
-  if (status_bad(st)) return;
+  if (__syncthreads_or(status_bad(st))) return;  // (another merge of this launch may be storing it)
   const int lo = blockIdx.x * 2 * half, mid = lo + half, hi = min(M, mid + half);
   const DcWs w = ws.at(lo, blockIdx.x);
   const int tid = threadIdx.x, nt = blockDim.x;
   const int n = hi - lo, n1 = half;
   const double beta = e[mid - 1];
   const double sg = beta < 0.0 ? -1.0 : 1.0;
-  double rho = 2.0 * fabs(beta);
+  auto field = [](double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); };
+  int bad = 0;
   double zmax = 0.0, dmax = 0.0, dall = 0.0;  // dmax: of the values that the rank-one term reaches
   for (int t = tid; t < n; t += nt) {
     double z = (t < n1) ? Z[GEP_IX(mid - 1, lo + t, ldz)] : sg * Z[GEP_IX(mid, lo + t, ldz)];
@@ -292,20 +293,25 @@ __global__ void __launch_bounds__(1024) k_prep(int M, int half, const double* __
     w.zs[t] = z;
     double dv = D[lo + t];
     w.dv[t] = dv;
+    bad |= max(field(z), field(dv)) == 0x7FF;
     zmax = fmax(zmax, fabs(z));
     dall = fmax(dall, fabs(dv));
     if (z != 0.0) dmax = fmax(dmax, fabs(dv));
+  }
+  // The orders below are indices into this merge's arrays: what is not a number has none.
+  if (__syncthreads_or(bad)) {
+    if (tid == 0) atomicCAS(st, 0, M + lo + 1);
+    return;
   }
   zmax = block_max(zmax, red);
   dmax = block_max(dmax, red);
   dall = block_max(dall, red);
   // The merge runs on numbers of order one: scaled by the power of two that brings those the rank-one term
   // reaches into [1, 2) (values of a decoupled block of another scale only pass through).
-  auto field = [](double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); };
-  const int top = field(fmax(dmax, rho));
+  const int top = field(fmax(dmax, fabs(beta)));
   const int sh = max(-1000, min(top ? 1023 - top : 0, min(1000, 2000 - field(dall))));
   const double f = pow2(sh);
-  rho *= f;
+  const double rho = 2.0 * (fabs(beta) * f);
   for (int t = tid; t < n; t += nt) w.dv[t] *= f;
   __syncthreads();
   const double tol = 8.0 * EPS * 2.0 * fmax(dmax * f, rho * zmax);
@@ -732,7 +738,7 @@ int tridiag_eig_dc(gep_handle_t h, int M, const double* d, const double* e, doub
     const int nm = (M - half + width - 1) / width;  // merges: those whose second half is not empty
     const int tail = nm * width;                    // rows from here on have no partner on this level
     const int nmax = M < width ? M : width;
-    k_prep<<<nm, nmax >= 1024 ? 1024 : (nmax + 31) / 32 * 32, 0, s>>>(M, half, e, w.D, cur, ldcur, w, stc);
+    k_prep<<<nm, nmax >= 1024 ? 1024 : (nmax + 31) / 32 * 32, 0, s>>>(M, half, e, w.D, cur, ldcur, w, h->d_status);
     GEP_CHECK(check_launch(h));
     k_secular<<<dim3((nmax + 7) / 8, nm), 256, 0, s>>>(width, w, stc);
     GEP_CHECK(check_launch(h));

@@ -140,3 +140,13 @@ def test_pushes_have_landed_before_a_cta_leaves(source, kernel):
     assert barriers[-2] < drain < barriers[-1]
     assert not re.search(r"\breturn\s*;", body[:barriers[-1]])
     assert "DRAIN" in open(os.path.join(CSRC, "cluster.cuh")).read()
+
+
+def test_merges_order_numbers_only():
+    """The orders that divide and conquer forms are used as indices, which comparisons with a NaN would leave unset: a
+    merge looks for numbers that are not finite before it forms any."""
+    text = open(os.path.join(CSRC, "dc.cu")).read()
+    body = {n: b for n, b, _ in functions(text)}["k_prep"]
+    check = body.index("__syncthreads_or(bad)")
+    assert "0x7FF" in body[:check] and "atomicCAS(st" in body[check:check + 120]
+    assert check < body.index("w.perm[")

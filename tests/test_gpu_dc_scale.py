@@ -64,3 +64,32 @@ def test_blocks(gep, m1, m2, p):
         ref = torch.linalg.eigvalsh(T)
         assert int(mine.sum()) == len(d) and not bool(Z[other][:, mine].any())
         assert float((w[mine] / q - ref).abs().max()) <= 200 * M * EPS * float(ref.abs().max())
+
+
+def test_coupling_near_overflow(gep):
+    """A coupling whose double overflows, at a tear: +-e and the rest, far below."""
+    import torch
+    M, big = 40, 1.2e308
+    d = torch.zeros(M, dtype=torch.float64)
+    e = torch.full((M - 1,), 1e290, dtype=torch.float64)
+    e[7] = big
+    w, Z, info = gep.tridiag_eig(d.cuda(), e.cuda())
+    assert info == 0
+    w, Z = w.cpu(), Z.cpu()
+    assert abs(float(w[0]) + big) <= 200 * M * EPS * big and abs(float(w[-1]) - big) <= 200 * M * EPS * big
+    assert float(w[1:-1].abs().max()) <= 200 * M * EPS * big
+    assert float((Z.t() @ Z - torch.eye(M, dtype=torch.float64)).abs().max()) <= 200 * M * EPS
+
+
+@pytest.mark.parametrize("M", [20, 40, 300])
+@pytest.mark.parametrize("where", ["d", "e"])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_not_a_number_is_a_failure(gep, M, where, bad):
+    import torch
+    d, e = _tridiagonal(M, M)
+    for i in (0, 7, 8, M // 2):
+        x, y = d.clone(), e.clone()
+        (x if where == "d" else y)[i] = bad
+        h = gep.Handle()
+        assert gep.tridiag_eig(x.cuda(), y.cuda(), handle=h)[2] > M
+        h.close()
