@@ -127,7 +127,7 @@ def test_one_cta_status(gep, M, minor):
     bad[minor - 1, minor - 1] = -1.0
     s = _one_cta(gep, [A, A], [B, bad])
     assert s.info() == minor
-    assert gep.solve(A, bad)[2] == minor
+    assert gep.solve(A, bad, handle=s.h)[2] == minor  # (a status stays with its handle)
     s.h.close()
     nan = A.clone()
     nan[5, 3] = nan[3, 5] = float("nan")
