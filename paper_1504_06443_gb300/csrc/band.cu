@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(PQ_ROWS) k_pqr_step(int n, int nb, int c, doub
     if (t == 0) {
       double alpha = prow_in[c], xn2 = sd[c];
       double tt = 0.0, sl = 0.0, be = alpha;
-      if (xn2 > 0.0) {
+      if (xn2 > 0.0 && !tiny_squares(alpha * alpha + xn2)) {
         be = -copysign(sqrt(alpha * alpha + xn2), alpha);
         tt = (be - alpha) / be;
         sl = 1.0 / (alpha - be);
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(PQ_ROWS) k_pqr_coop(int n, int nb, int rp, dou
       if (t == 0) {
         double alpha = __ldcg(rin + c), xn2 = sd[c];
         double tt = 0.0, sl = 0.0, be = alpha;
-        if (xn2 > 0.0) {
+        if (xn2 > 0.0 && !tiny_squares(alpha * alpha + xn2)) {
           be = -copysign(sqrt(alpha * alpha + xn2), alpha);
           tt = (be - alpha) / be;
           sl = 1.0 / (alpha - be);
@@ -401,8 +401,8 @@ __global__ void __launch_bounds__(32 * (PQW + 1)) k_panel_qr(PanelArgs a) {
                      ((red[4][lane] + red[5][lane]) + (red[6][lane] + red[7][lane]));
           const double xn2 = __shfl_sync(0xffffffffu, s, c), alpha = __shfl_sync(0xffffffffu, pr, c);
           double tt = 0.0, sl = 0.0, be = alpha;
-          if (xn2 > 0.0) {
-            const double n2 = fma(alpha, alpha, xn2);
+          const double n2 = fma(alpha, alpha, xn2);
+          if (xn2 > 0.0 && !tiny_squares(n2)) {
             const double ri = rsqrt(n2);
             be = -copysign(n2 * ri, alpha);
             sl = 1.0 / (alpha - be);
@@ -613,27 +613,36 @@ __host__ __device__ __forceinline__ size_t diamond_index(int Q, int j, int k) {
   return (size_t)j * (Q + 1) - (size_t)j * (j - 1) / 2 + k;
 }
 
-// dlarfg on x[0..len) (shared): v[0] = 1, v[i] = x[i] / (alpha - beta); returns tau, beta in out[0..1].
+// dlarfg on x[0..len) (shared): v[0] = 1, v[i] = x[i] / (alpha - beta); returns tau, beta in out[0..1].  The
+// squares are those of x scaled by the power of two out[3] into [1, 2): the bands that run in FP64 are those with
+// rows of very different scale.
 __device__ void house(const double* x, int len, double* v, double* out, int b) {
   const int t = threadIdx.x;
   if (t < 32) {
+    int E = 0;
+    for (int i = t; i < len; i += 32) E = max(E, (int)((__double_as_longlong(x[i]) >> 52) & 0x7FF));
+    E = min(max(__reduce_max_sync(0xffffffffu, E), 23), 2023);
+    const double f = __longlong_as_double((ll)(2046 - E) << 52), fi = __longlong_as_double((ll)E << 52);
     double s = 0.0;
-    for (int i = 1 + t; i < len; i += 32) s += x[i] * x[i];
+    for (int i = 1 + t; i < len; i += 32) s += (x[i] * f) * (x[i] * f);
     for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (t < 2) {  // lane 0 forms tau, lane 1 the scale: one division sequence for both
-      double alpha = x[0], be = alpha, q = 0.0;
+      double alpha = x[0] * f, be = alpha, q = 0.0;
       if (s > 0.0) {
         be = -copysign(sqrt(alpha * alpha + s), alpha);
         const double num = (t == 0) ? be - alpha : 1.0, den = (t == 0) ? be : alpha - be;
         q = num / den;
       }
       out[t == 0 ? 0 : 2] = q;
-      if (t == 0) out[1] = be;
+      if (t == 0) {
+        out[1] = be * fi;
+        out[3] = f;
+      }
     }
   }
   __syncthreads();
-  double sl = out[2];
-  for (int i = t; i < b; i += blockDim.x) v[i] = (i == 0) ? 1.0 : (i < len ? x[i] * sl : 0.0);
+  const double sl = out[2], f = out[3];
+  for (int i = t; i < b; i += blockDim.x) v[i] = (i == 0) ? 1.0 : (i < len ? (x[i] * f) * sl : 0.0);
   __syncthreads();
 }
 
@@ -684,7 +693,7 @@ __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
   double* xv = vc + BMAX;                   // column to annihilate / scratch
   double* pw = xv + BMAX;
   double* red = pw + BMAX;                  // 4*BMAX + 1
-  double* hs = red + 4 * BMAX + 8;          // tau, beta, scale
+  double* hs = red + 4 * BMAX + 8;          // tau, beta, the two factors of the scale
   __shared__ int abort_flag;
   const int t = threadIdx.x, M = a.M, b = a.b, ldab = a.ldab;
   if (t == 0) abort_flag = 0;

@@ -280,6 +280,11 @@ int small_gep_batched(gep_handle_t h, cudaStream_t s, int count, const int* M, d
                       double* const* w, double* const* Y, const int* order, double* scratch, int ctas, int* next,
                       int* info);
 
+// A column whose sum of squares (alpha's included) lies below 2^-1010 is taken as zero beside its first entry (H = I):
+// squares that underflow would give a reflector that is not orthogonal.  Its entries are below 2^-505.  (Compared
+// as integers: an FP64 instruction holds a scheduler for 64 clocks.)
+__device__ __forceinline__ bool tiny_squares(double n2) { return __double2hiint(n2) < (13 << 20); }
+
 // Kernel-side helper: returns true when an earlier stage recorded an error.
 __device__ __forceinline__ bool status_bad(const int* st) { return st != nullptr && (st[0] != 0 || st[1] != 0); }
 

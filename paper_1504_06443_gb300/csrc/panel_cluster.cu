@@ -196,8 +196,9 @@ __global__ void __cluster_dims__(QC, 1, 1) __launch_bounds__(QTHREADS, 1) k_pane
             const double pr = qr_dbl(sh.rrow[c & 1][lane]);
             const double xn2 = __shfl_sync(0xffffffffu, s, c), alpha = __shfl_sync(0xffffffffu, pr, c);
             double tt = 0.0, sl = 0.0, be = alpha;
-            if (xn2 > 0.0) {
-              const double n2 = fma(alpha, alpha, xn2), ri = rsqrt(n2);
+            const double n2 = fma(alpha, alpha, xn2);
+            if (xn2 > 0.0 && !tiny_squares(n2)) {
+              const double ri = rsqrt(n2);
               be = -copysign(n2 * ri, alpha);
               sl = 1.0 / (alpha - be);
               tt = fma(fabs(alpha), ri, 1.0);

@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(1024) k_householder(int M, int c, int i, doubl
   double sig = block_sum(s, red);
   double alpha = x[0];
   double beta, tv, scal;
-  if (sig == 0.0) {
+  const bool none = sig == 0.0 || tiny_squares(alpha * alpha + sig);
+  if (none) {
     tv = 0.0; beta = alpha; scal = 0.0;
   } else {
     double nrm = sqrt(alpha * alpha + sig);
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(1024) k_householder(int M, int c, int i, doubl
   double* v = Vp + (size_t)i * ldp;
   for (int r = threadIdx.x; r <= c; r += blockDim.x) v[r] = 0.0;
   for (int t = 1 + threadIdx.x; t < n; t += blockDim.x) {
-    double vt = (sig == 0.0) ? 0.0 : x[t] * scal;
+    double vt = none ? 0.0 : x[t] * scal;
     x[t] = vt;
     v[c + 1 + t] = vt;
   }
@@ -659,8 +660,9 @@ __global__ void __launch_bounds__(TRD_T) k_trd_panel(TrdArgs a) {
     if (warp == 0) {
       const double al = sc[2], ss = red8(red, lane);
       double tvv = 0.0, beta = al, sl = 0.0;
-      if (ss != 0.0) {
-        const double n2 = fma(al, al, ss), ri = rsqrt(n2), nrm = n2 * ri;
+      const double n2 = fma(al, al, ss);
+      if (ss != 0.0 && !tiny_squares(n2)) {
+        const double ri = rsqrt(n2), nrm = n2 * ri;
         beta = al >= 0.0 ? -nrm : nrm;
         sl = 1.0 / (al - beta);
         tvv = fma(fabs(al), ri, 1.0);

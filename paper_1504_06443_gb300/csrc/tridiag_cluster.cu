@@ -155,8 +155,10 @@ __device__ __forceinline__ void trc_columns(const TrcArgs& p, TrcShared& sh, cg:
     if (F64 && warp == 0) {
       const double s2 = trc_sum(lane < TRC_WARPS ? trc_dbl(sh.zs[lane]) : 0.0), xa = trc_dbl(sh.xa);
       double m = 0.0, tau = 0.0, beta = xa;
-      if (s2 != 0.0) {
-        const double n2 = fma(xa, xa, s2), ri = rsqrt(n2);
+      const double n2 = fma(xa, xa, s2);
+      const bool some = s2 != 0.0 && !tiny_squares(n2);
+      if (some) {
+        const double ri = rsqrt(n2);
         beta = -copysign(n2 * ri, xa);
         m = 1.0 / (xa - beta);
         tau = fma(fabs(xa), ri, 1.0);
@@ -164,7 +166,7 @@ __device__ __forceinline__ void trc_columns(const TrcArgs& p, TrcShared& sh, cg:
       if (lane == 0) {
         sh.mq = trc_int2(m);
         sh.tauq = sh.tau[i] = __double_as_longlong(tau);
-        sh.zero = s2 == 0.0;
+        sh.zero = !some;
         sh.e[i] = __double_as_longlong(beta);
       }
     } else if (warp == 0) {
