@@ -135,7 +135,7 @@ void mark(gep_handle_t h, const gep_options* o, int i) {
 // with vectors D&C then writes all eigenvalues to wt and all eigenvectors of T to Zt (M x M)
 // and only the first n columns are copied to Z and back-transformed.  timed: record marks 3
 // (after TRD/BAND) and 4 (after D&C) and the S1b/S1c split of the caller's timers.
-int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, double* dvec, double* evec,
+int sep_solve_scaled(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, double* dvec, double* evec,
               double* tvec, double* q2, char* uni, size_t uni_bytes, int eng, double* w, double* Z, int ldz,
               bool timed, int n = 0, double* Zt = nullptr, double* wt = nullptr, double* q2u = nullptr) {
   if (n <= 0 || n > M) n = M;
@@ -193,6 +193,23 @@ int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, d
     return backtransform_q(h, M, n, C, ldc, tvec, Z, ldz, (double*)uni, uni_bytes / sizeof(double), eng, bw);
   }
   return backtransform_q(h, M, n, C, ldc, tvec, Z, ldz, (double*)uni, uni_bytes / sizeof(double), eng);
+}
+
+// The SEP solver on C times the power of two that brings its largest entry into [1, 2), for the tensor-core engines:
+// their products take a row [W V] of a rank-2b update as one operand, whose digits are relative to its largest
+// entry.  With W of C's size and V of order one, V would lose as many bits as C's norm is away from one.
+int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, double* dvec, double* evec,
+              double* tvec, double* q2, char* uni, size_t uni_bytes, int eng, double* w, double* Z, int ldz,
+              bool timed, int n = 0, double* Zt = nullptr, double* wt = nullptr, double* q2u = nullptr) {
+  const bool scaled = eng != GEP_PREC_FP64 && !jacobi(o);
+  int* ex = h->d_status + STATUS_EXPONENTS + 2;
+  if (scaled) {
+    GEP_CUDA(cudaMemsetAsync(ex, 0, sizeof(int), h->stream));
+    GEP_CHECK(max_exponent(h, M, C, ldc, ex));
+    GEP_CHECK(scale_pow2(h, M, M, C, ldc, C, ldc, nullptr, ex));
+  }
+  GEP_CHECK(sep_solve_scaled(h, M, C, ldc, o, dvec, evec, tvec, q2, uni, uni_bytes, eng, w, Z, ldz, timed, n, Zt, wt, q2u));
+  return scaled ? scale_pow2(h, n > 0 && n < M ? n : M, 1, w, M, w, M, ex, nullptr) : GEP_OK;
 }
 
 }  // namespace
@@ -734,10 +751,19 @@ int gep_solve(gep_handle_t h, int M, double* A, int lda, double* B, int ldb, dou
     GEP_CHECK(copy_lower(h, M, B, ldb, Bf, M));
     GEP_CHECK(symmetrize_lower(h, M, Bf, M));
   }
-  if (!o->overwrite) {
+  // On the tensor-core engines A takes the size of B (a power of two, undone in w), so that the reduction's
+  // rank-2 updates [A21 L21] have rows of one size (see sep_solve).
+  int* ex = h->d_status + STATUS_EXPONENTS;
+  const bool scaled = eng != GEP_PREC_FP64;
+  if (scaled) {
+    GEP_CUDA(cudaMemsetAsync(ex, 0, 2 * sizeof(int), h->stream));
+    GEP_CHECK(max_exponent(h, M, A, lda, ex));
+    GEP_CHECK(max_exponent(h, M, B, ldb, ex + 1));
+    GEP_CHECK(scale_pow2(h, M, M, A, lda, Cw, ldcw, ex + 1, ex));
+  } else if (!o->overwrite) {
     GEP_CHECK(copy_lower(h, M, A, lda, Cw, ldcw));
-    GEP_CHECK(copy_lower(h, M, B, ldb, Lw, ldlw));
   }
+  if (!o->overwrite) GEP_CHECK(copy_lower(h, M, B, ldb, Lw, ldlw));
   double* wB = tvec + (M + 1);  // eigenvalues D of B (Cholesky-free reducer)
   double* wT = wB + (M + 1);     // all eigenvalues of T when only the lowest n are wanted
   double* Zt = partial_vectors(M, o) ? (double*)(base + Ly.zt) : nullptr;
@@ -762,6 +788,7 @@ int gep_solve(gep_handle_t h, int M, double* A, int lda, double* B, int ldb, dou
     GEP_CHECK(sep_solve(h, M, Cw, ldcw, o, dvec, evec, tvec, q2, uni, Ly.uni_bytes, eng, w, Z, ldlw, true, n, Zt,
                         wT, q2u));
     if (!o->want_vectors) {
+      if (scaled) GEP_CHECK(scale_pow2(h, n, 1, w, M, w, M, ex, ex + 1));
       mark(h, o, 5);
       mark(h, o, 6);
       mark(h, o, 7);
@@ -788,6 +815,7 @@ int gep_solve(gep_handle_t h, int M, double* A, int lda, double* B, int ldb, dou
     GEP_CHECK(sep_solve(h, M, Cw, ldcw, o, dvec, evec, tvec, q2, uni, Ly.uni_bytes, eng, w,
                         o->want_vectors ? Y : nullptr, ldy, true, n, Zt, wT, q2u));
     if (!o->want_vectors) {
+      if (scaled) GEP_CHECK(scale_pow2(h, n, 1, w, M, w, M, ex, ex + 1));
       mark(h, o, 5);
       mark(h, o, 6);
       mark(h, o, 7);
@@ -804,6 +832,7 @@ int gep_solve(gep_handle_t h, int M, double* A, int lda, double* B, int ldb, dou
     }
     mark(h, o, 6);
   }
+  if (scaled) GEP_CHECK(scale_pow2(h, n, 1, w, M, w, M, ex, ex + 1));
   h->refine_steps = 0;
   if (mixed && o->refine_iters >= 0) {
     GEP_CHECK(refine_eigenpairs(h, M, Af, Bf, Y, ldy, w, (double*)uni, o->refine_iters, GEP_PREC_FP64_EMULATED));

@@ -21,6 +21,31 @@ __global__ void k_copy_lower(int m, const double* __restrict__ s, int lds, doubl
     if (i < m && i >= j) d[GEP_IX(i, j, ldd)] = s[GEP_IX(i, j, lds)];
 }
 
+// Largest exponent field of the lower triangle (zero on entry).
+__global__ void __launch_bounds__(256) k_max_exponent(int M, const double* __restrict__ A, int lda, int* __restrict__ ex,
+                                                      const int* st) {
+  if (status_bad(st)) return;
+  int m = 0;
+  for (int j = blockIdx.x; j < M; j += gridDim.x) {
+#pragma unroll 4
+    for (int i = j + threadIdx.x; i < M; i += 256)
+      m = max(m, (int)((__double_as_longlong(A[GEP_IX(i, j, lda)]) >> 52) & 0x7FF));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(ex, m);
+}
+
+// The lower triangle (cols = 1: a vector) times 2^(*up - *down) (nothing where one of them is zero); in place or not.
+__global__ void k_scale_pow2(int m, int cols, const double* s, int lds, double* d, int ldd, const int* up,
+                             const int* down, const int* st) {
+  if (status_bad(st)) return;
+  const int eu = up ? *up : 1023, ed = down ? *down : 1023, e = eu && ed ? eu - ed : 0, h = e / 2;
+  const double f = __longlong_as_double((long long)(1023 + h) << 52), g = __longlong_as_double((long long)(1023 + e - h) << 52);
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int j = blockIdx.y; j < cols; j += gridDim.y)
+    if (i < m && i >= j) d[GEP_IX(i, j, ldd)] = s[GEP_IX(i, j, lds)] * f * g;
+}
+
 __global__ void k_set(int m, int n, double off, double dia, double* A, int lda) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   for (int j = blockIdx.y; j < n; j += gridDim.y)
@@ -146,6 +171,19 @@ int copy_matrix(gep_handle_t h, int m, int n, const double* src, int lds, double
 int copy_lower(gep_handle_t h, int M, const double* src, int lds, double* dst, int ldd) {
   if (M <= 0) return GEP_OK;
   k_copy_lower<<<grid2(M, M), 256, 0, h->stream>>>(M, src, lds, dst, ldd);
+  return check_launch(h);
+}
+
+int max_exponent(gep_handle_t h, int M, const double* A, int lda, int* ex) {
+  if (M <= 0) return GEP_OK;
+  k_max_exponent<<<M < 4 * h->sm_count ? M : 4 * h->sm_count, 256, 0, h->stream>>>(M, A, lda, ex, h->d_status);
+  return check_launch(h);
+}
+
+int scale_pow2(gep_handle_t h, int m, int cols, const double* src, int lds, double* dst, int ldd, const int* up,
+               const int* down) {
+  if (m <= 0 || cols <= 0) return GEP_OK;
+  k_scale_pow2<<<grid2(m, cols), 256, 0, h->stream>>>(m, cols, src, lds, dst, ldd, up, down, h->d_status);
   return check_launch(h);
 }
 

@@ -61,6 +61,8 @@ struct gep_handle_s {
 
 namespace gep {
 
+constexpr int STATUS_EXPONENTS = 16;  // ints of the status block: exponents of A, B and C of a solve
+
 // Bump allocator over the caller's workspace.
 struct Arena {
   char* base;
@@ -199,6 +201,11 @@ int dgemm_oz_sym_planes(gep_handle_t h, const OzSymPlanes& P, int row0, int n, d
 int copy_matrix(gep_handle_t h, int m, int n, const double* src, int lds, double* dst, int ldd);
 int copy_lower(gep_handle_t h, int M, const double* src, int lds, double* dst, int ldd);
 int set_matrix(gep_handle_t h, int m, int n, double offdiag, double diag, double* A, int lda);
+// *ex (zero on entry) := largest exponent field of the lower triangle of A
+int max_exponent(gep_handle_t h, int M, const double* A, int lda, int* ex);
+// lower triangle (cols = m) or vector (cols = 1): dst = src 2^(*up - *down), device exponent fields, null: that of 1
+int scale_pow2(gep_handle_t h, int m, int cols, const double* src, int lds, double* dst, int ldd, const int* up,
+               const int* down);
 int symmetrize_lower(gep_handle_t h, int M, double* A, int lda);  // upper := lower^T
 int transpose(gep_handle_t h, int m, int n, const double* src, int lds, double* dst, int ldd);
 int zero_upper(gep_handle_t h, int M, double* A, int lda);          // strict upper := 0
