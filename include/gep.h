@@ -178,9 +178,9 @@ int sep_backtransform(gep_handle_t h, int M, int ncol, const double* C, int ldc,
  *   NULL when only eigenvalues are wanted) receives the bulge-chasing reflectors.
  *   C's band itself is not modified by the second stage.
  *   With b <= 32 panels of up to 2048 rows are held in 64-bit fixed point with one unit a column,
- *   2^-60 of its norm, and with b = 32 or 64 the second stage's band with one unit, about 2^-61 of
- *   its largest absolute row sum, where the rows of the matrix (their largest entries; of the band
- *   their sums) lie within a factor of 16, and in FP64 otherwise.
+ *   2^-60 of its norm, where the absolute row sums of C lie within a factor of 16, and with b = 32
+ *   or 64 the second stage's band with one unit, about 2^-61 of its largest absolute row sum, where
+ *   those of neighbouring rows lie within 16 and all within 256; in FP64 otherwise.
  * sep_backtransform_2stage: Z (M x ncol) is overwritten by Q1 (Q2 Z) using C, tau1 and
  *   q2 from sep_tridiag_2stage with the same M and b.
  * Both take their scratch from the handle workspace (size it with gep_workspace_size

@@ -162,46 +162,50 @@ __device__ __forceinline__ void st_release(int* p, int v) {
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Largest exponent field of every row of the symmetric matrix in the lower triangle of C (zero on entry), a
-// 64 x 64 tile a CTA; one pass over the triangle: order 8192 about 50 us.
-__global__ void __launch_bounds__(256) k_row_exponents(int M, const double* __restrict__ C, int ldc, int* __restrict__ ex,
-                                                       const int* st) {
-  __shared__ int row[64], col[64];
+// Absolute row sums (zero on entry) of the symmetric matrix in the lower triangle of C, as integers: in units of
+// 2^-40 of the power of two of the largest entry (*ex its exponent field), an entry that is not zero at least
+// one.  A 64 x 64 tile a CTA; integer sums, so that the rule below gives the same answer every time.  One pass over the
+// triangle: order 8192 about 60 us.
+__global__ void __launch_bounds__(256) k_row_sums(int M, const double* __restrict__ C, int ldc, const int* __restrict__ ex,
+                                                  unsigned long long* __restrict__ sum, const int* st) {
+  __shared__ unsigned long long row[64], col[64];
   if (blockIdx.x < blockIdx.y || status_bad(st)) return;
-  const int t = threadIdx.x, r0 = blockIdx.x * 64, c0 = blockIdx.y * 64, r = r0 + (t & 63);
+  const int t = threadIdx.x, r0 = blockIdx.x * 64, c0 = blockIdx.y * 64, r = r0 + (t & 63), sh = 1023 - *ex + 40;
   if (t < 64) row[t] = col[t] = 0;
   __syncthreads();
-  int m = 0;
+  ll m = 0;
 #pragma unroll
   for (int u = 0; u < 16; ++u) {
     const int q = (t >> 6) + 4 * u, c = c0 + q;
-    const int x = r < M && c <= r ? (int)((__double_as_longlong(C[r + (size_t)c * ldc]) >> 52) & 0x7FF) : 0;
-    m = max(m, x);
-    const int w = __reduce_max_sync(0xffffffffu, x);
-    if ((t & 31) == 0) atomicMax(&col[q], w);
+    const ll x = r < M && c <= r ? __double_as_longlong(C[r + (size_t)c * ldc]) & ~(1ll << 63) : 0;
+    const ll v = max(qfix(x, sh), (ll)(x != 0));
+    m += v;
+    const ll w = qwarp_sum(r != c ? v : 0);
+    if ((t & 31) == 0) atomicAdd(&col[q], (unsigned long long)w);
   }
-  atomicMax(&row[t & 63], m);
+  atomicAdd(&row[t & 63], (unsigned long long)m);
   __syncthreads();
-  if (t < 64 && r0 + t < M) atomicMax(ex + r0 + t, row[t]);
-  else if (t >= 64 && t < 128 && c0 + t - 64 < M) atomicMax(ex + c0 + t - 64, col[t - 64]);
+  if (t < 64 && r0 + t < M) atomicAdd(sum + r0 + t, row[t]);
+  else if (t >= 64 && t < 128 && c0 + t - 64 < M) atomicAdd(sum + c0 + t - 64, col[t - 64]);
 }
 
-// *wide: whether the rows that are not zero lie further apart than 2^4.
-__global__ void __launch_bounds__(1024) k_row_spread(int M, const int* __restrict__ ex, int* __restrict__ wide, const int* st) {
-  __shared__ int hi, lo;
+// *wide: whether the sums of the rows that are not zero lie further apart than 2^4.
+__global__ void __launch_bounds__(1024) k_row_spread(int M, const unsigned long long* __restrict__ sum,
+                                                     const int* __restrict__ ex, int* __restrict__ wide, const int* st) {
+  __shared__ unsigned long long hi, lo;
   if (status_bad(st)) return;
   if (threadIdx.x == 0) {
     hi = 0;
-    lo = 0x7FF;
+    lo = ~0ull;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < M; i += 1024)
-    if (ex[i]) {
-      atomicMax(&hi, ex[i]);
-      atomicMin(&lo, ex[i]);
+    if (sum[i]) {
+      atomicMax(&hi, sum[i]);
+      atomicMin(&lo, sum[i]);
     }
   __syncthreads();
-  if (threadIdx.x == 0) *wide = hi < 0x7FF && hi - lo > 4;
+  if (threadIdx.x == 0) *wide = *ex < 0x7FF && hi != 0 && lo < hi >> 4;
 }
 
 // The whole panel QR in one cooperative launch: CTA g keeps panel rows [rp g, rp g + rp)
@@ -676,12 +680,17 @@ __device__ void two_sided(double* D, int len, const double* v, double tau, doubl
   __syncthreads();
 }
 
-// Norm bounds of the band (k_band_rowsum): mx[0] largest absolute row sum, mx[1] the complement of the
-// smallest one beside the first column (bits of doubles).  With the rows further apart than 2^4 the band stays
-// FP64: one fixed-point unit for all of it would take the relative accuracy of its small blocks.
+// Norm bounds of the band (k_band_rowsum): mx[0] largest absolute row sum, mx[1] the complement of the smallest one
+// beside the first column (bits of doubles), mx[2] bit 0: two neighbours further apart than 2^4, bit 1: a row of
+// zeros.  One fixed-point unit for the whole band, 2^-61 of mx[0], takes the relative accuracy of a block far below the
+// rest if that is decoupled: such a block begins with a jump between neighbours (or beyond a row of zeros),
+// and the band stays FP64.  Where the rows fall off slowly FP64 mixes them as well; there the unit has to
+// be no coarser than FP64's at the smallest row.  Decoupled blocks at 2^-4, 2^-6, 2^-8 of the rest, order 500: mean
+// error of their eigenvalues 0.8, 1.6, 5.4e-15 in fixed point, 0.7e-15 in FP64.  Tight-binding bands of order
+// 512 to 16384 have neighbours within 5.2 and rows within 13 to 106: 57 ms at order 8192 instead of 182.
 __device__ __forceinline__ bool band_wide(const unsigned long long* mx) {
   const double hi = __longlong_as_double((ll)mx[0]), lo = __longlong_as_double((ll)~mx[1]);
-  return mx[1] != 0 && (mx[0] >> 52) < 0x7FF && lo < 0.0625 * hi;
+  return mx[1] != 0 && (mx[0] >> 52) < 0x7FF && ((mx[2] & 1) || lo < ((mx[2] & 2) ? 0x1p-4 : 0x1p-8) * hi);
 }
 
 __global__ void __launch_bounds__(256) k_bulge(BulgeArgs a) {
@@ -1214,24 +1223,33 @@ __global__ void __launch_bounds__(bulge_threads<N>()) k_bulge_ws(BulgeArgs a) {
 __global__ void k_band_rowsum(int M, int b, const double* __restrict__ AB, int ldab, unsigned long long* mx,
                               const int* st) {
   if (status_bad(st)) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  double rest = 0.0, first = 0.0;  // first: the entry of the first column (of row 0: the diagonal)
-  if (i < M) {
-    first = i <= b ? fabs(AB[i]) : 0.0;
-    for (int o = i == 0 ? 1 : 0; o <= b && i + o < M; ++o) rest += fabs(AB[o + (size_t)i * ldab]);
-    for (int o = 1; o <= b && o < i; ++o) rest += fabs(AB[o + (size_t)(i - o) * ldab]);
-  }
-  unsigned long long v = (unsigned long long)__double_as_longlong(rest + first);
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  // row r beside the first column, and first: its entry there (of row 0: the diagonal)
+  auto beside = [&](int r, double& first) {
+    double s = 0.0;
+    first = r <= b ? fabs(AB[r]) : 0.0;
+    for (int o = r == 0 ? 1 : 0; o <= b && r + o < M; ++o) s += fabs(AB[o + (size_t)r * ldab]);
+    for (int o = 1; o <= b && o < r; ++o) s += fabs(AB[o + (size_t)(r - o) * ldab]);
+    return s;
+  };
+  double rest = 0.0, first = 0.0;
+  if (i < M) rest = beside(i, first);
+  unsigned long long v = (unsigned long long)__double_as_longlong(rest + first), bits = i < M && rest == 0.0 ? 2 : 0;
   if (i == 0 && rest == 0.0) rest = first;  // a decoupled first row
+  double above = __shfl_up_sync(0xffffffffu, rest, 1), unused;
+  if (lane == 0) above = i > 1 && i < M ? beside(i - 1, unused) : rest;
+  if (i > 1 && i < M && rest > 0.0 && above > 0.0 && fmin(rest, above) < 0x1p-4 * fmax(rest, above)) bits |= 1;
   unsigned long long u = rest > 0.0 ? ~(unsigned long long)__double_as_longlong(rest) : 0;
   for (int o = 16; o; o >>= 1) {
     const unsigned long long q = __shfl_xor_sync(0xffffffffu, v, o), p = __shfl_xor_sync(0xffffffffu, u, o);
     if (q > v) v = q;
     if (p > u) u = p;
+    bits |= __shfl_xor_sync(0xffffffffu, bits, o);
   }
-  if ((threadIdx.x & 31) == 0) {
+  if (lane == 0) {
     if (v) atomicMax(mx, v);
     if (u) atomicMax(mx + 1, u);
+    if (bits) atomicOr(mx + 2, bits);
   }
 }
 
@@ -1630,13 +1648,16 @@ int band_reduce(gep_handle_t h, int M, double* C, int ldc, int b, double* tau1, 
   w.part_elems = oz_sym_part_elems(M, b);
   w.parts = take(w.part_elems);
   const int levels = eng == GEP_PREC_MIXED_REFINED ? 4 : 9;
-  if (b <= PQN) {  // the arithmetic of the panels in a cluster (the exponents in V, not yet in use)
-    int* ex = reinterpret_cast<int*>(w.V);
-    GEP_CUDA(cudaMemsetAsync(ex, 0, sizeof(int) * (size_t)M, h->stream));
+  if (b <= PQN) {  // the arithmetic of the panels in a cluster (the sums in V, not yet in use)
+    unsigned long long* sum = reinterpret_cast<unsigned long long*>(w.V);
+    int* ex = w.wide + 1;
+    GEP_CUDA(cudaMemsetAsync(sum, 0, sizeof(unsigned long long) * (size_t)M, h->stream));
+    GEP_CUDA(cudaMemsetAsync(w.wide, 0, 2 * sizeof(int), h->stream));
     const int nt = (M + 63) / 64;
-    k_row_exponents<<<dim3(nt, nt), 256, 0, h->stream>>>(M, C, ldc, ex, h->d_status);
+    GEP_CHECK(max_exponent(h, M, C, ldc, ex));
+    k_row_sums<<<dim3(nt, nt), 256, 0, h->stream>>>(M, C, ldc, ex, sum, h->d_status);
     GEP_CHECK(check_launch(h));
-    k_row_spread<<<1, 1024, 0, h->stream>>>(M, ex, w.wide, h->d_status);
+    k_row_spread<<<1, 1024, 0, h->stream>>>(M, sum, ex, w.wide, h->d_status);
     GEP_CHECK(check_launch(h));
   }
   for (int pb = 0; M - pb - b >= 2;) {
@@ -1767,7 +1788,7 @@ int band_to_tridiag(gep_handle_t h, int M, const double* C, int ldc, int b, doub
     a.wait_ns = h->wait_limit_ns;
     a.drop_sweep = h->fault_drop_sweep;
     if (fixed) {
-      GEP_CUDA(cudaMemsetAsync(mx, 0, 2 * sizeof(unsigned long long), h->stream));
+      GEP_CUDA(cudaMemsetAsync(mx, 0, 3 * sizeof(unsigned long long), h->stream));
       k_band_rowsum<<<(M + 255) / 256, 256, 0, h->stream>>>(M, b, AB, ldab, mx, h->d_status);
       GEP_CHECK(check_launch(h));
       k_band_fix<<<std::min(M, 4 * h->sm_count), 256, 0, h->stream>>>(M, AB, ldab, mx, h->d_status);

@@ -9,7 +9,7 @@
 // sums, so that a pivot column that has become tiny still gives an orthogonal reflector.  The
 // scalars of a reflector are formed by warp 0 of every CTA; an extra warp of CTA 0 accumulates T in FP64.
 //
-// A column's unit is fair to rows of like size only: where the rows of the matrix lie further apart than 2^4
+// A column's unit is fair to rows of like size only: where the row sums of the matrix lie further apart than 2^4
 // (band.cu's scan) the same exchange carries FP64 numbers, columns scaled by powers of two.
 //
 // A column: every CTA pushes its sums (and the owner of the pivot row that row) to all 16

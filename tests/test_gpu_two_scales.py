@@ -115,3 +115,24 @@ def test_panel_rows_of_two_scales(gep, M, m1, b, s):
     ref = torch.geqrf(C[b:, :b].cpu())[0].tril(-1)
     scale = ref.abs().amax(1, keepdim=True)
     assert bool(((V - ref).abs() <= 200 * M * EPS * scale).all())
+
+
+@pytest.mark.parametrize("M", [300, 1000])
+def test_a_slowly_falling_band_keeps_the_fast_route(gep, M):
+    """A tight-binding matrix (neighbouring rows alike, the smallest of a band far below the largest): its bulge chasing is
+    not the FP64 one, which takes several times as long.  Two blocks 1e-4 apart take the FP64 one."""
+    import torch
+    import gep_inputs as gi
+    p = gi.tight_binding(M, 0)
+    A, B = (torch.as_tensor(p[x], device="cuda") for x in "AB")
+    h = gep.Handle()
+
+    def chase_ms(a, b):
+        t = []
+        for _ in range(4):
+            assert gep.solve(a, b, sep="2stage", precision="fp64_emulated", timers=True, handle=h)[2] == 0
+            t.append(h.band_times()[1])
+        return min(t[1:])
+    eye = torch.eye(M, dtype=torch.float64, device="cuda")
+    assert 1.5 * chase_ms(A, B) < chase_ms(_blocks(M, M // 2, 1e-4, 1), eye)
+    h.close()
