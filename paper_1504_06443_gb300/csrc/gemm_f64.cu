@@ -256,7 +256,7 @@ int dgemm_f64(gep_handle_t h, char ta, char tb, char uplo, int m, int n, int k, 
   if (SA && (TB || k != m)) return GEP_ERR_UNSUPPORTED;
   dim3 grid((m + BM - 1) / BM, (n + BN - 1) / BN);
   // Tile choice: the largest tile that still gives every SM about four CTAs, else 16 x 16 tiles
-  // with the depth split over clusters until there are two CTAs per SM (slices of at least 32)
+  // with the depth split over CTAs until there are two CTAs per SM (slices of at least 32)
   auto tiles_of = [&](int t) {
     long long gx = (m + t - 1) / t, gy = (n + t - 1) / t;
     return lower ? gx * gy - (gy < gx ? gy : gx) * ((gy < gx ? gy : gx) - 1) / 2 : gx * gy;

@@ -13,7 +13,7 @@
 //     X = sum_i t_i (P / m_i) - q P,   q = nearest integer of sum_i t_i / m_i.
 //
 // Three steps: residues of both operands (k_res_split), the 16 products (k_res_gemm: one item per
-// modulus and 128 x 256 tile, bytes out), the reconstruction (k_res_crt: 128-bit integers, then the
+// modulus and 256 x 256 tile of a CTA pair, bytes out), the reconstruction (k_res_crt: 128-bit integers, then the
 // double nearest to the value, alpha and beta).  Against the digit planes the operands take twice the bytes
 // and every output 32 bytes more, so this pays where K is large: see res_product_wins.
 //

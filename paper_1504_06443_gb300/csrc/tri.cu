@@ -356,7 +356,7 @@ int potrf_rec(gep_handle_t h, int o, int n, double* B, int ldb, double* invD, do
 
 }  // namespace
 
-// X := L^-1 X (forward substitution); tmp holds max(NB x n) doubles.
+// X := L^-1 X (forward substitution); tmp holds TRI_NB x n doubles.
 int trsm_lln(gep_handle_t h, int M, int n, const double* L, int ldl, const double* invD, int nb,
              double* X, int ldx, double* tmp, int engine) {
   if (nb != TRI_NB) return GEP_ERR_UNSUPPORTED;
@@ -372,8 +372,8 @@ int trsm_llt(gep_handle_t h, int M, int n, const double* L, int ldl, const doubl
   return llt_rec(h, 0, M, n, L, ldl, invD, X, ldx, tmp, engine);
 }
 
-// Eq. 4: recursive Cholesky.  invD receives the inverses of the NB x NB diagonal
-// blocks (reused by the reduction and the back-substitution).  tmp (M x NB doubles)
+// Eq. 4: recursive Cholesky.  invD receives the inverses of the TRI_NB x TRI_NB diagonal
+// blocks (reused by the reduction and the back-substitution).  tmp (M x TRI_NB doubles)
 // follows invD in the caller's workspace.
 int cholesky(gep_handle_t h, int M, double* B, int ldb, double* invD, int engine) {
   if (M <= 0) return GEP_OK;
@@ -393,11 +393,11 @@ int cholesky(gep_handle_t h, int M, double* B, int ldb, double* invD, int engine
 // and the trailing matrix is reduced the same way.  About M^3 flops in products (two
 // thirds in the symmetric rank-2nb updates, one third in the solves), against 2 M^3 for two
 // full triangular solves.  A (lower) is overwritten by the full symmetric C; X is an M x M
-// scratch matrix, tmp an NB x M one.
+// scratch matrix, tmp a TRI_NB x M one.
 int reduce_twosided(gep_handle_t h, int M, double* A, int lda, const double* L, int ldl,
                     const double* invD, double* X, double* tmp, int engine) {
   if (M <= 0) return GEP_OK;
-  // Panel width: a multiple of NB (the triangular recursions split at multiples of NB), half the
+  // Panel width: a multiple of TRI_NB (the triangular recursions split there), half the
   // matrix up to 2048.  Every panel is a chain of some twenty launches that depend on one another,
   // and its rank-2 nb update splits its operands anew; wide panels have fewer chains and give the
   // tensor engine deep products.  R2 at 1501 / 2047 / 3000 / 4000 / 6000 / 8192: with M / 8 up to
@@ -446,7 +446,7 @@ int reduce_explicit_inv(gep_handle_t h, int M, double* A, int lda, double* L, in
                         const double* invD, double* X, double* tmp, int engine) {
   if (M <= 0) return GEP_OK;
   double* T = tmp;                    // M x M
-  double* tmp_small = tmp + (size_t)M * M;  // NB x M
+  double* tmp_small = tmp + (size_t)M * M;  // TRI_NB x M
   GEP_CHECK(set_matrix(h, M, M, 0.0, 1.0, X, M));
   GEP_CHECK(trsm_lln(h, M, M, L, ldl, invD, TRI_NB, X, M, tmp_small, engine));  // X = R = L^-1
   GEP_CHECK(symmetrize_lower(h, M, A, lda));

@@ -500,8 +500,8 @@ __global__ void __launch_bounds__(256) k_w_finish(int n, int nblk, const double*
 //      formed by every CTA for itself.                                              [barrier]
 // Bound: the two barriers (1.2 us each on 152 SMs) and the latency of the reductions between
 // them; native FP64 tiles also by FP64 issue (two FMAs per element).  Measured per column (six
-// launches before): order 500 FP64 69 -> 11.3 us, order 1501 float pairs 72 -> 13.6 us, order 64
-// 58 -> 9.9 us.
+// launches before): order 1501 float pairs 72 -> 13.6 us; where no cluster takes the last 512 columns
+// (tridiag_cluster.cu) also order 500 FP64 69 -> 11.3 us, order 64 58 -> 9.9 us.
 constexpr int TRD_COOP_MAX = 4096;  // vs and the tiles fit shared memory; beyond, the SYMV is bound by HBM anyway
 constexpr int TRD_T = 256;          // threads
 constexpr int LPR = 16;             // lanes per owned row

@@ -344,19 +344,23 @@ __global__ void __launch_bounds__(TRC_THREADS, 1) k_trd_cluster(TrcArgs p) {
 #pragma unroll
   for (int u = 0; u < RPW; ++u) {
     const int r = (warp + TRC_WARPS * u) * CL + k;
-    ll s = 0, any = 0, first = 0;
+    ll s = 0, any = 0, first = 0, corner = 0;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
       const ll m = a[u][t] & ~(1ll << 63), q = qfix(m, sh0);
       s += q;
-      if (t == 0 && lane == 0) first = q;
-      else any |= m;
+      if (t == 0 && lane == 0) {
+        first = q;
+        corner = m;
+      } else {
+        any |= m;
+      }
     }
     s = qwarp_sum(s);
     rs = max(rs, s);
     const ll rest = s - __shfl_sync(0xffffffffu, first, 0);
     if (__any_sync(0xffffffffu, any != 0)) low = max(low, (1ll << 62) - rest);
-    else if (r == 0 && s > 0) low = max(low, (1ll << 62) - s);  // a decoupled first row: its diagonal
+    else if (r == 0 && __shfl_sync(0xffffffffu, corner, 0) != 0) low = max(low, (1ll << 62) - s);  // its diagonal alone
   }
   trc_cluster_max(cl, sh, rs, low);
   const bool wide = finite && low > 0 && (1ll << 62) - low < rs >> TRC_SPREAD;

@@ -55,6 +55,15 @@ def test_tridiagonal_blocks(gep, M, m1, s):
         assert _backward(Q, C, T, rows) <= 200 * M * EPS
 
 
+@pytest.mark.parametrize("M", [2, 40, 300])
+@pytest.mark.parametrize("s", [1e-3, 1e-30, 1e-200])
+def test_decoupled_first_row(gep, M, s):
+    C = _blocks(M, 1, 1.0, M)
+    C[0, 0] = s
+    d, e, _, _ = gep.tridiag_1stage(C)
+    assert float(d[0]) == s and float(e[0]) == 0.0
+
+
 @pytest.mark.parametrize("M", [33, 200, 512])
 @pytest.mark.parametrize("s", [1e-3, 1e-12, 1e-25])
 def test_tridiagonal_large_first_column(gep, M, s):
