@@ -542,36 +542,44 @@ def run_peaks(a):
     print(json.dumps(out), flush=True)
 
 
-# DRAM traffic of one product-kernel launch from a committed ncu capture
-# (profiles/k_oz_gemm_4096x4096x4096.md: dram__bytes_read.sum + dram__bytes_write.sum of one
-# 4096^3 launch, 36 plane products).  It is scaled to the timed launches by their tensor
-# flops and reported only while the kernel source is the one that was captured.
-OZ_CAPTURE = {"dram_bytes": 2.207139e9 + 0.128895e9, "tensor_flops": 36 * 2.0 * 4096 ** 3,
-              "kernel_sha1": "bdc5e708ee9c66f2b06441be1106e9861aafa325",
-              "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one 4096^3 k_oz_gemm launch "
-                      "(profiles/k_oz_gemm_4096x4096x4096.md), scaled to the average timed launch by its "
-                      "tensor flops; null when the kernel source differs from the captured one"}
+# DRAM traffic of one launch of each product kernel from ncu captures (dram__bytes_read.sum +
+# dram__bytes_write.sum).  They are scaled to the timed launches by their tensor flops (36 and 16 plane products per FP64 product) and reported only
+# while the kernel sources are the ones that were captured.
+PRODUCT_CAPTURES = {
+    "digits": {"dram_bytes": 2.225633e9 + 0.169617e9, "tensor_flops": 36 * 2.0 * 4096 ** 3, "planes": 36,
+               "source": "gemm_oz.cu", "from": "template <int SC, int LC, int TNC = TN>", "to": "size_t smem_bytes_for",
+               "kernel_sha1": "12e778370d0c233aad0046fed42ad573ed9f796c"},
+    "residues": {"dram_bytes": 0.802419e9 + 0.109109e9, "tensor_flops": 16 * 2.0 * 4096 * 2048 * 4096, "planes": 16,
+                 "source": "gemm_res.cu", "from": "__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(RTHREADS",
+                 "to": "// ------------------------------------------------------------------ reconstruction",
+                 "kernel_sha1": "8bbf5a52937995625464c284537cdaa1e8861dd0"}}
+TRAFFIC_NOTE = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of one 4096^3 k_oz_gemm launch and one 4096 x 2048 x 4096 "
+                "k_res_gemm launch, scaled to the average timed launch by its tensor flops; null when a kernel source "
+                "differs from the captured one")
 
 
-def oz_kernel_sha1():
-    """sha1 of the product kernel's source text (from its template line to the end of the
-    kernel), so that a capture taken of another version is not reported."""
+def product_kernel_sha1(c):
+    """sha1 of a product kernel's source text, so that a capture of another version is not reported."""
     import hashlib
-    path = os.path.join(ROOT, "paper_1504_06443_gb300", "csrc", "gemm_oz.cu")
+    path = os.path.join(ROOT, "paper_1504_06443_gb300", "csrc", c["source"])
     try:
         src = open(path).read()
-        i = src.index("template <int SC, int LC>")
-        j = src.index("size_t smem_bytes_for", i)
+        i = src.index(c["from"])
+        j = src.index(c["to"], i)
         return hashlib.sha1(src[i:j].encode()).hexdigest()
     except (OSError, ValueError):
         return None
 
 
 def product_traffic(prof):
-    if not prof["launches"] or OZ_CAPTURE["kernel_sha1"] != oz_kernel_sha1():
+    if not prof["launches"] or any(c["kernel_sha1"] != product_kernel_sha1(c) for c in PRODUCT_CAPTURES.values()):
         return None
-    per_launch_flops = prof["tensor_flops"] / prof["launches"]
-    return OZ_CAPTURE["dram_bytes"] * per_launch_flops / OZ_CAPTURE["tensor_flops"]
+    d, r = PRODUCT_CAPTURES["digits"], PRODUCT_CAPTURES["residues"]
+    # the launches' FP64 flops by form, from their total and the tensor flops they took
+    digits = max(prof["tensor_flops"] - r["planes"] * prof["fp64_flops"], 0.0) / (d["planes"] - r["planes"])
+    residues = prof["fp64_flops"] - digits
+    total = sum(c["dram_bytes"] * c["planes"] * f / c["tensor_flops"] for c, f in ((d, digits), (r, residues)))
+    return total / prof["launches"]
 
 
 STAGE_NAMES = ["R1_cholesky", "R2_reduce", "S1_tridiag", "S2_dc", "S3_back_q", "R3_backsub", "MP3_refine"]
@@ -615,7 +623,9 @@ def stage_rooflines(M, stages, band_ms, vectors, sep, b, bf16_peak, f64pk, reduc
             if f64:
                 r["frac_of_fp64_dgemm"] = tf / f64
             if tensor and bf16_peak:
+                # digits take 36 plane products per FP64 product (above 1 where the deep products' 16 residues do)
                 r["frac_of_bf16_sustained_36_planes"] = tf * 36 / bf16_peak
+                r["frac_of_bf16_sustained_16_planes"] = tf * 16 / bf16_peak
         return r
 
     for nm, t in zip(names, stages):
@@ -798,7 +808,7 @@ def main():
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": (achieved / peak) if achieved else None,
             "traffic": product_traffic(prof),
-            "traffic_note": OZ_CAPTURE["note"],
+            "traffic_note": TRAFFIC_NOTE,
             "peak_kind": f"{pk_kind} bf16 dense sustained",
             "fp64_equiv_tflops": (prof["fp64_flops"] / (prof["ms"] * 1e-3) / 1e12) if prof["ms"] > 0 else None,
             "kernel_ms_per_step": t_kernel_ms, "timed_launches": prof["launches"], "untimed_launches": prof["skipped"],
