@@ -103,7 +103,7 @@ typedef struct gep_options {
  * gep_get_info reports k and the later stages become no-ops.
  * GEP_PREC_MIXED_REFINED (needs want_vectors = 1): every dense product of the solve runs
  * on the FP32-grade split-BF16 engine and the SYMVs in FP32; FP64 stays in the diagonal
- * blocks, the secular equations and deflation; then all eigenpairs are refined in FP64
+ * blocks, the T factors, the secular equations and deflation; then all eigenpairs are refined in FP64
  * (B-Rayleigh quotients and the first-order correction X <- X (I + E) from S = X^T A X,
  * R = X^T B X formed with FP64-accurate products; pairs whose gap is below
  * max(64 |S_ij - lambda_j R_ij|, 16 max_ij |S_ij - lambda_j R_ij|, 1e-6 max|lambda|) are
@@ -343,7 +343,10 @@ const char* gep_status_string(int code);
  * k = m, transb 'N') and only its lower triangle is read.  uplo 'F' (full) or 'L' (only
  * entries i >= j of C are computed and written).  engine: GEP_PREC_FP64 (FP64 FMA)
  * or GEP_PREC_FP64_EMULATED (split-BF16 tensor cores, FP64-accurate).  On the tensor cores a row of
- * op(A) or a column of op(B) that holds a NaN or an infinity makes its row or column of C NaN. */
+ * op(A) or a column of op(B) that holds a NaN or an infinity makes its row or column of C NaN, and the
+ * error of an entry is relative to (largest entry of its row of op(A)) x (largest of its column of
+ * op(B)) x K: about 2^-54 for FP64_EMULATED, 2^-20 for MIXED_REFINED.  Products that are cheaper on the
+ * FP64 units (by size: 128^3, or fewer than 32 rows, 16 columns or a depth of 16) run there. */
 int gep_dgemm(gep_handle_t h, char transa, char transb, char uplo, int m, int n, int k, double alpha,
               const double* A, int lda, const double* B, int ldb, double beta, double* C, int ldc,
               int engine);
