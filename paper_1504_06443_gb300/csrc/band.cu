@@ -1447,7 +1447,11 @@ __global__ void __launch_bounds__(256) k_q2_tile_build(int b, int Q, const doubl
   double* Ut = U + (size_t)blockIdx.x * W * W;  // U - I, W x W column-major
   for (int idx = t; idx < W * TB_COLS; idx += blockDim.x) {
     int r = idx % W, cc = idx / W;
-    if (c0 + cc < W) Ut[r + (size_t)(c0 + cc) * W] = (double)(Us[r * TB_LD + cc] - (r == c0 + cc ? ONE : 0)) * 0x1p-62;
+    if (c0 + cc >= W) continue;
+    // (on the diagonal of a tile with reflections U may be -1 and a rounding: one less than -2^63 as an integer)
+    const ll u = Us[r * TB_LD + cc];
+    const bool dia = r == c0 + cc;
+    Ut[r + (size_t)(c0 + cc) * W] = dia && u < 0 ? (double)u * 0x1p-62 - 1.0 : (double)(u - (dia ? ONE : 0)) * 0x1p-62;
   }
 }
 

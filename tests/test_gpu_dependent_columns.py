@@ -69,3 +69,27 @@ def test_two_stage(gep, M, b, kind, clusters, rows):
     d, e, tau1, q2, Cr = gep.tridiag_2stage(C, b, handle=h)
     _check(C, gep.sep_backtransform_2stage(Cr, tau1, q2, b, torch.eye(M, dtype=torch.float64, device="cuda"), handle=h), d, e)
     h.close()
+
+
+@pytest.mark.parametrize("kind", ["ones", "falling", "rank_two", "signs"])
+@pytest.mark.parametrize("M,b", [(30, 2), (130, 2), (257, 5), (400, 16), (400, 32), (700, 64)])
+def test_tiles_of_reflections(gep, M, b, kind):
+    """Reflectors whose tails vanish beside their first entry are reflections (-1 on the diagonal of a tile of Q2)."""
+    import torch
+    i = torch.arange(M, device="cuda", dtype=torch.float64)
+    if kind == "falling":
+        g = torch.Generator(device="cuda").manual_seed(M)
+        G = torch.randn(M, M, generator=g, dtype=torch.float64, device="cuda")
+        C = (G + G.t()) * torch.exp(-0.2 * (i[:, None] + i[None, :]))
+    elif kind == "signs":  # a band of one subdiagonal and, b below the diagonal, entries beside which the others vanish
+        C = torch.diag(torch.cos(i)) + 0.5 * torch.diag(torch.ones(M - 1, dtype=torch.float64, device="cuda"), -1)
+        C = C + torch.diag(1e-14 * torch.ones(M - b, dtype=torch.float64, device="cuda"), -b)
+        C = C.tril() + C.tril(-1).t()
+    else:
+        C = _matrix(kind, M)
+    eye = torch.eye(M, dtype=torch.float64, device="cuda")
+    w, Y, info = gep.solve(C, eye, sep="2stage", bandwidth=b, precision="fp64_emulated")
+    assert info == 0
+    n = float(torch.linalg.matrix_norm(C, 2))
+    assert float((Y.t() @ Y - eye).abs().max()) <= 200 * M * EPS
+    assert float((C @ Y - Y * w).abs().max()) <= 200 * M * EPS * n
