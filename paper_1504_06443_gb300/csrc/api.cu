@@ -195,13 +195,15 @@ int sep_solve_scaled(gep_handle_t h, int M, double* C, int ldc, const gep_option
   return backtransform_q(h, M, n, C, ldc, tvec, Z, ldz, (double*)uni, uni_bytes / sizeof(double), eng);
 }
 
-// The SEP solver on C times the power of two that brings its largest entry into [1, 2), for the tensor-core engines:
-// their products take a row [W V] of a rank-2b update as one operand, whose digits are relative to its largest
-// entry.  With W of C's size and V of order one, V would lose as many bits as C's norm is away from one.
+// The SEP solver on C times the power of two that brings its largest entry into [1, 2).  On the tensor-core engines
+// the products take a row [W V] of a rank-2b update as one operand, whose digits are relative to its largest
+// entry: with W of C's size and V of order one, V would lose as many bits as C's norm is away from one.  On the
+// FP64 engine the kernels that sum plain squares (all but the cluster's, which scales for itself) would over- or
+// underflow from 2^+-500 on.
 int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, double* dvec, double* evec,
               double* tvec, double* q2, char* uni, size_t uni_bytes, int eng, double* w, double* Z, int ldz,
               bool timed, int n = 0, double* Zt = nullptr, double* wt = nullptr, double* q2u = nullptr) {
-  const bool scaled = eng != GEP_PREC_FP64 && !jacobi(o);
+  const bool scaled = !jacobi(o) && (eng != GEP_PREC_FP64 || two_stage(o) || M > 512);
   int* ex = h->d_status + STATUS_EXPONENTS + 2;
   if (scaled) {
     GEP_CUDA(cudaMemsetAsync(ex, 0, sizeof(int), h->stream));

@@ -63,3 +63,22 @@ def test_scaled_values_lowest_and_overwritten(gep, pencils, pa, sep):
     assert float((A @ Y - B @ Y * (w * 2.0 ** -pa)).norm() / (A.norm() * 700)) <= 1e-13
     w, Y, info = gep.solve(A * 2.0 ** pa, B.clone(), sep=sep, precision="fp64_emulated", overwrite=True)
     assert info == 0 and float((w * 2.0 ** -pa - ref).abs().max()) <= 1e-11 * n
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp64_emulated"])
+@pytest.mark.parametrize("sep,b", [("1stage", 0), ("2stage", 0), ("2stage", 48), ("2stage", 64)])
+@pytest.mark.parametrize("M", [300, 700])
+@pytest.mark.parametrize("p", [-660, 660])
+def test_squares_beyond_the_range(gep, pencils, M, p, sep, b, precision):
+    """Norms whose squares over- or underflow, with B = I."""
+    import torch
+    A = pencils[M][0]
+    ref = torch.linalg.eigvalsh(A.cpu()).cuda()
+    eye = torch.eye(M, dtype=torch.float64, device="cuda")
+    n = float(ref.abs().max())
+    w, Y, info = gep.solve(A * 2.0 ** p, eye, sep=sep, bandwidth=b, precision=precision)
+    assert info == 0
+    assert float((w * 2.0 ** -p - ref).abs().max()) <= 1e-11 * n
+    assert float((Y.t() @ Y - eye).abs().max()) <= 1e-12
+    assert float((gep.solve(A * 2.0 ** p, eye, sep=sep, bandwidth=b, precision=precision, want_vectors=False)[0] * 2.0 ** -p
+                  - ref).abs().max()) <= 1e-11 * n
