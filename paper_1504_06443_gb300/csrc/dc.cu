@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(32) k_leaf(int M, const double* __restrict__ d
   const double sc = pow2(sh), isc = pow2(-sh);
   if (lane < LEAF) {
     dl[lane] = dv * sc;
-    el[lane] = ev * sc;
+    el[lane] = fabs(ev * sc) < 0x1p-900 ? 0.0 : ev * sc;  // (a rotation of subnormal numbers is not orthogonal)
   }
 #pragma unroll
   for (int c = 0; c < LEAF; ++c) Zs[c][lane] = (lane == c) ? 1.0 : 0.0;
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(1024) k_prep(int M, int half, const double* __
   // The merge runs on numbers of order one: scaled by the power of two that brings those the rank-one term
   // reaches into [1, 2) (values of a decoupled block of another scale only pass through).
   const int top = field(fmax(dmax, fabs(beta)));
-  const int sh = max(-1000, min(top ? 1023 - top : 0, min(1000, 2000 - field(dall))));
+  const int sh = max(-1000, min(top ? 1023 - top : 1000, min(1000, 2000 - field(dall))));  // (top 0: subnormal)
   const double f = pow2(sh);
   const double rho = 2.0 * (fabs(beta) * f);
   for (int t = tid; t < n; t += nt) w.dv[t] *= f;

@@ -93,3 +93,29 @@ def test_not_a_number_is_a_failure(gep, M, where, bad):
         h = gep.Handle()
         assert gep.tridiag_eig(x.cuda(), y.cuda(), handle=h)[2] > M
         h.close()
+
+
+@pytest.mark.parametrize("M", [9, 40, 300])
+@pytest.mark.parametrize("ordinary", [False, True])
+def test_subnormal_numbers(gep, M, ordinary):
+    """A matrix (or a decoupled block) of subnormal numbers, whose reciprocals overflow."""
+    import torch
+    g = torch.Generator().manual_seed(M)
+    d = torch.randint(-40, 41, (M,), generator=g).double()
+    e = torch.randint(1, 30, (M - 1,), generator=g).double()
+    ds, es = d * 2.0 ** -1000 * 2.0 ** -74, e * 2.0 ** -1000 * 2.0 ** -74
+    if ordinary:
+        d1, e1 = _tridiagonal(30, 1)
+        ds, es = torch.cat([d1, ds]), torch.cat([e1, torch.zeros(1, dtype=torch.float64), es])
+    w, Z, info = gep.tridiag_eig(ds.cuda(), es.cuda())
+    assert info == 0
+    w, Z = w.cpu(), Z.cpu()
+    N = len(ds)
+    assert float((Z.t() @ Z - torch.eye(N, dtype=torch.float64)).abs().max()) <= 200 * N * EPS
+    if ordinary:  # (couplings below 2^-900 of their leaf's largest entry count as zero)
+        ref = torch.sort(torch.cat([torch.linalg.eigvalsh(_dense(d1, e1)), torch.zeros(M, dtype=torch.float64)]))[0]
+        assert float((w - ref).abs().max()) <= 200 * N * EPS * float(ref.abs().max())
+        return
+    ref = torch.linalg.eigvalsh(_dense(d, e))
+    got = w * 2.0 ** 1000 * 2.0 ** 74  # every level rounds to whole units
+    assert float((got - ref).abs().max()) <= 8.0
