@@ -195,19 +195,19 @@ int sep_solve_scaled(gep_handle_t h, int M, double* C, int ldc, const gep_option
   return backtransform_q(h, M, n, C, ldc, tvec, Z, ldz, (double*)uni, uni_bytes / sizeof(double), eng);
 }
 
-// The SEP solver on C times the power of two that brings its largest entry into [1, 2).  On the tensor-core engines
-// the products take a row [W V] of a rank-2b update as one operand, whose digits are relative to its largest
-// entry: with W of C's size and V of order one, V would lose as many bits as C's norm is away from one.  On the
-// FP64 engine the kernels that sum plain squares (all but the cluster's, which scales for itself) would over- or
-// underflow from 2^+-500 on.
+// The SEP solver on C times the power of two that brings its root mean square eigenvalue to one.  On the tensor-core
+// engines the products take a row [W V] of a rank-2b update as one operand, whose digits are relative to its largest
+// entry: with W of C's size and V of order one, V would lose as many bits as C's norm is above one.  The largest
+// entry does not serve as the norm: in a dense matrix it is sqrt(M) / 4 below it (order 8192, eigenvectors off by
+// 1.55e-12 with the largest entry brought to one, 1.02e-12 unscaled, 7.9e-13 so).  On the FP64 engine the kernels
+// that sum plain squares (all but the cluster's, which scales for itself) would over- or underflow from 2^+-500 on.
 int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, double* dvec, double* evec,
               double* tvec, double* q2, char* uni, size_t uni_bytes, int eng, double* w, double* Z, int ldz,
               bool timed, int n = 0, double* Zt = nullptr, double* wt = nullptr, double* q2u = nullptr) {
   const bool scaled = !jacobi(o) && (eng != GEP_PREC_FP64 || two_stage(o) || M > 512);
   int* ex = h->d_status + STATUS_EXPONENTS + 2;
   if (scaled) {
-    GEP_CUDA(cudaMemsetAsync(ex, 0, sizeof(int), h->stream));
-    GEP_CHECK(max_exponent(h, M, C, ldc, ex));
+    GEP_CHECK(norm_exponent(h, M, C, ldc, ex));
     GEP_CHECK(scale_pow2(h, M, M, C, ldc, C, ldc, nullptr, ex));
   }
   GEP_CHECK(sep_solve_scaled(h, M, C, ldc, o, dvec, evec, tvec, q2, uni, uni_bytes, eng, w, Z, ldz, timed, n, Zt, wt, q2u));

@@ -35,6 +35,41 @@ __global__ void __launch_bounds__(256) k_max_exponent(int M, const double* __res
   if ((threadIdx.x & 31) == 0 && m) atomicMax(ex, m);
 }
 
+// Sum of the squares of the symmetric matrix in the lower triangle, in units of 2^-26 of the square of the largest
+// entry's power of two (*ex its exponent field), from the leading 14 bits of every entry: integers, so that the
+// sum does not depend on the order.
+__global__ void __launch_bounds__(256) k_sum_squares(int M, const double* __restrict__ A, int lda, const int* __restrict__ ex,
+                                                     unsigned long long* __restrict__ sum, const int* st) {
+  __shared__ unsigned long long part[8];
+  if (status_bad(st)) return;
+  const int E = *ex;
+  unsigned long long s = 0;
+  for (int j = blockIdx.x; j < M; j += gridDim.x) {
+#pragma unroll 4
+    for (int i = j + threadIdx.x; i < M; i += 256) {
+      const unsigned hi = (unsigned)__double2hiint(A[GEP_IX(i, j, lda)]);
+      const int e = (int)((hi >> 20) & 0x7FF), d = E - e;
+      const unsigned m = (1u << 13) | ((hi & 0xFFFFF) >> 7);
+      if (e && d < 14) s += (unsigned long long)((m * m) >> (2 * d)) << (i != j);
+    }
+  }
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < 8; ++q) s += part[q];
+    if (s) atomicAdd(sum, s);
+  }
+}
+
+// *ex := exponent field of the power of two nearest to the root mean square eigenvalue, ||A||_F / sqrt(M).
+__global__ void k_norm_exponent(int M, const int* __restrict__ top, const unsigned long long* __restrict__ sum,
+                                int* __restrict__ ex, const int* st) {
+  if (status_bad(st)) return;
+  const int h = *sum ? (int)rint(0.5 * log2((double)*sum * 0x1p-26 / M)) : 0;
+  *ex = *top ? min(max(*top + h, 1), 2046) : 0;
+}
+
 // The lower triangle (cols = 1: a vector) times 2^(*up - *down) (nothing where one of them is zero); in place or not.
 __global__ void k_scale_pow2(int m, int cols, const double* s, int lds, double* d, int ldd, const int* up,
                              const int* down, const int* st) {
@@ -177,6 +212,18 @@ int copy_lower(gep_handle_t h, int M, const double* src, int lds, double* dst, i
 int max_exponent(gep_handle_t h, int M, const double* A, int lda, int* ex) {
   if (M <= 0) return GEP_OK;
   k_max_exponent<<<M < 4 * h->sm_count ? M : 4 * h->sm_count, 256, 0, h->stream>>>(M, A, lda, ex, h->d_status);
+  return check_launch(h);
+}
+
+int norm_exponent(gep_handle_t h, int M, const double* A, int lda, int* ex) {
+  if (M <= 0) return GEP_OK;
+  int* top = h->d_status + STATUS_SCRATCH;
+  unsigned long long* sum = reinterpret_cast<unsigned long long*>(top + 2);
+  GEP_CUDA(cudaMemsetAsync(top, 0, 16, h->stream));
+  GEP_CHECK(max_exponent(h, M, A, lda, top));
+  k_sum_squares<<<M < 4 * h->sm_count ? M : 4 * h->sm_count, 256, 0, h->stream>>>(M, A, lda, top, sum, h->d_status);
+  GEP_CHECK(check_launch(h));
+  k_norm_exponent<<<1, 1, 0, h->stream>>>(M, top, sum, ex, h->d_status);
   return check_launch(h);
 }
 
