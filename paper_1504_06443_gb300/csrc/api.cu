@@ -195,12 +195,14 @@ int sep_solve_scaled(gep_handle_t h, int M, double* C, int ldc, const gep_option
   return backtransform_q(h, M, n, C, ldc, tvec, Z, ldz, (double*)uni, uni_bytes / sizeof(double), eng);
 }
 
-// The SEP solver on C times the power of two that brings its root mean square eigenvalue to one.  On the tensor-core
+// The SEP solver on C times the power of two that brings its root mean square eigenvalue to two.  On the tensor-core
 // engines the products take a row [W V] of a rank-2b update as one operand, whose digits are relative to its largest
 // entry: with W of C's size and V of order one, V would lose as many bits as C's norm is above one.  The largest
 // entry does not serve as the norm: in a dense matrix it is sqrt(M) / 4 below it (order 8192, eigenvectors off by
-// 1.55e-12 with the largest entry brought to one, 1.02e-12 unscaled, 7.9e-13 so).  On the FP64 engine the kernels
-// that sum plain squares (all but the cluster's, which scales for itself) would over- or underflow from 2^+-500 on.
+// 1.55e-12 with the largest entry brought to one, 1.02e-12 unscaled, 7.8e-13 so).  From 0.7 to 2.8 the errors are
+// flat (order 2047: 2.14e-13, 2.03e-13 and 2.01e-13 at 0.7, 1.4 and 2.8), beyond they grow both ways.  On the FP64
+// engine the kernels that sum plain squares (all but the cluster's, which scales for itself) would over- or
+// underflow from 2^+-500 on.
 int sep_solve(gep_handle_t h, int M, double* C, int ldc, const gep_options* o, double* dvec, double* evec,
               double* tvec, double* q2, char* uni, size_t uni_bytes, int eng, double* w, double* Z, int ldz,
               bool timed, int n = 0, double* Zt = nullptr, double* wt = nullptr, double* q2u = nullptr) {

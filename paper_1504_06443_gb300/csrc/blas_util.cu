@@ -62,11 +62,11 @@ __global__ void __launch_bounds__(256) k_sum_squares(int M, const double* __rest
   }
 }
 
-// *ex := exponent field of the power of two nearest to the root mean square eigenvalue, ||A||_F / sqrt(M).
+// *ex := exponent field of the power of two nearest to half of the root mean square eigenvalue, ||A||_F / sqrt(M).
 __global__ void k_norm_exponent(int M, const int* __restrict__ top, const unsigned long long* __restrict__ sum,
                                 int* __restrict__ ex, const int* st) {
   if (status_bad(st)) return;
-  const int h = *sum ? (int)rint(0.5 * log2((double)*sum * 0x1p-26 / M)) : 0;
+  const int h = *sum ? (int)rint(0.5 * log2((double)*sum * 0x1p-26 / M)) - 1 : 0;
   *ex = *top ? min(max(*top + h, 1), 2046) : 0;
 }
 

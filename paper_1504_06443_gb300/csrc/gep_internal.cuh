@@ -204,7 +204,7 @@ int copy_lower(gep_handle_t h, int M, const double* src, int lds, double* dst, i
 int set_matrix(gep_handle_t h, int m, int n, double offdiag, double diag, double* A, int lda);
 // *ex (zero on entry) := largest exponent field of the lower triangle of A
 int max_exponent(gep_handle_t h, int M, const double* A, int lda, int* ex);
-// *ex := exponent field of the power of two nearest to ||A||_F / sqrt(M) (0 for a zero matrix), A symmetric, lower
+// *ex := exponent field of the power of two nearest to ||A||_F / (2 sqrt(M)) (0 for a zero matrix), A symmetric, lower
 int norm_exponent(gep_handle_t h, int M, const double* A, int lda, int* ex);
 // lower triangle (cols = m) or vector (cols = 1): dst = src 2^(*up - *down), device exponent fields, null: that of 1
 int scale_pow2(gep_handle_t h, int m, int cols, const double* src, int lds, double* dst, int ldd, const int* up,
